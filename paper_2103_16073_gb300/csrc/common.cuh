@@ -245,15 +245,42 @@ struct RcrTask {
                          // 5: staged with tensor-core rotations and coaxial step
     int32_t pad;
 };
-struct RcrTile {
-    int32_t task, col0, nb, pad;
+// One class of tile columns (rcr_tiles.cu): slots [slot0, slot0 + nslot),
+// polar-angle group g, coaxial tables at coax_off (complex entries of the
+// tile kernel's tables), built for order pc.
+struct RcrClass {
+    int32_t slot0, nslot, p_in, p_out;
+    int32_t g, pc;
+    int64_t coax_off;
 };
-// Tiles of an RCR plan for a number of right-hand sides: the columns of a
-// task are its (pair, rhs) combinations, pair-major.
+// columns [col0, col0 + ncol) of a class, 2^lcw per tile at most
+struct RcrColTile {
+    int32_t cls, col0, ncol, lcw;
+};
+namespace stg {
+struct StgSlot;
+}
+// Classes and slots of a plan's tiles, and the tiles per number of
+// right-hand sides (a class's columns are its (slot, rhs) combinations,
+// slot-major; the sets for more than one are built on first use).
 struct RcrTileSet {
-    RcrTile* tiles = nullptr;
-    int ntiles = 0;
-    size_t smem = 0;
+    struct Tiles {
+        RcrColTile* tiles = nullptr;      // three launches: one, two, three CTAs per SM
+        int ntiles[3] = {0, 0, 0};
+        size_t smem[3] = {0, 0, 0};
+    };
+    std::vector<RcrClass> h_cls;
+    RcrClass* cls = nullptr;
+    stg::StgSlot* slots = nullptr;
+    std::map<int, Tiles> tiles;
+};
+// Tables of the tile kernel in one arithmetic type, orders <= P.
+struct RcrTables {
+    void* rot = nullptr;                  // per polar-angle group: rotation, back-rotation
+    void* coax = nullptr;
+    int64_t per = 0;                      // entries of one rotation table
+    int P = 0;
+    std::map<int64_t, int64_t> coax_at;   // coaxial set -> offset in `coax`
 };
 // Large orders run as staged batched GEMM passes (rcr_staged.cu) instead of
 // per-pair tiles: a pair's rotation and coaxial blocks must then be shared
@@ -266,19 +293,12 @@ bool fb_rcr_tile_fits(int p_in, int p_out, size_t csize);
 int fb_rcr_default_staged(int p_in, int p_out, size_t csize);
 struct RcrPlan {
     std::vector<RcrTask> h_tasks;
-    std::vector<RcrTile> h_tiles;
-    RcrTask* tasks = nullptr;
-    RcrTile* tiles = nullptr;
     const int32_t* src_idx = nullptr;
     const int32_t* dst_idx = nullptr;
-    int ntiles = 0;
-    int nb = 1;          // box pairs per CTA
-    size_t smem = 0;     // dynamic shared memory per CTA (bytes)
     size_t csize = 0;    // bytes per complex coefficient
     void* stg = nullptr;        // staged passes of the large-order tasks
     int64_t stg_elems = 0;      // staging coefficients they need per buffer
-    std::map<int, RcrTileSet> multi;   // tiles for nrhs > 1 (built on first use), key 2 nrhs + df
-    RcrTileSet df_tiles;        // tiles of the double-FP32 tasks (one right-hand side)
+    RcrTileSet tiles, df_tiles;   // tiles in the operator's precision / in double-FP32
 };
 void fb_rcr_free(RcrPlan& p);
 bool fb_stg_staged(const RcrTask& tk);
@@ -314,7 +334,6 @@ void fb_stg_level_info(const void* plan, int li, int64_t* src_base, int64_t* dst
 struct fb_op;
 fb_status fb_stg_op_pass_times(fb_op* op, cudaStream_t s, double* ms, int* form);
 fb_status fb_stg_df_tables(fb_op* op, cudaStream_t s);
-fb_status fb_rcr_df_factors(fb_op* op, int P);
 fb_status fb_near_bf16(fb_op* op, int enable, cudaStream_t s);
 // Creates an operator; `donor` (an FP64 FMM operator of the same mesh, tree,
 // k and kind, or NULL) lends its near-field entries.
@@ -402,9 +421,9 @@ struct fb_op {
     int near16 = 0;                          // 1: the matvec reads nf16 instead of nf32
     df* rotf_df = nullptr;                   // FP64 operators: folded tables and coaxial sets in
     cx<df>* coax_df = nullptr;               // double-FP32 for the staged levels that use it
-    df* rotd_df = nullptr;                   // ... and the real factors of degrees < rotd_df_P
-    int rotd_df_P = 0;                       // (per-pair tiles in double-FP32)
-    int64_t rotd_df_per = 0;                 // values per direction
+    RcrTables rcr_tab, rcr_df;               // tables of the tile kernel (operator's precision, double-FP32)
+    uint32_t* rcr_lut = nullptr;             // its (n, m) index table
+    std::vector<std::pair<int, int64_t>> coax_sets;   // (order, offset in coax64) of every coaxial set, ascending
     std::vector<int> dir_of_code;            // M2L offset code -> direction (-1: near)
     // RCR form per level: 1 = staged passes, 0 = per-pair tiles (M2L of
     // level l; M2M and L2L between levels l-1 and l)
@@ -489,6 +508,13 @@ fb_status fb_fmm_create(fb_op* op, double d0, int pmin, cudaStream_t s);
 fb_status fb_fmm_apply(fb_op* op, const cd* x, cd* y, cudaStream_t s, PhaseTimer* pt = nullptr,
                        int nrhs = 1);
 fb_status fb_fmm_apply_noalloc(fb_op* op, const cd* x, cd* y, cudaStream_t s);
+// Tiles of a plan (rcr_tiles.cu): built from its tasks, run, freed.
+fb_status fb_rcr_tiles_build(fb_op* op, RcrPlan& pl, bool want_df);
+fb_status fb_rcr_tiles_run_f(const fb_op* op, RcrPlan& pl, const cf* src, cf* dst, cudaStream_t s, int nrhs,
+                             int64_t rstride);
+fb_status fb_rcr_tiles_run_d(const fb_op* op, RcrPlan& pl, const cd* src, cd* dst, cudaStream_t s, int nrhs,
+                             int64_t rstride);
+void fb_rcr_tiles_free(RcrTileSet& t);
 fb_status fb_rcr_upload(fb_op* op, RcrPlan& pl, const int32_t* src, const int32_t* dst, size_t csize);
 fb_status fb_tree_rotations(fb_tree* t, int P, const std::vector<double>& dirs, cudaStream_t s,
                             const fb_tree::RotSet** out);

@@ -207,398 +207,11 @@ __global__ void k_near_l2p(int P, const int32_t* __restrict__ leaf_start, const 
 }
 
 
-// ------------------------------------------------------- RCR translation ----
-// Rotation - coaxial translation - back-rotation (Sec. 3.3) applied per box
-// pair: for a group of pairs sharing one translation vector (one direction,
-// one |t|) each CTA takes nb pairs.  The rotations run folded by the
-// symmetry of the real factors, d^n_{-mu,-m} = d^n_{mu,m}: with the phased
-// input x_m = e^{i m phi} src_m and s_m = x_m + x_{-m}, t_m = x_m - x_{-m}
-// (m > 0), s_0 = x_0,
-//   E_mu = u_mu + u_{-mu} = 2 d_{mu,0} s_0 + sum_{m>0} (d_{mu,m} + d_{mu,-m}) s_m   (mu = 0..n)
-//   O_mu = u_mu - u_{-mu} =                  sum_{m>0} (d_{mu,m} - d_{mu,-m}) t_m   (mu = 1..n)
-// (half the multiplications of u = d x); the coaxial blocks, which depend
-// on |m| only, map E to E and O to O; the back-rotation folds the same way,
-//   Y+_{m'} = y_{m'} + y_{-m'} = d_{0,m'} E_0 + sum_{mu>0} (d_{mu,m'} + d_{-mu,m'}) E_mu
-//   Y-_{m'} = y_{m'} - y_{-m'} =               sum_{mu>0} (d_{mu,m'} - d_{-mu,m'}) O_mu
-// and y_{+-m'} = (Y+ +- Y-)/2, e^{-+ i m' phi} applied, scatter-added into the
-// target (atomic adds: the groups of one launch may share targets).  Folded
-// layout of degree n within a vector: [0..n] even part, [n+1..2n] odd part.
-__device__ __forceinline__ void nm_of(int e, int& n, int& m) {
-    n = (int)sqrtf((float)e);
-    while (n * n > e) --n;
-    while ((n + 1) * (n + 1) <= e) ++n;
-    m = e - n * n - n;
-}
-// (n, j) of a folded degree-major index e = n^2 + j, j in [0, 2n]
-__device__ __forceinline__ void nj_of(int e, int& n, int& j) {
-    nm_of(e, n, j);
-    j += n;
-}
-// pair index e -> (n1, m') for m' = 0..n1 (e = n1 (n1 + 1) / 2 + m')
-__device__ __forceinline__ void tri_of(int e, int& n, int& m) {
-    n = (int)((sqrtf(8.0f * (float)e + 1.0f) - 1.0f) * 0.5f);
-    while (n * (n + 1) / 2 > e) --n;
-    while ((n + 1) * (n + 2) / 2 <= e) ++n;
-    m = e - n * (n + 1) / 2;
-}
-
-// Each thread owns one (folded) coefficient and computes it for a chunk of W
-// pairs at once, so every rotation / coaxial entry it loads is used W times
-// from registers; the pair operands come from shared memory, where the
-// threads of a warp that share a degree read the same word (broadcast).
-// Full chunks use W = RcrChunk, the remainder of a tile one pair at a time.
-template <class R> struct RcrChunk { static constexpr int value = 8; };
-template <> struct RcrChunk<double> { static constexpr int value = 4; };
-template <> struct RcrChunk<df> { static constexpr int value = 4; };
-// CTAs per SM the register budget must allow: FP64 tiles (48 KB of shared
-// memory each) are latency bound and want four resident CTAs, FP32 tiles
-// (96 KB) fit two.
-template <class R> struct RcrMinBlocks { static constexpr int value = 2; };
-template <> struct RcrMinBlocks<double> { static constexpr int value = 4; };
-template <> struct RcrMinBlocks<df> { static constexpr int value = 4; };
-
-// acc += a x for real a
-template <class R>
-__device__ __forceinline__ void rmac(cx<R>& acc, R a, const cx<R>& x) {
-    acc.re = fma(a, x.re, acc.re);
-    acc.im = fma(a, x.im, acc.im);
-}
-
-// folded rotation of degree n, output j (E_j for j <= n, O_{j-n} otherwise);
-// Dc points at d_{0,0} of the degree-n block (row stride w = 2n + 1)
-template <int W, class R>
-__device__ __forceinline__ void rcr_rotate(const R* Dc, int n, int j, const cx<R>* xs, int Pin, int b0, int e,
-                                           cx<R>* us) {
-    cx<R> acc[W];
-#pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = mk<R>(0, 0);
-    const int w = 2 * n + 1;
-    const cx<R>* xb = xs + b0 * Pin + n * n;
-    if (j <= n) {
-        const R* row = Dc + (int64_t)j * w;
-        {
-            const R a = R(2) * row[0];
-#pragma unroll
-            for (int q = 0; q < W; ++q) rmac(acc[q], a, xb[q * Pin]);
-        }
-#pragma unroll 4
-        for (int m = 1; m <= n; ++m) {
-            const R a = row[m] + row[-m];
-#pragma unroll
-            for (int q = 0; q < W; ++q) rmac(acc[q], a, xb[q * Pin + m]);
-        }
-    } else {
-        const R* row = Dc + (int64_t)(j - n) * w;
-#pragma unroll 4
-        for (int m = 1; m <= n; ++m) {
-            const R a = row[m] - row[-m];
-#pragma unroll
-            for (int q = 0; q < W; ++q) rmac(acc[q], a, xb[q * Pin + n + m]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < W; ++q) us[(b0 + q) * Pin + e] = acc[q];
-}
-
-// coaxial step on folded data: output (n1, j1) of order am (even or odd part)
-// input of degree n at n^2 + withn * n + a: folded even part (withn = 0,
-// a = am), folded odd part (1, am), or unfolded order mu (1, mu)
-template <int W, class R>
-__device__ __forceinline__ void rcr_coax(const cx<R>* Cr, int am, int withn, int a, int pmid, const cx<R>* us,
-                                         int Pin, int Pout, int b0, int e, cx<R>* vs) {
-    cx<R> acc[W];
-#pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = mk<R>(0, 0);
-    const cx<R>* ub = us + b0 * Pin;
-#pragma unroll 4
-    for (int n = am; n < pmid; ++n) {
-        cx<R> c = Cr[n];
-        int o = n * n + withn * n + a;
-#pragma unroll
-        for (int q = 0; q < W; ++q) cmac(acc[q], c, ub[q * Pin + o]);
-    }
-#pragma unroll
-    for (int q = 0; q < W; ++q) vs[(b0 + q) * Pout + e] = acc[q];
-}
-
-// folded back-rotation of degree n1 for the output pair +-m' (m' >= 0),
-// inner range |mu| <= mmax; Dc at d_{0,0} of the degree-n1 block
-template <int W, class R>
-__device__ __forceinline__ void rcr_back(const R* Dc, int n1, int mp, int mmax, cx<R> ph, const cx<R>* vs,
-                                         int Pout, int b0, const int64_t* dsto, cx<R>* dst) {
-    cx<R> yp[W], ym[W];
-#pragma unroll
-    for (int q = 0; q < W; ++q) {
-        yp[q] = mk<R>(0, 0);
-        ym[q] = mk<R>(0, 0);
-    }
-    const int w = 2 * n1 + 1;
-    const cx<R>* vb = vs + b0 * Pout + n1 * n1;
-    {
-        const R a = Dc[mp];
-#pragma unroll
-        for (int q = 0; q < W; ++q) rmac(yp[q], a, vb[q * Pout]);
-    }
-#pragma unroll 4
-    for (int mu = 1; mu <= mmax; ++mu) {
-        const R dp = Dc[(int64_t)mu * w + mp], dm = Dc[-(int64_t)mu * w + mp];
-        const R ap = dp + dm, am = dp - dm;
-#pragma unroll
-        for (int q = 0; q < W; ++q) {
-            rmac(yp[q], ap, vb[q * Pout + mu]);
-            rmac(ym[q], am, vb[q * Pout + n1 + mu]);
-        }
-    }
-#pragma unroll
-    for (int q = 0; q < W; ++q) {
-        cx<R>* d = dst + dsto[b0 + q] + n1 * n1 + n1;
-        if (mp == 0) {
-            const cx<R> y = R(0.5) * yp[q];
-            atomicAdd(&d->re, y.re);
-            atomicAdd(&d->im, y.im);
-        } else {
-            const cx<R> y1 = (R(0.5) * (yp[q] + ym[q])) * conjg(ph);
-            const cx<R> y2 = (R(0.5) * (yp[q] - ym[q])) * ph;
-            atomicAdd(&d[mp].re, y1.re);
-            atomicAdd(&d[mp].im, y1.im);
-            atomicAdd(&d[-mp].re, y2.re);
-            atomicAdd(&d[-mp].im, y2.im);
-        }
-    }
-}
-
-// Unfolded forms (u = d x over all m, each output m' on its own), used by the
-// FP64 tiles: they are bound by FP64 latency rather than multiplies, and the
-// folded form's wider per-thread state costs them more than it saves.
-template <int W, class R>
-__device__ __forceinline__ void rcr_rotate_full(const R* dn, int n, const cx<R>* xs, int Pin, int b0, int e,
-                                                cx<R>* us) {
-    cx<R> acc[W];
-#pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = mk<R>(0, 0);
-    const cx<R>* xb = xs + b0 * Pin + n * n;
-#pragma unroll 4
-    for (int m = 0; m <= 2 * n; ++m) {
-        R d = dn[m];
-#pragma unroll
-        for (int q = 0; q < W; ++q) rmac(acc[q], d, xb[q * Pin + m]);
-    }
-#pragma unroll
-    for (int q = 0; q < W; ++q) us[(b0 + q) * Pin + e] = acc[q];
-}
-template <int W, class R, class O>
-__device__ __forceinline__ void rcr_back_full(const R* dn, int n1, cx<O> phc, const cx<R>* vs, int Pout, int b0,
-                                              int e, const int64_t* dsto, cx<O>* dst) {
-    cx<R> acc[W];
-#pragma unroll
-    for (int q = 0; q < W; ++q) acc[q] = mk<R>(0, 0);
-    int w = 2 * n1 + 1;
-    const cx<R>* vb = vs + b0 * Pout + n1 * n1;
-#pragma unroll 4
-    for (int mu = 0; mu < w; ++mu) {
-        R d = dn[(int64_t)mu * w];
-#pragma unroll
-        for (int q = 0; q < W; ++q) rmac(acc[q], d, vb[q * Pout + mu]);
-    }
-#pragma unroll
-    for (int q = 0; q < W; ++q) {
-        cx<O> y = cx_out<O, R>(acc[q]) * phc;
-        cx<O>* d = dst + dsto[b0 + q] + e;
-        atomicAdd(&d->re, y.re);
-        atomicAdd(&d->im, y.im);
-    }
-}
-
-// R: arithmetic and tables (rotd, coax), O: expansions and phases (R = O,
-// or R = double-FP32 on FP64 expansions); rot_stride: values per direction
-// in rotd.
-template <class R, class O>
-__global__ void __launch_bounds__(256, RcrMinBlocks<R>::value) k_rcr(const RcrTask* __restrict__ tasks, const RcrTile* __restrict__ tiles,
-                                             const R* __restrict__ rotd, const cx<O>* __restrict__ rph,
-                                             int64_t per_dir, int64_t rot_stride, int prot,
-                                             const cx<R>* __restrict__ coax,
-                                             const int32_t* __restrict__ src_idx,
-                                             const int32_t* __restrict__ dst_idx,
-                                             const cx<O>* __restrict__ src, cx<O>* __restrict__ dst,
-                                             int nrhs, int64_t rstride) {
-    constexpr int BCH = RcrChunk<R>::value;
-    constexpr bool kFold = sizeof(R) == 4;   // FP32: folded rotations; FP64, double-FP32: unfolded
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ int64_t s_dst_off[16];
-    RcrTile tl = tiles[blockIdx.x];
-    RcrTask tk = tasks[tl.task];
-    const int nb = tl.nb;
-    const int Pin = tk.p_in * tk.p_in, Pout = tk.p_out * tk.p_out;
-    const int pmid = tk.p_in;   // the rotated input keeps degrees n < p_in
-    cx<R>* buf = (cx<R>*)smem_raw;
-    cx<R>* xs = buf;                    // [nb][Pin] folded phased input, later reused for vs
-    cx<R>* us = buf + nb * max(Pin, Pout);   // [nb][Pin]
-    cx<R>* vs = buf;                    // [nb][Pout] (xs is dead after the rotation)
-    int tid = threadIdx.x, nth = blockDim.x;
-    // column b of the tile: pair (col0 + b) / nrhs, right-hand side (col0 + b) % nrhs
-    for (int b = tid; b < nb; b += nth) {
-        int col = tl.col0 + b;
-        int pr = col / nrhs, rh = col - pr * nrhs;
-        s_dst_off[b] = rh * rstride + tk.dst_base + (int64_t)dst_idx[tk.pair_off + pr] * Pout;
-    }
-    const int64_t dir = tk.rot_off / per_dir;
-    const cx<O>* ph = rph + dir * (2 * prot - 1) + (prot - 1);   // ph[m] = e^{i m phi}
-    for (int q = tid; q < nb * Pin; q += nth) {
-        int b = q / Pin, e = q % Pin;
-        int col = tl.col0 + b;
-        int pr = col / nrhs, rh = col - pr * nrhs;
-        int sb = src_idx[tk.pair_off + pr];
-        int n, j;
-        nj_of(e, n, j);
-        const cx<O>* x = src + rh * rstride + tk.src_base + (int64_t)sb * Pin + (int64_t)n * n + n;   // (n, 0)
-        cx<O> v;
-        if constexpr (!kFold) {
-            v = x[j - n] * ph[j - n];   // plain phased input, degree-major
-        } else if (j == 0) {
-            v = x[0];
-        } else {
-            const int m = j <= n ? j : j - n;
-            const cx<O> xp = x[m] * ph[m], xm = x[-m] * ph[-m];
-            v = j <= n ? xp + xm : xp - xm;
-        }
-        xs[q] = cx_to<R, O>(v);
-    }
-    __syncthreads();
-    const R* D = rotd + dir * rot_stride;
-    // chunk widths BCH, then 4, 2, 1 for the rest of the tile
-#define RCR_CHUNKS(CALL)                                              \
-    {                                                                 \
-        int b0 = 0;                                                   \
-        for (; b0 + BCH <= nb; b0 += BCH) CALL(BCH);                  \
-        if (BCH > 4 && b0 + 4 <= nb) { CALL(4); b0 += 4; }            \
-        if (b0 + 2 <= nb) { CALL(2); b0 += 2; }                       \
-        if (b0 < nb) CALL(1);                                         \
-    }
-    // rotation: folded E_j / O_{j-n}, or u_{n,mu} = sum_m d_{mu,m} x_m unfolded
-    for (int e = tid; e < Pin; e += nth) {
-        int n, j;
-        nj_of(e, n, j);
-        const R* Dc = D + (int64_t)n * (2 * n - 1) * (2 * n + 1) / 3 + (int64_t)n * (2 * n + 1) + n;
-        if constexpr (kFold) {
-#define RCR_ROT(W) rcr_rotate<(W)>(Dc, n, j, xs, Pin, b0, e, us)
-            RCR_CHUNKS(RCR_ROT)
-#undef RCR_ROT
-        } else {
-            const R* Dn = Dc + (int64_t)(j - n) * (2 * n + 1) - n;   // row mu = j - n
-#define RCR_ROT(W) rcr_rotate_full<(W)>(Dn, n, xs, Pin, b0, e, us)
-            RCR_CHUNKS(RCR_ROT)
-#undef RCR_ROT
-        }
-    }
-    __syncthreads();
-    // coaxial: v^{am}_{n'} = sum_n C^{am}_{n'n} u^{am}_n on the even and odd parts
-    const cx<R>* C = coax + tk.coax_off;
-    const int pc = tk.pc;
-    for (int e = tid; e < Pout; e += nth) {
-        int n1, j1;
-        nj_of(e, n1, j1);
-        // folded: even part of order j1 or odd part of order j1 - n1; unfolded:
-        // order mu = j1 - n1 at offset n^2 + n + mu
-        const bool odd = kFold && j1 > n1;
-        const int am = kFold ? (odd ? j1 - n1 : j1) : abs(j1 - n1);
-        const int withn = (kFold && !odd) ? 0 : 1;
-        const int a = kFold ? am : j1 - n1;
-        const cx<R>* Cr = C + ((int64_t)am * pc + n1) * pc;
-        const int hi = am < pmid ? pmid : am;   // empty sum when |mu| >= p_in
-#define RCR_COAX(W) rcr_coax<(W)>(Cr, am, withn, a, hi, us, Pin, Pout, b0, e, vs)
-        RCR_CHUNKS(RCR_COAX)
-#undef RCR_COAX
-    }
-    __syncthreads();
-    if constexpr (!kFold) {
-        // back-rotate: y_{n'}^{m'} = sum_mu d^{n'}_{mu,m'} v_{n'}^mu, e^{-i m' phi}, scatter-add
-        for (int e = tid; e < Pout; e += nth) {
-            int n1, m1;
-            nm_of(e, n1, m1);
-            const R* Dn = D + (int64_t)n1 * (2 * n1 - 1) * (2 * n1 + 1) / 3 + (m1 + n1);
-            const cx<O> phc = conjg(ph[m1]);
-#define RCR_BACK(W) rcr_back_full<(W)>(Dn, n1, phc, vs, Pout, b0, e, s_dst_off, dst)
-            RCR_CHUNKS(RCR_BACK)
-#undef RCR_BACK
-        }
-    } else {
-        // folded back-rotation of every pair +-m' of every degree n' < p_out, then scatter-add
-        const int npairs_out = tk.p_out * (tk.p_out + 1) / 2;
-        for (int e = tid; e < npairs_out; e += nth) {
-            int n1, mp;
-            tri_of(e, n1, mp);
-            const R* Dc = D + (int64_t)n1 * (2 * n1 - 1) * (2 * n1 + 1) / 3 + (int64_t)n1 * (2 * n1 + 1) + n1;
-            const int mmax = min(n1, pmid - 1);
-            const cx<R> phm = ph[mp];
-#define RCR_BACK(W) rcr_back<(W)>(Dc, n1, mp, mmax, phm, vs, Pout, b0, s_dst_off, dst)
-            RCR_CHUNKS(RCR_BACK)
-#undef RCR_BACK
-        }
-    }
-#undef RCR_CHUNKS
-}
-
-// Tiles of up to 16 columns per CTA within a shared-memory budget: 96 KB for
-// FP32 (two CTAs per SM; the columns of a tile reuse each rotation / coaxial
-// entry from registers, so larger tiles raise the arithmetic per load) and
-// 48 KB for FP64 (bound by the FP64 pipe, it wants more resident warps).
-// Tasks of large order are left to the staged passes (fb_stg_staged).
-// want_df: the tiles of the tasks in double-FP32 arithmetic (staged == 4),
-// else the others.
-static void rcr_make_tiles(const RcrPlan& pl, int nrhs, std::vector<RcrTile>& tiles, size_t& smem,
-                           bool want_df = false) {
-    const size_t budget = pl.csize == sizeof(cf) ? 96 * 1024 : 48 * 1024;
-    tiles.clear();
-    smem = 0;
-    for (int t = 0; t < (int)pl.h_tasks.size(); ++t) {
-        const RcrTask& tk = pl.h_tasks[t];
-        if (fb_stg_staged(tk) || (tk.staged == 4) != want_df) continue;
-        int64_t elems = (int64_t)tk.p_in * tk.p_in + std::max(tk.p_in * tk.p_in, tk.p_out * tk.p_out);
-        size_t per = (size_t)elems * pl.csize;
-        int nb = (int)std::max<size_t>(1, std::min<size_t>(16, budget / per));
-        int ncol = tk.npairs * nrhs;
-        for (int c = 0; c < ncol; c += nb) {
-            int k = std::min(nb, ncol - c);
-            tiles.push_back(RcrTile{t, c, k, 0});
-            smem = std::max(smem, per * k);
-        }
-    }
-}
-
-static fb_status rcr_tiles_for(RcrPlan& pl, int nrhs, RcrTileSet* out, bool want_df = false) {
-    if (nrhs == 1) {
-        if (want_df) {
-            *out = pl.df_tiles;
-            return FB_OK;
-        }
-        out->tiles = pl.tiles;
-        out->ntiles = pl.ntiles;
-        out->smem = pl.smem;
-        return FB_OK;
-    }
-    auto it = pl.multi.find(2 * nrhs + (want_df ? 1 : 0));
-    if (it == pl.multi.end()) {
-        std::vector<RcrTile> h;
-        RcrTileSet ts;
-        rcr_make_tiles(pl, nrhs, h, ts.smem, want_df);
-        ts.ntiles = (int)h.size();
-        if (!h.empty()) {
-            FB_CHECK(dalloc(&ts.tiles, h.size()));
-            FB_CUDA(cudaMemcpy(ts.tiles, h.data(), sizeof(RcrTile) * h.size(), cudaMemcpyHostToDevice));
-        }
-        it = pl.multi.emplace(2 * nrhs + (want_df ? 1 : 0), ts).first;
-    }
-    *out = it->second;
-    return FB_OK;
-}
-
-// Rotation data of an operator for the RCR kernels: real factors, phase
-// tables and their strides.
+// Data of an operator for the staged RCR passes: phase tables, staging
+// buffers, folded rotation tables.
 template <class R>
 struct RotArgs {
-    const R* d;
     const cx<R>* ph;
-    int64_t per_dir;
     int prot;
     cx<R>* U;   // staging buffers of the large-order passes
     cx<R>* V;
@@ -606,15 +219,11 @@ struct RotArgs {
     int64_t fper;
     StcTabs tc;       // tables of the tensor-core staged passes (single precision)
     DfTabs dft;       // tables of the double-FP32 staged passes (FP64 operators)
-    const df* d_df;   // real factors in double-FP32 (degrees < the tiles' largest order)
-    int64_t per_dir_df;
 };
 template <class R>
 static RotArgs<R> rot_args(const fb_op* op) {
     RotArgs<R> a;
-    a.d = (const R*)(sizeof(R) == 8 ? (const void*)op->rotd64 : (const void*)op->rotd32);
     a.ph = (const cx<R>*)(sizeof(R) == 8 ? (const void*)op->rph64 : (const void*)op->rph32);
-    a.per_dir = op->per_dir;
     a.prot = op->Prot;
     a.U = (cx<R>*)op->stg_u;
     a.V = (cx<R>*)op->stg_v;
@@ -622,8 +231,6 @@ static RotArgs<R> rot_args(const fb_op* op) {
     a.fper = op->rotf_per;
     a.tc = StcTabs{op->stc_tab, op->stc_off, op->stc_per, op->stc_err};
     a.dft = DfTabs{op->rotf_df, op->coax_df};
-    a.d_df = op->rotd_df;
-    a.per_dir_df = op->rotd_df_per;
     return a;
 }
 static fb_status stg_run(void* plan, const RotArgs<float>& r, const cf* coax, const cf* src, cf* dst,
@@ -694,61 +301,21 @@ fb_status fb_stg_op_pass_times(fb_op* op, cudaStream_t s, double* ms, int* tc) {
     return st;
 }
 
+// The tiles of a plan in the operator's precision (FP64: also those in double-FP32).
+static fb_status rcr_tiles_run(const fb_op* op, RcrPlan& pl, const cf* src, cf* dst, cudaStream_t s, int nrhs,
+                               int64_t rstride) {
+    return fb_rcr_tiles_run_f(op, pl, src, dst, s, nrhs, rstride);
+}
+static fb_status rcr_tiles_run(const fb_op* op, RcrPlan& pl, const cd* src, cd* dst, cudaStream_t s, int nrhs,
+                               int64_t rstride) {
+    return fb_rcr_tiles_run_d(op, pl, src, dst, s, nrhs, rstride);
+}
+
 template <class R>
-static fb_status run_rcr(RcrPlan& pl, const RotArgs<R>& rot, const cx<R>* coax, const cx<R>* src, cx<R>* dst,
-                         cudaStream_t s, int nrhs = 1, int64_t rstride = 0) {
-    RcrTileSet ts;
-    FB_CHECK(rcr_tiles_for(pl, nrhs, &ts));
-    if (ts.ntiles > 0) {
-        FB_CHECK(fb_smem_cap((const void*)k_rcr<R, R>, ts.smem));
-        k_rcr<R, R><<<ts.ntiles, 256, ts.smem, s>>>(pl.tasks, ts.tiles, rot.d, rot.ph, rot.per_dir, rot.per_dir,
-                                                    rot.prot, coax, pl.src_idx, pl.dst_idx, src, dst, nrhs, rstride);
-        FB_LAUNCH_CHECK();
-        fb_count_launch();
-    }
-    if constexpr (sizeof(R) == 8) {
-        // tiles in double-FP32 arithmetic on the FP64 expansions
-        FB_CHECK(rcr_tiles_for(pl, nrhs, &ts, true));
-        if (ts.ntiles > 0) {
-            if (!rot.d_df || !rot.dft.coax) return fb_fail(FB_ERR_STATE, "RCR tiles: double-FP32 tables missing");
-            FB_CHECK(fb_smem_cap((const void*)k_rcr<df, double>, ts.smem));
-            k_rcr<df, double><<<ts.ntiles, 256, ts.smem, s>>>(pl.tasks, ts.tiles, rot.d_df, rot.ph, rot.per_dir,
-                                                              rot.per_dir_df, rot.prot, rot.dft.coax, pl.src_idx,
-                                                              pl.dst_idx, src, dst, nrhs, rstride);
-            FB_LAUNCH_CHECK();
-            fb_count_launch();
-        }
-    }
+static fb_status run_rcr(const fb_op* op, RcrPlan& pl, const RotArgs<R>& rot, const cx<R>* coax, const cx<R>* src,
+                         cx<R>* dst, cudaStream_t s, int nrhs = 1, int64_t rstride = 0) {
+    FB_CHECK(rcr_tiles_run(op, pl, src, dst, s, nrhs, rstride));
     if (pl.stg) FB_CHECK(stg_run(pl.stg, rot, coax, src, dst, s, nrhs, rstride));
-    return FB_OK;
-}
-
-static __global__ void k_d_to_df(const double* __restrict__ in, int64_t per_in, int64_t per_out, int ndir,
-                                 df* __restrict__ out) {
-    const int64_t total = (int64_t)ndir * per_out;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t d = i / per_out, e = i - d * per_out;
-        out[i] = df_from(in[d * per_in + e]);
-    }
-}
-
-// Real rotation factors of every direction in double-FP32, degrees < P (the
-// largest order of the tiles that use them), rebuilt when a larger P is asked.
-fb_status fb_rcr_df_factors(fb_op* op, int P) {
-    if (op->rotd_df && op->rotd_df_P >= P) return FB_OK;
-    if (!op->rotd64 || P > op->Prot) return fb_fail(FB_ERR_STATE, "RCR tiles: no FP64 rotation factors");
-    const int ndir = (int)(op->rot_count / op->per_dir);
-    const int64_t per = (int64_t)P * (2 * P - 1) * (2 * P + 1) / 3;   // sum_{n<P} (2n+1)^2
-    FB_CUDA(cudaDeviceSynchronize());
-    dfree(op->rotd_df);
-    FB_CHECK(dalloc(&op->rotd_df, (size_t)ndir * per));
-    k_d_to_df<<<(unsigned)std::min<int64_t>(((int64_t)ndir * per + 255) / 256, 8192), 256>>>(op->rotd64, op->per_dir,
-                                                                                          per, ndir, op->rotd_df);
-    FB_CUDA(cudaDeviceSynchronize());
-    op->rotd_df_P = P;
-    op->rotd_df_per = per;
-    op->buf_gen++;   // captured graphs refer to the old factors
-    fb_count_launch();
     return FB_OK;
 }
 
@@ -770,29 +337,9 @@ fb_status fb_rcr_upload(fb_op* op, RcrPlan& pl, const int32_t* src, const int32_
     for (RcrTask& tk : pl.h_tasks)
         if ((tk.staged == 0 || tk.staged == 4) && !fb_rcr_tile_fits(tk.p_in, tk.p_out, csize))
             tk.staged = tk.staged == 4 ? 3 : 1;
-    rcr_make_tiles(pl, 1, pl.h_tiles, pl.smem);
-    pl.ntiles = (int)pl.h_tiles.size();
     if (pl.h_tasks.empty()) return FB_OK;
-    FB_CHECK(dalloc(&pl.tasks, pl.h_tasks.size()));
-    FB_CUDA(cudaMemcpy(pl.tasks, pl.h_tasks.data(), sizeof(RcrTask) * pl.h_tasks.size(), cudaMemcpyHostToDevice));
-    if (pl.ntiles) {
-        FB_CHECK(dalloc(&pl.tiles, pl.h_tiles.size()));
-        FB_CUDA(cudaMemcpy(pl.tiles, pl.h_tiles.data(), sizeof(RcrTile) * pl.h_tiles.size(), cudaMemcpyHostToDevice));
-    }
-    {
-        std::vector<RcrTile> h;
-        rcr_make_tiles(pl, 1, h, pl.df_tiles.smem, true);
-        pl.df_tiles.ntiles = (int)h.size();
-        if (!h.empty()) {
-            int pmax = 0;
-            for (const RcrTask& tk : pl.h_tasks)
-                if (tk.staged == 4) pmax = std::max(pmax, std::max(tk.p_in, tk.p_out));
-            FB_CHECK(fb_rcr_df_factors(op, pmax));
-            FB_CHECK(fb_stg_df_tables(op, cudaStreamLegacy));   // coaxial sets in double-FP32
-            FB_CHECK(dalloc(&pl.df_tiles.tiles, h.size()));
-            FB_CUDA(cudaMemcpy(pl.df_tiles.tiles, h.data(), sizeof(RcrTile) * h.size(), cudaMemcpyHostToDevice));
-        }
-    }
+    FB_CHECK(fb_rcr_tiles_build(op, pl, false));
+    FB_CHECK(fb_rcr_tiles_build(op, pl, true));
     FB_CHECK(fb_stg_build(pl, op->theta_slot, op->per_dir, op->coax64, &pl.stg, &pl.stg_elems));
     if (fb_stg_uses_tc(pl.stg)) FB_CHECK(fb_stc_tables(op, cudaStreamLegacy));
     if (fb_stg_uses_df(pl.stg)) FB_CHECK(fb_stg_df_tables(op, cudaStreamLegacy));
@@ -868,7 +415,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
         if (composed) FB_CHECK(run_plan<R>(op->m2m[l], T, mp, mp, s));
         else if (auto_tc && op->tc_m2m[l])
             FB_CHECK(fb_tc_run(op, op->tc_m2m[l], (const cf*)mp, (cf*)mp, s, nrhs, cnt));
-        else FB_CHECK(run_rcr<R>(op->m2m_rcr[l], rot, coax, mp, mp, s, nrhs, cnt));
+        else FB_CHECK(run_rcr<R>(op, op->m2m_rcr[l], rot, coax, mp, mp, s, nrhs, cnt));
     }
     mark(2);
     // phase [2] is the tensor-core part of M2L: empty unless it runs below
@@ -877,7 +424,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
     if (composed) {
         FB_CHECK(run_plan<R>(op->m2l, T, mp, loc, s));
     } else if (op->method == FB_TRANS_RCR) {
-        FB_CHECK(run_rcr<R>(op->m2l_rcr, rot, coax, mp, loc, s, nrhs, cnt));
+        FB_CHECK(run_rcr<R>(op, op->m2l_rcr, rot, coax, mp, loc, s, nrhs, cnt));
     } else {
         if constexpr (sizeof(R) == 4) {
             if (op->method == FB_TRANS_TENSOR) {
@@ -885,12 +432,12 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
             } else if (op->tc_plan) {
                 FB_CHECK(fb_tc_run(op, op->tc_plan, (const cf*)mp, (cf*)loc, s, nrhs, cnt));
                 mark(3);
-                FB_CHECK(run_rcr<R>(op->m2l_rcr_rest, rot, coax, mp, loc, s, nrhs, cnt));
+                FB_CHECK(run_rcr<R>(op, op->m2l_rcr_rest, rot, coax, mp, loc, s, nrhs, cnt));
             } else {
-                FB_CHECK(run_rcr<R>(op->m2l_rcr, rot, coax, mp, loc, s, nrhs, cnt));
+                FB_CHECK(run_rcr<R>(op, op->m2l_rcr, rot, coax, mp, loc, s, nrhs, cnt));
             }
         } else {
-            FB_CHECK(run_rcr<R>(op->m2l_rcr, rot, coax, mp, loc, s, nrhs, cnt));
+            FB_CHECK(run_rcr<R>(op, op->m2l_rcr, rot, coax, mp, loc, s, nrhs, cnt));
         }
     }
     mark(4);
@@ -898,7 +445,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
         if (composed) FB_CHECK(run_plan<R>(op->l2l[l], T, loc, loc, s));
         else if (auto_tc && op->tc_l2l[l])
             FB_CHECK(fb_tc_run(op, op->tc_l2l[l], (const cf*)loc, (cf*)loc, s, nrhs, cnt));
-        else FB_CHECK(run_rcr<R>(op->l2l_rcr[l], rot, coax, loc, loc, s, nrhs, cnt));
+        else FB_CHECK(run_rcr<R>(op, op->l2l_rcr[l], rot, coax, loc, loc, s, nrhs, cnt));
     }
     mark(5);
     int maxK = 0;
@@ -1033,8 +580,8 @@ fb_status fb_rcr_restage(fb_op* op, const int* m2l, const int* pair) {
 // One RCR plan on the operator's expansion buffers (precision of the op).
 fb_status fb_rcr_run_op(fb_op* op, RcrPlan& pl, void* src, void* dst, cudaStream_t s, int nrhs, int64_t rstride) {
     if (op->prec == FB_PREC_MIXED_FMM)
-        return run_rcr<float>(pl, rot_args<float>(op), op->coax32, (const cf*)src, (cf*)dst, s, nrhs, rstride);
-    return run_rcr<double>(pl, rot_args<double>(op), op->coax64, (const cd*)src, (cd*)dst, s, nrhs, rstride);
+        return run_rcr<float>(op, pl, rot_args<float>(op), op->coax32, (const cf*)src, (cf*)dst, s, nrhs, rstride);
+    return run_rcr<double>(op, pl, rot_args<double>(op), op->coax64, (const cd*)src, (cd*)dst, s, nrhs, rstride);
 }
 
 fb_status fb_fmm_apply(fb_op* op, const cd* x, cd* y, cudaStream_t s, PhaseTimer* pt, int nrhs) {
@@ -1048,14 +595,10 @@ static void free_plan(TransPlan& p) {
     dfree(p.tiles);
 }
 void fb_rcr_free(RcrPlan& p) {
-    dfree(p.tasks);
-    dfree(p.tiles);
-    dfree(p.df_tiles.tiles);
-    p.df_tiles = RcrTileSet();
+    fb_rcr_tiles_free(p.tiles);
+    fb_rcr_tiles_free(p.df_tiles);
     fb_stg_free(p.stg);
     p.stg_elems = 0;
-    for (auto& kv : p.multi) dfree(kv.second.tiles);
-    p.multi.clear();
 }
 static void free_plan(RcrPlan& p) { fb_rcr_free(p); }
 
@@ -1106,7 +649,11 @@ void fb_fmm_destroy(fb_op* op) {
     dfree(op->stc_err);
     dfree(op->rotf_df);
     dfree(op->coax_df);
-    dfree(op->rotd_df);
+    for (RcrTables* t : {&op->rcr_tab, &op->rcr_df}) {
+        dfree(t->rot);
+        dfree(t->coax);
+    }
+    dfree(op->rcr_lut);
 }
 
 // ---------------------------------------------------------------------------

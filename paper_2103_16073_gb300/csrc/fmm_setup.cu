@@ -793,6 +793,9 @@ fb_status fb_fmm_create(fb_op* op, double d0, int pmin, cudaStream_t s) {
     // the rotation blocks and coaxial sets stay with the operator (RCR form)
     op->coax64 = coax;
     op->coax_count = std::max<int64_t>(coax_total, 1);
+    op->coax_sets.clear();
+    for (const auto& cs : sets) op->coax_sets.emplace_back(cs.p, cs.out_off);
+    std::sort(op->coax_sets.begin(), op->coax_sets.end());
     coax = nullptr;
     op->rot64 = rot;
     op->rotd64 = rset->d64;
