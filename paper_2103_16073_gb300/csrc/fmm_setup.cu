@@ -22,33 +22,99 @@ __global__ void k_d2f(const cd* a, cf* b, int64_t n) {
 }
 
 // ------------------------------------------------------------ near field ----
-__global__ void k_near_fill(Geom g, int kind, double k, double rc, const int32_t* __restrict__ perm,
-                            const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ ucnt,
-                            const int32_t* __restrict__ ulist, const int64_t* __restrict__ nf_off,
-                            const int32_t* __restrict__ nf_ncol, cd* __restrict__ out) {
-    int t = blockIdx.x;
+// One CTA per (leaf, NF_COLS columns of its block): a thread keeps one source
+// element in registers and runs over the leaf's rows (coalesced stores along
+// the columns).  The closed-form entries (within r_c, a tenth of the block)
+// cost about ten times a far one: they are collected in shared memory and
+// then shared out over all threads, instead of holding up every warp that
+// has one.  FP64-pipe bound; L-room at 609 Hz (53,396 elements): 56.1 ms
+// with one thread per entry and the library's sqrt, divisions and sincos,
+// 12.7 ms in this form.
+constexpr int NF_COLS = 128, NF_ROWS = 32;
+template <int KIND>
+__global__ void __launch_bounds__(NF_COLS) k_near_fill(Geom g, double k, double rc, const int32_t* __restrict__ perm,
+                                                       const int32_t* __restrict__ leaf_start,
+                                                       const int32_t* __restrict__ ucnt,
+                                                       const int32_t* __restrict__ ulist,
+                                                       const int64_t* __restrict__ nf_off,
+                                                       const int32_t* __restrict__ nf_ncol, cd* __restrict__ out) {
+    const int t = blockIdx.x;
+    const int K = nf_ncol[t], c0 = blockIdx.y * NF_COLS;
+    if (c0 >= K) return;
+    __shared__ double2 s_sc[fm::SC_TAB];
     __shared__ int s_start[FB_ULIST], s_cum[FB_ULIST + 1];
-    int nu = ucnt[t];
-    if (threadIdx.x == 0) {
+    __shared__ int s_elem[NF_COLS];
+    __shared__ V3 s_x[NF_ROWS], s_n[NF_ROWS];
+    __shared__ int s_row[NF_ROWS];
+    __shared__ uint16_t s_near[NF_ROWS * NF_COLS];
+    __shared__ int s_cnt;
+    const int nu = ucnt[t], tid = threadIdx.x;
+    fm::sc_load(s_sc);
+    if (tid == 0) {
         s_cum[0] = 0;
         for (int i = 0; i < nu; ++i) {
-            int s = ulist[(int64_t)t * FB_ULIST + i];
+            const int s = ulist[(int64_t)t * FB_ULIST + i];
             s_start[i] = leaf_start[s];
             s_cum[i + 1] = s_cum[i] + (leaf_start[s + 1] - leaf_start[s]);
         }
     }
     __syncthreads();
-    int r0 = leaf_start[t];
-    int nr = leaf_start[t + 1] - r0;
-    int K = nf_ncol[t];
-    int64_t base = nf_off[t];
-    for (int64_t e = threadIdx.x; e < (int64_t)nr * K; e += blockDim.x) {
-        int r = (int)(e / K), c = (int)(e % K);
+    const int c = c0 + tid;
+    const bool has = c < K;
+    int64_t j = 0;
+    V3 y[3], cj, nj;
+    double area = 0.0;
+    cd ikb = mk(0.0, 0.0);
+    if (has) {
         int u = 0;
         while (s_cum[u + 1] <= c) ++u;
-        int col_pos = s_start[u] + (c - s_cum[u]);
-        int64_t i = perm[r0 + r], j = perm[col_pos];
-        out[base + e] = op_entry(g, kind, i, j, k, rc);
+        j = perm[s_start[u] + (c - s_cum[u])];
+        for (int q = 0; q < 3; ++q) y[q] = v3(g.gx[3 * j + q], g.gy[3 * j + q], g.gz[3 * j + q]);
+        cj = v3(g.cx[j], g.cy[j], g.cz[j]);
+        nj = v3(g.nx[j], g.ny[j], g.nz[j]);
+        area = g.area[j];
+        if (KIND == FB_OP_A) {
+            const cd b = g.beta[j];
+            ikb = mk(-k * b.im, k * b.re);
+        }
+    }
+    s_elem[tid] = (int)j;
+    const int r0 = leaf_start[t], nr = leaf_start[t + 1] - r0;
+    cd* blk = out + nf_off[t];
+    for (int rb = 0; rb < nr; rb += NF_ROWS) {
+        const int rows = min(NF_ROWS, nr - rb);
+        if (tid < rows) {
+            const int e = perm[r0 + rb + tid];
+            s_row[tid] = e;
+            s_x[tid] = v3(g.cx[e], g.cy[e], g.cz[e]);
+            s_n[tid] = v3(g.nx[e], g.ny[e], g.nz[e]);
+        }
+        if (tid == 0) s_cnt = 0;
+        __syncthreads();
+        if (has) {
+            for (int r = 0; r < rows; ++r) {
+                const V3 x = s_x[r];
+                const V3 dc = x - cj;
+                if (s_row[r] == (int)j || dot(dc, dc) < rc * rc) {
+                    s_near[atomicAdd(&s_cnt, 1)] = (uint16_t)(r * NF_COLS + tid);
+                    continue;
+                }
+                cd v;
+                if constexpr (KIND == FB_OP_MP) {
+                    v = mk(0.0, 0.0);
+                    for (int q = 0; q < 3; ++q) v = v + (area / 3.0) * kernel_nn(k, y[q] - x, s_n[r], nj);
+                } else {
+                    v = far_entry<KIND>(s_sc, k, y, area, -dot(nj, dc), x, s_n[r], ikb);
+                }
+                blk[(int64_t)(rb + r) * K + c] = v;
+            }
+        }
+        __syncthreads();
+        for (int i = tid; i < s_cnt; i += NF_COLS) {
+            const int r = s_near[i] / NF_COLS, cc = s_near[i] % NF_COLS;
+            blk[(int64_t)(rb + r) * K + c0 + cc] = op_entry(g, KIND, s_row[r], s_elem[cc], k, rc);
+        }
+        __syncthreads();
     }
 }
 
@@ -68,52 +134,180 @@ __global__ void k_absmax(const cd* a, int64_t n, double* out) {
 // ----------------------------------------------------------- P2M / L2P ----
 // W[pos][nm] = ik A_j sum_q w_q [dip n_j.grad R_n^{-m}(y_q - c) + mono_j R_n^{-m}(y_q - c)]
 // V[pos][nm] = R_n^m(x_i - c)  (L' : n_i . grad R_n^m(x_i - c))
-__global__ void k_p2m_l2p(Geom g, int kind, double k, int P, int64_t n, const int32_t* __restrict__ perm,
-                          const int32_t* __restrict__ leaf_of, const double* __restrict__ centers,
-                          double* scratch, int scratch_stride, cd* __restrict__ W, cd* __restrict__ V) {
-    int64_t tid = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-    int64_t nthreads = (int64_t)gridDim.x * blockDim.x;
-    double* sc = scratch + tid * (int64_t)scratch_stride;
-    int Pp1 = P + 1;
-    cd* Rv = (cd*)sc;                                  // (P+1)^2 complex
-    double* wrk = sc + 2 * Pp1 * Pp1;
-    for (int64_t pos = tid; pos < n; pos += nthreads) {
-        int64_t e = perm[pos];
-        int b = leaf_of[pos];
-        V3 c = v3(centers[3 * b], centers[3 * b + 1], centers[3 * b + 2]);
-        V3 nj = v3(g.nx[e], g.ny[e], g.nz[e]);
-        cd* Wr = W + pos * (int64_t)P * P;
-        cd* Vr = V + pos * (int64_t)P * P;
-        for (int q = 0; q < P * P; ++q) Wr[q] = mk(0.0, 0.0);
-        cd mono = mk(0.0, 0.0);
-        double dip = 0.0;
-        if (kind == FB_OP_L || kind == FB_OP_LP) mono = mk(1.0, 0.0);
-        if (kind == FB_OP_M || kind == FB_OP_MP) dip = 1.0;
-        if (kind == FB_OP_A) {
-            cd b = g.beta[e];
-            mono = mk(k * b.im, -k * b.re);   // -i k beta
-            dip = 1.0;
+//
+// One CTA per group of E elements.  R_n^{-m} = conj R_n^m, so only orders
+// m >= 0 are computed, and since the three Gauss points of a flat element
+// share weight and normal their R are summed before the gradient:
+//   A  one thread per (element, point): direction, j_n(k r), powers of
+//      e^{i phi} and of sin theta;
+//   B  one thread per (element, order m): the Legendre recursion up in n for
+//      the points side by side, S_n^m = sum_q R_n^m into shared memory;
+//   C  one thread per (element, n, m): gradient and stores of +m and -m.
+// The recursion and gradient factors come from tables.  FP64-pipe bound;
+// one thread per element with its arrays in global memory took 12.8 ms at
+// 53,396 elements (order 12), this form 1.07 ms (and 3.3 -> 0.1 ms at 1,500
+// to 6,000 elements).
+struct SphTab {
+    const double* leg;   // [n (n + 1) / 2 + m] (A, B) pairs of the Legendre recursion
+    const double* diag;  // Q_m^m = diag[m] sin^m theta
+    const double* ga;    // a_n^m at [n (M + 1) + m]
+    const double* gb;    // b_n^m at [n (2 M + 1) + m + M]
+    int M;
+};
+
+__global__ void k_sph_tables(int P, int M, double* __restrict__ leg, double* __restrict__ diag,
+                             double* __restrict__ ga, double* __restrict__ gb) {
+    const int tid = blockIdx.x * blockDim.x + threadIdx.x, nth = gridDim.x * blockDim.x;
+    for (int i = tid; i < P * P; i += nth) {
+        const int n = i / P, m = i % P;
+        if (m > n) continue;
+        double A = 0.0, B = 0.0;
+        const double nn = (double)n * n, mm = (double)m * m;
+        if (n > m) A = sqrt((4.0 * nn - 1.0) / (nn - mm));
+        if (n > m + 1)
+            B = sqrt(((n - 1.0) * (n - 1.0) - mm) * (2.0 * n + 1.0) / ((2.0 * n - 3.0) * (nn - mm)));
+        leg[2 * (n * (n + 1) / 2 + m)] = A;
+        leg[2 * (n * (n + 1) / 2 + m) + 1] = B;
+    }
+    for (int m = tid; m < P; m += nth) {
+        double v = 0.28209479177387814347;   // 1/sqrt(4 pi)
+        for (int i = 1; i <= m; ++i) v *= sqrt((2.0 * i + 1.0) / (2.0 * i));
+        diag[m] = v;
+    }
+    const int w = 2 * M + 1;
+    for (int i = tid; i < (P + 1) * w; i += nth) {
+        const int n = i / w, m = i % w - M;
+        gb[i] = coef_b(n, m);
+        if (m >= 0) ga[n * (M + 1) + m] = coef_a(n, m);
+    }
+}
+
+// bytes of shared memory per element of a group: S (unless in global memory),
+// and j_n, e^{i m phi}, Q_m^m and cos theta of its four points
+__host__ __device__ inline size_t p2m_elem_bytes(int Pp1, bool s_global) {
+    return (s_global ? 0 : (size_t)Pp1 * (Pp1 + 1) / 2 * sizeof(cd)) + 4 * (size_t)Pp1 * 32 + 4 * 8;
+}
+
+__global__ void __launch_bounds__(128) k_p2m_l2p(Geom g, int kind, double k, int P, int64_t n, int E, SphTab tab,
+                                                 const int32_t* __restrict__ perm, const int32_t* __restrict__ leaf_of,
+                                                 const double* __restrict__ centers, cd* __restrict__ s_global,
+                                                 cd* __restrict__ W, cd* __restrict__ V) {
+    extern __shared__ __align__(16) unsigned char p2m_smem[];
+    const int Pp1 = P + 1, H = Pp1 * (Pp1 + 1) / 2, tid = threadIdx.x, nth = blockDim.x, npt = 4 * E;
+    cd* em = (cd*)p2m_smem;                          // [point][m]
+    cd* S = s_global ? s_global + (int64_t)blockIdx.x * E * H : em + (size_t)npt * Pp1;   // [element][n (n + 1) / 2 + m]
+    double* jn = (double*)(s_global ? em + (size_t)npt * Pp1 : S + (size_t)E * H);        // [point][n]
+    double* dg = jn + npt * Pp1;                     // [point][m]
+    double* ct = dg + npt * Pp1;                     // [point]
+    const bool grad = kind != FB_OP_L && kind != FB_OP_LP;
+    const bool grad_v = kind == FB_OP_LP || kind == FB_OP_MP;
+    for (int64_t g0 = (int64_t)blockIdx.x * E; g0 < n; g0 += (int64_t)gridDim.x * E) {
+        const int ne = (int)min((int64_t)E, n - g0);
+        // ---- A: points (element, 0..2 Gauss points, 3 centroid)
+        for (int pt = tid; pt < 4 * ne; pt += nth) {
+            const int64_t pos = g0 + (pt >> 2), e = perm[pos];
+            const int q = pt & 3, b = leaf_of[pos];
+            const V3 c = v3(centers[3 * b], centers[3 * b + 1], centers[3 * b + 2]);
+            const V3 y = q < 3 ? v3(g.gx[3 * e + q], g.gy[3 * e + q], g.gz[3 * e + q]) : v3(g.cx[e], g.cy[e], g.cz[e]);
+            const V3 r = y - c;
+            const double rho = norm(r);
+            V3 u = v3(0.0, 0.0, 1.0);   // r = 0: R_0^0 = 1/sqrt(4 pi), all others vanish with j_n(0)
+            if (rho > 0.0) u = v3(r.x / rho, r.y / rho, r.z / rho);
+            const double st = sqrt(u.x * u.x + u.y * u.y);
+            const cd e1 = st > 0.0 ? mk(u.x / st, u.y / st) : mk(1.0, 0.0);
+            cd z = mk(1.0, 0.0);
+            double sm = 1.0;
+            for (int m = 0; m < Pp1; ++m) {
+                em[pt * Pp1 + m] = z;
+                dg[pt * Pp1 + m] = tab.diag[m] * sm;
+                z = z * e1;
+                sm *= st;
+            }
+            ct[pt] = u.z;
+            sph_bessel_j(P, k * rho, jn + pt * Pp1);
         }
-        // ik A_j w_q, w_q = 1/3
-        cd pref = mk(0.0, k * g.area[e] / 3.0);
-        for (int qp = 0; qp < 3; ++qp) {
-            V3 y = v3(g.gx[3 * e + qp], g.gy[3 * e + qp], g.gz[3 * e + qp]);
-            regular_all(Pp1, k, y - c, wrk, Rv);
-            for (int nn = 0; nn < P; ++nn)
-                for (int m = -nn; m <= nn; ++m) {
-                    cd v = mono * Rv[nm_idx(nn, -m)];
-                    if (dip != 0.0) v = v + ndot_grad_regular(Rv, P, k, nj, nn, -m);
-                    Wr[nm_idx(nn, m)] = Wr[nm_idx(nn, m)] + pref * v;
+        __syncthreads();
+        for (int pass = 0; pass < 2; ++pass) {   // the Gauss points for W, the centroid for V
+            // ---- B: S_n^m, every n of one order m
+            for (int i = tid; i < ne * Pp1; i += nth) {
+                const int el = i / Pp1, m = i % Pp1;
+                const int p0 = 4 * el + (pass ? 3 : 0), np = pass ? 1 : 3;
+                double q1[3], q2[3], x[3];
+                cd z[3];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    const int pt = p0 + (q < np ? q : 0);
+                    q1[q] = dg[pt * Pp1 + m];
+                    q2[q] = 0.0;
+                    x[q] = ct[pt];
+                    z[q] = em[pt * Pp1 + m];
                 }
-        }
-        V3 x = v3(g.cx[e], g.cy[e], g.cz[e]);
-        regular_all(Pp1, k, x - c, wrk, Rv);
-        if (kind == FB_OP_LP || kind == FB_OP_MP) {
-            V3 ni = nj;
-            for (int nn = 0; nn < P; ++nn)
-                for (int m = -nn; m <= nn; ++m) Vr[nm_idx(nn, m)] = ndot_grad_regular(Rv, P, k, ni, nn, m);
-        } else {
-            for (int q = 0; q < P * P; ++q) Vr[q] = Rv[q];
+                for (int nn = m; nn < Pp1; ++nn) {
+                    const double A = tab.leg[2 * (nn * (nn + 1) / 2 + m)], B = tab.leg[2 * (nn * (nn + 1) / 2 + m) + 1];
+                    cd acc = mk(0.0, 0.0);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        if (q >= np) continue;
+                        if (nn > m) {
+                            const double t = A * x[q] * q1[q] - B * q2[q];
+                            q2[q] = q1[q];
+                            q1[q] = t;
+                        }
+                        const double v = jn[(p0 + q) * Pp1 + nn] * q1[q];
+                        acc.re += v * z[q].re;
+                        acc.im += v * z[q].im;
+                    }
+                    S[(size_t)el * H + nn * (nn + 1) / 2 + m] = acc;
+                }
+            }
+            __syncthreads();
+            // ---- C
+            const int h = P * (P + 1) / 2;
+            for (int i = tid; i < ne * h; i += nth) {
+                const int el = i / h, t = i % h;
+                int nn = (int)((sqrtf(8.0f * (float)t + 1.0f) - 1.0f) * 0.5f);
+                while (nn * (nn + 1) / 2 > t) --nn;
+                while ((nn + 1) * (nn + 2) / 2 <= t) ++nn;
+                const int m = t - nn * (nn + 1) / 2;
+                const int64_t pos = g0 + el, e = perm[pos];
+                const cd* Se = S + (size_t)el * H;
+                auto get = [&](int a, int u) {   // S_a^u for u >= -1
+                    if (a < 0 || abs(u) > a) return mk(0.0, 0.0);
+                    const cd v = Se[a * (a + 1) / 2 + abs(u)];
+                    return u < 0 ? conjg(v) : v;
+                };
+                const cd Sv = Se[nn * (nn + 1) / 2 + m];
+                cd G = mk(0.0, 0.0);
+                if (pass ? grad_v : grad) {   // n . grad S_n^m
+                    const int M = tab.M;
+                    auto fa = [&](int a, int u) { return a < 0 ? 0.0 : tab.ga[a * (M + 1) + u]; };
+                    auto fb = [&](int a, int u) { return tab.gb[a * (2 * M + 1) + u + M]; };
+                    const V3 nv = v3(g.nx[e], g.ny[e], g.nz[e]);
+                    const cd dz = fa(nn - 1, m) * get(nn - 1, m) - fa(nn, m) * get(nn + 1, m);
+                    const cd dp = fb(nn + 1, -m - 1) * get(nn + 1, m + 1) - fb(nn, m) * get(nn - 1, m + 1);
+                    const cd dm = fb(nn + 1, m - 1) * get(nn + 1, m - 1) - fb(nn, -m) * get(nn - 1, m - 1);
+                    const cd hp = mk(0.5 * nv.x, -0.5 * nv.y), hm = mk(0.5 * nv.x, 0.5 * nv.y);
+                    G = k * (hp * dp + hm * dm + nv.z * dz);
+                }
+                cd* o = (pass ? V : W) + pos * (int64_t)P * P + nn * nn + nn;
+                if (pass) {
+                    const cd v = grad_v ? G : Sv;
+                    o[m] = v;
+                    if (m) o[-m] = conjg(v);
+                } else {
+                    cd mono = mk(0.0, 0.0);
+                    if (kind == FB_OP_L || kind == FB_OP_LP) mono = mk(1.0, 0.0);
+                    if (kind == FB_OP_A) {
+                        const cd be = g.beta[e];
+                        mono = mk(k * be.im, -k * be.re);   // -i k beta
+                    }
+                    const double f = k * g.area[e] / 3.0;   // ik A_j w_q, w_q = 1/3
+                    const cd vp = mono * conjg(Sv) + conjg(G), vm = mono * Sv + G;
+                    o[m] = mk(-f * vp.im, f * vp.re);
+                    if (m) o[-m] = mk(-f * vm.im, f * vm.re);
+                }
+            }
+            __syncthreads();
         }
     }
 }
@@ -126,7 +320,13 @@ __global__ void k_p2m_l2p(Geom g, int kind, double k, int P, int64_t n, const in
 //  k tau >= 1: 3.1 zonal (Eq. shft7), 3.2 diagonal + two subdiagonals
 //     (Eq. shft8; third formula with b_n^{-m-1}), 3 propagation in n'
 //     (Eq. shift6), 4 symmetry.
-// One thread per coefficient set.  out: [m][n'][n] with stride p (p^3 complex).
+// One CTA per coefficient set: every step is a chain along one index with
+// the other two free, so the threads take the free ones and a barrier
+// separates the links (about 5 p of them); the diagonals (3.2) advance as a
+// wavefront, order m + 1 one step behind order m.  The recursion factors
+// a_n^m and b_n^m are the same for every set and come from a table.  L-room
+// at 609 Hz (orders to 36): one thread per set took 24.4 ms, this form 0.34 ms.
+// out: [m][n'][n] with stride p (p^3 complex).
 struct CoaxSet {
     double ktau;
     int p;
@@ -134,79 +334,109 @@ struct CoaxSet {
     int64_t out_off;
 };
 
-__global__ void k_coaxial(const CoaxSet* sets, int nsets, cd* scratch, int64_t scratch_stride,
-                          double* fscratch, int64_t fstride, cd* out) {
-    int sid = blockIdx.x * blockDim.x + threadIdx.x;
-    if (sid >= nsets) return;
-    CoaxSet cs = sets[sid];
-    int p = cs.p;
-    int W2 = 2 * p + 2, W3 = p + 2;
-    cd* X = scratch + sid * scratch_stride;
+// a_n^m at [n (M + 1) + m], b_n^{m} at [n (2 M + 1) + m + M], n < N, |m| <= M
+__global__ void k_coaxial_factors(int N, int M, double* __restrict__ a, double* __restrict__ b) {
+    const int w = 2 * M + 1;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < N * w; i += gridDim.x * blockDim.x) {
+        const int n = i / w, m = i % w - M;
+        b[i] = coef_b(n, m);
+        if (m >= 0) a[n * (M + 1) + m] = coef_a(n, m);
+    }
+}
+
+__global__ void __launch_bounds__(512) k_coaxial(const CoaxSet* sets, cd* scratch, int64_t scratch_stride,
+                                                 double* fscratch, int64_t fstride, const double* __restrict__ ca,
+                                                 const double* __restrict__ cb, int M, cd* out) {
+    const CoaxSet cs = sets[blockIdx.x];
+    const int p = cs.p, tid = threadIdx.x, nth = blockDim.x;
+    const int W2 = 2 * p + 2, W3 = p + 2;
+    cd* X = scratch + blockIdx.x * scratch_stride;
     auto at = [&](int m, int n1, int n) -> cd& { return X[((int64_t)m * W2 + n1) * W3 + n]; };
-    for (int64_t i = 0; i < (int64_t)(p + 1) * W2 * W3; ++i) X[i] = mk(0.0, 0.0);
-    int P2 = 2 * p;
-    double* fj = fscratch + sid * fstride;
+    auto fa = [&](int n, int m) { return n < 0 ? 0.0 : ca[n * (M + 1) + m]; };
+    auto fb = [&](int n, int m) { return n < 0 ? 0.0 : cb[n * (2 * M + 1) + m + M]; };
+    for (int64_t i = tid; i < (int64_t)(p + 1) * W2 * W3; i += nth) X[i] = mk(0.0, 0.0);
+    const int P2 = 2 * p;
+    double* fj = fscratch + blockIdx.x * fstride;
     double* fy = fj + P2 + 1;
-    sph_bessel_j(P2 - 1, cs.ktau, fj);
-    if (cs.kind == 0) sph_bessel_y(P2 - 1, cs.ktau, fy);
-    for (int n1 = 0; n1 < P2; ++n1) {
+    if (tid == 0) sph_bessel_j(P2 - 1, cs.ktau, fj);
+    if (tid == 32 && cs.kind == 0) sph_bessel_y(P2 - 1, cs.ktau, fy);
+    __syncthreads();
+    for (int n1 = tid; n1 < P2; n1 += nth) {
         double sg = (n1 & 1) ? -1.0 : 1.0;
         double s = sg * sqrt(2.0 * n1 + 1.0);
         at(0, n1, 0) = cs.kind == 0 ? mk(s * fj[n1], s * fy[n1]) : mk(s * fj[n1], 0.0);
     }
-    for (int m = 0; m < p - 1; ++m)
-        for (int n1 = m + 1; n1 < P2 - 1 - m; ++n1)
-            at(m + 1, n1, m + 1) = (1.0 / coef_b(m + 1, -m - 1)) *
-                                   (coef_b(n1, -m - 1) * at(m, n1 - 1, m) - coef_b(n1 + 1, m) * at(m, n1 + 1, m));
+    __syncthreads();
+    for (int m = 0; m < p - 1; ++m) {
+        for (int n1 = m + 1 + tid; n1 < P2 - 1 - m; n1 += nth)
+            at(m + 1, n1, m + 1) = (1.0 / fb(m + 1, -m - 1)) *
+                                   (fb(n1, -m - 1) * at(m, n1 - 1, m) - fb(n1 + 1, m) * at(m, n1 + 1, m));
+        __syncthreads();
+    }
     if (cs.ktau < 1.0) {
-        for (int m = 0; m < p; ++m)
-            for (int n = m; n < p - 1; ++n)
-                for (int n1 = n; n1 < 2 * p - 1 - n; ++n1)
-                    at(m, n1, n + 1) = (1.0 / coef_a(n, m)) *
-                                       (coef_a(n - 1, m) * (n >= 1 ? at(m, n1, n - 1) : mk(0.0, 0.0)) -
-                                        coef_a(n1, m) * at(m, n1 + 1, n) +
-                                        coef_a(n1 - 1, m) * (n1 >= 1 ? at(m, n1 - 1, n) : mk(0.0, 0.0)));
-    } else {
-        for (int n = 0; n < p - 1; ++n)
-            for (int n1 = n + 1; n1 < 2 * p - n - 2; ++n1)
-                at(0, n1, n + 1) = (1.0 / coef_a(n, 0)) *
-                                   (coef_a(n - 1, 0) * (n >= 1 ? at(0, n1, n - 1) : mk(0.0, 0.0)) -
-                                    coef_a(n1, 0) * at(0, n1 + 1, n) + coef_a(n1 - 1, 0) * at(0, n1 - 1, n));
-        for (int m = 0; m < p - 2; ++m)
-            for (int n = m + 1; n < p - 1; ++n) {
-                if (n >= m + 2)
-                    at(m + 1, n + 1, n) = (1.0 / coef_b(n + 1, -m - 1)) *
-                                          (coef_b(n + 1, m) * at(m, n + 1, n) + coef_b(n, -m - 1) * at(m, n, n - 1) -
-                                           coef_b(n, m) * at(m + 1, n, n - 1));
-                at(m + 1, n + 1, n + 1) = (1.0 / coef_b(n + 1, -m - 1)) *
-                                          (coef_b(n, m) * at(m + 1, n + 1, n - 1) - coef_b(n + 2, m) * at(m, n + 2, n) +
-                                           coef_b(n + 1, -m - 1) * at(m, n, n));
-                if (n >= m + 2)
-                    at(m + 1, n + 2, n) = (1.0 / coef_b(n + 2, -m - 1)) *
-                                          (coef_b(n + 1, m) * at(m + 1, n, n) - coef_b(n + 1, m) * at(m, n + 1, n + 1) +
-                                           coef_b(n, -m - 1) * at(m, n + 1, n - 1));
+        // every order m advances in n together: step n uses columns n and n - 1
+        for (int n = 0; n < p - 1; ++n) {
+            const int len = 2 * p - 1 - 2 * n;   // n1 = n .. 2p - 2 - n
+            for (int i = tid; i < (n + 1) * len; i += nth) {
+                const int m = i / len, n1 = n + i % len;
+                at(m, n1, n + 1) = (1.0 / fa(n, m)) *
+                                   (fa(n - 1, m) * (n >= 1 ? at(m, n1, n - 1) : mk(0.0, 0.0)) -
+                                    fa(n1, m) * at(m, n1 + 1, n) +
+                                    fa(n1 - 1, m) * (n1 >= 1 ? at(m, n1 - 1, n) : mk(0.0, 0.0)));
             }
-        for (int m = 1; m < p; ++m)
-            for (int n1 = m + 3; n1 < p - 1; ++n1)
-                for (int n = m + 1; n < n1 - 1; ++n)
-                    at(m, n1 + 1, n) = (1.0 / coef_a(n1, m)) *
-                                       (coef_a(n - 1, m) * at(m, n1, n - 1) - coef_a(n, m) * at(m, n1, n + 1) +
-                                        coef_a(n1 - 1, m) * at(m, n1 - 1, n));
+            __syncthreads();
+        }
+    } else {
+        for (int n = 0; n < p - 1; ++n) {
+            for (int n1 = n + 1 + tid; n1 < 2 * p - n - 2; n1 += nth)
+                at(0, n1, n + 1) = (1.0 / fa(n, 0)) *
+                                   (fa(n - 1, 0) * (n >= 1 ? at(0, n1, n - 1) : mk(0.0, 0.0)) -
+                                    fa(n1, 0) * at(0, n1 + 1, n) + fa(n1 - 1, 0) * at(0, n1 - 1, n));
+            __syncthreads();
+        }
+        // order m at step s takes n = s - m: order m - 1 has done n one step before
+        for (int s = 1; s <= 2 * p - 5; ++s) {
+            for (int m = tid; m < p - 2; m += nth) {
+                const int n = s - m;
+                if (n < m + 1 || n >= p - 1) continue;
+                if (n >= m + 2)
+                    at(m + 1, n + 1, n) = (1.0 / fb(n + 1, -m - 1)) *
+                                          (fb(n + 1, m) * at(m, n + 1, n) + fb(n, -m - 1) * at(m, n, n - 1) -
+                                           fb(n, m) * at(m + 1, n, n - 1));
+                at(m + 1, n + 1, n + 1) = (1.0 / fb(n + 1, -m - 1)) *
+                                          (fb(n, m) * at(m + 1, n + 1, n - 1) - fb(n + 2, m) * at(m, n + 2, n) +
+                                           fb(n + 1, -m - 1) * at(m, n, n));
+                if (n >= m + 2)
+                    at(m + 1, n + 2, n) = (1.0 / fb(n + 2, -m - 1)) *
+                                          (fb(n + 1, m) * at(m + 1, n, n) - fb(n + 1, m) * at(m, n + 1, n + 1) +
+                                           fb(n, -m - 1) * at(m, n + 1, n - 1));
+            }
+            __syncthreads();
+        }
+        for (int n1 = 4; n1 < p - 1; ++n1) {   // m = 1 .. n1 - 3, n = m + 1 .. n1 - 2
+            const int side = n1 - 3;
+            for (int i = tid; i < side * side; i += nth) {
+                const int m = 1 + i / side, n = 2 + i % side;
+                if (n <= m) continue;
+                at(m, n1 + 1, n) = (1.0 / fa(n1, m)) * (fa(n - 1, m) * at(m, n1, n - 1) - fa(n, m) * at(m, n1, n + 1) +
+                                                        fa(n1 - 1, m) * at(m, n1 - 1, n));
+            }
+            __syncthreads();
+        }
     }
     cd* o = out + cs.out_off;
-    for (int m = 0; m < p; ++m)
-        for (int n1 = 0; n1 < p; ++n1)
-            for (int n = 0; n < p; ++n) {
-                cd v = mk(0.0, 0.0);
-                if (n1 >= m && n >= m) {
-                    if (n1 >= n) v = at(m, n1, n);
-                    else {
-                        v = at(m, n, n1);
-                        if ((n + n1) & 1) v = mk(-v.re, -v.im);
-                    }
-                }
-                o[((int64_t)m * p + n1) * p + n] = v;
+    for (int64_t i = tid; i < (int64_t)p * p * p; i += nth) {
+        const int n = (int)(i % p), n1 = (int)(i / p % p), m = (int)(i / ((int64_t)p * p));
+        cd v = mk(0.0, 0.0);
+        if (n1 >= m && n >= m) {
+            if (n1 >= n) v = at(m, n1, n);
+            else {
+                v = at(m, n, n1);
+                if ((n + n1) & 1) v = mk(-v.re, -v.im);
             }
+        }
+        o[i] = v;
+    }
 }
 
 // ------------------------------------------------------------ rotations ----
@@ -597,8 +827,16 @@ fb_status fb_fmm_create(fb_op* op, double d0, int pmin, cudaStream_t s) {
         // the same entries: copy them instead of integrating again
         FB_CUDA(cudaMemcpyAsync(op->nf64, dn->nf64, sizeof(cd) * op->nf_count, cudaMemcpyDeviceToDevice, s));
     } else {
-        k_near_fill<<<nleaf, 256, 0, s>>>(m->g, op->kind, k, m->rc, t->perm, t->leaf_start, t->ucnt, t->ulist,
-                                          op->nf_off, op->nf_ncol, op->nf64);
+        int maxK = 1;
+        for (int b = 0; b < nleaf; ++b) maxK = std::max(maxK, op->h_nf_ncol[b]);
+        const dim3 grid((unsigned)nleaf, (unsigned)div_up(maxK, NF_COLS));
+        auto fill = op->kind == FB_OP_L    ? k_near_fill<FB_OP_L>
+                    : op->kind == FB_OP_M  ? k_near_fill<FB_OP_M>
+                    : op->kind == FB_OP_LP ? k_near_fill<FB_OP_LP>
+                    : op->kind == FB_OP_MP ? k_near_fill<FB_OP_MP>
+                                           : k_near_fill<FB_OP_A>;
+        fill<<<grid, NF_COLS, 0, s>>>(m->g, k, m->rc, t->perm, t->leaf_start, t->ucnt, t->ulist, op->nf_off,
+                                      op->nf_ncol, op->nf64);
         FB_LAUNCH_CHECK();
     }
     // ---- box centres of every level
@@ -614,23 +852,33 @@ fb_status fb_fmm_create(fb_op* op, double d0, int pmin, cudaStream_t s) {
     // ---- P2M / L2P operators
     {
         int32_t* leaf_of = nullptr;
-        double* scratch = nullptr;
-        int nthreads = 152 * 256;
-        int Pp1 = pL + 1;
-        // even stride: each thread's slice starts with complex values (16-byte aligned)
-        int sstride = (2 * Pp1 * Pp1 + Pp1 * (Pp1 + 1) / 2 + Pp1 + 32 + 1) & ~1;
+        double* tabs = nullptr;
+        cd* sg = nullptr;
+        const int Pp1 = pL + 1, M = pL + 1;
+        // elements per CTA: up to 8 within 64 KB; S in global memory where one element's does not fit
+        const bool s_global = p2m_elem_bytes(Pp1, false) > 200 * 1024;
+        const size_t per = p2m_elem_bytes(Pp1, s_global);
+        const int E = s_global ? 1 : (int)std::max<size_t>(1, std::min<size_t>(8, 64 * 1024 / per));
+        const unsigned grid = (unsigned)std::min<int64_t>(div_up(n, E), s_global ? 304 : 1 << 30);
+        const size_t nleg = (size_t)Pp1 * (Pp1 + 1), nga = (size_t)(Pp1 + 1) * (M + 1), ngb = (size_t)(Pp1 + 1) * (2 * M + 1);
         fb_status st;
-        if ((st = dalloc(&leaf_of, n)) || (st = dalloc(&scratch, (size_t)nthreads * sstride)) ||
-            (st = dalloc(&op->w64, (size_t)n * PL)) || (st = dalloc(&op->v64, (size_t)n * PL))) {
-            dfree(leaf_of); dfree(scratch); free_centers();
+        if ((st = dalloc(&leaf_of, n)) || (st = dalloc(&tabs, nleg + Pp1 + nga + ngb)) ||
+            (s_global && (st = dalloc(&sg, (size_t)grid * E * (Pp1 * (Pp1 + 1) / 2)))) ||
+            (st = dalloc(&op->w64, (size_t)n * PL)) || (st = dalloc(&op->v64, (size_t)n * PL)) ||
+            (st = fb_smem_cap((const void*)k_p2m_l2p, E * per))) {
+            dfree(leaf_of); dfree(tabs); dfree(sg); free_centers();
             return st;
         }
         k_leaf_of<<<nleaf, 64, 0, s>>>(t->leaf_start, nleaf, leaf_of);
-        k_p2m_l2p<<<nthreads / 128, 128, 0, s>>>(m->g, op->kind, k, pL, n, t->perm, leaf_of, centers[L],
-                                                  scratch, sstride, op->w64, op->v64);
+        SphTab tab{tabs, tabs + nleg, tabs + nleg + Pp1, tabs + nleg + Pp1 + nga, M};
+        k_sph_tables<<<std::min(div_up((int64_t)Pp1 * Pp1, 128), 152), 128, 0, s>>>(
+            Pp1, M, tabs, tabs + nleg, tabs + nleg + Pp1, tabs + nleg + Pp1 + nga);
+        k_p2m_l2p<<<grid, 128, E * per, s>>>(m->g, op->kind, k, pL, n, E, tab, t->perm, leaf_of, centers[L], sg, op->w64,
+                                             op->v64);
         cudaError_t e = cudaStreamSynchronize(s);
         dfree(leaf_of);
-        dfree(scratch);
+        dfree(tabs);
+        dfree(sg);
         if (e != cudaSuccess) { free_centers(); return fb_fail(FB_ERR_CUDA, std::string("P2M/L2P setup: ") + cudaGetErrorString(e)); }
     }
     free_centers();
@@ -757,9 +1005,24 @@ fb_status fb_fmm_create(fb_op* op, double d0, int pmin, cudaStream_t s) {
     }
     if (!sets.empty()) {
         FB_CUDA(cudaMemcpyAsync(dsets, sets.data(), sizeof(CoaxSet) * sets.size(), cudaMemcpyHostToDevice, s));
-        k_coaxial<<<div_up((int64_t)sets.size(), 32), 32, 0, s>>>(dsets, (int)sets.size(), cscr, scr_stride,
-                                                                  fscr, f_stride, coax);
-        FB_LAUNCH_CHECK();
+        int P = 1;
+        for (const auto& cs : sets) P = std::max(P, cs.p);
+        const int N = 2 * P + 2, M = P + 1;   // factors of degrees < N, orders <= M
+        double* fac = nullptr;
+        if ((st = dalloc(&fac, (size_t)N * (3 * M + 2)))) {
+            free_coax();
+            return st;
+        }
+        double* facb = fac + (size_t)N * (M + 1);
+        k_coaxial_factors<<<std::min(div_up((int64_t)N * (2 * M + 1), 256), 1024), 256, 0, s>>>(N, M, fac, facb);
+        k_coaxial<<<(unsigned)sets.size(), 512, 0, s>>>(dsets, cscr, scr_stride, fscr, f_stride, fac, facb, M, coax);
+        const cudaError_t ce = cudaGetLastError();
+        cudaStreamSynchronize(s);
+        dfree(fac);
+        if (ce != cudaSuccess) {
+            free_coax();
+            return fb_fail(FB_ERR_CUDA, std::string("coaxial sets: ") + cudaGetErrorString(ce));
+        }
     }
     // rotation blocks of every direction up to pmax (cached in the tree: they
     // depend only on the directions, not on k or the operator)

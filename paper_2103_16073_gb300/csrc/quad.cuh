@@ -14,6 +14,7 @@
 #pragma once
 
 #include "common.cuh"
+#include "fastmath.cuh"
 
 #define FB_PI 3.14159265358979323846
 #define FB_INV4PI 0.079577471545947667884
@@ -65,19 +66,27 @@ __device__ __forceinline__ EdgeSums edge_sums(V3 x, const Tri& t) {
     for (int e = 0; e < 3; ++e) {
         V3 p0 = vs[e], p1 = vs[(e + 1) % 3];
         V3 ed = p1 - p0;
-        double le = norm(ed);
-        V3 tg = (1.0 / le) * ed;
+        double rle = rsqrt(dot(ed, ed));
+        V3 tg = rle * ed;
         V3 m = cross(tg, t.n);
         double lm = dot(p0 - x0, tg);
         double lp = dot(p1 - x0, tg);
         double P = dot(p0 - x0, m);
         double R0sq = P * P + d * d;
-        double R0 = sqrt(R0sq);
-        double R0s = fmax(R0, 1e-30 * le);
-        double Rm = sqrt(R0sq + lm * lm);
-        double Rp = sqrt(R0sq + lp * lp);
-        double E = asinh(lp / R0s) - asinh(lm / R0s);
-        s.inv_r += P * E - ad * (atan2(P * lp, R0sq + ad * Rp) - atan2(P * lm, R0sq + ad * Rm));
+        double R0s = fmax(R0sq, 1e-60 / (rle * rle));
+        double Rm = sqrt(R0s + lm * lm);
+        double Rp = sqrt(R0s + lp * lp);
+        // asinh(lp / R0) - asinh(lm / R0) as one logarithm, (R - l)(R + l) = R0^2
+        // keeping its argument free of cancellation
+        double num = lp >= 0.0 ? lp + Rp : Rm - lm, den = lp >= 0.0 ? lm + Rm : Rp - lp;
+        if (lp >= 0.0 && lm < 0.0) {
+            num = num * (Rm - lm);
+            den = R0s;
+        }
+        double E = log(num / den);
+        // atan2(P lp, xp) - atan2(P lm, xm) as one, both arguments right of the axis
+        double xp = R0sq + ad * Rp, xm = R0sq + ad * Rm;
+        s.inv_r += P * E - ad * atan2(P * lp * xm - P * lm * xp, xp * xm + P * P * lp * lm);
         s.medge = s.medge + E * m;
     }
     return s;
@@ -103,22 +112,58 @@ __device__ __forceinline__ cd em1(double kr) {
 //   g = G or G - 1/(4piR);  f such that dG/dn_y = (n_y.r) f / (4pi R^3),
 //   dG/dn_x = -(n_x.r) f / (4pi R^3);  f = e^{ikR}(ikR - 1) (+1 if smooth).
 __device__ __forceinline__ void kernel_pt(double k, V3 r, bool smooth, cd& g, cd& f, double& inv4piR3) {
-    double R = norm(r);
-    double kr = k * R;
-    double s, c;
-    sincos(kr, &s, &c);
-    cd E = mk(c, s);
-    cd ikR = mk(0.0, kr);
-    double i4R = FB_INV4PI / R;
+    double R;
+    const double ri = fm::inv_and_r(dot(r, r), &R);
+    const double kr = k * R;
+    const double i4R = FB_INV4PI * ri;
     if (smooth) {
-        cd e1 = em1(kr);
+        const cd e1 = em1(kr);
+        const cd E = mk(1.0 + e1.re, e1.im);
         g = i4R * e1;
-        f = ikR * E - e1;
+        f = mk(-kr * E.im - e1.re, kr * E.re - e1.im);   // ikR E - e1
     } else {
+        double s, c;
+        sincos(kr, &s, &c);
+        const cd E = mk(c, s);
         g = i4R * E;
         f = E * mk(-1.0, kr);
     }
-    inv4piR3 = i4R / (R * R);
+    inv4piR3 = i4R * (ri * ri);
+}
+
+// Far entry (3-point rule) of operator kind KIND (FB_OP_L, M, LP or A): the
+// sum of a w_q / (4 pi R) e^{ikR} z over the Gauss points y_q, with
+//   z = 1 (L),  dn (ikR - 1) (M),  -dx (ikR - 1) (L'),  dn (ikR - 1) - ik beta (A),
+// dn = n_y.r / R^2 and dx = n_x.r / R^2; on a flat element n_y.r is the same
+// for every point, n_y.(c - x).  About 45 FP64 operations per point.
+template <int KIND>
+__device__ __forceinline__ cd far_entry(const double2* sc, double k, const V3 (&y)[3], double area, double nr, V3 x,
+                                        V3 nx, cd ikb) {
+    cd acc = mk(0.0, 0.0);
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        const V3 r = y[q] - x;
+        double R, s, c;
+        const double w = fm::inv_and_r(dot(r, r), &R);
+        const double kr = k * R;
+        fm::sincos_tab(sc, kr, &s, &c);
+        double zr = 1.0, zi = 0.0;
+        if (KIND != FB_OP_L) {
+            const double d = (KIND == FB_OP_LP ? -dot(nx, r) : nr) * (w * w);
+            zr = -d;
+            zi = d * kr;
+            if (KIND == FB_OP_A) {
+                zr -= ikb.re;
+                zi -= ikb.im;
+            }
+            acc.re = fma(w, c * zr - s * zi, acc.re);
+            acc.im = fma(w, c * zi + s * zr, acc.im);
+        } else {
+            acc.re = fma(w, c, acc.re);
+            acc.im = fma(w, s, acc.im);
+        }
+    }
+    return (area * (FB_INV4PI / 3.0)) * acc;
 }
 
 // Degree-5 seven-point rule (Radon): barycentrics and weights.

@@ -54,10 +54,11 @@ __device__ inline void sph_bessel_j(int nmax, double x, double* j) {
         return;
     }
     int start = nmax + 24 + (int)x;
+    const double ix = 1.0 / x;
     double fp = 0.0, f = 1e-280;
     for (int n = 0; n <= nmax; ++n) j[n] = 0.0;
     for (int n = start; n >= 1; --n) {
-        double fm = (2.0 * n + 1.0) / x * f - fp;
+        double fm = (2.0 * n + 1.0) * ix * f - fp;
         fp = f;
         f = fm;             // f = f_{n-1}, fp = f_n
         if (n - 1 <= nmax) j[n - 1] = f;
@@ -100,38 +101,4 @@ __device__ inline void ylm_unit(int P, double ux, double uy, double uz, double* 
         }
         em = em * e1;
     }
-}
-
-// R_n^m(r) for n < P: out[nm_idx(n,m)].  scratch: P(P+1)/2 + P + 24 doubles.
-__device__ inline void regular_all(int P, double k, V3 r, double* scratch, cd* out) {
-    double rho = norm(r);
-    double* q = scratch;
-    double* jn = scratch + P * (P + 1) / 2;
-    if (rho == 0.0) {
-        for (int i = 0; i < P * P; ++i) out[i] = mk(0.0, 0.0);
-        out[0] = mk(0.28209479177387814347, 0.0);
-        return;
-    }
-    ylm_unit(P, r.x / rho, r.y / rho, r.z / rho, q, out);
-    sph_bessel_j(P - 1, k * rho, jn);
-    for (int n = 0; n < P; ++n)
-        for (int m = -n; m <= n; ++m) out[nm_idx(n, m)] = jn[n] * out[nm_idx(n, m)];
-}
-
-// n . grad R_n^mu for n < P from R up to degree P (array Rv of (P+1)^2):
-//   dz R_n^u      = k [a_{n-1}^u R_{n-1}^u - a_n^u R_{n+1}^u]
-//   (dx+idy) R_n^u = k [-b_n^u R_{n-1}^{u+1} + b_{n+1}^{-u-1} R_{n+1}^{u+1}]
-//   (dx-idy) R_n^u = k [-b_n^{-u} R_{n-1}^{u-1} + b_{n+1}^{u-1} R_{n+1}^{u-1}]
-//   n.grad = (nx - i ny)/2 (dx+idy) + (nx + i ny)/2 (dx-idy) + nz dz
-__device__ __forceinline__ cd rget(const cd* Rv, int Pp1, int n, int m) {
-    if (n < 0 || n >= Pp1 || abs(m) > n) return mk(0.0, 0.0);
-    return Rv[nm_idx(n, m)];
-}
-__device__ inline cd ndot_grad_regular(const cd* Rv, int P, double k, V3 nv, int n, int u) {
-    int Pp1 = P + 1;
-    cd dz = k * (coef_a(n - 1, u) * rget(Rv, Pp1, n - 1, u) - coef_a(n, u) * rget(Rv, Pp1, n + 1, u));
-    cd dp = k * ((-coef_b(n, u)) * rget(Rv, Pp1, n - 1, u + 1) + coef_b(n + 1, -u - 1) * rget(Rv, Pp1, n + 1, u + 1));
-    cd dm = k * ((-coef_b(n, -u)) * rget(Rv, Pp1, n - 1, u - 1) + coef_b(n + 1, u - 1) * rget(Rv, Pp1, n + 1, u - 1));
-    cd hp = mk(0.5 * nv.x, -0.5 * nv.y), hm = mk(0.5 * nv.x, 0.5 * nv.y);
-    return hp * dp + hm * dm + nv.z * dz;
 }
