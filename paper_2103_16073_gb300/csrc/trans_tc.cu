@@ -1,4 +1,5 @@
-// Stacked M2L translations on the 5th-generation tensor cores (tcgen05).
+// Stacked translations of composed matrices on the 5th-generation tensor
+// cores (tcgen05).
 //
 // All box pairs of one level that share a translation vector share one
 // composed translation matrix T (p^2 x p^2 complex, Sec. 3.3 RCR composed in
@@ -7,29 +8,49 @@
 // columns,
 //     [Y_re(r)]   [ T_re  -T_im ] [X_re]
 //     [Y_im(r)] = [ T_im   T_re ] [X_im],
+// transposed, so that the matrix rows are the MMA's N:
+//     D[pair][row] = sum_k X[pair][k] T[row][k]
 // in 3xTF32: every FP32 operand is split into hi (TF32) + lo, and
-// D += A_hi B_hi + A_hi B_lo + A_lo B_hi with FP32 accumulation in tensor
+// D += X_hi T_hi + X_lo T_hi + X_hi T_lo with FP32 accumulation in tensor
 // memory.
 //
-// Operands:  A = real T rows, M = 128 per tile, pre-split and stored in
-// global memory already in the canonical no-swizzle K-major layout, one
-// 16 KB (hi + lo) block per (row tile, K chunk of 16) -> one bulk TMA copy.
-// B = gathered X columns, N <= 256 per tile, from hi/lo planes of the level
-// multipoles written once per matvec by k_tc_split -> 16-byte cp.async
-// pieces into the canonical layout.
+// Tile: 128 pairs x a block of rows of T (at most 224, in equal blocks padded
+// to 16), accumulators double-buffered in tensor memory.
 //
-// Pipeline (8 warps, 2 shared-memory stages of 48 KB, two CTAs per SM):
-//   warps 0-5  B producers (cp.async, completion tracked by the stage's
-//              "full" mbarrier), warp 6 lane 0 A producer (bulk copy with
-//              transaction count), warp 7 lane 0 MMA issuer (waits "full",
-//              issues 6 MMAs, commits to the stage's "empty" mbarrier);
-//   epilogue   all warps: tcgen05.ld of the accumulator (warps w and w+4
-//              share lane quadrant w % 4 and split the columns), atomic
-//              scatter-add into the target locals.
+// Operands:  A = gathered X rows, read as FP32 and split by the producer
+// warps on the way into the canonical layout.  B = T, pre-split and stored in
+// global memory already in the canonical no-swizzle K-major layout, one block
+// (hi then lo) per (row tile, K chunk of 16).  Streaming T for every 128
+// pairs is what bounds a dense level (order 12: 663 KB per 128 pairs, at 6.6
+// TB/s out of L2 0.74 ms of level 7 below), so the tiles of one matrix run in
+// clusters of four that load a share each and multicast it to the others'
+// stages.
+//
+// Persistent: every cluster walks over its share of the tiles with each role
+// running ahead of the next (a tile's setup, a chain of dependent loads, and
+// its scatter cost as much as its MMAs at order 12):
+//   warps 0-7    A producers: warp w takes every fourth chunk (w % 4) of 64
+//                pairs (w / 4), so that a chunk's fixed cost (waits, proxy
+//                fence, arrival) is spread over eight pieces per lane, with
+//                the loads of its next chunk in flight;
+//   warp 8       lane 0: bulk copies of T (transaction count);
+//   warp 9       lane 0: MMA issuer (6 MMAs per chunk, commits to the stage's
+//                "empty" barrier in every CTA of the cluster, which keeps the
+//                four in step);
+//   warps 10-17  epilogue: accumulator rows (lane = pair) through shared
+//                memory, so that the atomic adds into the targets are
+//                coalesced runs of one pair's coefficients;
+//   warp 18      source offsets of the next tiles into a ring in shared
+//                memory, ahead of the producers.
+// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 1.20 ms (the
+// MMAs alone 0.68 ms); 1.87 ms with pairs as N, one tile per CTA and hi/lo
+// planes of X split in a pass of its own.  The three tensor levels together
+// 2.21 ms against 3.54 ms; of the shoebox at 1 kHz 0.26 against 0.36 ms.
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // flag, drains its own copies and MMAs (bounded) and releases tensor memory.
 #include <algorithm>
 #include <atomic>
+#include <functional>
 
 #include <map>
 
@@ -38,23 +59,50 @@
 
 namespace {
 
-constexpr int TC_M = 128;       // real output rows per tile
-constexpr int TC_NMAX = 256;    // box pairs per tile
-constexpr int TC_KC = 16;       // real K per stage
-constexpr int TC_STAGES = 2;   // two 48 KB stages: two CTAs (and 2 x 256 TMEM columns) per SM
-constexpr int A_BLOCK = TC_M * TC_KC;       // floats per (hi or lo) A block
-constexpr int B_BLOCK = TC_NMAX * TC_KC;    // floats per (hi or lo) B block
-constexpr int STAGE_FLOATS = 2 * A_BLOCK + 2 * B_BLOCK;
-constexpr int NPROD = 192;                  // B producer threads (warps 0-5)
+constexpr int TC_PAIRS = 128;     // box pairs per tile (MMA M)
+constexpr int TC_RMAX = 224;      // real output rows per tile (MMA N <= 256; four stages must fit)
+constexpr int TC_KC = 16;         // real K per stage
+constexpr int TC_STAGES = 6;      // at most
+constexpr int A_BLOCK = TC_PAIRS * TC_KC;   // floats per (hi or lo) block of X
+constexpr int PROD_WARPS = 8;     // warps 0-7
+constexpr int EPI_WARPS = 8;      // warps 10-17
+constexpr int IDX_WARP = 10 + EPI_WARPS;
+constexpr int TC_THREADS = 32 * (IDX_WARP + 1);
+constexpr int TC_RING = 4;        // tiles of source offsets in shared memory
+constexpr int TC_CS = 32;         // accumulator columns staged per epilogue pass
+constexpr int TC_STAGING = EPI_WARPS * 32 * (TC_CS + 4);   // floats
+constexpr int TC_CLUSTER = 4;     // CTAs per cluster
+// drain bound of the shared copies: they land within microseconds, but after
+// a peer's timeout a stage may never get that peer's share
+constexpr long long SHARE_DRAIN = 1LL << 20;
 using tcx::canon;
 using tcx::DRAIN_LIMIT;
 using tcx::LBO;
+using tcx::mbar_init;
 using tcx::mbar_wait;
+using tcx::mma_commit;
 using tcx::mma_tf32;
 using tcx::smem_u32;
 using tcx::tf32_hi;
 using tcx::umma_desc;
 static_assert(TC_KC == tcx::KC, "one canonical block width");
+
+__device__ __forceinline__ uint32_t cluster_rank() {
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+    asm volatile("barrier.cluster.arrive.release.aligned;");
+    asm volatile("barrier.cluster.wait.acquire.aligned;");
+}
+// arrives on `bar` in every CTA of the mask once the MMAs issued so far are complete
+__device__ __forceinline__ void mma_commit_to(uint64_t* bar, uint16_t mask) {
+    asm volatile(
+        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
+            smem_u32(bar)),
+        "h"(mask));
+}
 
 }  // namespace
 
@@ -62,26 +110,31 @@ struct TcTask {
     int64_t a_off;          // float offset of the pre-split tiles of T
     int64_t pair_off;
     int32_t npairs, nrt, nkc, p_out2;   // p_out2 = complex rows P_out
+    int32_t rt_rows;                    // real rows per row tile (multiple of 16, <= TC_RMAX)
     int32_t p_in2;                      // complex columns P_in
-    int32_t stride_f;                   // floats per box vector in the hi/lo planes
-    int64_t plane_base;                 // float offset of the level in the planes
-    int64_t dst_base;                   // complex offset of the target level
-    int32_t nbox_src;                   // boxes of the source level (planes hold nrhs sets)
-    int32_t pad;
+    int64_t src_base, dst_base;         // complex offsets of the source and target levels
 };
-struct TcTile {
-    int32_t task, rt, col0, ncol;
+// Columns [col0, col0 + ncol) of a task (ncol = 0 fills a cluster), real rows
+// from row0 on.  Its T is shared by the scount (1, 2 or 4) CTAs of the cluster
+// from rank sbase on.  The four tiles of a cluster have the same nkc and nrow.
+struct alignas(16) TcTile {
+    int64_t t_off, pair_off, src_base, dst_base;
+    int32_t p_in2, p_out2, nkc, nrow;
+    int32_t row0, col0;
+    int16_t ncol, sbase, scount, pad;
 };
 
 // Pre-split canonical tiles of the real interleaved form of a complex matrix.
-__global__ void k_tc_pack(const cd* __restrict__ T, int rows, int cols, int nrt, int nkc, float* __restrict__ out) {
-    int64_t total = (int64_t)nrt * nkc * A_BLOCK;
+__global__ void k_tc_pack(const cd* __restrict__ T, int rows, int cols, int nrt, int nkc, int rt_rows,
+                          float* __restrict__ out) {
+    const int blk_f = rt_rows * TC_KC;
+    int64_t total = (int64_t)nrt * nkc * blk_f;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t blk = i / A_BLOCK;
-        int e = (int)(i % A_BLOCK);
+        int64_t blk = i / blk_f;
+        int e = (int)(i % blk_f);
         int rt = (int)(blk / nkc), kc = (int)(blk % nkc);
         int ri = e / TC_KC, ki = e % TC_KC;
-        int rr = rt * TC_M + ri, kk = kc * TC_KC + ki;
+        int rr = rt * rt_rows + ri, kk = kc * TC_KC + ki;
         int r = rr >> 1, sr = rr & 1, k = kk >> 1, sk = kk & 1;
         double v = 0.0;
         if (r < rows && k < cols) {
@@ -91,252 +144,527 @@ __global__ void k_tc_pack(const cd* __restrict__ T, int rows, int cols, int nrt,
         float f = (float)v;
         float hi = tf32_hi(f);
         float lo = (float)(v - (double)hi);
-        float* base = out + blk * 2 * A_BLOCK;
+        float* base = out + blk * 2 * blk_f;
         int off = canon(ri, ki) >> 2;
         base[off] = hi;
-        base[A_BLOCK + off] = lo;
+        base[blk_f + off] = lo;
     }
 }
 
-// hi/lo planes of the multipoles of the tensor-core levels: box vectors of
-// 2P floats padded to stride_f (multiple of 4) with zeros.
-struct SplitLevel {
-    int64_t src_base;     // complex offset of the level in the multipoles
-    int64_t plane_base;   // float offset in the planes
-    int32_t nbox, P, stride_f, pad;
+struct TcArgs {
+    const TcTile* tiles;
+    int nct;           // clusters of tiles
+    const float* T;
+    const int32_t* src_idx;
+    const int32_t* dst_idx;
+    const cf* src;
+    cf* dst;
+    int* err;
+    int nrhs;
+    int64_t rstride;
+    long long wait_limit;
+    int inject_stall;
+    int nst;           // pipeline stages
+    int stage_floats;  // A hi, A lo, then the largest T block (hi, lo)
+    int acc_cols;      // tensor memory columns of one accumulator
 };
-// With nrhs right-hand sides a level's planes hold nrhs sets of nbox vectors
-// (plane_base scaled by nrhs), set r read from mp + r * rstride.
-__global__ void k_tc_split(const SplitLevel* __restrict__ lv, int nlev, const cf* __restrict__ mp,
-                           float* __restrict__ hi, float* __restrict__ lo, int nrhs, int64_t rstride) {
-    int l = blockIdx.y;
-    if (l >= nlev) return;
-    SplitLevel L = lv[l];
-    int64_t per = (int64_t)L.nbox * L.stride_f;
-    int64_t total = per * nrhs;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < total; i += (int64_t)gridDim.x * blockDim.x) {
-        int64_t r = i / per, ib = i - r * per;
-        int64_t b = ib / L.stride_f;
-        int k = (int)(ib % L.stride_f);
-        const float* src = (const float*)(mp + r * rstride + L.src_base);
-        float v = k < 2 * L.P ? src[b * 2 * L.P + k] : 0.f;
-        float h = tf32_hi(v);
-        hi[L.plane_base * nrhs + i] = h;
-        lo[L.plane_base * nrhs + i] = v - h;
-    }
+
+// 32 consecutive accumulator columns of this thread's lane
+__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
+    asm volatile(
+        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
+        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
+          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
+          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
+          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
+        : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
-__global__ void __launch_bounds__(256, 2) k_trans_tc(const TcTask* __restrict__ tasks, const TcTile* __restrict__ tiles,
-                                                      const float* __restrict__ Abuf, const int32_t* __restrict__ src_idx,
-                                                      const int32_t* __restrict__ dst_idx,
-                                                      const float* __restrict__ plane_hi,
-                                                      const float* __restrict__ plane_lo, cf* __restrict__ dst,
-                                                      int* __restrict__ err, int nrhs, int64_t rstride,
-                                                      long long wait_limit, int inject_stall) {
+__global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[TC_STAGES];    // B producers' cp.async pieces
-    __shared__ __align__(8) uint64_t a_bar[TC_STAGES];       // the A producer's bulk copy
-    __shared__ __align__(8) uint64_t empty_bar[TC_STAGES];
+    __shared__ __align__(8) uint64_t full_bar[TC_STAGES];    // A producers' stores
+    __shared__ __align__(8) uint64_t b_bar[TC_STAGES];       // the bulk copies of T
+    __shared__ __align__(8) uint64_t empty_bar[TC_STAGES];   // the MMAs of every CTA of the cluster
+    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
     __shared__ __align__(8) uint64_t done_bar;
     __shared__ __align__(8) uint64_t never_bar;              // test hook: nothing arrives on it
+    __shared__ __align__(8) uint64_t idx_full[TC_RING], idx_empty[TC_RING];
+    __shared__ int64_t s_src[TC_RING][TC_PAIRS];   // source expansion (complex), -1: no pair
+    __shared__ int s_nkc[TC_RING], s_len[TC_RING];  // chunks; floats of a source expansion
     __shared__ uint32_t tmem_holder;
-    __shared__ int s_src[TC_NMAX];       // source vector index in the planes (rhs * nbox + box)
-    __shared__ int s_dst[TC_NMAX];
-    __shared__ int s_rhs[TC_NMAX];
     __shared__ int s_fail;
-    uint32_t raw = smem_u32(smem_raw);
-    uint32_t pad = (1024 - (raw & 1023)) & 1023;
+    const uint32_t raw = smem_u32(smem_raw);
+    const uint32_t pad = (1024 - (raw & 1023)) & 1023;
     float* stage0 = (float*)(smem_raw + pad);
 
-    const TcTile tl = tiles[blockIdx.x];
-    const TcTask tk = tasks[tl.task];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int ncol = tl.ncol;
-    const int nmma = (ncol + 15) & ~15;
-    const int nkc = tk.nkc;
-    // column j: pair (col0 + j) / nrhs, right-hand side (col0 + j) % nrhs
-    for (int j = tid; j < TC_NMAX; j += blockDim.x) {
-        bool ok = j < ncol;
-        int col = tl.col0 + j;
-        int pr = col / nrhs, rh = col - pr * nrhs;
-        s_src[j] = ok ? rh * tk.nbox_src + src_idx[tk.pair_off + pr] : -1;
-        s_dst[j] = ok ? dst_idx[tk.pair_off + pr] : -1;
-        s_rhs[j] = ok ? rh : 0;
-    }
+    const int nst = a.nst, rank = (int)cluster_rank();
+    const int ct0 = blockIdx.x / TC_CLUSTER, ncl = gridDim.x / TC_CLUSTER;
+    const TcTile* tiles = a.tiles + rank;   // this CTA's tile of cluster tile ct: tiles[ct * TC_CLUSTER]
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(TC_NMAX));
+                     "r"(2 * a.acc_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
         s_fail = 0;
         for (int s = 0; s < TC_STAGES; ++s) {
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&full_bar[s])), "r"(NPROD));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&a_bar[s])), "r"(1));
-            asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&empty_bar[s])), "r"(1));
+            mbar_init(&full_bar[s], PROD_WARPS / 4);   // the two warps of a chunk
+            mbar_init(&b_bar[s], 1);
+            mbar_init(&empty_bar[s], TC_CLUSTER);
         }
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&done_bar)), "r"(1));
-        asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(&never_bar)), "r"(1));
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], EPI_WARPS);
+        }
+        for (int r = 0; r < TC_RING; ++r) {
+            mbar_init(&idx_full[r], 1);
+            mbar_init(&idx_empty[r], PROD_WARPS);
+        }
+        mbar_init(&done_bar, 1);
+        mbar_init(&never_bar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;");
     }
     asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
+    cluster_sync();   // every CTA's barriers are there before a peer signals them
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_holder;
 
-    if (warp < 6) {
-        // ---------------- B producers: 16-byte cp.async pieces -------------
-        const int npieces = nmma * (TC_KC / 4) * 2;   // columns x K pieces x {hi, lo}
-        for (int c = 0; c < nkc; ++c) {
-            const int s = c % TC_STAGES, u = c / TC_STAGES;
-            if (u > 0 && !mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, wait_limit)) {
+    if (warp < PROD_WARPS) {
+        // ---------------- A producers: 8 (pair, 4 K values) pieces a lane ----
+        // eight consecutive lanes store one 128-byte core matrix (no bank conflicts)
+        const int quarter = lane >> 3, jb = (warp >> 2) * 64 + (lane & 7);   // pairs jb + 8 i
+        const int d0 = canon(jb, 4 * quarter) >> 2, dstep = tcx::SBO / 4;     // stage offset of piece i: d0 + i dstep
+        const float* g[8];
+        int len = 0;             // floats of a source expansion from the lane's quarter on
+        uint32_t has = 0;        // pieces with a pair
+        bool al = true;          // every piece 16-byte aligned
+        int c = warp & 3, nkc = 0, it = -1, ct = ct0 - ncl;   // load cursor: chunk of tile it
+        bool fail = false;
+        // moves the cursor to this warp's next chunk; false at the end
+        auto seek = [&]() -> bool {
+            while (c >= nkc) {
+                if (it >= 0 && lane == 0)   // the tile's offsets are no longer needed
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_empty[it % TC_RING])));
+                c -= nkc;
+                nkc = 0;
+                ++it;
+                ct += ncl;
+                if (ct >= a.nct) return false;
+                const int r = it % TC_RING;
+                const bool ok = mbar_wait(smem_u32(&idx_full[r]), (it / TC_RING) & 1, a.wait_limit);
+                if (!__all_sync(0xffffffffu, ok)) {
+                    atomicExch(&s_fail, 1);
+                    fail = true;
+                    return false;
+                }
+                nkc = s_nkc[r];
+                if (c < nkc) {
+                    len = s_len[r] - 4 * quarter;
+                    has = 0;
+                    al = true;
+#pragma unroll
+                    for (int i = 0; i < 8; ++i) {
+                        const int64_t o = s_src[r][jb + 8 * i];
+                        if (o >= 0) has |= 1u << i;
+                        g[i] = (const float*)(a.src + (o >= 0 ? o : 0)) + 4 * quarter;
+                        al = al && ((uintptr_t)g[i] & 15) == 0;
+                    }
+                }
+                __syncwarp();
+            }
+            return true;
+        };
+        auto fetch = [&](float4 (&v)[8]) {
+            const int n = len - c * TC_KC;   // an even count
+            if (al && n >= 4) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    v[i] = has >> i & 1 ? __ldg(reinterpret_cast<const float4*>(g[i] + c * TC_KC))
+                                        : make_float4(0.f, 0.f, 0.f, 0.f);
+            } else {
+#pragma unroll
+                for (int i = 0; i < 8; ++i) {
+                    float2 p = make_float2(0.f, 0.f), q = p;
+                    if ((has >> i & 1) && n >= 2) p = __ldg(reinterpret_cast<const float2*>(g[i] + c * TC_KC));
+                    if ((has >> i & 1) && n >= 4) q = __ldg(reinterpret_cast<const float2*>(g[i] + c * TC_KC) + 1);
+                    v[i] = make_float4(p.x, p.y, q.x, q.y);
+                }
+            }
+            c += 4;
+        };
+        float4 cur[8], nxt[8];
+        bool more = seek();
+        if (more) fetch(cur);
+        for (int s = warp & 3, u = 0; more; s += 4) {   // stage s of its u-th use
+            const bool next = seek();
+            if (next) fetch(nxt);
+            while (s >= nst) {
+                s -= nst;
+                ++u;
+            }
+            const bool ok = u == 0 || mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, a.wait_limit);
+            if (!__all_sync(0xffffffffu, ok)) {
                 atomicExch(&s_fail, 1);
                 break;
             }
-            float* sBh = stage0 + s * STAGE_FLOATS + 2 * A_BLOCK;
-            for (int i = tid; i < npieces; i += NPROD) {
-                int plane = i & 1;
-                int q = (i >> 1) % (TC_KC / 4);
-                int j = (i >> 1) / (TC_KC / 4);
-                int k = c * TC_KC + 4 * q;
-                int sb = s_src[j];
-                const float* pl = plane ? plane_lo : plane_hi;
-                const int64_t base = tk.plane_base * nrhs;
-                const float* g = pl + base;   // valid address even when nothing is read
-                int bytes = 0;
-                if (sb >= 0 && k < tk.stride_f) {
-                    g = pl + base + (int64_t)sb * tk.stride_f + k;
-                    bytes = 16;
-                }
-                uint32_t d = smem_u32(sBh + plane * B_BLOCK) + canon(j, 4 * q);
-                asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(g), "r"(bytes));
+            float* st = stage0 + (size_t)s * a.stage_floats + d0;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                const float4 x = cur[i];
+                const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+                *reinterpret_cast<float4*>(st + i * dstep) = h;
+                *reinterpret_cast<float4*>(st + A_BLOCK + i * dstep) =
+                    make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+                cur[i] = nxt[i];
             }
-            asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" ::"r"(smem_u32(&full_bar[s])));
+            // generic-proxy stores become visible to the tensor core's reads
+            asm volatile("fence.proxy.async.shared::cta;");
+            __syncwarp();
+            if (lane == 0)
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])));
+            more = next;
         }
-        asm volatile("cp.async.wait_all;");
-    } else if (warp == 6) {
-        // ---------------- A producer: one bulk copy per stage ----------------
+    } else if (warp == 8) {
+        // ---------------- T: this CTA's share of every stage, to all sharers --
         if (lane == 0) {
-            const float* Atile = Abuf + tk.a_off + (int64_t)tl.rt * nkc * 2 * A_BLOCK;
-            int issued = 0;
-            for (int c = 0; c < nkc; ++c) {
-                const int s = c % TC_STAGES, u = c / TC_STAGES;
-                if (u > 0 && !mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, wait_limit)) {
-                    atomicExch(&s_fail, 1);
-                    break;
+            int64_t cc = 0;
+            int s = 0;
+            uint32_t ph = 1;
+            bool fail = false;
+            TcTile tn;
+            if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
+            for (int ct = ct0; ct < a.nct && !fail; ct += ncl) {
+                const TcTile tl = tn;
+                if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
+                const int blk = 2 * tl.nrow * TC_KC, part = blk / tl.scount, off = (rank - tl.sbase) * part;
+                const uint16_t smask = (uint16_t)(((1 << tl.scount) - 1) << tl.sbase);
+                const float* g = a.T + tl.t_off + off;
+                for (int c = 0; c < tl.nkc; ++c, ++cc, g += blk) {
+                    if (cc >= nst && !mbar_wait(smem_u32(&empty_bar[s]), ph, a.wait_limit)) {
+                        atomicExch(&s_fail, 1);
+                        fail = true;
+                        break;
+                    }
+                    const uint32_t bb = smem_u32(&b_bar[s]);
+                    const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_BLOCK + off);
+                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb),
+                                 "r"((uint32_t)(blk * sizeof(float))));
+                    if (tl.scount == 1)
+                        asm volatile(
+                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                dB),
+                            "l"(g), "r"((uint32_t)(blk * sizeof(float))), "r"(bb));
+                    else
+                        asm volatile(
+                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
+                            "[%1], %2, [%3], %4;" ::"r"(dB),
+                            "l"(g), "r"((uint32_t)(part * sizeof(float))), "r"(bb), "h"(smask));
+                    if (++s == nst) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
-                uint32_t ab = smem_u32(&a_bar[s]);
-                uint32_t dA = smem_u32(stage0 + s * STAGE_FLOATS);
-                const float* g = Atile + (int64_t)c * 2 * A_BLOCK;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(ab), "r"(2 * A_BLOCK * 4));
-                asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dA),
-                    "l"(g), "r"(2 * A_BLOCK * 4), "r"(ab));
-                ++issued;
             }
-            // every bulk copy this CTA issued lands before the CTA may exit
-            // (on success the MMA issuer has already waited for each of them)
-            for (int c = max(0, issued - TC_STAGES); c < issued; ++c)
-                mbar_wait(smem_u32(&a_bar[c % TC_STAGES]), (c / TC_STAGES) & 1, DRAIN_LIMIT);
+            // every copy into this CTA lands before it may exit (on success the
+            // MMA issuer has already waited for each of them)
+            for (int64_t k = cc > nst ? cc - nst : 0; k < cc; ++k)
+                mbar_wait(smem_u32(&b_bar[k % nst]), (uint32_t)(k / nst) & 1, SHARE_DRAIN);
         }
         __syncwarp();
-    } else {
+    } else if (warp == 9) {
         // ---------------- MMA issuer ----------------------------------------
         if (lane == 0) {
-            const uint32_t idesc = (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(nmma >> 3) << 17) |
-                                   ((uint32_t)(TC_M >> 4) << 24);
             // test hook: a wait on a barrier nothing arrives on runs out
-            const bool stalled = inject_stall && !mbar_wait(smem_u32(&never_bar), 0, wait_limit);
-            if (stalled) atomicExch(&s_fail, 1);
-            for (int c = 0; c < nkc && !stalled; ++c) {
-                const int s = c % TC_STAGES, u = c / TC_STAGES;
-                if (!mbar_wait(smem_u32(&full_bar[s]), u & 1, wait_limit) ||
-                    !mbar_wait(smem_u32(&a_bar[s]), u & 1, wait_limit)) {
+            bool fail = a.inject_stall && !mbar_wait(smem_u32(&never_bar), 0, a.wait_limit);
+            if (fail) atomicExch(&s_fail, 1);
+            int s = 0, it = 0;
+            uint32_t ph = 0;
+            // operand descriptors differ in their start address alone, a field of
+            // 16-byte units that no sum below carries out of (shared memory ends
+            // below its 256 KB): one add each, the single thread's issue chain
+            // being as long as the MMAs themselves otherwise
+            const uint64_t dsc0 = umma_desc(smem_u32(stage0)), dstep = (uint64_t)(a.stage_floats * 4) >> 4;
+            uint64_t dsc = dsc0;
+            int nkc_n = 0, nrow_n = 0;
+            if (ct0 < a.nct) {
+                nkc_n = tiles[(int64_t)ct0 * TC_CLUSTER].nkc;
+                nrow_n = tiles[(int64_t)ct0 * TC_CLUSTER].nrow;
+            }
+            for (int ct = ct0; ct < a.nct && !fail; ct += ncl, ++it) {
+                const int nkc = nkc_n, nrow = nrow_n;
+                if (ct + ncl < a.nct) {
+                    nkc_n = tiles[(int64_t)(ct + ncl) * TC_CLUSTER].nkc;
+                    nrow_n = tiles[(int64_t)(ct + ncl) * TC_CLUSTER].nrow;
+                }
+                const int b = it & 1;
+                if (it >= 2 && !mbar_wait(smem_u32(&acc_empty[b]), ((it >> 1) - 1) & 1, a.wait_limit)) {
                     atomicExch(&s_fail, 1);
                     break;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                float* st = stage0 + s * STAGE_FLOATS;
-                uint32_t aH = smem_u32(st), aL = smem_u32(st + A_BLOCK);
-                uint32_t bH = smem_u32(st + 2 * A_BLOCK), bL = smem_u32(st + 2 * A_BLOCK + B_BLOCK);
+                const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols);
+                const uint32_t idesc = tcx::idesc_tf32(TC_PAIRS, nrow);
+                const uint64_t blo = (uint64_t)(nrow * TC_KC * 4) >> 4;   // from T's hi block to its lo block
+                for (int c = 0; c < nkc; ++c) {
+                    if (!mbar_wait(smem_u32(&full_bar[s]), ph, a.wait_limit) ||
+                        !mbar_wait(smem_u32(&b_bar[s]), ph, a.wait_limit)) {
+                        atomicExch(&s_fail, 1);
+                        fail = true;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-                for (int ks = 0; ks < TC_KC / 8; ++ks) {
-                    uint32_t o = ks * 2 * LBO;
-                    uint32_t first = (c == 0 && ks == 0) ? 0u : 1u;
-                    mma_tf32(tmem, umma_desc(aH + o), umma_desc(bH + o), idesc, first);
-                    mma_tf32(tmem, umma_desc(aH + o), umma_desc(bL + o), idesc, 1u);
-                    mma_tf32(tmem, umma_desc(aL + o), umma_desc(bH + o), idesc, 1u);
+                    for (int ks = 0; ks < TC_KC / 8; ++ks) {
+                        const uint64_t aH = dsc + (uint64_t)((ks * 2 * LBO) >> 4), bH = aH + ((2 * A_BLOCK * 4) >> 4);
+                        mma_tf32(acc, aH, bH, idesc, ks == 0 ? (uint32_t)c : 1u);
+                        mma_tf32(acc, aH + ((A_BLOCK * 4) >> 4), bH, idesc, 1u);
+                        mma_tf32(acc, aH, bH + blo, idesc, 1u);
+                    }
+                    mma_commit_to(&empty_bar[s], (uint16_t)((1 << TC_CLUSTER) - 1));
+                    dsc += dstep;
+                    if (++s == nst) {
+                        s = 0;
+                        ph ^= 1;
+                        dsc = dsc0;
+                    }
                 }
-                asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                    smem_u32(&empty_bar[s])));
+                if (!fail) mma_commit(&acc_full[b]);
             }
             // completion of every MMA issued above (also on failure)
-            asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(
-                smem_u32(&done_bar)));
+            mma_commit(&done_bar);
         }
         __syncwarp();
-    }
-
-    // ---------------- epilogue ------------------------------------------------
-    bool done = mbar_wait(smem_u32(&done_bar), 0, DRAIN_LIMIT);
-    __syncthreads();
-    const bool ok = done && s_fail == 0;
-    if (!ok && tid == 0) atomicExch(err, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok) {
-        const int quad = warp & 3;
-        const int half = warp >> 2;
-        const int rr = tl.rt * TC_M + quad * 32 + lane;      // real output row
-        const int r = rr >> 1, part = rr & 1;
-        const int cmid = ((nmma / 16 + 1) / 2) * 16;        // split on 16-column boundaries
-        const int cbeg = half ? cmid : 0;
-        const int cend = half ? nmma : cmid;
-        for (int c0 = cbeg; c0 < cend; c0 += 16) {
-            uint32_t v[16];
-            uint32_t taddr = tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)c0;
-            asm volatile(
-                "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-                : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-                  "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15])
-                : "r"(taddr));
-            asm volatile("tcgen05.wait::ld.sync.aligned;");
-            if (r < tk.p_out2) {
+    } else if (warp == IDX_WARP) {
+        // ---------------- source offsets, up to TC_RING tiles ahead -----------
+        TcTile tn;
+        if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
+        int it = 0;
+        for (int ct = ct0; ct < a.nct; ct += ncl, ++it) {
+            const TcTile tl = tn;
+            if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
+            int64_t o[TC_PAIRS / 32];
 #pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    int j = c0 + q;
-                    int db = s_dst[j];
-                    if (db < 0) continue;
-                    float* d = (float*)(dst + s_rhs[j] * rstride + tk.dst_base + (int64_t)db * tk.p_out2 + r) +
-                               part;
-                    atomicAdd(d, __uint_as_float(v[q]));
+            for (int q = 0; q < TC_PAIRS / 32; ++q) {
+                const int j = q * 32 + lane;
+                o[q] = -1;
+                if (j < tl.ncol) {
+                    const int col = tl.col0 + j, pr = col / a.nrhs;
+                    o[q] = (int64_t)(col - pr * a.nrhs) * a.rstride + tl.src_base +
+                           (int64_t)a.src_idx[tl.pair_off + pr] * tl.p_in2;
                 }
             }
+            const int r = it % TC_RING;
+            const bool ok = it < TC_RING || mbar_wait(smem_u32(&idx_empty[r]), (it / TC_RING - 1) & 1, a.wait_limit);
+            if (!__all_sync(0xffffffffu, ok)) {
+                atomicExch(&s_fail, 1);
+                break;
+            }
+#pragma unroll
+            for (int q = 0; q < TC_PAIRS / 32; ++q) s_src[r][q * 32 + lane] = o[q];
+            if (lane == 0) {
+                s_nkc[r] = tl.nkc;
+                s_len[r] = 2 * tl.p_in2;
+            }
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_full[r])));
+        }
+    } else {
+        // ---------------- epilogue: accumulator lanes 32 quad .. 32 quad + 31,
+        // every second group of TC_CS columns (two warps per quadrant) --------
+        const int ew = warp - 10, quad = warp & 3, half = ew >> 2;
+        float* sg = stage0 + (size_t)nst * a.stage_floats + ew * 32 * (TC_CS + 4);
+        float* row = sg + lane * (TC_CS + 4);
+        TcTile tn;
+        if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
+        int it = 0;
+        for (int ct = ct0; ct < a.nct; ct += ncl, ++it) {
+            const TcTile tl = tn;
+            const int j = quad * 32 + lane;   // this lane's pair
+            int64_t dst = 0;                  // its target expansion (floats)
+            if (j < tl.ncol) {
+                const int col = tl.col0 + j, pr = col / a.nrhs;
+                dst = 2 * ((int64_t)(col - pr * a.nrhs) * a.rstride + tl.dst_base +
+                           (int64_t)a.dst_idx[tl.pair_off + pr] * tl.p_out2) + tl.row0;
+            }
+            if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
+            const int b = it & 1;
+            const bool full = mbar_wait(smem_u32(&acc_full[b]), (it >> 1) & 1, a.wait_limit);
+            if (!__all_sync(0xffffffffu, full)) {   // the whole warp goes on or none of it
+                atomicExch(&s_fail, 1);
+                break;
+            }
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            const int npair = min(32, tl.ncol - quad * 32), rows = min(tl.nrow, 2 * tl.p_out2 - tl.row0);
+            const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols) + ((uint32_t)(quad * 32) << 16);
+            // 16-byte adds where every target of the warp is aligned to them
+            const bool wide = __all_sync(0xffffffffu, (dst & 3) == 0 && (((uintptr_t)a.dst) & 15) == 0);
+            int c0 = half * TC_CS;
+            for (; c0 < tl.nrow; c0 += 2 * TC_CS) {
+                uint32_t v[32];   // (columns past the block lie within the accumulator's)
+                tmem_ld32(acc + (uint32_t)c0, v);
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                    *reinterpret_cast<uint4*>(row + 4 * q) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                __syncwarp();
+                float* dp = (float*)a.dst + c0;
+                const int rn = rows - c0;   // an even count
+                if (wide) {   // 8 lanes a pair, 4 pairs at a time
+                    const int k = 4 * (lane & 7);
+#pragma unroll 4
+                    for (int t = lane >> 3; t < 32; t += 4) {
+                        const int64_t dt = __shfl_sync(0xffffffffu, dst, t);
+                        const float4 x = *reinterpret_cast<const float4*>(sg + t * (TC_CS + 4) + k);
+                        if (t < npair) {
+                            if (k + 4 <= rn) atomicAdd(reinterpret_cast<float4*>(dp + dt + k), x);
+                            else if (k + 2 <= rn) atomicAdd(reinterpret_cast<float2*>(dp + dt + k), make_float2(x.x, x.y));
+                        }
+                    }
+                } else {      // 16 lanes a pair, 2 pairs at a time
+                    const int k = 2 * (lane & 15);
+#pragma unroll 4
+                    for (int t = lane >> 4; t < 32; t += 2) {
+                        const int64_t dt = __shfl_sync(0xffffffffu, dst, t);
+                        const float2 x = *reinterpret_cast<const float2*>(sg + t * (TC_CS + 4) + k);
+                        if (t < npair && k + 2 <= rn) atomicAdd(reinterpret_cast<float2*>(dp + dt + k), x);
+                    }
+                }
+                __syncwarp();
+            }
+            // this warp's share of the accumulator is read
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])));
         }
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+
+    const bool done = mbar_wait(smem_u32(&done_bar), 0, DRAIN_LIMIT);
     __syncthreads();
-    if (warp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(TC_NMAX));
+    if ((!done || s_fail) && tid == 0) atomicExch(a.err, 1);
+    asm volatile("tcgen05.fence::after_thread_sync;");
+    if (warp == 0)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * a.acc_cols));
+    cluster_sync();   // no CTA leaves while a peer may still write its shared memory or signal its barriers
 }
 
 // ------------------------------------------------------------- host side ----
+// One launch: the tiles of the tasks with the same accumulator size.
+struct TcLaunch {
+    int rows_max = 0, acc_cols = 0;
+    std::vector<int> tasks;
+    int nst = 0, resident = 1;   // pipeline stages, clusters resident at once
+    size_t smem = 0;
+};
+struct TcTiles {
+    TcTile* d = nullptr;
+    std::vector<int> count;   // clusters of tiles per launch, consecutive in d
+};
 struct TcPlanImpl {
     std::vector<TcTask> h_tasks;
-    std::vector<TcTile> h_tiles;
-    std::vector<SplitLevel> h_split;
-    TcTask* tasks = nullptr;
-    TcTile* tiles = nullptr;
-    SplitLevel* split = nullptr;
+    std::vector<TcLaunch> launches;
     float* A = nullptr;
-    float* plane_hi = nullptr;
-    float* plane_lo = nullptr;
     int* err = nullptr;
     const int32_t* src_idx = nullptr;
     const int32_t* dst_idx = nullptr;
-    int64_t a_floats = 0, plane_floats = 0;
-    int max_split = 0;
-    int plane_nrhs = 1;                     // right-hand sides the planes hold
-    std::map<int, std::pair<TcTile*, int>> multi;   // tiles for nrhs > 1
+    int64_t a_floats = 0;
+    std::map<int, TcTiles> tiles;   // per number of right-hand sides (built on first use beyond one)
 };
+
+static size_t tc_stage_bytes(int rows) { return (size_t)(2 * A_BLOCK + 2 * rows * TC_KC) * sizeof(float); }
+
+static void tc_launch_config(const TcLaunch& ln, int clusters, cudaStream_t s, cudaLaunchConfig_t* cfg,
+                             cudaLaunchAttribute* at) {
+    *cfg = {};
+    cfg->gridDim = dim3((unsigned)(TC_CLUSTER * clusters));
+    cfg->blockDim = dim3(TC_THREADS);
+    cfg->dynamicSmemBytes = ln.smem;
+    cfg->stream = s;
+    at->id = cudaLaunchAttributeClusterDimension;
+    at->val.clusterDim.x = TC_CLUSTER;
+    at->val.clusterDim.y = 1;
+    at->val.clusterDim.z = 1;
+    cfg->attrs = at;
+    cfg->numAttrs = 1;
+}
+// Stages and shared memory of a launch (one CTA per SM: at least a share
+// such that no second CTA's allocation waits for tensor memory).  At least
+// four stages: a producer warp stores every fourth chunk, so when it waits
+// for a stage's last use, all uses before that one must be known complete
+// (its previous chunk's wait covers them from four stages on), or the
+// barrier's phase parity would be ambiguous.
+static fb_status tc_configure(TcLaunch& ln) {
+    const size_t stage = tc_stage_bytes(ln.rows_max), fixed = TC_STAGING * sizeof(float) + 1024;
+    ln.nst = (int)std::max<size_t>(2, std::min<size_t>(TC_STAGES, (220 * 1024 - fixed) / stage));
+    if (ln.nst < 4) return fb_fail(FB_ERR_STATE, "tensor-core translation: fewer than four pipeline stages");
+    ln.smem = std::max(ln.nst * stage + fixed, (size_t)116 * 1024);
+    FB_CHECK(fb_smem_cap((const void*)k_trans_tc, ln.smem));
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    tc_launch_config(ln, 1, nullptr, &cfg, &at);
+    FB_CUDA(cudaOccupancyMaxActiveClusters(&ln.resident, k_trans_tc, &cfg));
+    ln.resident = std::max(1, ln.resident);
+    return FB_OK;
+}
+
+// Tiles of the plan for nrhs right-hand sides, in clusters of TC_CLUSTER:
+// per (chunks, rows) whole clusters of one matrix first, then the remaining
+// pairs and single tiles packed together.
+static void tc_make_tiles(const TcPlanImpl* pl, int nrhs, std::vector<TcTile>& out, std::vector<int>& count) {
+    for (const TcLaunch& ln : pl->launches) {
+        std::map<std::pair<int, int>, std::vector<int>, std::greater<std::pair<int, int>>> by;   // most work first
+        for (int ti : ln.tasks) by[{pl->h_tasks[ti].nkc, pl->h_tasks[ti].rt_rows}].push_back(ti);
+        const size_t first = out.size();
+        for (const auto& kv : by) {
+            std::vector<TcTile> two, one;
+            for (int ti : kv.second) {
+                const TcTask& tk = pl->h_tasks[ti];
+                const int ncol = tk.npairs * nrhs, nc = div_up(ncol, TC_PAIRS);
+                for (int rt = 0; rt < tk.nrt; ++rt) {
+                    auto tile = [&](int c, int scount) {
+                        TcTile t;
+                        t.t_off = tk.a_off + (int64_t)rt * tk.nkc * 2 * tk.rt_rows * TC_KC;
+                        t.pair_off = tk.pair_off;
+                        t.src_base = tk.src_base;
+                        t.dst_base = tk.dst_base;
+                        t.p_in2 = tk.p_in2;
+                        t.p_out2 = tk.p_out2;
+                        t.nkc = tk.nkc;
+                        t.nrow = tk.rt_rows;
+                        t.row0 = rt * tk.rt_rows;
+                        t.col0 = c * TC_PAIRS;
+                        t.ncol = (int16_t)std::min(TC_PAIRS, ncol - c * TC_PAIRS);
+                        t.sbase = 0;
+                        t.scount = (int16_t)scount;
+                        t.pad = 0;
+                        return t;
+                    };
+                    int c = 0;
+                    for (; c + TC_CLUSTER <= nc; c += TC_CLUSTER)
+                        for (int i = 0; i < TC_CLUSTER; ++i) out.push_back(tile(c + i, TC_CLUSTER));
+                    if (TC_CLUSTER > 2 && c + 2 <= nc) {
+                        two.push_back(tile(c, 2));
+                        two.push_back(tile(c + 1, 2));
+                        c += 2;
+                    }
+                    if (c < nc) one.push_back(tile(c, 1));
+                }
+            }
+            out.insert(out.end(), two.begin(), two.end());
+            out.insert(out.end(), one.begin(), one.end());
+            while ((out.size() - first) % TC_CLUSTER) {   // a tile without columns
+                TcTile t = out.back();
+                t.ncol = 0;
+                t.scount = 1;
+                out.push_back(t);
+            }
+        }
+        // rank of the first sharer: groups of 4, 2 and 1 lie aligned to their size
+        for (size_t i = first; i < out.size(); ++i)
+            out[i].sbase = (int16_t)((int)((i - first) % TC_CLUSTER) / out[i].scount * out[i].scount);
+        count.push_back((int)((out.size() - first) / TC_CLUSTER));
+    }
+}
 
 // Bound of the pipeline's device waits (mbarrier polls) and the test hook
 // that makes one of them run out; library-wide, read at each launch.
@@ -347,83 +675,71 @@ int fb_tc_set_inject_stall(int on) { return g_inject_stall.exchange(on ? 1 : 0);
 long long fb_tc_wait_limit() { return g_wait_limit.load(); }
 int fb_tc_inject_stall() { return g_inject_stall.load(); }
 
-size_t fb_tc_smem_bytes() { return (size_t)TC_STAGES * STAGE_FLOATS * sizeof(float) + 1024; }
+static fb_status tc_tiles_for(TcPlanImpl* pl, int nrhs, const TcTiles** out) {
+    auto it = pl->tiles.find(nrhs);
+    if (it == pl->tiles.end()) {
+        std::vector<TcTile> h;
+        TcTiles t;
+        tc_make_tiles(pl, nrhs, h, t.count);
+        FB_CHECK(dalloc(&t.d, h.size()));
+        FB_CUDA(cudaMemcpy(t.d, h.data(), sizeof(TcTile) * h.size(), cudaMemcpyHostToDevice));
+        it = pl->tiles.emplace(nrhs, t).first;
+    }
+    if (out) *out = &it->second;
+    return FB_OK;
+}
 
 // Builds a tensor-core plan for groups of box pairs; each group shares one
 // composed translation matrix (job) and reads the source expansions of one
-// level (hi/lo planes split once per run).
+// level.
 fb_status fb_tc_build_groups(fb_op* op, const std::vector<TcGroup>& groups, const int32_t* src_idx,
                              const int32_t* dst_idx, void** slot, cudaStream_t s) {
-    const fb_tree* t = op->tree;
     TcPlanImpl* pl = new TcPlanImpl();
     *slot = pl;
     pl->src_idx = src_idx;
     pl->dst_idx = dst_idx;
-    std::vector<int> split_of(FB_MAXLEV + 1, -1);
     for (const TcGroup& g : groups) {
-        int ls = g.src_level;
-        if (split_of[ls] < 0) {
-            int Pin = op->p[ls] * op->p[ls];
-            SplitLevel sl;
-            sl.src_base = op->lev_off[ls];
-            sl.plane_base = pl->plane_floats;
-            sl.nbox = t->nbox[ls];
-            sl.P = Pin;
-            sl.stride_f = (2 * Pin + TC_KC - 1) / TC_KC * TC_KC;   // whole K chunks, 16-byte pieces
-            sl.pad = 0;
-            split_of[ls] = (int)pl->h_split.size();
-            pl->h_split.push_back(sl);
-            pl->plane_floats += (int64_t)sl.nbox * sl.stride_f;
-            pl->max_split = std::max<int>(pl->max_split,
-                                          (int)std::min<int64_t>((int64_t)sl.nbox * sl.stride_f / 256 + 1, 4096));
-        }
-        const SplitLevel& sl = pl->h_split[split_of[ls]];
         const ComposeJob& jb = op->h_jobs[g.job];
-        int Pout = jb.p_out * jb.p_out;
+        const int Pin = jb.p_in * jb.p_in, Pout = jb.p_out * jb.p_out;
         TcTask tk;
         tk.a_off = pl->a_floats;
         tk.pair_off = g.pair_off;
         tk.npairs = g.npairs;
-        tk.nrt = (2 * Pout + TC_M - 1) / TC_M;
-        tk.nkc = sl.stride_f / TC_KC;
+        tk.nrt = div_up(2 * Pout, TC_RMAX);
+        tk.rt_rows = (div_up(2 * Pout, tk.nrt) + 15) & ~15;
+        tk.nkc = div_up(2 * Pin, TC_KC);
         tk.p_out2 = Pout;
-        tk.p_in2 = sl.P;
-        tk.stride_f = sl.stride_f;
-        tk.plane_base = sl.plane_base;
+        tk.p_in2 = Pin;
+        tk.src_base = op->lev_off[g.src_level];
         tk.dst_base = op->lev_off[g.dst_level];
-        tk.nbox_src = sl.nbox;
-        tk.pad = 0;
-        int ti = (int)pl->h_tasks.size();
+        int cols = 32;
+        while (cols < tk.rt_rows) cols *= 2;
+        auto ln = std::find_if(pl->launches.begin(), pl->launches.end(),
+                               [&](const TcLaunch& l) { return l.acc_cols == cols; });
+        if (ln == pl->launches.end()) {
+            TcLaunch l;
+            l.acc_cols = cols;
+            ln = pl->launches.insert(pl->launches.end(), l);
+        }
+        ln->rows_max = std::max(ln->rows_max, (int)tk.rt_rows);
+        ln->tasks.push_back((int)pl->h_tasks.size());
         pl->h_tasks.push_back(tk);
-        for (int rt = 0; rt < tk.nrt; ++rt)
-            for (int c0 = 0; c0 < tk.npairs; c0 += TC_NMAX)
-                pl->h_tiles.push_back(TcTile{ti, rt, c0, std::min(TC_NMAX, tk.npairs - c0)});
-        pl->a_floats += (int64_t)tk.nrt * tk.nkc * 2 * A_BLOCK;
+        pl->a_floats += (int64_t)tk.nrt * tk.nkc * 2 * tk.rt_rows * TC_KC;
     }
     if (pl->h_tasks.empty()) return FB_OK;
     FB_CHECK(dalloc(&pl->A, pl->a_floats));
-    FB_CHECK(dalloc(&pl->plane_hi, pl->plane_floats));
-    FB_CHECK(dalloc(&pl->plane_lo, pl->plane_floats));
-    FB_CHECK(dalloc(&pl->tasks, pl->h_tasks.size()));
-    FB_CHECK(dalloc(&pl->tiles, pl->h_tiles.size()));
-    FB_CHECK(dalloc(&pl->split, pl->h_split.size()));
     FB_CHECK(dalloc(&pl->err, 1));
     FB_CUDA(cudaMemsetAsync(pl->err, 0, sizeof(int), s));
-    FB_CUDA(cudaMemcpyAsync(pl->tasks, pl->h_tasks.data(), sizeof(TcTask) * pl->h_tasks.size(),
-                            cudaMemcpyHostToDevice, s));
-    FB_CUDA(cudaMemcpyAsync(pl->tiles, pl->h_tiles.data(), sizeof(TcTile) * pl->h_tiles.size(),
-                            cudaMemcpyHostToDevice, s));
-    FB_CUDA(cudaMemcpyAsync(pl->split, pl->h_split.data(), sizeof(SplitLevel) * pl->h_split.size(),
-                            cudaMemcpyHostToDevice, s));
+    for (TcLaunch& ln : pl->launches) FB_CHECK(tc_configure(ln));
+    FB_CHECK(tc_tiles_for(pl, 1, nullptr));
     for (size_t i = 0; i < groups.size(); ++i) {
         const TcTask& tk = pl->h_tasks[i];
         const ComposeJob& jb = op->h_jobs[groups[i].job];
-        int64_t total = (int64_t)tk.nrt * tk.nkc * A_BLOCK;
+        int64_t total = (int64_t)tk.nrt * tk.nkc * tk.rt_rows * TC_KC;
         k_tc_pack<<<(unsigned)std::min<int64_t>(div_up(total, 256), 4096), 256, 0, s>>>(
-            op->T64 + jb.t_off, tk.p_out2, jb.p_in * jb.p_in, tk.nrt, tk.nkc, pl->A + tk.a_off);
+            op->T64 + jb.t_off, tk.p_out2, jb.p_in * jb.p_in, tk.nrt, tk.nkc, tk.rt_rows, pl->A + tk.a_off);
     }
     FB_LAUNCH_CHECK();
-    FB_CHECK(fb_smem_cap((const void*)k_trans_tc, fb_tc_smem_bytes()));
     return FB_OK;
 }
 
@@ -446,46 +762,34 @@ fb_status fb_tc_build(fb_op* op, const std::vector<int>& levels, void** slot, cu
 // the translation matrix is loaded once for all right-hand sides.
 fb_status fb_tc_run(fb_op* op, void* plan, const cf* src, cf* dst, cudaStream_t s, int nrhs, int64_t rstride) {
     TcPlanImpl* pl = (TcPlanImpl*)plan;
-    if (!pl || pl->h_tiles.empty()) return FB_OK;
-    const TcTile* tiles = pl->tiles;
-    int ntiles = (int)pl->h_tiles.size();
-    if (nrhs > 1) {
-        if (nrhs > pl->plane_nrhs) {
-            cudaStreamSynchronize(s);
-            dfree(pl->plane_hi);
-            dfree(pl->plane_lo);
-            FB_CHECK(dalloc(&pl->plane_hi, pl->plane_floats * nrhs));
-            FB_CHECK(dalloc(&pl->plane_lo, pl->plane_floats * nrhs));
-            pl->plane_nrhs = nrhs;
-            op->buf_gen++;   // captured graphs of this operator refer to the old planes
-        }
-        auto it = pl->multi.find(nrhs);
-        if (it == pl->multi.end()) {
-            std::vector<TcTile> h;
-            for (int ti = 0; ti < (int)pl->h_tasks.size(); ++ti) {
-                const TcTask& tk = pl->h_tasks[ti];
-                int ncol = tk.npairs * nrhs;
-                for (int rt = 0; rt < tk.nrt; ++rt)
-                    for (int c0 = 0; c0 < ncol; c0 += TC_NMAX)
-                        h.push_back(TcTile{ti, rt, c0, std::min(TC_NMAX, ncol - c0)});
-            }
-            TcTile* d = nullptr;
-            FB_CHECK(dalloc(&d, h.size()));
-            FB_CUDA(cudaMemcpy(d, h.data(), sizeof(TcTile) * h.size(), cudaMemcpyHostToDevice));
-            it = pl->multi.emplace(nrhs, std::make_pair(d, (int)h.size())).first;
-        }
-        tiles = it->second.first;
-        ntiles = it->second.second;
+    if (!pl || pl->h_tasks.empty()) return FB_OK;
+    const TcTiles* tiles = nullptr;
+    FB_CHECK(tc_tiles_for(pl, nrhs, &tiles));
+    TcArgs a;
+    a.tiles = tiles->d;
+    a.T = pl->A;
+    a.src_idx = pl->src_idx;
+    a.dst_idx = pl->dst_idx;
+    a.src = src;
+    a.dst = dst;
+    a.err = pl->err;
+    a.nrhs = nrhs;
+    a.rstride = rstride;
+    a.wait_limit = g_wait_limit.load();
+    a.inject_stall = g_inject_stall.load();
+    for (size_t i = 0; i < pl->launches.size(); a.tiles += (size_t)tiles->count[i] * TC_CLUSTER, ++i) {
+        const TcLaunch& ln = pl->launches[i];
+        a.nct = tiles->count[i];
+        a.acc_cols = ln.acc_cols;
+        a.nst = ln.nst;
+        a.stage_floats = (int)(tc_stage_bytes(ln.rows_max) / sizeof(float));
+        FB_CHECK(fb_smem_cap((const void*)k_trans_tc, ln.smem));
+        cudaLaunchAttribute at;
+        cudaLaunchConfig_t cfg;
+        tc_launch_config(ln, std::min(ln.resident, a.nct), s, &cfg, &at);
+        FB_CUDA(cudaLaunchKernelEx(&cfg, k_trans_tc, a));
+        fb_count_launch();
     }
-    dim3 sg(pl->max_split, (unsigned)pl->h_split.size());
-    k_tc_split<<<sg, 256, 0, s>>>(pl->split, (int)pl->h_split.size(), src, pl->plane_hi, pl->plane_lo, nrhs,
-                                  rstride);
-    k_trans_tc<<<(unsigned)ntiles, 256, fb_tc_smem_bytes(), s>>>(pl->tasks, tiles, pl->A, pl->src_idx,
-                                                                 pl->dst_idx, pl->plane_hi, pl->plane_lo, dst,
-                                                                 pl->err, nrhs, rstride, g_wait_limit.load(),
-                                                                 g_inject_stall.load());
-    FB_LAUNCH_CHECK();
-    fb_count_launch(2);
     return FB_OK;
 }
 
@@ -522,13 +826,8 @@ void fb_tc_free(void*& plan) {
     TcPlanImpl* pl = (TcPlanImpl*)plan;
     if (!pl) return;
     dfree(pl->A);
-    dfree(pl->plane_hi);
-    dfree(pl->plane_lo);
-    dfree(pl->tasks);
-    dfree(pl->tiles);
-    dfree(pl->split);
     dfree(pl->err);
-    for (auto& kv : pl->multi) dfree(kv.second.first);
+    for (auto& kv : pl->tiles) dfree(kv.second.d);
     delete pl;
     plan = nullptr;
 }
