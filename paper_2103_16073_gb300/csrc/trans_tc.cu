@@ -42,10 +42,10 @@
 //                coalesced runs of one pair's coefficients;
 //   warp 18      source offsets of the next tiles into a ring in shared
 //                memory, ahead of the producers.
-// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 1.20 ms (the
+// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 1.16 ms (the
 // MMAs alone 0.68 ms); 1.87 ms with pairs as N, one tile per CTA and hi/lo
 // planes of X split in a pass of its own.  The three tensor levels together
-// 2.21 ms against 3.54 ms; of the shoebox at 1 kHz 0.26 against 0.36 ms.
+// 2.14 ms against 3.54 ms; of the shoebox at 1 kHz 0.24 against 0.36 ms.
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // flag, drains its own copies and MMAs (bounded) and releases tensor memory.
 #include <algorithm>
@@ -79,6 +79,7 @@ using tcx::canon;
 using tcx::DRAIN_LIMIT;
 using tcx::LBO;
 using tcx::mbar_init;
+using tcx::mbar_test;
 using tcx::mbar_wait;
 using tcx::mma_commit;
 using tcx::mma_tf32;
@@ -382,12 +383,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             if (fail) atomicExch(&s_fail, 1);
             int s = 0, it = 0;
             uint32_t ph = 0;
-            // operand descriptors differ in their start address alone, a field of
+            // Operand descriptors differ in their start address alone, a field of
             // 16-byte units that no sum below carries out of (shared memory ends
-            // below its 256 KB): one add each, the single thread's issue chain
-            // being as long as the MMAs themselves otherwise
-            const uint64_t dsc0 = umma_desc(smem_u32(stage0)), dstep = (uint64_t)(a.stage_floats * 4) >> 4;
-            uint64_t dsc = dsc0;
+            // below its 256 KB).
+            const uint64_t d0 = umma_desc(smem_u32(stage0));
+            const uint32_t dlo = (uint32_t)d0, dhi = (uint32_t)(d0 >> 32), dstep = (uint32_t)(a.stage_floats * 4) >> 4;
+            auto desc = [dhi](uint32_t lo) { return (uint64_t)dhi << 32 | lo; };
+            uint32_t dof = dlo;
+            // A wait costs this thread some 200 cycles behind the other warps'
+            // shared-memory traffic: a stage's barriers are looked at while the
+            // one before is issued.
+            bool ready = false;
             int nkc_n = 0, nrow_n = 0;
             if (ct0 < a.nct) {
                 nkc_n = tiles[(int64_t)ct0 * TC_CLUSTER].nkc;
@@ -406,29 +412,29 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 }
                 const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols);
                 const uint32_t idesc = tcx::idesc_tf32(TC_PAIRS, nrow);
-                const uint64_t blo = (uint64_t)(nrow * TC_KC * 4) >> 4;   // from T's hi block to its lo block
+                const uint32_t blo = (uint32_t)(nrow * TC_KC * 4) >> 4;   // from T's hi block to its lo block
                 for (int c = 0; c < nkc; ++c) {
-                    if (!mbar_wait(smem_u32(&full_bar[s]), ph, a.wait_limit) ||
-                        !mbar_wait(smem_u32(&b_bar[s]), ph, a.wait_limit)) {
+                    if (!ready && (!mbar_wait(smem_u32(&full_bar[s]), ph, a.wait_limit) ||
+                                   !mbar_wait(smem_u32(&b_bar[s]), ph, a.wait_limit))) {
                         atomicExch(&s_fail, 1);
                         fail = true;
                         break;
                     }
+                    const int s1 = s + 1 == nst ? 0 : s + 1;
+                    const uint32_t p1 = s1 == 0 ? ph ^ 1 : ph;
+                    ready = mbar_test(smem_u32(&full_bar[s1]), p1) & mbar_test(smem_u32(&b_bar[s1]), p1);
                     asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
                     for (int ks = 0; ks < TC_KC / 8; ++ks) {
-                        const uint64_t aH = dsc + (uint64_t)((ks * 2 * LBO) >> 4), bH = aH + ((2 * A_BLOCK * 4) >> 4);
-                        mma_tf32(acc, aH, bH, idesc, ks == 0 ? (uint32_t)c : 1u);
-                        mma_tf32(acc, aH + ((A_BLOCK * 4) >> 4), bH, idesc, 1u);
-                        mma_tf32(acc, aH, bH + blo, idesc, 1u);
+                        const uint32_t aH = dof + ((ks * 2 * LBO) >> 4), bH = aH + ((2 * A_BLOCK * 4) >> 4);
+                        mma_tf32(acc, desc(aH), desc(bH), idesc, ks == 0 ? (uint32_t)c : 1u);
+                        mma_tf32(acc, desc(aH + ((A_BLOCK * 4) >> 4)), desc(bH), idesc, 1u);
+                        mma_tf32(acc, desc(aH), desc(bH + blo), idesc, 1u);
                     }
                     mma_commit_to(&empty_bar[s], (uint16_t)((1 << TC_CLUSTER) - 1));
-                    dsc += dstep;
-                    if (++s == nst) {
-                        s = 0;
-                        ph ^= 1;
-                        dsc = dsc0;
-                    }
+                    dof = s1 == 0 ? dlo : dof + dstep;
+                    s = s1;
+                    ph = p1;
                 }
                 if (!fail) mma_commit(&acc_full[b]);
             }
