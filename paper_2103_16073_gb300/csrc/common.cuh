@@ -313,7 +313,6 @@ struct DfTabs {
 // tables of the tensor-core rotation passes of the staged levels that use them
 struct StcTabs {
     const float* tab;
-    const int64_t* off;
     int64_t per;
     int* err;
 };

@@ -229,7 +229,7 @@ static RotArgs<R> rot_args(const fb_op* op) {
     a.V = (cx<R>*)op->stg_v;
     a.rf = op->rotf;
     a.fper = op->rotf_per;
-    a.tc = StcTabs{op->stc_tab, op->stc_off, op->stc_per, op->stc_err};
+    a.tc = StcTabs{op->stc_tab, op->stc_per, op->stc_err};
     a.dft = DfTabs{op->rotf_df, op->coax_df};
     return a;
 }

@@ -317,11 +317,13 @@ __global__ void __launch_bounds__(STHREADS, 2) k_stg_rot(const StgTile* __restri
 // O^{am}_{n'} (V[slot][n'^2 + n' + am]) = sum_k C^{am}_{n', am+k} O^{am}_{am+k}   (odd columns, am > 0)
 // for n' = am + row (degree-major folded, as u)
 // with E^{am}_n = U[slot][n^2 + am], O^{am}_n = U[slot][n^2 + n + am].
-template <class R>
+// INNER: u and v are [coefficient][slot] (levels whose rotations run on the
+// tensor cores) with S slots instead of [slot][coefficient] with S coefficients.
+template <class R, bool INNER>
 __global__ void __launch_bounds__(STHREADS, 2) k_stg_coax(const StgCTile* __restrict__ tiles,
                                                           const int32_t* __restrict__ cidx,
                                                           const cx<R>* __restrict__ coax, const cx<R>* __restrict__ U,
-                                                          cx<R>* __restrict__ V, int S, int pout) {
+                                                          cx<R>* __restrict__ V, int S) {
     extern __shared__ __align__(16) unsigned char stg_smem[];
     StgSmem<R, true>& sm = *reinterpret_cast<StgSmem<R, true>*>(stg_smem);
     const StgCTile tl = tiles[blockIdx.x];
@@ -332,7 +334,7 @@ __global__ void __launch_bounds__(STHREADS, 2) k_stg_coax(const StgCTile* __rest
             const int v = tl.vc0 + tid;
             const int slot = am == 0 ? cidx[tl.c0 + v] : cidx[tl.c0 + (v >> 1)];
             const int odd = (am != 0 && (v & 1)) ? 1 : 0;
-            sm.col_off[tid] = (int64_t)slot * S;
+            sm.col_off[tid] = INNER ? slot : (int64_t)slot * S;
             sm.col_aux[tid] = odd;
         } else {
             sm.col_off[tid] = -1;
@@ -348,7 +350,8 @@ __global__ void __launch_bounds__(STHREADS, 2) k_stg_coax(const StgCTile* __rest
         const int64_t o = sm.col_off[c];
         if (o < 0 || k >= K) return nullptr;
         const int nn = am + k;
-        return U + o + (int64_t)nn * nn + (sm.col_aux[c] ? nn : 0) + am;
+        const int64_t e = (int64_t)nn * nn + (sm.col_aux[c] ? nn : 0) + am;
+        return U + o + (INNER ? e * S : e);
     };
     cx<R> acc[4][4];
     stg_mainloop<R, true>(sm, K, aptr, xptr, (const void*)coax, acc);
@@ -357,13 +360,14 @@ __global__ void __launch_bounds__(STHREADS, 2) k_stg_coax(const StgCTile* __rest
     for (int j = 0; j < 4; ++j) {
         const int c = tx + 16 * j;
         if (c >= tl.nvc) continue;
-        cx<R>* v = V + sm.col_off[c] + am;
+        cx<R>* v = V + sm.col_off[c];
         const int odd = sm.col_aux[c];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const int r = ty * 4 + i;
             const int n1 = am + tl.row0 + r;
-            if (r < M) v[(int64_t)n1 * n1 + (odd ? n1 : 0)] = acc[i][j];
+            const int64_t e = (int64_t)n1 * n1 + (odd ? n1 : 0) + am;
+            if (r < M) v[INNER ? e * S : e] = acc[i][j];
         }
     }
 }
@@ -462,12 +466,12 @@ struct StgLevel {
     int tc = 0;
     int tcc = 0;  // ... and the coaxial pass too
     int df = 0;   // passes in double-FP32 arithmetic (FP64 expansions)
-    StcTile* rtc = nullptr;
-    StcTile* btc = nullptr;
+    StcItem* rtc = nullptr;
+    StcItem* btc = nullptr;
     int nrtc = 0, nbtc = 0;
-    // coaxial pass on the tensor cores (tc levels): tiles and the plan's
+    // coaxial pass on the tensor cores (tc levels): items and the plan's
     // pre-split coaxial blocks
-    StcCTile* ctc = nullptr;
+    StcItem* ctc = nullptr;
     int nctc = 0;
     float* ctab = nullptr;
 };
@@ -557,7 +561,7 @@ fb_status fb_stg_build(const RcrPlan& pl, const std::vector<int>& theta_slot, in
         std::vector<StgSlot> slots;
         std::vector<int> slot_task;
         std::vector<StgTile> rt, bt;
-        std::vector<StcTile> rtc, btc;
+        std::vector<StcItem> rtc, btc;
         for (int rep : group_order) {
             const int g0 = (int)slots.size();
             for (int t : groups[rep]) {
@@ -581,8 +585,12 @@ fb_status fb_stg_build(const RcrPlan& pl, const std::vector<int>& theta_slot, in
             }
             const int g1 = (int)slots.size();
             if (lv.tc) {
-                fb_stc_group_tiles(rep, g0, g1, p_in, 0, p_in, rtc);
-                fb_stc_group_tiles(rep, g0, g1, p_out, 1, p_in, btc);
+                fb_stc_group_items(rep, g0, g1, p_in, 0, p_in, rtc);
+                fb_stc_group_items(rep, g0, g1, p_out, 1, p_in, btc);
+                while (slots.size() % STC_ALIGN) {   // slots of no pair
+                    slots.push_back(StgSlot{0, 0, 0, 0});
+                    slot_task.push_back(-1);
+                }
                 continue;
             }
             // folded blocks: even rows n + 1, odd rows n (none for n = 0)
@@ -605,13 +613,14 @@ fb_status fb_stg_build(const RcrPlan& pl, const std::vector<int>& theta_slot, in
         std::map<int64_t, std::vector<int32_t>> sets;   // coax_off -> slots
         std::map<int64_t, int> set_pc;
         for (int s = 0; s < (int)slots.size(); ++s) {
+            if (slot_task[s] < 0) continue;
             const RcrTask& tk = pl.h_tasks[slot_task[s]];
             sets[tk.coax_off].push_back(s);
             set_pc[tk.coax_off] = tk.pc;
         }
         std::vector<int32_t> cidx;
         std::vector<StgCTile> ct;
-        std::vector<StcCTile> ctc;
+        std::vector<StcItem> ctc;
         std::vector<StcCBlock> cblocks;
         int64_t ctab_floats = 0;
         const int q = std::min(p_in, p_out);
@@ -657,23 +666,9 @@ fb_status fb_stg_build(const RcrPlan& pl, const std::vector<int>& theta_slot, in
         lv.nrt = (int)rt.size();
         lv.nct = (int)ct.size();
         lv.nbt = (int)bt.size();
-        // heaviest tensor-core tiles first (K chunks x columns), for the tail
-        auto heavier = [&](int pass) {
-            return [pass, p_in](const StcTile& x, const StcTile& y) {
-                auto w = [&](const StcTile& t) {
-                    int64_t c = 0;
-                    for (int n = t.n0; n < t.n1; ++n) {
-                        const int N = n + 1 - t.part;
-                        const int K = pass == 0 ? N : std::min(n, p_in - 1) + 1 - t.part;
-                        c += (int64_t)stc_pad16(N) * ((K + 15) / 16);
-                    }
-                    return c;
-                };
-                return w(x) > w(y);
-            };
-        };
-        std::stable_sort(rtc.begin(), rtc.end(), heavier(0));
-        std::stable_sort(btc.begin(), btc.end(), heavier(1));
+        fb_stc_sort(rtc);
+        fb_stc_sort(btc);
+        fb_stc_sort(ctc);
         lv.nrtc = (int)rtc.size();
         lv.nbtc = (int)btc.size();
         lv.nctc = (int)ctc.size();
@@ -779,11 +774,8 @@ fb_status fb_stg_df_tables(fb_op* op, cudaStream_t s) {
 static fb_status stc_pass(const StgLevel& lv, int pass, const StcTabs* tc, const cf* X, cf* out, const cf* rph,
                           int prot, cudaStream_t s) {
     if (!tc || !tc->tab) return fb_fail(FB_ERR_STATE, "staged RCR: tensor-core tables missing");
-    const int np = std::max(lv.p_in, lv.p_out);
-    return pass == 0 ? fb_stc_run(0, lv.rtc, lv.nrtc, np, tc->off, tc->tab, tc->per, lv.slots, X, out, lv.S, lv.p_in,
-                                  lv.p_out, rph, prot, tc->err, s)
-                     : fb_stc_run(1, lv.btc, lv.nbtc, np, tc->off, tc->tab, tc->per, lv.slots, X, out, lv.S, lv.p_in,
-                                  lv.p_out, rph, prot, tc->err, s);
+    return fb_stc_run(pass, pass == 0 ? lv.rtc : lv.btc, pass == 0 ? lv.nrtc : lv.nbtc, std::max(lv.p_in, lv.p_out),
+                      tc->tab, tc->per, lv.slots, nullptr, X, out, lv.nslot, rph, prot, tc->err, s);
 }
 template <class X, class Y, class Ph>
 static fb_status stc_pass(const StgLevel&, int, const StcTabs*, const X*, Y*, const Ph*, int, cudaStream_t) {
@@ -792,7 +784,8 @@ static fb_status stc_pass(const StgLevel&, int, const StcTabs*, const X*, Y*, co
 // Tensor-core coaxial pass of a level (single precision only).
 static fb_status stc_coax(const StgLevel& lv, const StcTabs* tc, const cf* U, cf* V, cudaStream_t s) {
     if (!tc) return fb_fail(FB_ERR_STATE, "staged RCR: tensor-core error flag missing");
-    return fb_stc_coax_run(lv.ctc, lv.nctc, lv.cidx, lv.ctab, U, V, lv.S, lv.p_out, tc->err, s);
+    return fb_stc_run(2, lv.ctc, lv.nctc, 2 * std::min(STC_CROWS, lv.p_out), lv.ctab, 0, nullptr, lv.cidx, U, V,
+                      lv.nslot, nullptr, 0, tc->err, s);
 }
 template <class X>
 static fb_status stc_coax(const StgLevel&, const StcTabs*, const X*, X*, cudaStream_t) {
@@ -809,7 +802,7 @@ static fb_status stg_level(const StgLevel& lv, int pass_mask, const R* rf, int64
                            const StcTabs* tc) {
     const size_t sm_rc = sizeof(StgSmem<R, false>), sm_c = sizeof(StgSmem<R, true>);
     FB_CHECK(fb_smem_cap((const void*)k_stg_rot<R>, sm_rc));
-    FB_CHECK(fb_smem_cap((const void*)k_stg_coax<R>, sm_c));
+    FB_CHECK(fb_smem_cap((const void*)k_stg_coax<R, false>, sm_c));
     FB_CHECK(fb_smem_cap((const void*)k_stg_back<R, O>, sm_rc));
     if ((pass_mask & 1) && !lv.tc) {   // the tensor-core rotation pass folds its inputs itself
         const int64_t tot = (int64_t)lv.nslot * lv.p_in * lv.p_in;
@@ -828,7 +821,13 @@ static fb_status stg_level(const StgLevel& lv, int pass_mask, const R* rf, int64
     if ((pass_mask & 4) && lv.nctc) {
         FB_CHECK(stc_coax(lv, tc, U, V, s));
     } else if ((pass_mask & 4) && lv.nct) {
-        k_stg_coax<R><<<lv.nct, STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.S, lv.p_out);
+        if constexpr (std::is_same<R, float>::value) {
+            if (lv.tc) {
+                FB_CHECK(fb_smem_cap((const void*)k_stg_coax<R, true>, sm_c));
+                k_stg_coax<R, true><<<lv.nct, STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.nslot);
+            }
+        }
+        if (!lv.tc) k_stg_coax<R, false><<<lv.nct, STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.S);
         fb_count_launch();
     }
     if (pass_mask & 8) {

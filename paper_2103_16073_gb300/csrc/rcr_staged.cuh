@@ -25,18 +25,25 @@ __host__ __device__ __forceinline__ int64_t fo(int n) {
     return (int64_t)(n - 1) * n * (2 * n - 1) / 3 + (int64_t)n * n;
 }
 
-// ---- tensor-core rotation passes ------------------------------------------
-// A tile of the tensor-core R or B pass: slots [s0, s0 + ns) (ns <= 64) of
-// one polar-angle group g, folded part `part`, degrees [n0, n1), whose
-// accumulators share the CTA's tensor memory.
-struct StcTile {
-    int32_t g, part;
-    int32_t n0, n1;
-    int32_t s0, ns;
-};
+// ---- tensor-core passes ----------------------------------------------------
+constexpr int STC_SLOTS = 64;     // slots per item (128 accumulator rows)
+constexpr int STC_COLS = 256;     // accumulator columns of an item, at most
+constexpr int STC_CROWS = 128;    // coaxial output rows (complex) per item
+// Slots of a level whose rotations run on the tensor cores start every
+// polar-angle group at a multiple of 16: whole 128-byte lines of u and v.
+constexpr int STC_ALIGN = 16;
 
-constexpr int STC_SLOTS = 64;        // slots per tile (128 real rows: re, im)
-constexpr int STC_TMEM_COLS = 256;   // accumulator columns per tile
+// One block of a pass applied to up to 64 slots.  R, B: degree n, folded part
+// `part`, slots s0 .. s0 + ns of polar-angle group g; C: order n, output
+// degrees from n + part on, slots cidx[s0 ..] of one |t| set.
+struct StcItem {
+    int64_t tab;      // float offset of its table block (R, B: within the group's table)
+    int32_t s0, ns;
+    int32_t n, part;
+    int32_t N, K;     // real columns and summed length
+    int32_t g;
+    int32_t uni;      // (set on the device)
+};
 
 // columns of the folded degree-n block (rows of the table), padded to 16
 __host__ __device__ __forceinline__ int stc_pad16(int v) { return (v + 15) & ~15; }
@@ -47,45 +54,32 @@ __host__ __device__ __forceinline__ int stc_pad16(int v) { return (v + 15) & ~15
 // TF32 part then the remainder); returns the floats per group and pass.
 int64_t fb_stc_layout(int P, std::vector<int64_t>& toff);
 
-// Appends the tiles of one polar-angle group (slots [g0, g1)) for degrees
+// Appends the items of one polar-angle group (slots [g0, g1)) for degrees
 // [0, nmax) of pass 0 (rotation) or 1 (back-rotation; K limited by p_in).
-void fb_stc_group_tiles(int g, int g0, int g1, int nmax, int pass, int p_in, std::vector<StcTile>& out);
+void fb_stc_group_items(int g, int g0, int g1, int nmax, int pass, int p_in, std::vector<StcItem>& out);
 
-// A tile of the tensor-core coaxial pass: virtual columns [vc0, vc0 + nvc)
-// (nvc <= 128; order 0: one slot each, order am > 0: slot (v / 2), even part
-// for even v and odd part for odd v) of one |t| set whose slots start at
-// cidx[c0], output degrees am + r0 .. am + r0 + nr - 1 (nr <= 128), summed
-// over the K = p_in - am input degrees; its pre-split coaxial block starts at
-// float toff of the plan's coaxial tables.
-struct StcCTile {
-    int64_t toff;
-    int32_t c0, vc0, nvc;
-    int32_t am, r0, nr, K;
-    int32_t pad;
-};
 // A pre-split coaxial block to build: C^{am}_{am + r0 + i, am + k} of the set
 // at coax offset cs_off (row stride pc), i < nr, k < K, at float toff.
 struct StcCBlock {
     int64_t cs_off, toff;
     int32_t pc, am, r0, nr, K, pad;
 };
-constexpr int STC_CROWS = 128;   // coaxial output rows (complex) per tile
 
-// Appends the coaxial tiles and table blocks of one |t| set (ns slots at
+// Appends the coaxial items and table blocks of one |t| set (ns slots at
 // cidx[c0], coefficients at cs_off, stride pc) of a level; *tfloats grows by
 // the floats of the new table blocks.
-void fb_stc_coax_set(int c0, int ns, int64_t cs_off, int pc, int p_in, int p_out, std::vector<StcCTile>& tiles,
+void fb_stc_coax_set(int c0, int ns, int64_t cs_off, int pc, int p_in, int p_out, std::vector<StcItem>& items,
                      std::vector<StcCBlock>& blocks, int64_t* tfloats);
+void fb_stc_sort(std::vector<StcItem>& items);
 // Builds the pre-split coaxial blocks (3xTF32 real form of the complex
 // blocks) from the FP64 coaxial sets.
 fb_status fb_stc_coax_tables(const StcCBlock* blocks, int nblocks, const cd* coax64, float* out, cudaStream_t s);
-// Launches the coaxial tiles: U -> V (both degree-major folded).
-fb_status fb_stc_coax_run(const StcCTile* tiles, int ntiles, const int32_t* cidx, const float* tab, const cf* U,
-                          cf* V, int S, int p_out, int* err, cudaStream_t s);
 
-// Launches the rotation (pass 0) or back-rotation (pass 1) tiles.
-fb_status fb_stc_run(int pass, const StcTile* tiles, int ntiles, int npmax, const int64_t* toff, const float* tab,
-                     int64_t tper, const StgSlot* slots, const cf* X, cf* out, int S, int p_in, int p_out,
-                     const cf* rph, int prot, int* err, cudaStream_t s);
+// Launches the items of a pass: rotation 0 (expansions -> u), back-rotation 1
+// (v -> expansions), coaxial 2 (u -> v); ncol_max bounds their columns; ns is
+// the level's number of slots, u and v are [coefficient][slot].
+fb_status fb_stc_run(int pass, const StcItem* items, int nitems, int ncol_max, const float* tab, int64_t tper,
+                     const StgSlot* slots, const int32_t* cidx, const cf* X, cf* out, int64_t ns, const cf* rph,
+                     int prot, int* err, cudaStream_t s);
 
 }  // namespace stg

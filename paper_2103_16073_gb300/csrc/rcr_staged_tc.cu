@@ -1,37 +1,48 @@
-// Rotation passes of the staged RCR translation (Sec. 3.3) on the tensor
+// The three passes of the staged RCR translation (Sec. 3.3) on the tensor
 // cores (tcgen05, 3xTF32).
 //
-// The rotation pass R and the back-rotation pass B of rcr_staged.cu are
-// real-by-complex GEMMs per (polar-angle group, degree n, folded part): the
-// folded real table block d (N x K, N = K = n + 1 or n) applied to the
-// complex vectors of every slot (pair) of the group.  Here they run
-// transposed, so that the short dimension of a degree block is the MMA's N:
-//     D[(slot, re/im)][row] = sum_k  x[slot][k].{re, im}  d[row][k]
-//   A = the slots' vectors: 64 slots per tile as 128 real rows (row 2j the
-//       real parts of slot j, row 2j + 1 the imaginary parts), loaded by
-//       producer warps with plain loads (pass R folds and phases the source
-//       expansions on the fly; pass B reads contiguous runs of v), split
-//       into TF32 hi + lo and stored in the canonical layout;
-//   B = the table block, K-major as stored (row-major [row][k]), pre-split
-//       into hi + lo and laid out canonically per K chunk of 16 at setup, so
-//       that one bulk copy moves a chunk;
-//   D = FP32 accumulators in tensor memory, one column range per degree; a
-//       tile packs consecutive degrees up to 256 columns.
-// 3xTF32: D += A_hi B_hi + A_hi B_lo + A_lo B_hi.
+// R and B (rotation, back-rotation) of rcr_staged.cu are real-by-complex
+// GEMMs per (polar-angle group, degree n, folded part): the folded real table
+// block d (N x K, N = K = n + 1 or n) applied to the complex vectors of every
+// slot (pair) of the group.  C (coaxial) is a complex GEMM per (|t|, order
+// |m|) over the degrees.  All three run transposed, slots along M and the
+// short dimension of a block as the MMA's N:
+//     D[row][col] = sum_k A[row][k] T[col][k],  128 rows = 64 slots x 2,
+//   R, B: row = 16 (j / 8) + 8 c + j % 8 is the real (c = 0) or imaginary
+//       (c = 1) part of slot j, T the table block;
+//   C: row = 64 part + j is the even or odd part of slot j (order 0: even
+//       alone), K interleaved: A[row][(k, c)] = u[k].c and
+//       T[(i, 0)][(k, .)] = (Re C, -Im C), T[(i, 1)][(k, .)] = (Im C, Re C),
+//       so columns 2 i, 2 i + 1 are the real and imaginary part of degree i.
+// T is K-major, pre-split into TF32 hi + lo and laid out canonically per K
+// chunk of 16 at setup, so that one bulk copy moves a chunk; A is split by the
+// producer warps.  3xTF32: D += A_hi T_hi + A_hi T_lo + A_lo T_hi.
 //
-// Pipeline (10 warps, 3 shared-memory stages):
-//   warps 0-7  A producers (each thread 4 consecutive K values of one slot
-//              per chunk, the next chunk's loads in flight while the current
-//              one is stored), then the epilogue;
-//   warp 8     lane 0: bulk copies of the table chunks (transaction count);
-//   warp 9     lane 0: MMA issuer (waits for both operands of a stage,
-//              6 MMAs per chunk, commits to the stage's "empty" barrier).
-//   epilogue   warps w and w + 4 read the accumulator lanes of quadrant
-//              w % 4 (even / odd 16-column groups); lanes 2j and 2j + 1
-//              hold the real and imaginary part of slot j and trade halves
-//              (one shuffle) so that each lane writes whole complex values:
-//              pass R stores u (degree-major, folded), pass B adds the
-//              phased y_{+-m'} = (Y+ +- Y-)/2 into the targets (atomics).
+// Layout of the staging buffers u and v: coefficient-major, slot innermost,
+// u[e * ns + slot] with e = n^2 (+ n for the odd part) + |m|.  The rows of
+// every tile are slots, so all three passes read and write whole lines along
+// the lanes (8 bytes of every 32-byte sector with slots outermost, where C
+// strides over the degrees and R and C store a column at a time).
+//
+// Persistent: one CTA per SM walks over items (one block T x 64 slots), every
+// role running ahead of the next, because an item is a few microseconds of
+// dependent latencies (descriptor, slots, operands, products, stores) around
+// a few hundred cycles of MMAs:
+//   12, 8 or 4 warps (R, C, B)  A producers: a warp takes every third, fourth
+//                or second chunk of K, with the loads of its next in flight;
+//   one warp     lane 0: bulk copies of the chunks of T (transaction count);
+//   one warp     lane 0: MMA issuer, two to four accumulators in tensor memory;
+//   4, 8 or 12 warps  epilogue: accumulator lanes 32 (w % 4) .., groups of 16
+//                columns in turn; R and C store u and v, B goes through
+//                shared memory so that the phased y_{+-m'} = (Y+ +- Y-)/2 are
+//                added (atomics) in runs of one target's coefficients;
+//   warps 18-19  items and their slots into a ring in shared memory, ahead of
+//                the others.
+// Room of 240 leaf boxes at 7.5 kHz (orders 116 and 66, M2L): R 0.44 ms, C
+// 0.34 ms, B 0.46 ms over both levels; together 3.34 ms with one tile per
+// CTA, degree-major u and v, and lanes along a row's K values.  C moves 1 GB
+// per pass out of L2 at 6 TB/s; R and B are bound by their warps' issue rate
+// around the waits of a chunk.
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // flag, drains its own bulk copies and MMAs (bounded) and frees its tensor
 // memory.
@@ -49,8 +60,8 @@ namespace {
 using tcx::canon;
 using tcx::DRAIN_LIMIT;
 using tcx::KC;
-using tcx::LBO;
 using tcx::mbar_init;
+using tcx::mbar_test;
 using tcx::mbar_wait;
 using tcx::mma_commit;
 using tcx::mma_tf32;
@@ -58,17 +69,39 @@ using tcx::smem_u32;
 using tcx::tf32_hi;
 using tcx::umma_desc;
 
-constexpr int STC_M = 2 * STC_SLOTS;         // real rows of a tile
-constexpr int STC_PRODW = 8;                 // producer / epilogue warps
-constexpr int STC_NPROD = STC_PRODW * 32;
-constexpr int STC_THREADS = STC_NPROD + 64;  // + bulk-copy warp + MMA warp
-constexpr int A_PLANE = STC_M * KC;          // floats of one (hi or lo) A block
-constexpr int STC_STAGES = 3;
-// at most two CTAs per SM, so that their tensor memory (2 x 256 columns)
-// is always free when they start
-constexpr size_t STC_SMEM_MIN = 80 * 1024;
+enum { ST_R = 0, ST_B = 1, ST_C = 2 };   // pass
 
-static_assert(STC_NPROD == STC_SLOTS * (KC / 4), "one producer thread per (slot, 4 K values)");
+constexpr int STC_M = 2 * STC_SLOTS;     // rows of a tile
+constexpr int STC_WORKW = 16;            // producer and epilogue warps
+constexpr int STC_IDXW = 2;              // warps 18-19
+constexpr int STC_IDX0 = STC_WORKW + 2;
+constexpr int STC_THREADS = 32 * (STC_IDX0 + STC_IDXW);
+constexpr int STC_STAGES = 8;            // at most
+// Items in shared memory.  A producer looks up the item of the chunk two of
+// its own ahead before it stores the current one, with one chunk per item 2 x
+// 4 items further: the ring has to hold more than those.
+constexpr int STC_RING = 12;
+constexpr int STC_ACC = 4;               // accumulators, at most
+constexpr int STC_SG = 20;               // floats of a staged accumulator row (16 columns, padded)
+constexpr size_t STC_SMEM_MAX = 214 * 1024;   // dynamic; the ring (< 11 KB) is static
+constexpr size_t STC_SMEM_MIN = 116 * 1024;   // one CTA per SM: its accumulators are always free
+
+// Every producer warp of pass R stores single K values of 16 consecutive m
+// (the order its loads coalesce in): core matrices 144 bytes apart put the
+// 16 values of two slots into 32 banks.  The other passes store 16-byte rows
+// and take the packed layout.
+template <int PASS>
+struct StcLayout {
+    static constexpr int LBO = PASS == ST_R ? 144 : tcx::LBO;
+    static constexpr int SBO = (KC / 4) * LBO;
+    static constexpr int PLANE = STC_M / 8 * SBO / 4;   // floats of one (hi or lo) A block
+    // producer and epilogue warps (R folds its inputs, B scatters with atomics);
+    // a producer warp takes every PERIOD-th chunk
+    static constexpr int PRODW = PASS == ST_R ? 12 : (PASS == ST_C ? 8 : 4), EPIW = STC_WORKW - PRODW;
+    static constexpr int PERIOD = PASS == ST_R ? 3 : (PASS == ST_C ? 4 : 2);
+    static constexpr int SHARES = EPIW / 4;             // epilogue warps per 32 accumulator lanes
+    static_assert(STC_RING > 2 * PERIOD, "a producer's look-ahead fits the ring");
+};
 
 // accumulator columns N (output rows of the table block) and summed length
 // K of degree n, folded part `part`, of pass R (0) or B (1)
@@ -78,120 +111,307 @@ __host__ __device__ __forceinline__ void stc_dims(int pass, int n, int part, int
 }
 
 struct StcArgs {
-    const StcTile* tiles;
-    const int64_t* toff;   // table block offsets [2 n + part]
-    const float* tab;      // group g: R table at g * 2 tper, B table at g * 2 tper + tper
+    const StcItem* items;
+    int nitems;
+    const float* tab;      // R, B: group g's R table at g * 2 tper, B table at g * 2 tper + tper; C: the coaxial blocks
     int64_t tper;
     const StgSlot* slots;
-    const cf* X;           // R: source expansions; B: v (degree-major, folded)
-    cf* out;               // R: u (degree-major, folded); B: target expansions
+    const int32_t* cidx;   // C: slots of a |t| set
+    const cf* X;           // R: source expansions; C: u; B: v
+    cf* out;               // R: u; C: v; B: target expansions
     const cf* rph;         // phases e^{i m phi} per direction
     int* err;
     long long wait_limit;
-    int S, p_in, p_out, prot;
-    int stage_floats;
+    int64_t ns;            // slots: the stride of a coefficient of u and v
+    int prot;
+    int nst;               // pipeline stages
+    int stage_floats;      // A hi, A lo, then the largest chunk of T (hi, lo)
+    int acc_cols, nacc;    // tensor memory columns of an accumulator, accumulators
     int inject_stall;
 };
 
-// 4 consecutive K values (k0 .. k0 + 3) of one slot's vector of degree n.
-// Pass R folds and phases the source expansion on the fly (m = part + k):
-// s_0 = x_0, s_m = x_m e^{i m phi} + x_{-m} e^{-i m phi}, t_m = the
-// difference; pass B reads E_mu / O_mu (mu = part + k) of v.
+__device__ __forceinline__ void arrive(uint64_t* bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)));
+}
+
+// stores a row's 4 K values as TF32 hi and remainder
+__device__ __forceinline__ void split_store(float* st, int plane, const float4& x) {
+    const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
+    *reinterpret_cast<float4*>(st) = h;
+    *reinterpret_cast<float4*>(st + plane) = make_float4(x.x - h.x, x.y - h.y, x.z - h.z, x.w - h.w);
+}
+
+// A producer's registers for one chunk: load() issues the loads of chunk c of
+// an item, take() makes them the current chunk, store() writes that one.  A
+// warp's issue rate is what bounds the producers, so addresses are one
+// multiply-add each and only the last chunk of an item pays for its ragged K.
+// Rows past the item's slots hold copies of its last slot and are not written
+// anywhere; K values past K are zero, as they are in T.
 template <int PASS>
-__device__ __forceinline__ void stc_load(const StcArgs& a, int64_t row, int dir, int n, int part, int K, int k0,
-                                         float (&v)[8]) {
-    const cf* ph = a.rph + (int64_t)dir * (2 * a.prot - 1) + (a.prot - 1);
+struct Producer;
+
+__device__ __forceinline__ float2 ldg2(const char* p) { return __ldg(reinterpret_cast<const float2*>(p)); }
+
+// R: folds and phases the source expansions on the way (m = part + k):
+// s_0 = x_0, s_m = x_m e^{i m phi} + x_{-m} e^{-i m phi}, t_m = the difference.
+// Lanes: 16 consecutive m of two slots 4 apart, 8 such units per warp and
+// chunk.  Slots are sorted by direction, so most groups of 16 share a phase.
+template <>
+struct Producer<ST_R> {
+    float2 xp[8], xm[8], ph[8], cur[8];
+    float sg;      // sign of x_{-m} (0: m = 0)
+    bool uni, in;  // one direction for all slots; k < K
+    __device__ __forceinline__ void load(const StcArgs& a, const StcItem& it, const int64_t* pos, const int32_t* dir,
+                                         int sub, int lane, int c) {
+        const int k = c * KC + (lane & 15), n = it.n, part = it.part, m = min(part + k, n);
+        sg = m == 0 ? 0.f : (part ? -1.f : 1.f);
+        in = k < it.K;
+        uni = it.uni >> sub & 1;
+        const int j0 = 16 * sub + 4 * (lane >> 4);
+        const char* xs = (const char*)(a.X + (int64_t)n * n + n);
+        const char *bp = xs + 8 * m, *bm = xs - 8 * m, *bh = (const char*)(a.rph + a.prot - 1 + m);
+        int64_t o[8];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const int k = k0 + i;
-        float2 x = make_float2(0.f, 0.f);
-        if (row >= 0 && k < K) {
-            if (PASS == 0) {
-                const cf* xs = a.X + row + (int64_t)n * n + n;   // (n, 0)
-                const int m = part + k;
-                if (m == 0) {
-                    x = __ldg(reinterpret_cast<const float2*>(xs));
-                } else {
-                    const float2 xp = __ldg(reinterpret_cast<const float2*>(xs + m));
-                    const float2 xm = __ldg(reinterpret_cast<const float2*>(xs - m));
-                    const float2 pp = __ldg(reinterpret_cast<const float2*>(ph + m));
-                    const float2 pm = __ldg(reinterpret_cast<const float2*>(ph - m));
-                    const float ar = xp.x * pp.x - xp.y * pp.y, ai = xp.x * pp.y + xp.y * pp.x;
-                    const float br = xm.x * pm.x - xm.y * pm.y, bi = xm.x * pm.y + xm.y * pm.x;
-                    x = part ? make_float2(ar - br, ai - bi) : make_float2(ar + br, ai + bi);
-                }
-            } else {
-                x = __ldg(reinterpret_cast<const float2*>(a.X + row + (int64_t)n * n + (part ? n : 0) + part + k));
+        for (int i = 0; i < 8; ++i) o[i] = pos[j0 + 8 * (i >> 2) + (i & 3)];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            xp[i] = ldg2(bp + 8 * o[i]);
+            xm[i] = ldg2(bm + 8 * o[i]);
+        }
+        const int pw = 8 * (2 * a.prot - 1);
+        ph[0] = ldg2(bh + (int64_t)dir[j0] * pw);
+        if (!uni) {
+#pragma unroll
+            for (int i = 1; i < 8; ++i) ph[i] = ldg2(bh + (int64_t)dir[j0 + 8 * (i >> 2) + (i & 3)] * pw);
+        }
+    }
+    __device__ __forceinline__ void fold(int i, float2 e) {
+        const float px = xp[i].x + sg * xm[i].x, py = xp[i].y + sg * xm[i].y;
+        const float qx = xp[i].x - sg * xm[i].x, qy = xp[i].y - sg * xm[i].y;
+        cur[i] = make_float2(px * e.x - qy * e.y, py * e.x + qx * e.y);
+    }
+    __device__ __forceinline__ void take() {
+        if (uni) {
+            const float2 e = in ? ph[0] : make_float2(0.f, 0.f);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) fold(i, e);
+        } else {
+#pragma unroll
+            for (int i = 0; i < 8; ++i) fold(i, in ? ph[i] : make_float2(0.f, 0.f));
+        }
+    }
+    __device__ __forceinline__ void store(float* st, int sub, int lane) const {
+        using L = StcLayout<ST_R>;
+        const int k = lane & 15;
+        st += ((k >> 2) * L::LBO + 4 * (lane >> 4) * 16 + 4 * sub * L::SBO) / 4 + (k & 3);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            float* d = st + (2 * (i >> 2) * L::SBO + (i & 3) * 16) / 4;   // row of the real part
+            const float hr = tf32_hi(cur[i].x), hi = tf32_hi(cur[i].y);
+            d[0] = hr;
+            d[L::PLANE] = cur[i].x - hr;
+            d[L::SBO / 4] = hi;
+            d[L::PLANE + L::SBO / 4] = cur[i].y - hi;
+        }
+    }
+};
+
+// C: lanes along the slots, one part per warp, 2 slots x 4 pairs of degrees a
+// lane.
+template <>
+struct Producer<ST_C> {
+    float4 nxt[8], cur[8];
+    __device__ __forceinline__ void load(const StcArgs& a, const StcItem& it, const int64_t* pos, const int32_t*,
+                                         int sub, int lane, int c) {
+        const int part = sub, am = it.n, left = it.K / 2 - c * (KC / 2);   // degrees
+        const char *x0 = (const char*)(a.X + pos[lane]), *x1 = (const char*)(a.X + pos[lane + 32]);
+        const int64_t es = 8 * a.ns;
+        int n = am + c * (KC / 2), e = n * n + (part ? n : 0) + am;
+        float2 x[2][KC / 2];
+#pragma unroll
+        for (int k = 0; k < KC / 2; ++k) {
+            x[0][k] = x[1][k] = make_float2(0.f, 0.f);
+            if (left >= KC / 2 || k < left) {
+                x[0][k] = ldg2(x0 + e * es);
+                x[1][k] = ldg2(x1 + e * es);
+            }
+            e += 2 * n + 1 + part;
+            ++n;
+        }
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            const float2 u = x[i & 1][i & ~1], v = x[i & 1][(i & ~1) + 1];
+            nxt[i] = make_float4(u.x, u.y, v.x, v.y);
+        }
+    }
+    __device__ __forceinline__ void take() {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
+    }
+    __device__ __forceinline__ void store(float* st, int sub, int lane) const {
+        st += canon(64 * sub + lane, 0) / 4;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            split_store(st + (canon(32 * (i & 1), 4 * (i >> 1)) >> 2), StcLayout<ST_C>::PLANE, cur[i]);
+    }
+};
+
+// B: E_mu / O_mu (mu = part + k) of v; lanes along the slots, 32 slots per
+// warp and chunk, 4 groups of 4 consecutive mu a lane.
+template <>
+struct Producer<ST_B> {
+    float2 nxt[16], cur[16];
+    __device__ __forceinline__ void load(const StcArgs& a, const StcItem& it, const int64_t*, const int32_t*, int sub,
+                                         int lane, int c) {
+        const int j = min(32 * sub + lane, it.ns - 1), left = it.K - c * KC, n = it.n;
+        const int64_t es = 8 * a.ns;
+        const char* v = (const char*)(a.X + it.s0 + j) + (n * n + (it.part ? n : 0) + it.part + c * KC) * es;
+        if (left >= KC) {
+#pragma unroll
+            for (int k = 0; k < KC; ++k) nxt[k] = ldg2(v + k * es);
+        } else {
+#pragma unroll
+            for (int k = 0; k < KC; ++k) {
+                nxt[k] = make_float2(0.f, 0.f);
+                if (k < left) nxt[k] = ldg2(v + k * es);
             }
         }
-        v[2 * i] = x.x;
-        v[2 * i + 1] = x.y;
     }
-}
-
-// stores them as rows 2j (real parts) and 2j + 1 (imaginary parts) of the
-// hi and lo A blocks of a stage
-__device__ __forceinline__ void stc_store(float* st, int j, int q, const float (&v)[8]) {
-    float4 rh, rl, ih, il;
-    float* prh = &rh.x;
-    float* prl = &rl.x;
-    float* pih = &ih.x;
-    float* pil = &il.x;
+    __device__ __forceinline__ void take() {
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float re = v[2 * i], im = v[2 * i + 1];
-        const float hr = tf32_hi(re), hi = tf32_hi(im);
-        prh[i] = hr;
-        prl[i] = re - hr;
-        pih[i] = hi;
-        pil[i] = im - hi;
+        for (int k = 0; k < KC; ++k) cur[k] = nxt[k];
     }
-    const int ore = canon(2 * j, 4 * q) >> 2, oim = canon(2 * j + 1, 4 * q) >> 2;
-    *reinterpret_cast<float4*>(st + ore) = rh;
-    *reinterpret_cast<float4*>(st + A_PLANE + ore) = rl;
-    *reinterpret_cast<float4*>(st + oim) = ih;
-    *reinterpret_cast<float4*>(st + A_PLANE + oim) = il;
+    __device__ __forceinline__ void store(float* st, int sub, int lane) const {
+        const int j = 32 * sub + lane;
+        st += canon(16 * (j >> 3) + (j & 7), 0) / 4;
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float2* x = cur + 4 * q;
+            float* d = st + q * (tcx::LBO / 4);
+            split_store(d, StcLayout<ST_B>::PLANE, make_float4(x[0].x, x[1].x, x[2].x, x[3].x));
+            split_store(d + tcx::SBO / 4, StcLayout<ST_B>::PLANE, make_float4(x[0].y, x[1].y, x[2].y, x[3].y));
+        }
+    }
+};
+
+// The accumulator of one item to its destination (one warp's share: 32 rows,
+// every SHARES-th group of 16 columns from the share-th on).  sg: 32 x STC_SG
+// floats of the warp (B).
+template <int PASS>
+__device__ __forceinline__ void stc_epilogue(const StcArgs& a, const StcItem& it, const int64_t* pos,
+                                             const int32_t* dir, uint32_t acc, int quad, int share, int lane,
+                                             float* sg) {
+    const int N = it.N, n = it.n, part = it.part, ns = it.ns;
+    const int64_t es = 8 * a.ns;
+    acc += (uint32_t)(quad * 32) << 16;
+    for (int c0 = 16 * share; c0 < N; c0 += 16 * StcLayout<PASS>::SHARES) {
+        uint32_t v[16];
+        if (PASS == ST_R) {
+            tcx::tmem_ld16(acc + (uint32_t)c0, v);
+            const int j = 16 * quad + 8 * (lane >> 4) + (lane & 7);
+            char* u = (char*)(a.out + it.s0 + j) + 4 * (lane >> 3 & 1) + (n * n + (part ? n : 0) + part + c0) * es;
+            const int left = j < ns ? N - c0 : 0;
+            if (left >= 16) {
+#pragma unroll
+                for (int i = 0; i < 16; ++i) *reinterpret_cast<uint32_t*>(u + i * es) = v[i];
+            } else {
+#pragma unroll
+                for (int i = 0; i < 16; ++i)
+                    if (i < left) *reinterpret_cast<uint32_t*>(u + i * es) = v[i];
+            }
+        } else if (PASS == ST_C) {
+            tcx::tmem_ld16(acc + (uint32_t)c0, v);
+            const int odd = quad >> 1, j = 32 * (quad & 1) + lane;   // (part: the block's first row)
+            const int left = j < ns && (odd == 0 || n > 0) ? (N - c0) / 2 : 0;
+            char* w = (char*)(a.out + pos[j]);
+            int n1 = n + part + c0 / 2, e = n1 * n1 + (odd ? n1 : 0) + n;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                if (t < left) *reinterpret_cast<uint2*>(w + e * es) = make_uint2(v[2 * t], v[2 * t + 1]);
+                e += 2 * n1 + 1 + odd;
+                ++n1;
+            }
+        } else {
+            // 16 lanes along m' of one slot, two slots 4 apart (their rows lie 16 banks apart)
+            const int i = lane & 15, mp = part + c0 + i, j0 = 16 * quad + 4 * (lane >> 4);
+            const bool in = c0 + i < N;
+            const char* bh = (const char*)(a.rph + a.prot - 1 + (in ? mp : 0));
+            const int pw = 8 * (2 * a.prot - 1);
+            int last = dir[j0];
+            float2 e = ldg2(bh + (int64_t)last * pw);   // (slots are sorted by direction)
+            tcx::tmem_ld16(acc + (uint32_t)c0, v);
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                *reinterpret_cast<uint4*>(sg + lane * STC_SG + 4 * q) =
+                    make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+            __syncwarp();
+            char* d0 = (char*)(a.out + (int64_t)n * n + n);   // entry (n, 0) of a target
+            char *dp = d0 + 8 * mp, *dm = d0 - 8 * mp;
+            const float sgn = part ? -0.5f : 0.5f;
+            const float* row = sg + 4 * (lane >> 4) * STC_SG + i;
+#pragma unroll
+            for (int t = 0; t < 8; ++t) {
+                const int j = j0 + 8 * (t >> 2) + (t & 3);
+                const float re = row[(16 * (t >> 2) + (t & 3)) * STC_SG], im = row[(16 * (t >> 2) + (t & 3) + 8) * STC_SG];
+                if (j < ns && in) {
+                    const int dj = dir[j];
+                    const int64_t o = 8 * pos[j];
+                    if (dj != last) {
+                        last = dj;
+                        e = ldg2(bh + (int64_t)dj * pw);
+                    }
+                    const float ex = 0.5f * e.x, ey = 0.5f * e.y, fx = sgn * e.x, fy = sgn * e.y;
+                    atomicAdd(reinterpret_cast<float2*>(dp + o), make_float2(re * ex + im * ey, im * ex - re * ey));
+                    if (mp > 0)
+                        atomicAdd(reinterpret_cast<float2*>(dm + o), make_float2(re * fx - im * fy, re * fy + im * fx));
+                }
+            }
+            __syncwarp();
+        }
+    }
 }
 
 template <int PASS>
-__global__ void __launch_bounds__(STC_THREADS, 2) k_stg_tc(const StcArgs a) {
+__device__ __forceinline__ void stc_body(const StcArgs& a) {
+    using L = StcLayout<PASS>;
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[STC_STAGES];    // A producers' stores
-    __shared__ __align__(8) uint64_t b_bar[STC_STAGES];       // the bulk copy of the table chunk
+    __shared__ __align__(8) uint64_t b_bar[STC_STAGES];       // the bulk copy of the chunk of T
     __shared__ __align__(8) uint64_t empty_bar[STC_STAGES];   // MMAs of the stage complete
+    __shared__ __align__(8) uint64_t acc_full[STC_ACC], acc_empty[STC_ACC];
+    __shared__ __align__(8) uint64_t idx_full[STC_RING], idx_empty[STC_RING];
     __shared__ __align__(8) uint64_t done_bar;
     __shared__ __align__(8) uint64_t never_bar;               // test hook: nothing arrives on it
+    __shared__ StcItem s_item[STC_RING];
+    __shared__ int64_t s_pos[STC_RING][STC_SLOTS];   // R: source, B: target expansion, C: slot
+    __shared__ int32_t s_dir[STC_RING][STC_SLOTS];   // R, B: direction (phases)
     __shared__ uint32_t tmem_holder;
-    __shared__ int64_t s_row[STC_SLOTS];   // slot * S (-1: padding row of zeros)
-    __shared__ int64_t s_dst[STC_SLOTS];   // pass R: the slot's row of u; pass B: its target expansion
-    __shared__ int32_t s_dir[STC_SLOTS];   // pass B: direction (phases)
     __shared__ int s_fail;
     const uint32_t raw = smem_u32(smem_raw);
     const uint32_t pad = (1024 - (raw & 1023)) & 1023;
     float* stage0 = (float*)(smem_raw + pad);
 
-    const StcTile tl = a.tiles[blockIdx.x];
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int part = tl.part;
-    if (tid < STC_SLOTS) {
-        const bool ok = tid < tl.ns;
-        const int sl = tl.s0 + tid;
-        // pass R: the source expansion of the slot; pass B: its row of v
-        s_row[tid] = ok ? (PASS == 0 ? a.slots[sl].src_off : (int64_t)sl * a.S) : -1;
-        s_dst[tid] = ok ? (PASS == 0 ? (int64_t)sl * a.S : a.slots[sl].dst_off) : 0;
-        s_dir[tid] = ok ? a.slots[sl].dir : 0;
-    }
+    const int nst = a.nst;
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(STC_TMEM_COLS));
+                     "r"(a.nacc * a.acc_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
         s_fail = 0;
         for (int s = 0; s < STC_STAGES; ++s) {
-            mbar_init(&full_bar[s], STC_NPROD);
+            mbar_init(&full_bar[s], L::PRODW / L::PERIOD);   // the warps of a chunk
             mbar_init(&b_bar[s], 1);
             mbar_init(&empty_bar[s], 1);
+        }
+        for (int b = 0; b < STC_ACC; ++b) {
+            mbar_init(&acc_full[b], 1);
+            mbar_init(&acc_empty[b], L::EPIW);
+        }
+        for (int r = 0; r < STC_RING; ++r) {
+            mbar_init(&idx_full[r], 1);
+            mbar_init(&idx_empty[r], STC_WORKW + 2);
         }
         mbar_init(&done_bar, 1);
         mbar_init(&never_bar, 1);
@@ -201,396 +421,299 @@ __global__ void __launch_bounds__(STC_THREADS, 2) k_stg_tc(const StcArgs a) {
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_holder;
-    const float* tabg = a.tab + (int64_t)tl.g * 2 * a.tper + (PASS ? a.tper : 0);
+    // this CTA's items: blockIdx.x, + gridDim.x, ...; the it-th is in ring entry it % STC_RING
+    const int nmine = (a.nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    auto item_wait = [&](int it) {
+        return mbar_wait(smem_u32(&idx_full[it % STC_RING]), (it / STC_RING) & 1, a.wait_limit);
+    };
 
-    if (warp < STC_PRODW) {
+    if (warp < L::PRODW) {
         // ---------------- A producers ---------------------------------------
-        const int j = tid >> 2, q = tid & 3;
-        const int64_t row = s_row[j];
-        const int dir = s_dir[j];
-        int n = tl.n0, kc = 0, N, K;
-        stc_dims(PASS, n, part, a.p_in, N, K);
-        float cur[8], nxt[8];
-        stc_load<PASS>(a, row, dir, n, part, K, 4 * q, cur);
-        for (int c = 0;; ++c) {
-            // the next chunk's loads go out before this one is stored
-            int n2 = n, kc2 = kc + 1, K2 = K;
-            if (kc2 * KC >= K) {
-                ++n2;
-                kc2 = 0;
-                if (n2 < tl.n1) stc_dims(PASS, n2, part, a.p_in, N, K2);
+        Producer<PASS> p;
+        constexpr int PER = L::PERIOD;
+        const int first = PASS == ST_R ? warp >> 2 : warp % PER, sub = PASS == ST_R ? warp & 3 : warp / PER;
+        int c = first, nkc = 0, it = -1;
+        // moves to this warp's next chunk; false at the end
+        auto seek = [&]() -> bool {
+            while (c >= nkc) {
+                __syncwarp();
+                if (it >= 0 && lane == 0) arrive(&idx_empty[it % STC_RING]);   // the item is no longer needed
+                c -= nkc;
+                nkc = 0;
+                if (++it >= nmine) return false;
+                if (!__all_sync(0xffffffffu, item_wait(it))) {
+                    atomicExch(&s_fail, 1);
+                    return false;
+                }
+                nkc = (s_item[it % STC_RING].K + KC - 1) / KC;
             }
-            const bool more = n2 < tl.n1;
-            if (more) stc_load<PASS>(a, row, dir, n2, part, K2, kc2 * KC + 4 * q, nxt);
-            const int s = c % STC_STAGES, u = c / STC_STAGES;
-            if (u > 0 && !mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, a.wait_limit)) {
+            return true;
+        };
+        auto load = [&]() {
+            const int r = it % STC_RING;
+            p.load(a, s_item[r], s_pos[r], s_dir[r], sub, lane, c);
+            c += PER;
+        };
+        bool more = seek(), next = false;
+        if (more) {
+            load();
+            next = seek();
+            p.take();
+        }
+        for (int s = first, u = 0; more; s += PER) {   // stage s of its u-th use
+            // the next chunk's loads go out before this one is stored, and its
+            // successor is looked up while they are on their way
+            if (next) load();
+            const bool after = next && seek();
+            while (s >= nst) {
+                s -= nst;
+                ++u;
+            }
+            const bool ok = u == 0 || mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, a.wait_limit);
+            if (!__all_sync(0xffffffffu, ok)) {
                 atomicExch(&s_fail, 1);
                 break;
             }
-            stc_store(stage0 + (size_t)s * a.stage_floats, j, q, cur);
+            p.store(stage0 + (size_t)s * a.stage_floats, sub, lane);
             // generic-proxy stores become visible to the tensor core's reads
             asm volatile("fence.proxy.async.shared::cta;");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])));
-            if (!more) break;
-#pragma unroll
-            for (int i = 0; i < 8; ++i) cur[i] = nxt[i];
-            n = n2;
-            kc = kc2;
-            K = K2;
+            __syncwarp();
+            if (lane == 0) arrive(&full_bar[s]);
+            if (next) p.take();
+            more = next;
+            next = after;
         }
-    } else if (warp == STC_PRODW) {
-        // ---------------- table chunks: one bulk copy per stage --------------
+    } else if (warp == L::PRODW) {
+        // ---------------- chunks of T: one bulk copy per stage ---------------
         if (lane == 0) {
-            int issued = 0;
+            int cc = 0, s = 0;
+            uint32_t ph = 1;
             bool fail = false;
-            for (int n = tl.n0, c = 0; n < tl.n1 && !fail; ++n) {
-                int N, K;
-                stc_dims(PASS, n, part, a.p_in, N, K);
-                const int np = stc_pad16(N), nkc = (K + KC - 1) / KC;
-                const float* tb = tabg + a.toff[2 * n + part];
-                const uint32_t bytes = (uint32_t)(2 * np * KC * sizeof(float));
-                for (int kc = 0; kc < nkc; ++kc, ++c) {
-                    const int s = c % STC_STAGES, u = c / STC_STAGES;
-                    if (u > 0 && !mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, a.wait_limit)) {
+            for (int it = 0; it < nmine && !fail; ++it) {
+                const int r = it % STC_RING;
+                if (!item_wait(it)) {
+                    atomicExch(&s_fail, 1);
+                    break;
+                }
+                const StcItem tl = s_item[r];
+                arrive(&idx_empty[r]);
+                const int blk = 2 * stc_pad16(tl.N) * KC, nkc = (tl.K + KC - 1) / KC;
+                const uint32_t bytes = (uint32_t)(blk * sizeof(float));
+                const float* g = a.tab + tl.tab + (PASS == ST_C ? 0 : ((int64_t)2 * tl.g + (PASS == ST_B)) * a.tper);
+                for (int c = 0; c < nkc; ++c, ++cc, g += blk) {
+                    if (cc >= nst && !mbar_wait(smem_u32(&empty_bar[s]), ph, a.wait_limit)) {
                         atomicExch(&s_fail, 1);
                         fail = true;
                         break;
                     }
                     const uint32_t bb = smem_u32(&b_bar[s]);
-                    const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_PLANE);
-                    const float* g = tb + (int64_t)kc * 2 * np * KC;
+                    const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * L::PLANE);
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb), "r"(bytes));
                     asm volatile(
                         "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
                             dB),
                         "l"(g), "r"(bytes), "r"(bb));
-                    ++issued;
+                    if (++s == nst) {
+                        s = 0;
+                        ph ^= 1;
+                    }
                 }
             }
             // every bulk copy this CTA issued lands before the CTA may exit
-            for (int c = std::max(0, issued - STC_STAGES); c < issued; ++c)
-                mbar_wait(smem_u32(&b_bar[c % STC_STAGES]), (c / STC_STAGES) & 1, DRAIN_LIMIT);
+            for (int k = cc > nst ? cc - nst : 0; k < cc; ++k)
+                mbar_wait(smem_u32(&b_bar[k % nst]), (uint32_t)(k / nst) & 1, DRAIN_LIMIT);
         }
         __syncwarp();
-    } else {
+    } else if (warp == L::PRODW + 1) {
         // ---------------- MMA issuer ----------------------------------------
         if (lane == 0) {
             // test hook: a wait on a barrier nothing arrives on runs out
-            const bool stalled = a.inject_stall && !mbar_wait(smem_u32(&never_bar), 0, a.wait_limit);
-            bool fail = stalled;
-            if (stalled) atomicExch(&s_fail, 1);
-            uint32_t col = 0;
-            for (int n = tl.n0, c = 0; n < tl.n1 && !fail; ++n) {
-                int N, K;
-                stc_dims(PASS, n, part, a.p_in, N, K);
-                const int np = stc_pad16(N), nkc = (K + KC - 1) / KC;
+            bool fail = a.inject_stall && !mbar_wait(smem_u32(&never_bar), 0, a.wait_limit);
+            if (fail) atomicExch(&s_fail, 1);
+            // operand descriptors: a stage's differ in their start address alone, a
+            // field of 16-byte units that no sum below carries out of
+            const uint32_t base = smem_u32(stage0);
+            const uint64_t dA0 = ((uint64_t)1 << 46) | ((uint64_t)(L::SBO >> 4) << 32) | ((uint64_t)(L::LBO >> 4) << 16) |
+                                 ((base & 0x3FFFF) >> 4);
+            const uint64_t dB0 = umma_desc(base + 2 * L::PLANE * 4);
+            const uint32_t a0 = (uint32_t)dA0, ahi = (uint32_t)(dA0 >> 32), b0 = (uint32_t)dB0, bhi = (uint32_t)(dB0 >> 32);
+            const uint32_t dstep = (uint32_t)(a.stage_floats * 4) >> 4;
+            auto desc = [](uint32_t lo, uint32_t hi) { return (uint64_t)hi << 32 | lo; };
+            int s = 0, b = 0;
+            uint32_t ph = 0, aph = 1, dof = 0;
+            // This thread's chain of waits (some 200 cycles each behind the other
+            // warps' shared-memory traffic) is longer than the MMAs: a stage's
+            // barriers are looked at while the one before is issued, the next
+            // item's while this one is.
+            bool ready = false, iready = false, aready = false;
+            int nN = 0, nK = 0;
+            auto peek_stage = [&](int s1, uint32_t p1) {
+                return mbar_test(smem_u32(&full_bar[s1]), p1) & mbar_test(smem_u32(&b_bar[s1]), p1);
+            };
+            for (int it = 0; it < nmine && !fail; ++it) {
+                const int r = it % STC_RING;
+                if (!iready) {
+                    if (!item_wait(it)) {
+                        atomicExch(&s_fail, 1);
+                        break;
+                    }
+                    nN = s_item[r].N;
+                    nK = s_item[r].K;
+                }
+                const int np = stc_pad16(nN), nkc = (nK + KC - 1) / KC;
+                arrive(&idx_empty[r]);
+                iready = false;
+                const int b1 = b + 1 == a.nacc ? 0 : b + 1;
+                const uint32_t ap1 = b1 == 0 ? aph ^ 1 : aph;
+                if (it + 1 < nmine) {   // (read early: valid if the barrier says so)
+                    const int r1 = (it + 1) % STC_RING;
+                    iready = mbar_test(smem_u32(&idx_full[r1]), ((it + 1) / STC_RING) & 1);
+                    nN = *(volatile int*)&s_item[r1].N;
+                    nK = *(volatile int*)&s_item[r1].K;
+                }
+                const bool adone = aready;
+                aready = it + 1 >= a.nacc && mbar_test(smem_u32(&acc_empty[b1]), ap1);
+                if (it >= a.nacc && !adone && !mbar_wait(smem_u32(&acc_empty[b]), aph, a.wait_limit)) {
+                    atomicExch(&s_fail, 1);
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols);
                 const uint32_t idesc = tcx::idesc_tf32(STC_M, np);
-                for (int kc = 0; kc < nkc; ++kc, ++c) {
-                    const int s = c % STC_STAGES, u = c / STC_STAGES;
-                    if (!mbar_wait(smem_u32(&full_bar[s]), u & 1, a.wait_limit) ||
-                        !mbar_wait(smem_u32(&b_bar[s]), u & 1, a.wait_limit)) {
+                const uint32_t blo = (uint32_t)(np * KC * 4) >> 4;   // from T's hi block to its lo block
+                for (int c = 0; c < nkc; ++c) {
+                    if (!ready && (!mbar_wait(smem_u32(&full_bar[s]), ph, a.wait_limit) ||
+                                   !mbar_wait(smem_u32(&b_bar[s]), ph, a.wait_limit))) {
                         atomicExch(&s_fail, 1);
                         fail = true;
                         break;
                     }
+                    const int s1 = s + 1 == nst ? 0 : s + 1;
+                    const uint32_t p1 = s1 == 0 ? ph ^ 1 : ph;
+                    ready = peek_stage(s1, p1);
                     asm volatile("tcgen05.fence::after_thread_sync;");
-                    const float* st = stage0 + (size_t)s * a.stage_floats;
-                    const uint32_t aH = smem_u32(st), aL = smem_u32(st + A_PLANE);
-                    const uint32_t bH = smem_u32(st + 2 * A_PLANE), bL = smem_u32(st + 2 * A_PLANE + np * KC);
 #pragma unroll
                     for (int ks = 0; ks < KC / 8; ++ks) {
-                        const uint32_t o = ks * 2 * LBO;
-                        const uint32_t first = (kc == 0 && ks == 0) ? 0u : 1u;
-                        mma_tf32(tmem + col, umma_desc(aH + o), umma_desc(bH + o), idesc, first);
-                        mma_tf32(tmem + col, umma_desc(aH + o), umma_desc(bL + o), idesc, 1u);
-                        mma_tf32(tmem + col, umma_desc(aL + o), umma_desc(bH + o), idesc, 1u);
+                        const uint32_t aH = a0 + dof + ((ks * 2 * L::LBO) >> 4), bH = b0 + dof + ((ks * 2 * tcx::LBO) >> 4);
+                        mma_tf32(acc, desc(aH, ahi), desc(bH, bhi), idesc, ks == 0 ? (uint32_t)c : 1u);
+                        mma_tf32(acc, desc(aH, ahi), desc(bH + blo, bhi), idesc, 1u);
+                        mma_tf32(acc, desc(aH + ((L::PLANE * 4) >> 4), ahi), desc(bH, bhi), idesc, 1u);
                     }
                     mma_commit(&empty_bar[s]);
+                    dof = s1 == 0 ? 0u : dof + dstep;
+                    s = s1;
+                    ph = p1;
                 }
-                col += np;
+                if (!fail) mma_commit(&acc_full[b]);
+                b = b1;
+                aph = ap1;
             }
             // completion of every MMA issued above (also on failure)
             mma_commit(&done_bar);
         }
         __syncwarp();
-    }
-
-    // ---------------- epilogue ------------------------------------------------
-    const bool done = mbar_wait(smem_u32(&done_bar), 0, DRAIN_LIMIT);
-    __syncthreads();
-    const bool ok = done && s_fail == 0;
-    if (!ok && tid == 0) atomicExch(a.err, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok && warp < STC_PRODW) {
-        const int quad = warp & 3, half = warp >> 2;
-        const int rr = quad * 32 + lane;           // accumulator lane = real row
-        const int j = rr >> 1, cpt = rr & 1;       // slot, 0: real / 1: imaginary part
-        const bool valid = j < tl.ns;
-        const float sgn = part ? -1.f : 1.f;
-        const cf* ph = a.rph + (int64_t)s_dir[j] * (2 * a.prot - 1) + (a.prot - 1);
-        uint32_t col = 0;
-        for (int n = tl.n0; n < tl.n1; ++n) {
-            int N, K;
-            stc_dims(PASS, n, part, a.p_in, N, K);
-            const int np = stc_pad16(N);
-            for (int g16 = half; g16 < np / 16; g16 += 2) {
-                uint32_t v[16];
-                tcx::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + col + (uint32_t)(g16 * 16), v);
-#pragma unroll
-                for (int qq = 0; qq < 8; ++qq) {
-                    // the real lane holds columns (c, c+1) of re, the imaginary
-                    // lane of im: trade so that each writes one complex value
-                    const float x0 = __uint_as_float(v[2 * qq]), x1 = __uint_as_float(v[2 * qq + 1]);
-                    const float recv = __shfl_xor_sync(0xffffffffu, cpt ? x0 : x1, 1);
-                    const float re = cpt ? recv : x0, im = cpt ? x1 : recv;
-                    const int i = g16 * 16 + 2 * qq + cpt;   // row of the degree block
-                    if (!valid || i >= N) continue;
-                    if (PASS == 0) {
-                        cf* u = a.out + s_dst[j] + (int64_t)n * n + (part ? n : 0) + part + i;
-                        *reinterpret_cast<float2*>(u) = make_float2(re, im);
-                    } else {
-                        const int mp = part + i;
-                        const float hr = 0.5f * re, hi = 0.5f * im;
-                        cf* d = a.out + s_dst[j] + (int64_t)n * n + n;   // entry (n, 0) of the target
-                        if (mp == 0) {
-                            atomicAdd(reinterpret_cast<float2*>(d), make_float2(hr, hi));
-                        } else {
-                            const cf e = ph[mp];
-                            atomicAdd(reinterpret_cast<float2*>(d + mp),
-                                      make_float2(hr * e.re + hi * e.im, hi * e.re - hr * e.im));
-                            atomicAdd(reinterpret_cast<float2*>(d - mp),
-                                      make_float2(sgn * (hr * e.re - hi * e.im), sgn * (hr * e.im + hi * e.re)));
-                        }
-                    }
-                }
-            }
-            col += np;
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(STC_TMEM_COLS));
-}
-
-// ---------------------------------------------------------------------------
-// Coaxial pass (complex blocks): D[v][(i, re/im)] = sum_k u_v[k] C[i][k] in
-// the real form with interleaved K (u as stored, complex = (re, im) pairs):
-//   A[v][(k, c)] = u_v[k].c  (v: virtual column = slot x even/odd part),
-//   B[(i, 0)][(k, 0)] = Re C,  B[(i, 0)][(k, 1)] = -Im C,
-//   B[(i, 1)][(k, 0)] = Im C,  B[(i, 1)][(k, 1)] = Re C,
-// so D[v][(i, 0)] = Re(sum u C), D[v][(i, 1)] = Im(sum u C): no zero blocks,
-// and each accumulator lane holds one output vector (degrees n' at a fixed
-// order), scattered into the degree-major folded v.
-struct StcCArgs {
-    const StcCTile* tiles;
-    const int32_t* cidx;
-    const float* tab;
-    const cf* U;
-    cf* V;
-    int* err;
-    long long wait_limit;
-    int S, p_out;
-    int stage_floats;
-    int nst;            // pipeline stages (<= STC_CSTAGES)
-    int inject_stall;
-};
-
-constexpr int STC_CSTAGES = 3;
-
-__global__ void __launch_bounds__(STC_THREADS, 2) k_stc_coax(const StcCArgs a) {
-    extern __shared__ unsigned char smem_raw[];
-    __shared__ __align__(8) uint64_t full_bar[STC_CSTAGES];
-    __shared__ __align__(8) uint64_t b_bar[STC_CSTAGES];
-    __shared__ __align__(8) uint64_t empty_bar[STC_CSTAGES];
-    __shared__ __align__(8) uint64_t done_bar;
-    __shared__ __align__(8) uint64_t never_bar;
-    __shared__ uint32_t tmem_holder;
-    __shared__ int64_t s_row[STC_M];   // slot * S (-1: padding row)
-    __shared__ int32_t s_odd[STC_M];
-    __shared__ int s_fail;
-    const uint32_t raw = smem_u32(smem_raw);
-    const uint32_t pad = (1024 - (raw & 1023)) & 1023;
-    float* stage0 = (float*)(smem_raw + pad);
-
-    const StcCTile tl = a.tiles[blockIdx.x];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int am = tl.am;
-    if (tid < STC_M) {
-        const int v = tl.vc0 + tid;
-        const bool ok = tid < tl.nvc;
-        const int slot = ok ? (am == 0 ? a.cidx[tl.c0 + v] : a.cidx[tl.c0 + (v >> 1)]) : 0;
-        s_row[tid] = ok ? (int64_t)slot * a.S : -1;
-        s_odd[tid] = (ok && am != 0 && (v & 1)) ? 1 : 0;
-    }
-    if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(STC_TMEM_COLS));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
-    }
-    if (tid == 0) {
-        s_fail = 0;
-        for (int s = 0; s < STC_CSTAGES; ++s) {
-            mbar_init(&full_bar[s], STC_NPROD);
-            mbar_init(&b_bar[s], 1);
-            mbar_init(&empty_bar[s], 1);
-        }
-        mbar_init(&done_bar, 1);
-        mbar_init(&never_bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
-    const uint32_t tmem = tmem_holder;
-    const int nst = a.nst;
-    const int np = stc_pad16(2 * tl.nr);
-    const int nkc = (2 * tl.K + KC - 1) / KC;   // K chunks of 8 complex input degrees
-
-    if (warp < STC_PRODW) {
-        // ---------------- A producers: 2 (row, 2 complex K values) units each
-        auto load = [&](int kc, int unit, float (&v)[4]) {
-            const int r = unit >> 2, q = unit & 3;
-            const int64_t row = s_row[r];
-#pragma unroll
-            for (int i = 0; i < 2; ++i) {
-                const int k = kc * (KC / 2) + 2 * q + i;
-                float2 x = make_float2(0.f, 0.f);
-                if (row >= 0 && k < tl.K) {
-                    const int n = am + k;
-                    x = __ldg(reinterpret_cast<const float2*>(a.U + row + (int64_t)n * n + (s_odd[r] ? n : 0) + am));
-                }
-                v[2 * i] = x.x;
-                v[2 * i + 1] = x.y;
-            }
-        };
-        float cur[2][4], nxt[2][4];
-        load(0, tid, cur[0]);
-        load(0, tid + STC_NPROD, cur[1]);
-        for (int c = 0; c < nkc; ++c) {
-            const bool more = c + 1 < nkc;
-            if (more) {
-                load(c + 1, tid, nxt[0]);
-                load(c + 1, tid + STC_NPROD, nxt[1]);
-            }
-            const int s = c % nst, u = c / nst;
-            if (u > 0 && !mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, a.wait_limit)) {
+    } else if (warp < STC_IDX0) {
+        // ---------------- epilogue --------------------------------------------
+        const int ew = warp - L::PRODW - 2, quad = warp & 3;
+        float* sg = stage0 + (size_t)nst * a.stage_floats + ew * 32 * STC_SG;
+        int b = 0;
+        uint32_t aph = 0;
+        for (int it = 0; it < nmine; ++it) {
+            const int r = it % STC_RING;
+            const bool known = mbar_test(smem_u32(&idx_full[r]), (it / STC_RING) & 1);
+            const bool ok = mbar_wait(smem_u32(&acc_full[b]), aph, a.wait_limit) && (known || item_wait(it));
+            if (!__all_sync(0xffffffffu, ok)) {   // the whole warp goes on or none of it
                 atomicExch(&s_fail, 1);
                 break;
             }
-            float* st = stage0 + (size_t)s * a.stage_floats;
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const int unit = tid + h * STC_NPROD;
-                const int r = unit >> 2, q = unit & 3;
-                float4 hi4, lo4;
-                float* ph = &hi4.x;
-                float* pl = &lo4.x;
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float t = tf32_hi(cur[h][i]);
-                    ph[i] = t;
-                    pl[i] = cur[h][i] - t;
-                }
-                const int o = canon(r, 4 * q) >> 2;
-                *reinterpret_cast<float4*>(st + o) = hi4;
-                *reinterpret_cast<float4*>(st + A_PLANE + o) = lo4;
+            asm volatile("tcgen05.fence::after_thread_sync;");
+            stc_epilogue<PASS>(a, s_item[r], s_pos[r], s_dir[r], tmem + (uint32_t)(b * a.acc_cols), quad,
+                               (ew / 4 + it) % L::SHARES, lane, sg);
+            // this warp's share of the accumulator is read
+            asm volatile("tcgen05.fence::before_thread_sync;");
+            __syncwarp();
+            if (lane == 0) {
+                arrive(&acc_empty[b]);
+                arrive(&idx_empty[r]);
             }
-            asm volatile("fence.proxy.async.shared::cta;");
-            asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])));
-            if (!more) break;
-#pragma unroll
-            for (int h = 0; h < 2; ++h)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) cur[h][i] = nxt[h][i];
-        }
-    } else if (warp == STC_PRODW) {
-        // ---------------- coaxial block chunks: one bulk copy per stage -----
-        if (lane == 0) {
-            int issued = 0;
-            const uint32_t bytes = (uint32_t)(2 * np * KC * sizeof(float));
-            for (int c = 0; c < nkc; ++c) {
-                const int s = c % nst, u = c / nst;
-                if (u > 0 && !mbar_wait(smem_u32(&empty_bar[s]), (u - 1) & 1, a.wait_limit)) {
-                    atomicExch(&s_fail, 1);
-                    break;
-                }
-                const uint32_t bb = smem_u32(&b_bar[s]);
-                const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_PLANE);
-                const float* g = a.tab + tl.toff + (int64_t)c * 2 * np * KC;
-                asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb), "r"(bytes));
-                asm volatile(
-                    "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dB),
-                    "l"(g), "r"(bytes), "r"(bb));
-                ++issued;
+            if (++b == a.nacc) {
+                b = 0;
+                aph ^= 1;
             }
-            for (int c = std::max(0, issued - nst); c < issued; ++c)
-                mbar_wait(smem_u32(&b_bar[c % nst]), (c / nst) & 1, DRAIN_LIMIT);
         }
-        __syncwarp();
     } else {
-        // ---------------- MMA issuer ----------------------------------------
-        if (lane == 0) {
-            const bool stalled = a.inject_stall && !mbar_wait(smem_u32(&never_bar), 0, a.wait_limit);
-            if (stalled) atomicExch(&s_fail, 1);
-            const uint32_t idesc = tcx::idesc_tf32(STC_M, np);
-            for (int c = 0; c < nkc && !stalled; ++c) {
-                const int s = c % nst, u = c / nst;
-                if (!mbar_wait(smem_u32(&full_bar[s]), u & 1, a.wait_limit) ||
-                    !mbar_wait(smem_u32(&b_bar[s]), u & 1, a.wait_limit)) {
-                    atomicExch(&s_fail, 1);
-                    break;
-                }
-                asm volatile("tcgen05.fence::after_thread_sync;");
-                const float* st = stage0 + (size_t)s * a.stage_floats;
-                const uint32_t aH = smem_u32(st), aL = smem_u32(st + A_PLANE);
-                const uint32_t bH = smem_u32(st + 2 * A_PLANE), bL = smem_u32(st + 2 * A_PLANE + np * KC);
+        // ---------------- items, up to STC_RING ahead; two warps in turn -----
+        auto slots_of = [&](const StcItem& tl, int64_t (&o)[2], int32_t (&d)[2]) {
 #pragma unroll
-                for (int ks = 0; ks < KC / 8; ++ks) {
-                    const uint32_t o = ks * 2 * LBO;
-                    const uint32_t first = (c == 0 && ks == 0) ? 0u : 1u;
-                    mma_tf32(tmem, umma_desc(aH + o), umma_desc(bH + o), idesc, first);
-                    mma_tf32(tmem, umma_desc(aH + o), umma_desc(bL + o), idesc, 1u);
-                    mma_tf32(tmem, umma_desc(aL + o), umma_desc(bH + o), idesc, 1u);
+            for (int q = 0; q < 2; ++q) {
+                const int j = tl.s0 + min(q * 32 + lane, tl.ns - 1);
+                d[q] = 0;
+                if (PASS == ST_C) {
+                    o[q] = __ldg(a.cidx + j);
+                } else {
+                    o[q] = PASS == ST_R ? __ldg(&a.slots[j].src_off) : __ldg(&a.slots[j].dst_off);
+                    d[q] = __ldg(&a.slots[j].dir);
                 }
-                mma_commit(&empty_bar[s]);
             }
-            mma_commit(&done_bar);
+        };
+        // every CTA starts elsewhere in its share (equal weights lie together):
+        // targets of different degrees at a time in B's adds
+        const int rot = (int)((int64_t)blockIdx.x * nmine / gridDim.x);
+        auto item_of = [&](int it) {
+            it += rot;
+            return a.items[blockIdx.x + (int64_t)(it < nmine ? it : it - nmine) * gridDim.x];
+        };
+        StcItem cur, nxt;
+        int64_t o[2], on[2];
+        int32_t d[2], dn[2];
+        int it = warp - STC_IDX0;
+        if (it < nmine) {
+            cur = item_of(it);
+            slots_of(cur, o, d);
         }
-        __syncwarp();
+        if (it + STC_IDXW < nmine) nxt = item_of(it + STC_IDXW);
+        for (; it < nmine; it += STC_IDXW) {
+            const int r = it % STC_RING;
+            if (it + STC_IDXW < nmine) slots_of(nxt, on, dn);
+            const bool ok = it < STC_RING || mbar_wait(smem_u32(&idx_empty[r]), (it / STC_RING - 1) & 1, a.wait_limit);
+            if (!__all_sync(0xffffffffu, ok)) {
+                atomicExch(&s_fail, 1);
+                break;
+            }
+            cur.uni = 0;
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (PASS == ST_R) {   // groups of 16 slots with one direction
+                    const uint32_t eq = __ballot_sync(0xffffffffu, d[q] == __shfl_sync(0xffffffffu, d[q], lane & 16));
+                    cur.uni |= (((eq & 0xffffu) == 0xffffu ? 1 : 0) | (eq >> 16 == 0xffffu ? 2 : 0)) << (2 * q);
+                }
+                s_pos[r][q * 32 + lane] = o[q];
+                s_dir[r][q * 32 + lane] = d[q];
+                o[q] = on[q];
+                d[q] = dn[q];
+            }
+            if (lane == 0) s_item[r] = cur;
+            __syncwarp();
+            if (lane == 0) arrive(&idx_full[r]);
+            cur = nxt;
+            if (it + 2 * STC_IDXW < nmine) nxt = item_of(it + 2 * STC_IDXW);
+        }
     }
 
-    // ---------------- epilogue: v[slot][n'^2 + (odd ? n' : 0) + am], n' = am + r0 + i
     const bool done = mbar_wait(smem_u32(&done_bar), 0, DRAIN_LIMIT);
     __syncthreads();
-    const bool ok = done && s_fail == 0;
-    if (!ok && tid == 0) atomicExch(a.err, 1);
+    if ((!done || s_fail) && tid == 0) atomicExch(a.err, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
-    if (ok && warp < STC_PRODW) {
-        const int quad = warp & 3, half = warp >> 2;
-        const int r = quad * 32 + lane;
-        const bool valid = r < tl.nvc;
-        cf* vout = a.V + (valid ? s_row[r] : 0) + am;
-        const int odd = s_odd[r];
-        for (int g16 = half; g16 < np / 16; g16 += 2) {
-            uint32_t v[16];
-            tcx::tmem_ld16(tmem + ((uint32_t)(quad * 32) << 16) + (uint32_t)(g16 * 16), v);
-            if (!valid) continue;
-#pragma unroll
-            for (int t = 0; t < 8; ++t) {
-                const int i = g16 * 8 + t;
-                const int n1 = am + tl.r0 + i;
-                if (i < tl.nr)
-                    *reinterpret_cast<float2*>(vout + (int64_t)n1 * n1 + (odd ? n1 : 0)) =
-                        make_float2(__uint_as_float(v[2 * t]), __uint_as_float(v[2 * t + 1]));
-            }
-        }
-    }
-    asm volatile("tcgen05.fence::before_thread_sync;");
-    __syncthreads();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(STC_TMEM_COLS));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.nacc * a.acc_cols));
 }
+
+// rotation (0) and back-rotation (1); coaxial pass
+template <int PASS>
+__global__ void __launch_bounds__(STC_THREADS, 1) k_stg_tc(const StcArgs a) {
+    stc_body<PASS>(a);
+}
+__global__ void __launch_bounds__(STC_THREADS, 1) k_stc_coax(const StcArgs a) { stc_body<ST_C>(a); }
 
 // Pre-split real-form coaxial blocks (grid: one CTA per block).
 __global__ void k_stc_coax_tables(const StcCBlock* __restrict__ blocks, const cd* __restrict__ coax,
@@ -670,58 +793,41 @@ int64_t fb_stc_layout(int P, std::vector<int64_t>& toff) {
     return off;
 }
 
-void fb_stc_group_tiles(int g, int g0, int g1, int nmax, int pass, int p_in, std::vector<StcTile>& out) {
-    for (int part = 0; part < 2; ++part) {
-        int n0 = -1, cols = 0;
-        auto flush = [&](int n1) {
-            if (n0 < 0) return;
-            for (int s0 = g0; s0 < g1; s0 += STC_SLOTS)
-                out.push_back(StcTile{g, part, n0, n1, s0, std::min(STC_SLOTS, g1 - s0)});
-            n0 = -1;
-            cols = 0;
-        };
-        for (int n = 0; n < nmax; ++n) {
-            int N, K;
-            stc_dims(pass, n, part, p_in, N, K);
-            if (N <= 0 || K <= 0) {
-                flush(n);
-                continue;
+void fb_stc_group_items(int g, int g0, int g1, int nmax, int pass, int p_in, std::vector<StcItem>& out) {
+    std::vector<int64_t> toff;
+    fb_stc_layout(nmax, toff);
+    for (int s0 = g0; s0 < g1; s0 += STC_SLOTS)
+        for (int n = 0; n < nmax; ++n)
+            for (int part = 0; part < 2; ++part) {
+                int N, K;
+                stc_dims(pass, n, part, p_in, N, K);
+                if (N > 0 && K > 0)
+                    out.push_back(StcItem{toff[2 * n + part], s0, std::min(STC_SLOTS, g1 - s0), n, part, N, K, g, 0});
             }
-            const int np = stc_pad16(N);
-            if (n0 >= 0 && cols + np > STC_TMEM_COLS) flush(n);
-            if (n0 < 0) n0 = n;
-            cols += np;
-        }
-        flush(nmax);
-    }
 }
 
-void fb_stc_coax_set(int c0, int ns, int64_t cs_off, int pc, int p_in, int p_out, std::vector<StcCTile>& tiles,
+void fb_stc_coax_set(int c0, int ns, int64_t cs_off, int pc, int p_in, int p_out, std::vector<StcItem>& items,
                      std::vector<StcCBlock>& blocks, int64_t* tfloats) {
-    const int q = std::min(p_in, p_out);
-    // one pre-split block per (order, row block)
-    std::vector<std::vector<int64_t>> toff(q);
-    for (int am = 0; am < q; ++am) {
+    for (int am = 0; am < std::min(p_in, p_out); ++am) {
         const int M = p_out - am, K = p_in - am;
         for (int r0 = 0; r0 < M; r0 += STC_CROWS) {
             const int nr = std::min(STC_CROWS, M - r0);
             const int np = stc_pad16(2 * nr), kp = ((2 * K + KC - 1) / KC) * KC;
             blocks.push_back(StcCBlock{cs_off, *tfloats, pc, am, r0, nr, K, 0});
-            toff[am].push_back(*tfloats);
+            for (int s0 = 0; s0 < ns; s0 += STC_SLOTS)
+                items.push_back(
+                    StcItem{*tfloats, c0 + s0, std::min(STC_SLOTS, ns - s0), am, r0, 2 * nr, 2 * K, 0, 0});
             *tfloats += (int64_t)2 * np * kp;
         }
     }
-    // slot blocks outermost, orders next (sectors of u and v shared by
-    // consecutive orders are used while in L2)
-    for (int sb = 0; sb < ns; sb += STC_M / 2)
-        for (int am = 0; am < q; ++am) {
-            const int M = p_out - am, K = p_in - am;
-            const int v0 = am == 0 ? sb : 2 * sb;
-            const int nvc = am == 0 ? std::min(STC_M / 2, ns - sb) : std::min(STC_M, 2 * (ns - sb));
-            int b = 0;
-            for (int r0 = 0; r0 < M; r0 += STC_CROWS, ++b)
-                tiles.push_back(StcCTile{toff[am][b], c0, v0, nvc, am, r0, std::min(STC_CROWS, M - r0), K, 0});
-        }
+}
+
+// the heaviest items first, in equal shares of every weight to the CTAs
+void fb_stc_sort(std::vector<StcItem>& items) {
+    std::stable_sort(items.begin(), items.end(), [](const StcItem& x, const StcItem& y) {
+        auto w = [](const StcItem& t) { return (int64_t)(stc_pad16(t.N) + 64) * ((t.K + KC - 1) / KC); };
+        return w(x) > w(y);
+    });
 }
 
 fb_status fb_stc_coax_tables(const StcCBlock* blocks, int nblocks, const cd* coax64, float* out, cudaStream_t s) {
@@ -732,61 +838,56 @@ fb_status fb_stc_coax_tables(const StcCBlock* blocks, int nblocks, const cd* coa
     return FB_OK;
 }
 
-fb_status fb_stc_coax_run(const StcCTile* tiles, int ntiles, const int32_t* cidx, const float* tab, const cf* U,
-                          cf* V, int S, int p_out, int* err, cudaStream_t s) {
-    if (ntiles == 0) return FB_OK;
-    const int npmax = stc_pad16(2 * std::min(STC_CROWS, p_out));
-    StcCArgs a;
-    a.tiles = tiles;
-    a.cidx = cidx;
-    a.tab = tab;
-    a.U = U;
-    a.V = V;
-    a.err = err;
-    a.wait_limit = fb_tc_wait_limit();
-    a.S = S;
-    a.p_out = p_out;
-    a.stage_floats = 2 * A_PLANE + 2 * npmax * KC;
-    // three stages while two CTAs still fit an SM, else two
-    a.nst = (size_t)STC_CSTAGES * a.stage_floats * sizeof(float) + 1024 <= 110 * 1024 ? STC_CSTAGES : 2;
-    a.inject_stall = fb_tc_inject_stall();
-    const size_t smem = std::max(STC_SMEM_MIN, (size_t)a.nst * a.stage_floats * sizeof(float) + 1024);
-    FB_CHECK(fb_smem_cap((const void*)k_stc_coax, smem));
-    k_stc_coax<<<(unsigned)ntiles, STC_THREADS, smem, s>>>(a);
-    FB_LAUNCH_CHECK();
-    fb_count_launch();
-    return FB_OK;
-}
-
-fb_status fb_stc_run(int pass, const StcTile* tiles, int ntiles, int npmax, const int64_t* toff, const float* tab,
-                     int64_t tper, const StgSlot* slots, const cf* X, cf* out, int S, int p_in, int p_out,
-                     const cf* rph, int prot, int* err, cudaStream_t s) {
-    if (ntiles == 0) return FB_OK;
-    if (npmax > STC_TMEM_COLS) return fb_fail(FB_ERR_ARG, "tensor-core staged RCR: order above 256");
+fb_status fb_stc_run(int pass, const StcItem* items, int nitems, int ncol_max, const float* tab, int64_t tper,
+                     const StgSlot* slots, const int32_t* cidx, const cf* X, cf* out, int64_t ns, const cf* rph,
+                     int prot, int* err, cudaStream_t s) {
+    if (nitems == 0) return FB_OK;
+    const int npmax = stc_pad16(ncol_max);
+    if (npmax > STC_COLS) return fb_fail(FB_ERR_ARG, "tensor-core staged RCR: order above 256");
     StcArgs a;
-    a.tiles = tiles;
-    a.toff = toff;
+    a.items = items;
+    a.nitems = nitems;
     a.tab = tab;
     a.tper = tper;
     a.slots = slots;
+    a.cidx = cidx;
     a.X = X;
     a.out = out;
     a.rph = rph;
     a.err = err;
     a.wait_limit = fb_tc_wait_limit();
-    a.S = S;
-    a.p_in = p_in;
-    a.p_out = p_out;
+    a.ns = ns;
     a.prot = prot;
-    a.stage_floats = 2 * A_PLANE + 2 * stc_pad16(npmax) * KC;
+    const int plane = pass == ST_R ? StcLayout<ST_R>::PLANE : StcLayout<ST_B>::PLANE;
+    a.stage_floats = 2 * plane + 2 * npmax * KC;
+    const size_t stage = a.stage_floats * sizeof(float);
+    const size_t fixed = 1024 + (pass == ST_B ? StcLayout<ST_B>::EPIW * 32 * STC_SG * sizeof(float) : 0);
+    a.nst = (int)std::min<size_t>(STC_STAGES, (STC_SMEM_MAX - fixed) / stage);
+    // a warp that stores every PERIOD-th chunk tells a stage's uses apart by
+    // their parity: at least as many stages
+    const int period = pass == ST_R   ? StcLayout<ST_R>::PERIOD
+                       : pass == ST_B ? StcLayout<ST_B>::PERIOD
+                                      : StcLayout<ST_C>::PERIOD;
+    if (a.nst < period) return fb_fail(FB_ERR_STATE, "tensor-core staged RCR: too few pipeline stages");
+    a.acc_cols = 32;
+    while (a.acc_cols < npmax) a.acc_cols *= 2;
+    a.nacc = std::min(STC_ACC, 2 * STC_COLS / a.acc_cols);
     a.inject_stall = fb_tc_inject_stall();
-    const size_t smem = std::max(STC_SMEM_MIN, (size_t)STC_STAGES * a.stage_floats * sizeof(float) + 1024);
-    const void* fn = pass == 0 ? (const void*)k_stg_tc<0> : (const void*)k_stg_tc<1>;
+    const size_t smem = std::max(STC_SMEM_MIN, a.nst * stage + fixed);
+    const void* fn = pass == ST_R   ? (const void*)k_stg_tc<ST_R>
+                     : pass == ST_B ? (const void*)k_stg_tc<ST_B>
+                                    : (const void*)k_stc_coax;
     FB_CHECK(fb_smem_cap(fn, smem));
-    if (pass == 0)
-        k_stg_tc<0><<<(unsigned)ntiles, STC_THREADS, smem, s>>>(a);
+    int dev = 0, sms = 0;
+    FB_CUDA(cudaGetDevice(&dev));
+    FB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    const unsigned grid = (unsigned)std::min(sms, nitems);
+    if (pass == ST_R)
+        k_stg_tc<ST_R><<<grid, STC_THREADS, smem, s>>>(a);
+    else if (pass == ST_B)
+        k_stg_tc<ST_B><<<grid, STC_THREADS, smem, s>>>(a);
     else
-        k_stg_tc<1><<<(unsigned)ntiles, STC_THREADS, smem, s>>>(a);
+        k_stc_coax<<<grid, STC_THREADS, smem, s>>>(a);
     FB_LAUNCH_CHECK();
     fb_count_launch();
     return FB_OK;
