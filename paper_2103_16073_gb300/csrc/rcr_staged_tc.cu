@@ -131,7 +131,7 @@ struct StcArgs {
 };
 
 __device__ __forceinline__ void arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)));
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
 
 // stores a row's 4 K values as TF32 hi and remainder
@@ -565,12 +565,8 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                 iready = false;
                 const int b1 = b + 1 == a.nacc ? 0 : b + 1;
                 const uint32_t ap1 = b1 == 0 ? aph ^ 1 : aph;
-                if (it + 1 < nmine) {   // (read early: valid if the barrier says so)
-                    const int r1 = (it + 1) % STC_RING;
-                    iready = mbar_test(smem_u32(&idx_full[r1]), ((it + 1) / STC_RING) & 1);
-                    nN = *(volatile int*)&s_item[r1].N;
-                    nK = *(volatile int*)&s_item[r1].K;
-                }
+                const int r1 = (it + 1) % STC_RING;
+                if (it + 1 < nmine) iready = mbar_test(smem_u32(&idx_full[r1]), ((it + 1) / STC_RING) & 1);
                 const bool adone = aready;
                 aready = it + 1 >= a.nacc && mbar_test(smem_u32(&acc_empty[b1]), ap1);
                 if (it >= a.nacc && !adone && !mbar_wait(smem_u32(&acc_empty[b]), aph, a.wait_limit)) {
@@ -603,6 +599,10 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                     dof = s1 == 0 ? 0u : dof + dstep;
                     s = s1;
                     ph = p1;
+                }
+                if (iready) {   // (read under the test's branch: never before its outcome is known)
+                    nN = s_item[r1].N;
+                    nK = s_item[r1].K;
                 }
                 if (!fail) mma_commit(&acc_full[b]);
                 b = b1;

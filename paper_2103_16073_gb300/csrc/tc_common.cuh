@@ -59,7 +59,8 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, long lo
             "{\n\t.reg .pred P1;\n\tmbarrier.try_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
             "selp.b32 %0, 1, 0, P1;\n\t}\n"
             : "=r"(ok)
-            : "r"(bar), "r"(parity));
+            : "r"(bar), "r"(parity)
+            : "memory");
         if (ok) return true;
     }
     return false;
@@ -72,7 +73,8 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
         "{\n\t.reg .pred P1;\n\tmbarrier.test_wait.parity.shared::cta.b64 P1, [%1], %2;\n\t"
         "selp.b32 %0, 1, 0, P1;\n\t}\n"
         : "=r"(ok)
-        : "r"(bar), "r"(parity));
+        : "r"(bar), "r"(parity)
+        : "memory");
     return ok != 0;
 }
 

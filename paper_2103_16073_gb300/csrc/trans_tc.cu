@@ -248,7 +248,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         auto seek = [&]() -> bool {
             while (c >= nkc) {
                 if (it >= 0 && lane == 0)   // the tile's offsets are no longer needed
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_empty[it % TC_RING])));
+                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_empty[it % TC_RING])) : "memory");
                 c -= nkc;
                 nkc = 0;
                 ++it;
@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             asm volatile("fence.proxy.async.shared::cta;");
             __syncwarp();
             if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])));
+                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])) : "memory");
             more = next;
         }
     } else if (warp == 8) {
@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 s_len[r] = 2 * tl.p_in2;
             }
             __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_full[r])));
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_full[r])) : "memory");
         }
     } else {
         // ---------------- epilogue: accumulator lanes 32 quad .. 32 quad + 31,
@@ -541,7 +541,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             // this warp's share of the accumulator is read
             asm volatile("tcgen05.fence::before_thread_sync;");
             __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])));
+            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
         }
     }
 
