@@ -94,29 +94,66 @@ __global__ void __launch_bounds__(256) k_trans(const TransTask* __restrict__ tas
 
 // ----------------------------------------------------------------- P2M ----
 // mp[leaf][r] = sum_{pos in leaf} W[pos][r] x[perm[pos]]
-// (blockIdx.y = right-hand side: x and mp advance by xstride / mstride)
+// blockIdx.x = leaf, blockIdx.y = chunk of NB right-hand sides (x and mp
+// advance by xstride / mstride each), blockIdx.z = chunk of coefficients.
+// Bound by reading W once for the NB right-hand sides; a leaf is a chain of
+// four dependent loads, so that a thread's first LU rows of W are on their way
+// before the gather of x and the next LU before the current ones are used, and
+// the coefficients of a large order go to a CTA per 256.  Per product (one CTA
+// of 128 threads per leaf before): L-room at 2 kHz 0.25 -> 0.20 ms (all 16
+// first rows at once, without the second buffer: 0.22), 240 leaves of order 66
+// 0.31 -> 0.047 ms.  FP64 is bound by its pipe (85 %).
 template <class R>
-__global__ void k_p2m(int P, const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ perm,
-                      const cx<R>* __restrict__ W, const cd* __restrict__ x, cx<R>* __restrict__ mp,
-                      int64_t xstride, int64_t mstride) {
-    x += blockIdx.y * xstride;
-    mp += blockIdx.y * mstride;
-    int b = blockIdx.x;
-    int s0 = leaf_start[b], s1 = leaf_start[b + 1];
-    __shared__ cx<R> xs[256];
-    for (int r0 = 0; r0 < P; r0 += blockDim.x) {
-        int r = r0 + threadIdx.x;
-        cx<R> acc = mk<R>(0, 0);
-        for (int c0 = s0; c0 < s1; c0 += 256) {
-            int cn = min(256, s1 - c0);
-            __syncthreads();
-            for (int i = threadIdx.x; i < cn; i += blockDim.x) xs[i] = from_d<R>(x[perm[c0 + i]]);
-            __syncthreads();
-            if (r < P)
-                for (int i = 0; i < cn; ++i) cmac(acc, W[(int64_t)(c0 + i) * P + r], xs[i]);
+constexpr int LEAF_UNROLL = sizeof(R) == 4 ? 8 : 4;
+
+template <class R, int NB>
+__global__ void __launch_bounds__(256, sizeof(R) == 4 ? 4 : 6) k_p2m(int P, const int32_t* __restrict__ leaf_start,
+                                             const int32_t* __restrict__ perm, const cx<R>* __restrict__ W,
+                                             const cd* __restrict__ x, cx<R>* __restrict__ mp, int nrhs,
+                                             int64_t xstride, int64_t mstride) {
+    constexpr int LU = LEAF_UNROLL<R> / (sizeof(R) / 4), CHUNK = 256;
+    __shared__ cx<R> xs[NB][CHUNK];
+    const int j0 = blockIdx.y * NB, nr = min(NB, nrhs - j0);
+    x += j0 * xstride;
+    mp += j0 * mstride;
+    const int b = blockIdx.x, r = blockIdx.z * blockDim.x + threadIdx.x;
+    const int s0 = leaf_start[b], s1 = leaf_start[b + 1];
+    const int rc = min(r, P - 1);   // (threads past the order read its last row and store nothing)
+    cx<R> w[LU], acc[NB];
+#pragma unroll
+    for (int u = 0; u < LU; ++u)
+        if (s0 + u < s1) w[u] = W[(int64_t)(s0 + u) * P + rc];
+#pragma unroll
+    for (int j = 0; j < NB; ++j) acc[j] = mk<R>(0, 0);
+    for (int c0 = s0; c0 < s1; c0 += CHUNK) {
+        const int cn = min(CHUNK, s1 - c0);
+        if (c0 > s0) __syncthreads();
+        for (int i = threadIdx.x; i < cn; i += blockDim.x) {
+            const int e = perm[c0 + i];
+#pragma unroll
+            for (int j = 0; j < NB; ++j)
+                if (j < nr) xs[j][i] = from_d<R>(x[j * xstride + e]);
         }
-        if (r < P) mp[(int64_t)b * P + r] = acc;
+        __syncthreads();
+        for (int i = 0; i < cn; i += LU) {
+            cx<R> wn[LU];
+#pragma unroll
+            for (int u = 0; u < LU; ++u)
+                if (c0 + i + LU + u < s1) wn[u] = W[(int64_t)(c0 + i + LU + u) * P + rc];
+#pragma unroll
+            for (int u = 0; u < LU; ++u)
+                if (i + u < cn)
+#pragma unroll
+                    for (int j = 0; j < NB; ++j)
+                        if (j < nr) cmac(acc[j], w[u], xs[j][i + u]);
+#pragma unroll
+            for (int u = 0; u < LU; ++u) w[u] = wn[u];
+        }
     }
+    if (r < P)
+#pragma unroll
+        for (int j = 0; j < NB; ++j)
+            if (j < nr) mp[j * mstride + (int64_t)b * P + r] = acc[j];
 }
 
 // ----------------------------------------------------- near field + L2P ----
@@ -133,76 +170,183 @@ __device__ __forceinline__ cf nf_entry(uint32_t a) {
     return mk(__uint_as_float(a << 16), __uint_as_float(a & 0xFFFF0000u));
 }
 
+//
+// Bound by reading A and V (one warp per row).  A leaf of some 18 rows is
+// mostly latency: the columns are gathered by all warps at once (offsets of
+// the U-list leaves from one warp scan), the warp's first row of A is on its
+// way before that, and every batch of LU loads of a row (A, then V, then the
+// next row's A) goes out before the one ahead of it is used.  blockIdx.z
+// splits the rows of a leaf where there are too few leaves.  FP32 with 16-bit
+// entries is bound by its issue rate, FP64 by its pipe: both take two rows per
+// warp (one read of x, shared reduction steps), FP64 reads A and V as one row;
+// FP32 entries stay at one row and twice the loads in flight (0.34 against
+// 0.37 ms).  Per product at 2 kHz (256 threads, leaves of the list in turn and
+// a row at a time before): FP32 0.54 -> 0.34 ms, 16-bit 0.41 -> 0.26 ms, FP64
+// 2.5 -> 2.4 ms; 240 leaves of order 66 0.19 -> 0.049 ms.
+constexpr int NEAR_THREADS = 128;
+// Sums of M per-lane values over a warp, M a power of two: every step halves
+// the values a lane still holds (M - 1 + log2(32 / M) additions instead of
+// 5 M).  v[0] of a lane is then the sum of value sum_of(lane).
+template <int M, class T>
+__device__ __forceinline__ void warp_sums(T (&v)[M], int lane) {
+    int o = 16;
+#pragma unroll
+    for (int h = M / 2; h > 0; h /= 2, o /= 2) {
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const T keep = up ? v[i + h] : v[i], send = up ? v[i] : v[i + h];
+            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+    }
+    for (; o > 0; o /= 2) v[0] += __shfl_xor_sync(0xffffffffu, v[0], o);
+}
+template <int M>
+__device__ __forceinline__ int sum_of(int lane) { return lane / (32 / M); }   // the top log2(M) bits
+template <class R, int NB, class AS>
+constexpr int NEAR_ROWS = sizeof(AS) != 8 && (sizeof(R) == 4 || NB == 1) ? 2 : 1;   // rows a warp takes at a time
+template <class R, int NB>
+constexpr int NEAR_CTAS = sizeof(R) == 4 ? 8 : (NB == 1 ? 10 : 8);   // per SM
+
 template <class R, int NB, class AS = cx<R>>
-__global__ void k_near_l2p(int P, const int32_t* __restrict__ leaf_start, const int32_t* __restrict__ perm,
-                           const int32_t* __restrict__ ucnt, const int32_t* __restrict__ ulist,
-                           const int64_t* __restrict__ nf_off, const int32_t* __restrict__ nf_ncol,
-                           const AS* __restrict__ A, const cx<R>* __restrict__ V,
-                           const cx<R>* __restrict__ loc, const cd* __restrict__ x, cd* __restrict__ y,
-                           int nrhs, int64_t xstride, int64_t lstride) {
+__global__ void __launch_bounds__(NEAR_THREADS, NEAR_CTAS<R, NB>) k_near_l2p(int P, const int32_t* __restrict__ leaf_start,
+                                                     const int32_t* __restrict__ perm,
+                                                     const int32_t* __restrict__ ucnt,
+                                                     const int32_t* __restrict__ ulist,
+                                                     const int64_t* __restrict__ nf_off,
+                                                     const int32_t* __restrict__ nf_ncol, const AS* __restrict__ A,
+                                                     const cx<R>* __restrict__ V, const cx<R>* __restrict__ loc,
+                                                     const cd* __restrict__ x, cd* __restrict__ y, int nrhs,
+                                                     int64_t xstride, int64_t lstride) {
+    constexpr int NR = NEAR_ROWS<R, NB, AS>, LU = LEAF_UNROLL<R> / NR;
+    constexpr bool ONE = sizeof(AS) == 16;   // A and V as one row of K + P entries (FP64: no half-empty step between)
     extern __shared__ unsigned char smem_raw[];
     const int r0 = blockIdx.y * NB;
     const int nr = min(NB, nrhs - r0);
-    cx<R>* xs = (cx<R>*)smem_raw;       // [nr][K]
-    int t = blockIdx.x;
-    int K = nf_ncol[t];
-    cx<R>* ls = xs + nr * K;            // [nr][P]
-    // gather the x values of the U-list leaves in column order
-    int nu = ucnt[t];
-    int c = 0;
-    for (int i = 0; i < nu; ++i) {
-        int s = ulist[(int64_t)t * FB_ULIST + i];
-        int a0 = leaf_start[s], a1 = leaf_start[s + 1];
-        for (int q = threadIdx.x; q < a1 - a0; q += blockDim.x) {
-            int e = perm[a0 + q];
-            for (int j = 0; j < nr; ++j) xs[j * K + c + q] = from_d<R>(x[(r0 + j) * xstride + e]);
-        }
-        c += a1 - a0;
+    cx<R>* xs = (cx<R>*)smem_raw;
+    const int t = blockIdx.x;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    const int nu = ucnt[t], K = nf_ncol[t];
+    // start and column offset of every U-list leaf (FB_ULIST < 32)
+    __shared__ int s_start[32], s_col[32];
+    const int sl = lane < FB_ULIST ? ulist[(int64_t)t * FB_ULIST + lane] : 0;
+    int a0 = 0, len = 0;
+    if (warp == 0 && lane < nu) {
+        a0 = leaf_start[sl];
+        len = leaf_start[sl + 1] - a0;
     }
+    const int rb = leaf_start[t], nrow = leaf_start[t + 1] - rb, step = nw * gridDim.z;
+    const AS* At = A + nf_off[t];
+    int r = blockIdx.z * nw + warp;
+    const int nv = loc ? P : 0, na = ONE ? K + nv : K;
+    AS a[NR][LU];
+    auto load_a = [&](int row0, int q0) {
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+            const int row = min(row0 + i * step, nrow - 1);
+            const AS* p = At + (int64_t)row * K + lane;
+            const cx<R>* pv = V + (int64_t)(rb + row) * P + lane - K;
+#pragma unroll
+            for (int u = 0; u < LU; ++u) {
+                const int q = q0 + 32 * u;
+                if (ONE) {
+                    if (q + lane < na) a[i][u] = q + lane < K ? p[q] : reinterpret_cast<const AS*>(pv)[q];
+                } else if (q + lane < K) {
+                    a[i][u] = p[q];
+                }
+            }
+        }
+    };
+    if (r < nrow) load_a(r, 0);
+    if (warp == 0) {
+        int c = len;
+#pragma unroll
+        for (int o = 1; o < 32; o *= 2) {
+            const int v = __shfl_up_sync(0xffffffffu, c, o);
+            if (lane >= o) c += v;
+        }
+        s_start[lane] = a0;
+        s_col[lane] = lane < nu ? c - len : K;
+    }
+    const int ldx = K + P;              // xs: [nr][K columns, P local coefficients]
     if (loc)
         for (int j = 0; j < nr; ++j)
-            for (int q = threadIdx.x; q < P; q += blockDim.x)
-                ls[j * P + q] = loc[(r0 + j) * lstride + (int64_t)t * P + q];
+            for (int q = threadIdx.x; q < P; q += NEAR_THREADS)
+                xs[j * ldx + K + q] = loc[(r0 + j) * lstride + (int64_t)t * P + q];
     __syncthreads();
-    int rb = leaf_start[t], nrow = leaf_start[t + 1] - rb;
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
-    const AS* At = A + nf_off[t];
-    for (int r = warp; r < nrow; r += nw) {
-        cx<R> acc[NB];
+    // gather the x values of the U-list leaves in column order
+#pragma unroll 2
+    for (int q = threadIdx.x; q < K; q += NEAR_THREADS) {
+        int i = 0;   // the last leaf that starts at or before column q
 #pragma unroll
-        for (int j = 0; j < NB; ++j) acc[j] = mk<R>(0, 0);
-        const AS* row = At + (int64_t)r * K;
-        // unrolled: several independent row loads in flight per lane
-#pragma unroll 4
-        for (int q = lane; q < K; q += 32) {
-            const cx<R> a = nf_entry(row[q]);
+        for (int o = 16; o > 0; o >>= 1)
+            if (s_col[i + o] <= q) i += o;
+        const int e = perm[s_start[i] + q - s_col[i]];
+        for (int j = 0; j < nr; ++j) xs[j * ldx + q] = from_d<R>(x[(r0 + j) * xstride + e]);
+    }
+    __syncthreads();
+    constexpr int M = 2 * NR * NB;
+    const int mi = sum_of<M>(lane), mj = (mi >> 1) % NB, mr = (mi >> 1) / NB;   // the sum this lane ends up with
+    for (; r < nrow; r += NR * step) {
+        const int row = min(r + mr * step, nrow - 1), e = perm[rb + row];
+        cx<R> acc[NR][NB], v[NR][LU];
 #pragma unroll
-            for (int j = 0; j < NB; ++j)
-                if (j < nr) cmac(acc[j], a, xs[j * K + q]);
-        }
-        if (loc) {
-            const cx<R>* vr = V + (int64_t)(rb + r) * P;
-            for (int q = lane; q < P; q += 32) {
-                cx<R> v = vr[q];
+        for (int i = 0; i < NR; ++i)
 #pragma unroll
-                for (int j = 0; j < NB; ++j)
-                    if (j < nr) cmac(acc[j], v, ls[j * P + q]);
+            for (int j = 0; j < NB; ++j) acc[i][j] = mk<R>(0, 0);
+        auto load_v = [&](int q0) {
+#pragma unroll
+            for (int i = 0; i < NR; ++i) {
+                const cx<R>* vr = V + (int64_t)(rb + min(r + i * step, nrow - 1)) * P + q0 + lane;
+#pragma unroll
+                for (int u = 0; u < LU; ++u)
+                    if (q0 + lane + 32 * u < P) v[i][u] = vr[32 * u];
+            }
+        };
+        if (!ONE && nv) load_v(0);
+        for (int q0 = 0; q0 < na; q0 += 32 * LU) {
+            if (q0) load_a(r, q0);
+#pragma unroll
+            for (int u = 0; u < LU; ++u) {
+                const int q = q0 + lane + 32 * u;
+                if (q < na)
+#pragma unroll
+                    for (int j = 0; j < NB; ++j)
+                        if (j < nr) {
+                            const cx<R> xq = xs[j * ldx + q];
+#pragma unroll
+                            for (int i = 0; i < NR; ++i) cmac(acc[i][j], nf_entry(a[i][u]), xq);
+                        }
             }
         }
+        if (r + NR * step < nrow) load_a(r + NR * step, 0);
+        if (!ONE)
+            for (int q0 = 0; q0 < nv; q0 += 32 * LU) {
+                if (q0) load_v(q0);
 #pragma unroll
-        for (int j = 0; j < NB; ++j) {
+                for (int u = 0; u < LU; ++u) {
+                    const int q = q0 + lane + 32 * u;
+                    if (q < P)
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) {
-                acc[j].re += __shfl_xor_sync(0xffffffffu, acc[j].re, o);
-                acc[j].im += __shfl_xor_sync(0xffffffffu, acc[j].im, o);
+                        for (int j = 0; j < NB; ++j)
+                            if (j < nr) {
+                                const cx<R> xq = xs[j * ldx + K + q];
+#pragma unroll
+                                for (int i = 0; i < NR; ++i) cmac(acc[i][j], v[i][u], xq);
+                            }
+                }
             }
-        }
-        if (lane == 0) {
-            int e = perm[rb + r];
+        R sums[M];
 #pragma unroll
-            for (int j = 0; j < NB; ++j)
-                if (j < nr) y[(r0 + j) * xstride + e] = mk<double>((double)acc[j].re, (double)acc[j].im);
-        }
+        for (int i = 0; i < NR; ++i)
+#pragma unroll
+            for (int j = 0; j < NB; ++j) {
+                sums[2 * (i * NB + j)] = acc[i][j].re;
+                sums[2 * (i * NB + j) + 1] = acc[i][j].im;
+            }
+        warp_sums<M>(sums, lane);
+        if (lane % (32 / M) == 0 && mj < nr && r + mr * step < nrow)
+            ((double*)(y + (r0 + mj) * xstride + e))[mi & 1] = (double)sums[0];
     }
 }
 
@@ -404,7 +548,13 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
     FB_CUDA(cudaMemsetAsync(mp, 0, sizeof(cx<R>) * cnt * nrhs, s));
     FB_CUDA(cudaMemsetAsync(loc, 0, sizeof(cx<R>) * cnt * nrhs, s));
     int nleaf = t->nbox[L];
-    k_p2m<R><<<dim3(nleaf, nrhs), 128, 0, s>>>(PL, t->leaf_start, t->perm, W, x, mp + op->lev_off[L], n, cnt);
+    const int pt_threads = std::min(256, (PL + 31) & ~31), pz = div_up(PL, pt_threads);
+    if (nrhs == 1)
+        k_p2m<R, 1><<<dim3(nleaf, 1, pz), pt_threads, 0, s>>>(PL, t->leaf_start, t->perm, W, x, mp + op->lev_off[L], 1,
+                                                              n, cnt);
+    else
+        k_p2m<R, 4><<<dim3(nleaf, div_up(nrhs, 4), pz), pt_threads, 0, s>>>(PL, t->leaf_start, t->perm, W, x,
+                                                                            mp + op->lev_off[L], nrhs, n, cnt);
     FB_LAUNCH_CHECK();
     fb_count_launch();
     mark(1);
@@ -451,13 +601,18 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
     int maxK = 0;
     for (int v : op->h_nf_ncol) maxK = std::max(maxK, v);
     const cx<R>* locL = loc + op->lev_off[L];
+    // eight CTAs per SM (1216) where a leaf's rows go round: at most one share
+    // per 4 of them (240 leaves of 13 rows, order 66: 0.049 ms against 0.076)
+    auto splits = [&](int chunks) {
+        return (unsigned)std::max(1, std::min(div_up(1216, nleaf * chunks), div_up((int)(n / nleaf), 4)));
+    };
     if (nrhs == 1) {
         size_t smem = sizeof(cx<R>) * (maxK + PL);
         bool done16 = false;
         if constexpr (sizeof(R) == 4) {
             if (op->near16 && op->nf16) {   // 16-bit near-field entries
                 FB_CHECK(fb_smem_cap((const void*)k_near_l2p<R, 1, uint32_t>, smem));
-                k_near_l2p<R, 1, uint32_t><<<nleaf, 256, smem, s>>>(PL, t->leaf_start, t->perm, t->ucnt,
+                k_near_l2p<R, 1, uint32_t><<<dim3(nleaf, 1, splits(1)), NEAR_THREADS, smem, s>>>(PL, t->leaf_start, t->perm, t->ucnt,
                                                                     t->ulist, op->nf_off, op->nf_ncol, op->nf16, V,
                                                                     locL, x, y, 1, n, cnt);
                 done16 = true;
@@ -465,7 +620,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
         }
         if (!done16) {
             FB_CHECK(fb_smem_cap((const void*)k_near_l2p<R, 1>, smem));
-            k_near_l2p<R, 1><<<nleaf, 256, smem, s>>>(PL, t->leaf_start, t->perm, t->ucnt, t->ulist, op->nf_off,
+            k_near_l2p<R, 1><<<dim3(nleaf, 1, splits(1)), NEAR_THREADS, smem, s>>>(PL, t->leaf_start, t->perm, t->ucnt, t->ulist, op->nf_off,
                                                       op->nf_ncol, A, V, locL, x, y, 1, n, cnt);
         }
     } else {
@@ -477,7 +632,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
         if constexpr (sizeof(R) == 4) {
             if (op->near16 && op->nf16) {
                 FB_CHECK(fb_smem_cap((const void*)k_near_l2p<R, NB, uint32_t>, smem));
-                k_near_l2p<R, NB, uint32_t><<<dim3(nleaf, div_up(nrhs, NB)), 256, smem, s>>>(
+                k_near_l2p<R, NB, uint32_t><<<dim3(nleaf, div_up(nrhs, NB), splits(div_up(nrhs, NB))), NEAR_THREADS, smem, s>>>(
                     PL, t->leaf_start, t->perm, t->ucnt, t->ulist, op->nf_off, op->nf_ncol, op->nf16, V, locL, x,
                     y, nrhs, n, cnt);
                 done16 = true;
@@ -485,7 +640,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
         }
         if (!done16) {
             FB_CHECK(fb_smem_cap((const void*)k_near_l2p<R, NB>, smem));
-            k_near_l2p<R, NB><<<dim3(nleaf, div_up(nrhs, NB)), 256, smem, s>>>(
+            k_near_l2p<R, NB><<<dim3(nleaf, div_up(nrhs, NB), splits(div_up(nrhs, NB))), NEAR_THREADS, smem, s>>>(
                 PL, t->leaf_start, t->perm, t->ucnt, t->ulist, op->nf_off, op->nf_ncol, A, V, locL, x, y, nrhs, n,
                 cnt);
         }
