@@ -15,7 +15,8 @@
 // memory.
 //
 // Tile: 128 pairs x a block of rows of T (at most 224, in equal blocks padded
-// to 16), accumulators double-buffered in tensor memory.
+// to 16; or two blocks of at most 160), accumulators double-buffered (two
+// blocks: a ring of three) in tensor memory.
 //
 // Operands:  A = gathered X rows, read as FP32 and split by the producer
 // warps on the way into the canonical layout.  B = T, pre-split and stored in
@@ -32,7 +33,8 @@
 //   warps 0-7    A producers: warp w takes every fourth chunk (w % 4) of 64
 //                pairs (w / 4), so that a chunk's fixed cost (waits, proxy
 //                fence, arrival) is spread over eight pieces per lane, with
-//                the loads of its next chunk in flight;
+//                the loads of its next chunk in flight (two blocks: every
+//                second chunk of 32 pairs, as only three stages fit);
 //   warp 8       lane 0: bulk copies of T (transaction count);
 //   warp 9       lane 0: MMA issuer (6 MMAs per chunk, commits to the stage's
 //                "empty" barrier in every CTA of the cluster, which keeps the
@@ -42,10 +44,13 @@
 //                coalesced runs of one pair's coefficients;
 //   warp 18      source offsets of the next tiles into a ring in shared
 //                memory, ahead of the producers.
-// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 1.16 ms (the
+// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 0.85 ms (the
 // MMAs alone 0.68 ms); 1.87 ms with pairs as N, one tile per CTA and hi/lo
 // planes of X split in a pass of its own.  The three tensor levels together
-// 2.14 ms against 3.54 ms; of the shoebox at 1 kHz 0.24 against 0.36 ms.
+// 1.83 ms against 3.54 ms; of the shoebox at 1 kHz 0.20 against 0.36 ms.
+// What is left is shared-memory bandwidth: the MMAs read 130 bytes per cycle
+// of it at their peak rate, the copies of T, the split X and the epilogue
+// share the rest.
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // flag, drains its own copies and MMAs (bounded) and releases tensor memory.
 #include <algorithm>
@@ -61,6 +66,11 @@ namespace {
 
 constexpr int TC_PAIRS = 128;     // box pairs per tile (MMA M)
 constexpr int TC_RMAX = 224;      // real output rows per tile (MMA N <= 256; four stages must fit)
+// ... of each of a tile's two blocks where one would not do: three accumulators
+// have to fit the 512 columns of tensor memory (the third takes the next tile's
+// first block while the last one's are read) and three stages shared memory
+constexpr int TC_RMAX2 = 160;
+constexpr int TC_ACC = 3;         // accumulators, at most
 constexpr int TC_KC = 16;         // real K per stage
 constexpr int TC_STAGES = 6;      // at most
 constexpr int A_BLOCK = TC_PAIRS * TC_KC;   // floats per (hi or lo) block of X
@@ -72,6 +82,8 @@ constexpr int TC_RING = 4;        // tiles of source offsets in shared memory
 constexpr int TC_CS = 32;         // accumulator columns staged per epilogue pass
 constexpr int TC_STAGING = EPI_WARPS * 32 * (TC_CS + 4);   // floats
 constexpr int TC_CLUSTER = 4;     // CTAs per cluster
+// a producer warp takes every fourth chunk, with two blocks every second one
+__host__ __device__ constexpr int tc_period(int nblk) { return nblk == 2 ? 2 : 4; }
 // drain bound of the shared copies: they land within microseconds, but after
 // a peer's timeout a stage may never get that peer's share
 constexpr long long SHARE_DRAIN = 1LL << 20;
@@ -115,14 +127,15 @@ struct TcTask {
     int32_t p_in2;                      // complex columns P_in
     int64_t src_base, dst_base;         // complex offsets of the source and target levels
 };
-// Columns [col0, col0 + ncol) of a task (ncol = 0 fills a cluster), real rows
-// from row0 on.  Its T is shared by the scount (1, 2 or 4) CTAs of the cluster
+// Columns [col0, col0 + ncol) of a task (ncol = 0 fills a cluster), NB blocks of
+// nrow real rows from row0 on (their chunks of T lie t_blk floats apart).  Its T is shared by the scount (1, 2 or 4) CTAs of the cluster
 // from rank sbase on.  The four tiles of a cluster have the same nkc and nrow.
 struct alignas(16) TcTile {
     int64_t t_off, pair_off, src_base, dst_base;
     int32_t p_in2, p_out2, nkc, nrow;
     int32_t row0, col0;
     int16_t ncol, sbase, scount, pad;
+    int64_t t_blk;
 };
 
 // Pre-split canonical tiles of the real interleaved form of a complex matrix.
@@ -168,6 +181,7 @@ struct TcArgs {
     int nst;           // pipeline stages
     int stage_floats;  // A hi, A lo, then the largest T block (hi, lo)
     int acc_cols;      // tensor memory columns of one accumulator
+    int nacc, tmem_cols;   // accumulators; columns to allocate
 };
 
 // 32 consecutive accumulator columns of this thread's lane
@@ -183,12 +197,14 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
     asm volatile("tcgen05.wait::ld.sync.aligned;");
 }
 
+template <int NB>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
+    constexpr int PER = tc_period(NB), NP = 2 * PER;   // a producer warp's chunks; its pieces of each per lane
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[TC_STAGES];    // A producers' stores
     __shared__ __align__(8) uint64_t b_bar[TC_STAGES];       // the bulk copies of T
     __shared__ __align__(8) uint64_t empty_bar[TC_STAGES];   // the MMAs of every CTA of the cluster
-    __shared__ __align__(8) uint64_t acc_full[2], acc_empty[2];
+    __shared__ __align__(8) uint64_t acc_full[TC_ACC], acc_empty[TC_ACC];
     __shared__ __align__(8) uint64_t done_bar;
     __shared__ __align__(8) uint64_t never_bar;              // test hook: nothing arrives on it
     __shared__ __align__(8) uint64_t idx_full[TC_RING], idx_empty[TC_RING];
@@ -206,17 +222,17 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     const TcTile* tiles = a.tiles + rank;   // this CTA's tile of cluster tile ct: tiles[ct * TC_CLUSTER]
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(2 * a.acc_cols));
+                     "r"(a.tmem_cols));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
     if (tid == 0) {
         s_fail = 0;
         for (int s = 0; s < TC_STAGES; ++s) {
-            mbar_init(&full_bar[s], PROD_WARPS / 4);   // the two warps of a chunk
+            mbar_init(&full_bar[s], PROD_WARPS / PER);   // the warps of a chunk
             mbar_init(&b_bar[s], 1);
             mbar_init(&empty_bar[s], TC_CLUSTER);
         }
-        for (int b = 0; b < 2; ++b) {
+        for (int b = 0; b < TC_ACC; ++b) {
             mbar_init(&acc_full[b], 1);
             mbar_init(&acc_empty[b], EPI_WARPS);
         }
@@ -234,15 +250,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     const uint32_t tmem = tmem_holder;
 
     if (warp < PROD_WARPS) {
-        // ---------------- A producers: 8 (pair, 4 K values) pieces a lane ----
+        // ---------------- A producers: NP (pair, 4 K values) pieces a lane ---
         // eight consecutive lanes store one 128-byte core matrix (no bank conflicts)
-        const int quarter = lane >> 3, jb = (warp >> 2) * 64 + (lane & 7);   // pairs jb + 8 i
+        const int quarter = lane >> 3, jb = warp / PER * (8 * NP) + (lane & 7);   // pairs jb + 8 i
         const int d0 = canon(jb, 4 * quarter) >> 2, dstep = tcx::SBO / 4;     // stage offset of piece i: d0 + i dstep
-        const float* g[8];
+        const float* g[NP];
         int len = 0;             // floats of a source expansion from the lane's quarter on
         uint32_t has = 0;        // pieces with a pair
         bool al = true;          // every piece 16-byte aligned
-        int c = warp & 3, nkc = 0, it = -1, ct = ct0 - ncl;   // load cursor: chunk of tile it
+        int c = warp % PER, nkc = 0, it = -1, ct = ct0 - ncl;   // load cursor: chunk of tile it
         bool fail = false;
         // moves the cursor to this warp's next chunk; false at the end
         auto seek = [&]() -> bool {
@@ -267,7 +283,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     has = 0;
                     al = true;
 #pragma unroll
-                    for (int i = 0; i < 8; ++i) {
+                    for (int i = 0; i < NP; ++i) {
                         const int64_t o = s_src[r][jb + 8 * i];
                         if (o >= 0) has |= 1u << i;
                         g[i] = (const float*)(a.src + (o >= 0 ? o : 0)) + 4 * quarter;
@@ -278,28 +294,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             }
             return true;
         };
-        auto fetch = [&](float4 (&v)[8]) {
+        auto fetch = [&](float4 (&v)[NP]) {
             const int n = len - c * TC_KC;   // an even count
             if (al && n >= 4) {
 #pragma unroll
-                for (int i = 0; i < 8; ++i)
+                for (int i = 0; i < NP; ++i)
                     v[i] = has >> i & 1 ? __ldg(reinterpret_cast<const float4*>(g[i] + c * TC_KC))
                                         : make_float4(0.f, 0.f, 0.f, 0.f);
             } else {
 #pragma unroll
-                for (int i = 0; i < 8; ++i) {
+                for (int i = 0; i < NP; ++i) {
                     float2 p = make_float2(0.f, 0.f), q = p;
                     if ((has >> i & 1) && n >= 2) p = __ldg(reinterpret_cast<const float2*>(g[i] + c * TC_KC));
                     if ((has >> i & 1) && n >= 4) q = __ldg(reinterpret_cast<const float2*>(g[i] + c * TC_KC) + 1);
                     v[i] = make_float4(p.x, p.y, q.x, q.y);
                 }
             }
-            c += 4;
+            c += PER;
         };
-        float4 cur[8], nxt[8];
+        float4 cur[NP], nxt[NP];
         bool more = seek();
         if (more) fetch(cur);
-        for (int s = warp & 3, u = 0; more; s += 4) {   // stage s of its u-th use
+        for (int s = warp % PER, u = 0; more; s += PER) {   // stage s of its u-th use
             const bool next = seek();
             if (next) fetch(nxt);
             while (s >= nst) {
@@ -313,7 +329,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             }
             float* st = stage0 + (size_t)s * a.stage_floats + d0;
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < NP; ++i) {
                 const float4 x = cur[i];
                 const float4 h = make_float4(tf32_hi(x.x), tf32_hi(x.y), tf32_hi(x.z), tf32_hi(x.w));
                 *reinterpret_cast<float4*>(st + i * dstep) = h;
@@ -352,17 +368,22 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     const uint32_t bb = smem_u32(&b_bar[s]);
                     const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_BLOCK + off);
                     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb),
-                                 "r"((uint32_t)(blk * sizeof(float))));
-                    if (tl.scount == 1)
-                        asm volatile(
-                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                dB),
-                            "l"(g), "r"((uint32_t)(blk * sizeof(float))), "r"(bb));
-                    else
-                        asm volatile(
-                            "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
-                            "[%1], %2, [%3], %4;" ::"r"(dB),
-                            "l"(g), "r"((uint32_t)(part * sizeof(float))), "r"(bb), "h"(smask));
+                                 "r"((uint32_t)(NB * blk * sizeof(float))));
+#pragma unroll
+                    for (int h = 0; h < NB; ++h) {
+                        const float* gh = g + h * tl.t_blk;
+                        const uint32_t dh = dB + (uint32_t)(h * blk * sizeof(float));
+                        if (tl.scount == 1)
+                            asm volatile(
+                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                                    dh),
+                                "l"(gh), "r"((uint32_t)(blk * sizeof(float))), "r"(bb));
+                        else
+                            asm volatile(
+                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
+                                "[%1], %2, [%3], %4;" ::"r"(dh),
+                                "l"(gh), "r"((uint32_t)(part * sizeof(float))), "r"(bb), "h"(smask));
+                    }
                     if (++s == nst) {
                         s = 0;
                         ph ^= 1;
@@ -381,8 +402,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             // test hook: a wait on a barrier nothing arrives on runs out
             bool fail = a.inject_stall && !mbar_wait(smem_u32(&never_bar), 0, a.wait_limit);
             if (fail) atomicExch(&s_fail, 1);
-            int s = 0, it = 0;
-            uint32_t ph = 0;
+            int s = 0, b = 0, unit = 0;   // unit: accumulators used so far
+            uint32_t ph = 0, aph = 1;
             // Operand descriptors differ in their start address alone, a field of
             // 16-byte units that no sum below carries out of (shared memory ends
             // below its 256 KB).
@@ -399,18 +420,28 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 nkc_n = tiles[(int64_t)ct0 * TC_CLUSTER].nkc;
                 nrow_n = tiles[(int64_t)ct0 * TC_CLUSTER].nrow;
             }
-            for (int ct = ct0; ct < a.nct && !fail; ct += ncl, ++it) {
+            for (int ct = ct0; ct < a.nct && !fail; ct += ncl) {
                 const int nkc = nkc_n, nrow = nrow_n;
                 if (ct + ncl < a.nct) {
                     nkc_n = tiles[(int64_t)(ct + ncl) * TC_CLUSTER].nkc;
                     nrow_n = tiles[(int64_t)(ct + ncl) * TC_CLUSTER].nrow;
                 }
-                const int b = it & 1;
-                if (it >= 2 && !mbar_wait(smem_u32(&acc_empty[b]), ((it >> 1) - 1) & 1, a.wait_limit)) {
-                    atomicExch(&s_fail, 1);
-                    break;
+                uint32_t acc[NB];
+                uint64_t* fullb[NB];
+#pragma unroll
+                for (int h = 0; h < NB; ++h, ++unit) {
+                    if (unit >= a.nacc && !fail && !mbar_wait(smem_u32(&acc_empty[b]), aph, a.wait_limit)) {
+                        atomicExch(&s_fail, 1);
+                        fail = true;
+                    }
+                    acc[h] = tmem + (uint32_t)(b * a.acc_cols);
+                    fullb[h] = &acc_full[b];
+                    if (++b == a.nacc) {
+                        b = 0;
+                        aph ^= 1;
+                    }
                 }
-                const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols);
+                if (fail) break;
                 const uint32_t idesc = tcx::idesc_tf32(TC_PAIRS, nrow);
                 const uint32_t blo = (uint32_t)(nrow * TC_KC * 4) >> 4;   // from T's hi block to its lo block
                 for (int c = 0; c < nkc; ++c) {
@@ -425,18 +456,23 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     ready = mbar_test(smem_u32(&full_bar[s1]), p1) & mbar_test(smem_u32(&b_bar[s1]), p1);
                     asm volatile("tcgen05.fence::after_thread_sync;");
 #pragma unroll
-                    for (int ks = 0; ks < TC_KC / 8; ++ks) {
-                        const uint32_t aH = dof + ((ks * 2 * LBO) >> 4), bH = aH + ((2 * A_BLOCK * 4) >> 4);
-                        mma_tf32(acc, desc(aH), desc(bH), idesc, ks == 0 ? (uint32_t)c : 1u);
-                        mma_tf32(acc, desc(aH + ((A_BLOCK * 4) >> 4)), desc(bH), idesc, 1u);
-                        mma_tf32(acc, desc(aH), desc(bH + blo), idesc, 1u);
-                    }
+                    for (int h = 0; h < NB; ++h)
+#pragma unroll
+                        for (int ks = 0; ks < TC_KC / 8; ++ks) {
+                            const uint32_t aH = dof + ((ks * 2 * LBO) >> 4),
+                                           bH = aH + ((2 * A_BLOCK * 4) >> 4) + h * 2 * blo;
+                            mma_tf32(acc[h], desc(aH), desc(bH), idesc, ks == 0 ? (uint32_t)c : 1u);
+                            mma_tf32(acc[h], desc(aH + ((A_BLOCK * 4) >> 4)), desc(bH), idesc, 1u);
+                            mma_tf32(acc[h], desc(aH), desc(bH + blo), idesc, 1u);
+                        }
                     mma_commit_to(&empty_bar[s], (uint16_t)((1 << TC_CLUSTER) - 1));
                     dof = s1 == 0 ? dlo : dof + dstep;
                     s = s1;
                     ph = p1;
                 }
-                if (!fail) mma_commit(&acc_full[b]);
+                if (!fail)
+#pragma unroll
+                    for (int h = 0; h < NB; ++h) mma_commit(fullb[h]);
             }
             // completion of every MMA issued above (also on failure)
             mma_commit(&done_bar);
@@ -484,8 +520,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         float* row = sg + lane * (TC_CS + 4);
         TcTile tn;
         if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
-        int it = 0;
-        for (int ct = ct0; ct < a.nct; ct += ncl, ++it) {
+        int b = 0;
+        uint32_t aph = 0;
+        bool fail = false;
+        for (int ct = ct0; ct < a.nct && !fail; ct += ncl) {
             const TcTile tl = tn;
             const int j = quad * 32 + lane;   // this lane's pair
             int64_t dst = 0;                  // its target expansion (floats)
@@ -495,53 +533,60 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                            (int64_t)a.dst_idx[tl.pair_off + pr] * tl.p_out2) + tl.row0;
             }
             if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
-            const int b = it & 1;
-            const bool full = mbar_wait(smem_u32(&acc_full[b]), (it >> 1) & 1, a.wait_limit);
-            if (!__all_sync(0xffffffffu, full)) {   // the whole warp goes on or none of it
-                atomicExch(&s_fail, 1);
-                break;
-            }
-            asm volatile("tcgen05.fence::after_thread_sync;");
-            const int npair = min(32, tl.ncol - quad * 32), rows = min(tl.nrow, 2 * tl.p_out2 - tl.row0);
-            const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols) + ((uint32_t)(quad * 32) << 16);
-            // 16-byte adds where every target of the warp is aligned to them
-            const bool wide = __all_sync(0xffffffffu, (dst & 3) == 0 && (((uintptr_t)a.dst) & 15) == 0);
-            int c0 = half * TC_CS;
-            for (; c0 < tl.nrow; c0 += 2 * TC_CS) {
-                uint32_t v[32];   // (columns past the block lie within the accumulator's)
-                tmem_ld32(acc + (uint32_t)c0, v);
+#pragma unroll 1
+            for (int h = 0; h < NB; ++h, dst += tl.nrow) {
+                const bool full = mbar_wait(smem_u32(&acc_full[b]), aph, a.wait_limit);
+                if (!__all_sync(0xffffffffu, full)) {   // the whole warp goes on or none of it
+                    atomicExch(&s_fail, 1);
+                    fail = true;
+                    break;
+                }
+                asm volatile("tcgen05.fence::after_thread_sync;");
+                const int npair = min(32, tl.ncol - quad * 32), rows = min(tl.nrow, 2 * tl.p_out2 - tl.row0 - h * tl.nrow);
+                const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols) + ((uint32_t)(quad * 32) << 16);
+                // 16-byte adds where every target of the warp is aligned to them
+                const bool wide = __all_sync(0xffffffffu, (dst & 3) == 0 && (((uintptr_t)a.dst) & 15) == 0);
+                int c0 = half * TC_CS;
+                for (; c0 < tl.nrow; c0 += 2 * TC_CS) {
+                    uint32_t v[32];   // (columns past the block lie within the accumulator's)
+                    tmem_ld32(acc + (uint32_t)c0, v);
 #pragma unroll
-                for (int q = 0; q < 8; ++q)
-                    *reinterpret_cast<uint4*>(row + 4 * q) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-                __syncwarp();
-                float* dp = (float*)a.dst + c0;
-                const int rn = rows - c0;   // an even count
-                if (wide) {   // 8 lanes a pair, 4 pairs at a time
-                    const int k = 4 * (lane & 7);
+                    for (int q = 0; q < 8; ++q)
+                        *reinterpret_cast<uint4*>(row + 4 * q) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
+                    __syncwarp();
+                    float* dp = (float*)a.dst + c0;
+                    const int rn = rows - c0;   // an even count
+                    if (wide) {   // 8 lanes a pair, 4 pairs at a time
+                        const int k = 4 * (lane & 7);
 #pragma unroll 4
-                    for (int t = lane >> 3; t < 32; t += 4) {
-                        const int64_t dt = __shfl_sync(0xffffffffu, dst, t);
-                        const float4 x = *reinterpret_cast<const float4*>(sg + t * (TC_CS + 4) + k);
-                        if (t < npair) {
-                            if (k + 4 <= rn) atomicAdd(reinterpret_cast<float4*>(dp + dt + k), x);
-                            else if (k + 2 <= rn) atomicAdd(reinterpret_cast<float2*>(dp + dt + k), make_float2(x.x, x.y));
+                        for (int t = lane >> 3; t < 32; t += 4) {
+                            const int64_t dt = __shfl_sync(0xffffffffu, dst, t);
+                            const float4 x = *reinterpret_cast<const float4*>(sg + t * (TC_CS + 4) + k);
+                            if (t < npair) {
+                                if (k + 4 <= rn) atomicAdd(reinterpret_cast<float4*>(dp + dt + k), x);
+                                else if (k + 2 <= rn) atomicAdd(reinterpret_cast<float2*>(dp + dt + k), make_float2(x.x, x.y));
+                            }
+                        }
+                    } else {      // 16 lanes a pair, 2 pairs at a time
+                        const int k = 2 * (lane & 15);
+#pragma unroll 4
+                        for (int t = lane >> 4; t < 32; t += 2) {
+                            const int64_t dt = __shfl_sync(0xffffffffu, dst, t);
+                            const float2 x = *reinterpret_cast<const float2*>(sg + t * (TC_CS + 4) + k);
+                            if (t < npair && k + 2 <= rn) atomicAdd(reinterpret_cast<float2*>(dp + dt + k), x);
                         }
                     }
-                } else {      // 16 lanes a pair, 2 pairs at a time
-                    const int k = 2 * (lane & 15);
-#pragma unroll 4
-                    for (int t = lane >> 4; t < 32; t += 2) {
-                        const int64_t dt = __shfl_sync(0xffffffffu, dst, t);
-                        const float2 x = *reinterpret_cast<const float2*>(sg + t * (TC_CS + 4) + k);
-                        if (t < npair && k + 2 <= rn) atomicAdd(reinterpret_cast<float2*>(dp + dt + k), x);
-                    }
+                    __syncwarp();
                 }
+                // this warp's share of the accumulator is read
+                asm volatile("tcgen05.fence::before_thread_sync;");
                 __syncwarp();
+                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
+                if (++b == a.nacc) {
+                    b = 0;
+                    aph ^= 1;
+                }
             }
-            // this warp's share of the accumulator is read
-            asm volatile("tcgen05.fence::before_thread_sync;");
-            __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
         }
     }
 
@@ -550,14 +595,14 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     if ((!done || s_fail) && tid == 0) atomicExch(a.err, 1);
     asm volatile("tcgen05.fence::after_thread_sync;");
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(2 * a.acc_cols));
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols));
     cluster_sync();   // no CTA leaves while a peer may still write its shared memory or signal its barriers
 }
 
 // ------------------------------------------------------------- host side ----
 // One launch: the tiles of the tasks with the same accumulator size.
 struct TcLaunch {
-    int rows_max = 0, acc_cols = 0;
+    int rows_max = 0, acc_cols = 0, nblk = 1, nacc = 2, tmem_cols = 0;
     std::vector<int> tasks;
     int nst = 0, resident = 1;   // pipeline stages, clusters resident at once
     size_t smem = 0;
@@ -578,6 +623,7 @@ struct TcPlanImpl {
 };
 
 static size_t tc_stage_bytes(int rows) { return (size_t)(2 * A_BLOCK + 2 * rows * TC_KC) * sizeof(float); }
+static const void* tc_kernel(int nblk) { return nblk == 2 ? (const void*)k_trans_tc<2> : (const void*)k_trans_tc<1>; }
 
 static void tc_launch_config(const TcLaunch& ln, int clusters, cudaStream_t s, cudaLaunchConfig_t* cfg,
                              cudaLaunchAttribute* at) {
@@ -594,21 +640,21 @@ static void tc_launch_config(const TcLaunch& ln, int clusters, cudaStream_t s, c
     cfg->numAttrs = 1;
 }
 // Stages and shared memory of a launch (one CTA per SM: at least a share
-// such that no second CTA's allocation waits for tensor memory).  At least
-// four stages: a producer warp stores every fourth chunk, so when it waits
-// for a stage's last use, all uses before that one must be known complete
-// (its previous chunk's wait covers them from four stages on), or the
-// barrier's phase parity would be ambiguous.
+// such that no second CTA's allocation waits for tensor memory).  At least as
+// many stages as a producer warp's period of chunks: when it waits for a
+// stage's last use, all uses before that one must be known complete (its
+// previous chunk's wait covers them then), or the barrier's phase parity
+// would be ambiguous.
 static fb_status tc_configure(TcLaunch& ln) {
-    const size_t stage = tc_stage_bytes(ln.rows_max), fixed = TC_STAGING * sizeof(float) + 1024;
+    const size_t stage = tc_stage_bytes(ln.nblk * ln.rows_max), fixed = TC_STAGING * sizeof(float) + 1024;
     ln.nst = (int)std::max<size_t>(2, std::min<size_t>(TC_STAGES, (220 * 1024 - fixed) / stage));
-    if (ln.nst < 4) return fb_fail(FB_ERR_STATE, "tensor-core translation: fewer than four pipeline stages");
+    if (ln.nst < tc_period(ln.nblk)) return fb_fail(FB_ERR_STATE, "tensor-core translation: too few pipeline stages");
     ln.smem = std::max(ln.nst * stage + fixed, (size_t)116 * 1024);
-    FB_CHECK(fb_smem_cap((const void*)k_trans_tc, ln.smem));
+    FB_CHECK(fb_smem_cap(tc_kernel(ln.nblk), ln.smem));
     cudaLaunchConfig_t cfg;
     cudaLaunchAttribute at;
     tc_launch_config(ln, 1, nullptr, &cfg, &at);
-    FB_CUDA(cudaOccupancyMaxActiveClusters(&ln.resident, k_trans_tc, &cfg));
+    FB_CUDA(cudaOccupancyMaxActiveClusters(&ln.resident, tc_kernel(ln.nblk), &cfg));
     ln.resident = std::max(1, ln.resident);
     return FB_OK;
 }
@@ -626,7 +672,7 @@ static void tc_make_tiles(const TcPlanImpl* pl, int nrhs, std::vector<TcTile>& o
             for (int ti : kv.second) {
                 const TcTask& tk = pl->h_tasks[ti];
                 const int ncol = tk.npairs * nrhs, nc = div_up(ncol, TC_PAIRS);
-                for (int rt = 0; rt < tk.nrt; ++rt) {
+                for (int rt = 0; rt < tk.nrt; rt += ln.nblk) {
                     auto tile = [&](int c, int scount) {
                         TcTile t;
                         t.t_off = tk.a_off + (int64_t)rt * tk.nkc * 2 * tk.rt_rows * TC_KC;
@@ -643,6 +689,7 @@ static void tc_make_tiles(const TcPlanImpl* pl, int nrhs, std::vector<TcTile>& o
                         t.sbase = 0;
                         t.scount = (int16_t)scount;
                         t.pad = 0;
+                        t.t_blk = (int64_t)tk.nkc * 2 * tk.rt_rows * TC_KC;
                         return t;
                     };
                     int c = 0;
@@ -711,7 +758,13 @@ fb_status fb_tc_build_groups(fb_op* op, const std::vector<TcGroup>& groups, cons
         tk.a_off = pl->a_floats;
         tk.pair_off = g.pair_off;
         tk.npairs = g.npairs;
+        // Two blocks of rows in one tile where that is all rows (orders 11 and
+        // 12): X is gathered and split once instead of twice, order 12 0.85
+        // against 1.16 ms (level 7 above).  With more tiles the three stages it
+        // leaves cost more than the gathers saved: order 20 in 3 x 2 blocks of
+        // 144 0.59 ms, in 4 of 208 0.56 ms.
         tk.nrt = div_up(2 * Pout, TC_RMAX);
+        const int nblk = tk.nrt == 2 && 2 * Pout <= 2 * TC_RMAX2 ? 2 : 1;
         tk.rt_rows = (div_up(2 * Pout, tk.nrt) + 15) & ~15;
         tk.nkc = div_up(2 * Pin, TC_KC);
         tk.p_out2 = Pout;
@@ -720,11 +773,15 @@ fb_status fb_tc_build_groups(fb_op* op, const std::vector<TcGroup>& groups, cons
         tk.dst_base = op->lev_off[g.dst_level];
         int cols = 32;
         while (cols < tk.rt_rows) cols *= 2;
+        if (nblk == 2) cols = std::min(cols, TC_RMAX2);
         auto ln = std::find_if(pl->launches.begin(), pl->launches.end(),
-                               [&](const TcLaunch& l) { return l.acc_cols == cols; });
+                               [&](const TcLaunch& l) { return l.acc_cols == cols && l.nblk == nblk; });
         if (ln == pl->launches.end()) {
             TcLaunch l;
             l.acc_cols = cols;
+            l.nblk = nblk;
+            l.nacc = nblk == 2 ? 3 : 2;
+            l.tmem_cols = nblk == 2 ? 512 : 2 * cols;
             ln = pl->launches.insert(pl->launches.end(), l);
         }
         ln->rows_max = std::max(ln->rows_max, (int)tk.rt_rows);
@@ -788,12 +845,17 @@ fb_status fb_tc_run(fb_op* op, void* plan, const cf* src, cf* dst, cudaStream_t 
         a.nct = tiles->count[i];
         a.acc_cols = ln.acc_cols;
         a.nst = ln.nst;
-        a.stage_floats = (int)(tc_stage_bytes(ln.rows_max) / sizeof(float));
-        FB_CHECK(fb_smem_cap((const void*)k_trans_tc, ln.smem));
+        a.nacc = ln.nacc;
+        a.tmem_cols = ln.tmem_cols;
+        a.stage_floats = (int)(tc_stage_bytes(ln.nblk * ln.rows_max) / sizeof(float));
+        FB_CHECK(fb_smem_cap(tc_kernel(ln.nblk), ln.smem));
         cudaLaunchAttribute at;
         cudaLaunchConfig_t cfg;
         tc_launch_config(ln, std::min(ln.resident, a.nct), s, &cfg, &at);
-        FB_CUDA(cudaLaunchKernelEx(&cfg, k_trans_tc, a));
+        if (ln.nblk == 2)
+            FB_CUDA(cudaLaunchKernelEx(&cfg, k_trans_tc<2>, a));
+        else
+            FB_CUDA(cudaLaunchKernelEx(&cfg, k_trans_tc<1>, a));
         fb_count_launch();
     }
     return FB_OK;
