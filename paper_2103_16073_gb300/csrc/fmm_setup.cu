@@ -584,9 +584,12 @@ fb_status fb_compose_jobs(fb_op* op, const std::vector<int>& which, cudaStream_t
         k_compose<<<grid, 256, 0, s>>>(djobs + j0, op->rot64, op->Prot, op->coax64, op->T64);
     }
     if (op->T32)
-        for (auto& jb : todo) {
-            int64_t cnt = (int64_t)jb.p_out * jb.p_out * jb.p_in * jb.p_in;
-            k_d2f<<<div_up(cnt, 256), 256, 0, s>>>(op->T64 + jb.t_off, op->T32 + jb.t_off, cnt);
+        for (size_t i = 0; i < todo.size();) {   // one launch per run of adjacent matrices
+            const int64_t t0 = todo[i].t_off;
+            int64_t t1 = t0;
+            for (; i < todo.size() && todo[i].t_off == t1; ++i)
+                t1 += (int64_t)todo[i].p_out * todo[i].p_out * todo[i].p_in * todo[i].p_in;
+            k_d2f<<<div_up(t1 - t0, 256), 256, 0, s>>>(op->T64 + t0, op->T32 + t0, t1 - t0);
         }
     FB_LAUNCH_CHECK();
     cudaError_t e = cudaStreamSynchronize(s);

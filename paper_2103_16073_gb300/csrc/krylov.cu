@@ -528,52 +528,66 @@ fb_status fb_self_blocks(const fb_op* op, const int64_t* d_off, cd* out, cudaStr
 
 // In-place Gauss-Jordan inverse with partial pivoting of the block of leaf t
 // (order `scale` x its element count; scale 2 for the indirect system).
+// The block stays in shared memory where it fits (room for `cap` rows), the
+// pivot is found by one warp and a warp updates a row at a time: 1,838 leaves
+// of 29 rows 2.95 ms in global memory with the pivot searched by one thread.
 __global__ void k_bj_invert(const int32_t* leaf_start, const int64_t* blk_off, cd* blocks, int* piv_scr,
-                            int* singular, int scale) {
+                            int* singular, int scale, int cap) {
     int t = blockIdx.x;
     int n = scale * (leaf_start[t + 1] - leaf_start[t]);
-    cd* a = blocks + blk_off[t];
+    cd* const ga = blocks + blk_off[t];
     int* piv = piv_scr + scale * leaf_start[t];
     extern __shared__ cd fcol[];
+    cd* a = n <= cap ? fcol + n : ga;
     __shared__ int s_p;
     __shared__ cd s_inv;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (a != ga)
+        for (int e = threadIdx.x; e < n * n; e += blockDim.x) a[e] = ga[e];
+    __syncthreads();
     for (int k = 0; k < n; ++k) {
-        if (threadIdx.x == 0) {
+        if (warp == 0) {
+            // the first row of the largest entry (k itself if that is no number)
             int p = k;
             double best = abs2(a[(int64_t)k * n + k]);
-            for (int i = k + 1; i < n; ++i) {
-                double v = abs2(a[(int64_t)i * n + k]);
-                if (v > best) { best = v; p = i; }
+            const bool num = best == best;
+            if (num)
+                for (int i = k + 1 + lane; i < n; i += 32) {
+                    const double v = abs2(a[(int64_t)i * n + k]);
+                    if (v > best) { best = v; p = i; }
+                }
+            for (int o = 16; num && o > 0; o >>= 1) {
+                const double v = __shfl_xor_sync(0xffffffffu, best, o);
+                const int q = __shfl_xor_sync(0xffffffffu, p, o);
+                if (v > best || (v == best && q < p)) { best = v; p = q; }
             }
-            piv[k] = p;
-            s_p = p;
-            if (best == 0.0) { atomicExch(singular, 1); s_inv = mk(0.0, 0.0); }
-            else {
-                cd d = a[(int64_t)p * n + k];
-                s_inv = (1.0 / best) * conjg(d);
+            if (lane == 0) {
+                piv[k] = p;
+                s_p = p;
+                if (best == 0.0) { atomicExch(singular, 1); s_inv = mk(0.0, 0.0); }
+                else {
+                    cd d = a[(int64_t)p * n + k];
+                    s_inv = (1.0 / best) * conjg(d);
+                }
             }
         }
         __syncthreads();
         int p = s_p;
-        if (p != k)
-            for (int j = threadIdx.x; j < n; j += blockDim.x) {
-                cd tmp = a[(int64_t)k * n + j];
-                a[(int64_t)k * n + j] = a[(int64_t)p * n + j];
-                a[(int64_t)p * n + j] = tmp;
-            }
+        const cd inv = s_inv;
+        // rows k and p change places, row k scaled
+        for (int j = threadIdx.x; j < n; j += blockDim.x) {
+            const cd u = a[(int64_t)k * n + j], v = a[(int64_t)p * n + j];
+            if (p != k) a[(int64_t)p * n + j] = u;
+            a[(int64_t)k * n + j] = inv * (j == k ? mk(1.0, 0.0) : v);
+        }
         __syncthreads();
-        cd inv = s_inv;
-        if (threadIdx.x == 0) a[(int64_t)k * n + k] = mk(1.0, 0.0);
-        __syncthreads();
-        for (int j = threadIdx.x; j < n; j += blockDim.x) a[(int64_t)k * n + j] = inv * a[(int64_t)k * n + j];
         for (int i = threadIdx.x; i < n; i += blockDim.x) fcol[i] = (i == k) ? mk(0.0, 0.0) : a[(int64_t)i * n + k];
         __syncthreads();
-        for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
-            int i = e / n, j = e % n;
+        for (int i = warp; i < n; i += nw) {
             if (i == k) continue;
-            cd f = fcol[i];
-            if (j == k) a[(int64_t)i * n + j] = mk(0.0, 0.0) - f * a[(int64_t)k * n + j];
-            else a[(int64_t)i * n + j] = a[(int64_t)i * n + j] - f * a[(int64_t)k * n + j];
+            const cd f = fcol[i];
+            for (int j = lane; j < n; j += 32)
+                a[(int64_t)i * n + j] = (j == k ? mk(0.0, 0.0) : a[(int64_t)i * n + j]) - f * a[(int64_t)k * n + j];
         }
         __syncthreads();
     }
@@ -587,6 +601,16 @@ __global__ void k_bj_invert(const int32_t* leaf_start, const int64_t* blk_off, c
             }
         __syncthreads();
     }
+    if (a != ga)
+        for (int e = threadIdx.x; e < n * n; e += blockDim.x) ga[e] = a[e];
+}
+
+// Rows a block in shared memory may have and the bytes to launch with, for
+// blocks of up to maxn rows (three CTAs per SM).
+static int bj_cap(int maxn, size_t* smem) {
+    const int cap = (size_t)maxn * (maxn + 1) * sizeof(cd) <= 72 * 1024 ? maxn : 0;
+    *smem = sizeof(cd) * (size_t)std::max(maxn, 1) * (cap + 1);
+    return cap;
 }
 
 template <class R>
@@ -730,14 +754,15 @@ static fb_status dbem5_bj_create(fb_op* op, cudaStream_t s, fb_precond** out) {
             self[q] = sub->self64;
         }
     }
+    size_t bj_smem = 0;
+    const int bj_rows = bj_cap(maxn, &bj_smem);
     if (st == FB_OK) {
         k_d5_bj_assemble<<<nleaf, 256, 0, s>>>(t->leaf_start, t->perm, pc->blk_off, self[0], self[1], op->ib_beta_m,
                                                op->k, pc->inv64);
-        st = fb_smem_cap((const void*)k_bj_invert, sizeof(cd) * std::max(maxn, 1));
+        st = fb_smem_cap((const void*)k_bj_invert, bj_smem);
     }
     if (st == FB_OK) {
-        k_bj_invert<<<nleaf, 256, sizeof(cd) * std::max(maxn, 1), s>>>(t->leaf_start, pc->blk_off, pc->inv64, piv,
-                                                                        sing, 1);
+        k_bj_invert<<<nleaf, 256, bj_smem, s>>>(t->leaf_start, pc->blk_off, pc->inv64, piv, sing, 1, bj_rows);
         int hs = 0;
         cudaMemcpyAsync(&hs, sing, sizeof(int), cudaMemcpyDeviceToHost, s);
         cudaError_t e = cudaStreamSynchronize(s);
@@ -802,15 +827,16 @@ static fb_status ibem_bj_create(fb_op* op, cudaStream_t s, fb_precond** out) {
             self[q] = sub->self64;
         }
     }
+    size_t bj_smem = 0;
+    const int bj_rows = bj_cap(2 * maxn, &bj_smem);
     if (st == FB_OK) {
         // sub-operators: 0 = M, 1 = L, 2 = M', 3 = L'
         k_ibem_bj_assemble<<<nleaf, 256, 0, s>>>(t->leaf_start, t->perm, d_off1, pc->blk_off, self[0], self[1],
                                                  self[2], self[3], op->ib_beta_p, op->ib_beta_m, op->k, pc->inv64);
-        st = fb_smem_cap((const void*)k_bj_invert, sizeof(cd) * 2 * std::max(maxn, 1));
+        st = fb_smem_cap((const void*)k_bj_invert, bj_smem);
     }
     if (st == FB_OK) {
-        k_bj_invert<<<nleaf, 256, sizeof(cd) * 2 * std::max(maxn, 1), s>>>(t->leaf_start, pc->blk_off, pc->inv64,
-                                                                            piv, sing, 2);
+        k_bj_invert<<<nleaf, 256, bj_smem, s>>>(t->leaf_start, pc->blk_off, pc->inv64, piv, sing, 2, bj_rows);
         int hs = 0;
         cudaMemcpyAsync(&hs, sing, sizeof(int), cudaMemcpyDeviceToHost, s);
         cudaError_t e = cudaStreamSynchronize(s);
@@ -1370,8 +1396,10 @@ fb_status fb_precond_create_impl(fb_op* op, int kind, cudaStream_t s, fb_precond
     FB_CUDA(cudaMemsetAsync(sing, 0, sizeof(int), s));
     if (op->nf64) FB_CHECK(fb_self_blocks(op, pc->blk_off, pc->inv64, s));
     else FB_CUDA(cudaMemcpyAsync(pc->inv64, op->self64, sizeof(cd) * off[nleaf], cudaMemcpyDeviceToDevice, s));
-    FB_CHECK(fb_smem_cap((const void*)k_bj_invert, sizeof(cd) * std::max(maxn, 1)));
-    k_bj_invert<<<nleaf, 256, sizeof(cd) * std::max(maxn, 1), s>>>(t->leaf_start, pc->blk_off, pc->inv64, piv, sing, 1);
+    size_t bj_smem = 0;
+    const int bj_rows = bj_cap(maxn, &bj_smem);
+    FB_CHECK(fb_smem_cap((const void*)k_bj_invert, bj_smem));
+    k_bj_invert<<<nleaf, 256, bj_smem, s>>>(t->leaf_start, pc->blk_off, pc->inv64, piv, sing, 1, bj_rows);
     int hs = 0;
     FB_CUDA(cudaMemcpyAsync(&hs, sing, sizeof(int), cudaMemcpyDeviceToHost, s));
     FB_CUDA(cudaStreamSynchronize(s));
