@@ -27,7 +27,8 @@
 // at n^2, folded within the degree: E_0..E_n, then O_1..O_n), so the
 // rotations read and write contiguous runs; the coaxial pass, which sums
 // over degrees at a fixed order, gathers its inputs and scatters its
-// outputs with a stride of one degree block.  One CTA computes a 64 x 64
+// outputs with a stride of one degree block (levels whose rotations run on
+// the tensor cores keep the slots innermost instead).  One CTA computes a 64 x 64
 // tile of one GEMM (256 threads, 4 x 4 complex outputs each, K in chunks
 // of 16, three-stage cp.async pipeline).
 #include <algorithm>
