@@ -317,14 +317,15 @@ struct StcTabs {
     int* err;
 };
 // Runs the staged passes of a plan (pass_mask bits: pre-pass, rotation,
-// coaxial, back-rotation; only_level >= 0: that level of the plan alone).
+// coaxial, back-rotation; only_level >= 0: that level of the plan alone), nb
+// right-hand sides at a time, their staging buffers ustride apart.
 fb_status fb_stg_run_f(void* plan, const float* rf, int64_t fper, const cf* rph, int prot, const cf* coax,
                        const cf* src, cf* dst, cf* U, cf* V, cudaStream_t s, int nrhs, int64_t rstride,
-                       const StcTabs& tc, int only_level = -1, int pass_mask = 15);
+                       const StcTabs& tc, int nb, int64_t ustride, int only_level = -1, int pass_mask = 15);
 bool fb_stg_uses_tc(const void* plan);
 fb_status fb_stg_run_d(void* plan, const double* rf, int64_t fper, const cd* rph, int prot, const cd* coax,
                        const cd* src, cd* dst, cd* U, cd* V, cudaStream_t s, int nrhs, int64_t rstride,
-                       const DfTabs& dft, int only_level = -1, int pass_mask = 15);
+                       const DfTabs& dft, int nb, int64_t ustride, int only_level = -1, int pass_mask = 15);
 bool fb_stg_uses_df(const void* plan);
 int fb_stg_level_count(const void* plan);
 // form: 1 CUDA cores, 2 rotations on the tensor cores, 3 double-FP32 arithmetic,
@@ -433,6 +434,7 @@ struct fb_op {
     void* stg_u = nullptr;
     void* stg_v = nullptr;
     int64_t stg_elems = 0;
+    int stg_nrhs = 1;   // right-hand sides they hold
     RcrPlan m2l_rcr, m2m_rcr[FB_MAXLEV + 1], l2l_rcr[FB_MAXLEV + 1];
     // tensor-core (3xTF32) stacked M2L: dense levels (auto) / every level
     void* tc_plan = nullptr;

@@ -246,7 +246,10 @@ __global__ void k_fold_tables(const double* __restrict__ rotd, int64_t per_dir, 
 // written once so that the rotation GEMMs read contiguous columns.
 template <class R, class O>
 __global__ void k_stg_prep(const StgSlot* __restrict__ slots, int nslot, const cx<O>* __restrict__ src,
-                           const cx<O>* __restrict__ rph, int prot, int Pin, int S, cx<R>* __restrict__ X0) {
+                           const cx<O>* __restrict__ rph, int prot, int Pin, int S, cx<R>* __restrict__ X0,
+                           int64_t rstride, int64_t ustride) {
+    src += blockIdx.y * rstride;
+    X0 += blockIdx.y * ustride;
     const int64_t total = (int64_t)nslot * Pin;
     for (int64_t q = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; q < total; q += (int64_t)gridDim.x * blockDim.x) {
         const int sl = (int)(q / Pin), e = (int)(q % Pin);
@@ -276,7 +279,9 @@ template <class R>
 __global__ void __launch_bounds__(STHREADS, 2) k_stg_rot(const StgTile* __restrict__ tiles,
                                                          const R* __restrict__ rf, int64_t fper,
                                                          const cx<R>* __restrict__ X0, cx<R>* __restrict__ U,
-                                                         int S) {
+                                                         int S, int64_t ustride) {
+    X0 += blockIdx.y * ustride;
+    U += blockIdx.y * ustride;
     extern __shared__ __align__(16) unsigned char stg_smem[];
     StgSmem<R, false>& sm = *reinterpret_cast<StgSmem<R, false>*>(stg_smem);
     const StgTile tl = tiles[blockIdx.x];
@@ -324,7 +329,9 @@ template <class R, bool INNER>
 __global__ void __launch_bounds__(STHREADS, 2) k_stg_coax(const StgCTile* __restrict__ tiles,
                                                           const int32_t* __restrict__ cidx,
                                                           const cx<R>* __restrict__ coax, const cx<R>* __restrict__ U,
-                                                          cx<R>* __restrict__ V, int S) {
+                                                          cx<R>* __restrict__ V, int S, int64_t ustride) {
+    U += blockIdx.y * ustride;
+    V += blockIdx.y * ustride;
     extern __shared__ __align__(16) unsigned char stg_smem[];
     StgSmem<R, true>& sm = *reinterpret_cast<StgSmem<R, true>*>(stg_smem);
     const StgCTile tl = tiles[blockIdx.x];
@@ -395,7 +402,9 @@ __global__ void __launch_bounds__(STHREADS, 2) k_stg_back(const StgTile* __restr
                                                           const R* __restrict__ rf, int64_t fper,
                                                           const cx<O>* __restrict__ rph, int prot,
                                                           const cx<R>* __restrict__ V, cx<O>* __restrict__ dst, int S,
-                                                          int pin, int pout) {
+                                                          int pin, int pout, int64_t rstride, int64_t ustride) {
+    V += blockIdx.y * ustride;
+    dst += blockIdx.y * rstride;
     extern __shared__ __align__(16) unsigned char stg_smem[];
     StgSmem<R, false>& sm = *reinterpret_cast<StgSmem<R, false>*>(stg_smem);
     const StgTile tl = tiles[blockIdx.x];
@@ -768,28 +777,34 @@ fb_status fb_stg_df_tables(fb_op* op, cudaStream_t s) {
 }
 
 // Runs the staged passes of a plan for nrhs right-hand sides (set r of the
-// expansions at src / dst + r * rstride), one right-hand side and one level
-// at a time: pre-pass (src -> V), rotation (V -> U), coaxial (U -> V),
+// expansions at src / dst + r * rstride), one level and as many right-hand
+// sides at a time as the staging buffers hold (nb, ustride apart): pre-pass (src -> V), rotation (V -> U), coaxial (U -> V),
 // back-rotation (V -> dst).
+// right-hand sides of one launch
+struct StgRhs {
+    int n;
+    int64_t rstride, ustride;
+};
 // Tensor-core rotation passes of a level (single precision only).
 static fb_status stc_pass(const StgLevel& lv, int pass, const StcTabs* tc, const cf* X, cf* out, const cf* rph,
-                          int prot, cudaStream_t s) {
+                          int prot, cudaStream_t s, const StgRhs& q) {
     if (!tc || !tc->tab) return fb_fail(FB_ERR_STATE, "staged RCR: tensor-core tables missing");
     return fb_stc_run(pass, pass == 0 ? lv.rtc : lv.btc, pass == 0 ? lv.nrtc : lv.nbtc, std::max(lv.p_in, lv.p_out),
-                      tc->tab, tc->per, lv.slots, nullptr, X, out, lv.nslot, rph, prot, tc->err, s);
+                      tc->tab, tc->per, lv.slots, nullptr, X, out, lv.nslot, rph, prot, tc->err, s, q.n, q.rstride, q.ustride);
 }
 template <class X, class Y, class Ph>
-static fb_status stc_pass(const StgLevel&, int, const StcTabs*, const X*, Y*, const Ph*, int, cudaStream_t) {
+static fb_status stc_pass(const StgLevel&, int, const StcTabs*, const X*, Y*, const Ph*, int, cudaStream_t,
+                          const StgRhs&) {
     return fb_fail(FB_ERR_ARG, "tensor-core staged RCR applies to single precision");
 }
 // Tensor-core coaxial pass of a level (single precision only).
-static fb_status stc_coax(const StgLevel& lv, const StcTabs* tc, const cf* U, cf* V, cudaStream_t s) {
+static fb_status stc_coax(const StgLevel& lv, const StcTabs* tc, const cf* U, cf* V, cudaStream_t s, const StgRhs& q) {
     if (!tc) return fb_fail(FB_ERR_STATE, "staged RCR: tensor-core error flag missing");
     return fb_stc_run(2, lv.ctc, lv.nctc, 2 * std::min(STC_CROWS, lv.p_out), lv.ctab, 0, nullptr, lv.cidx, U, V,
-                      lv.nslot, nullptr, 0, tc->err, s);
+                      lv.nslot, nullptr, 0, tc->err, s, q.n, q.rstride, q.ustride);
 }
 template <class X>
-static fb_status stc_coax(const StgLevel&, const StcTabs*, const X*, X*, cudaStream_t) {
+static fb_status stc_coax(const StgLevel&, const StcTabs*, const X*, X*, cudaStream_t, const StgRhs&) {
     return fb_fail(FB_ERR_ARG, "tensor-core staged RCR applies to single precision");
 }
 
@@ -800,7 +815,8 @@ static fb_status stc_coax(const StgLevel&, const StcTabs*, const X*, X*, cudaStr
 template <class R, class O>
 static fb_status stg_level(const StgLevel& lv, int pass_mask, const R* rf, int64_t fper, const cx<O>* rph, int prot,
                            const cx<R>* coax, const cx<O>* sr, cx<O>* dr, cx<R>* U, cx<R>* V, cudaStream_t s,
-                           const StcTabs* tc) {
+                           const StcTabs* tc, const StgRhs& q) {
+    const unsigned nr = (unsigned)q.n;
     const size_t sm_rc = sizeof(StgSmem<R, false>), sm_c = sizeof(StgSmem<R, true>);
     FB_CHECK(fb_smem_cap((const void*)k_stg_rot<R>, sm_rc));
     FB_CHECK(fb_smem_cap((const void*)k_stg_coax<R, false>, sm_c));
@@ -808,35 +824,38 @@ static fb_status stg_level(const StgLevel& lv, int pass_mask, const R* rf, int64
     if ((pass_mask & 1) && !lv.tc) {   // the tensor-core rotation pass folds its inputs itself
         const int64_t tot = (int64_t)lv.nslot * lv.p_in * lv.p_in;
         const int pb = (int)std::min<int64_t>((tot + 255) / 256, 152 * 16);
-        k_stg_prep<R, O><<<pb, 256, 0, s>>>(lv.slots, lv.nslot, sr, rph, prot, lv.p_in * lv.p_in, lv.S, V);
+        k_stg_prep<R, O><<<dim3(pb, nr), 256, 0, s>>>(lv.slots, lv.nslot, sr, rph, prot, lv.p_in * lv.p_in, lv.S, V,
+                                                      q.rstride, q.ustride);
         fb_count_launch();
     }
     if (pass_mask & 2) {
         if (lv.tc) {
-            FB_CHECK(stc_pass(lv, 0, tc, sr, U, rph, prot, s));
+            FB_CHECK(stc_pass(lv, 0, tc, sr, U, rph, prot, s, q));
         } else if (lv.nrt) {
-            k_stg_rot<R><<<lv.nrt, STHREADS, sm_rc, s>>>(lv.rt, rf, fper, V, U, lv.S);
+            k_stg_rot<R><<<dim3(lv.nrt, nr), STHREADS, sm_rc, s>>>(lv.rt, rf, fper, V, U, lv.S, q.ustride);
             fb_count_launch();
         }
     }
     if ((pass_mask & 4) && lv.nctc) {
-        FB_CHECK(stc_coax(lv, tc, U, V, s));
+        FB_CHECK(stc_coax(lv, tc, U, V, s, q));
     } else if ((pass_mask & 4) && lv.nct) {
         if constexpr (std::is_same<R, float>::value) {
             if (lv.tc) {
                 FB_CHECK(fb_smem_cap((const void*)k_stg_coax<R, true>, sm_c));
-                k_stg_coax<R, true><<<lv.nct, STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.nslot);
+                k_stg_coax<R, true><<<dim3(lv.nct, nr), STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.nslot,
+                                                                             q.ustride);
             }
         }
-        if (!lv.tc) k_stg_coax<R, false><<<lv.nct, STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.S);
+        if (!lv.tc)
+            k_stg_coax<R, false><<<dim3(lv.nct, nr), STHREADS, sm_c, s>>>(lv.ct, lv.cidx, coax, U, V, lv.S, q.ustride);
         fb_count_launch();
     }
     if (pass_mask & 8) {
         if (lv.tc) {
-            FB_CHECK(stc_pass(lv, 1, tc, V, dr, rph, prot, s));
+            FB_CHECK(stc_pass(lv, 1, tc, V, dr, rph, prot, s, q));
         } else if (lv.nbt) {
-            k_stg_back<R, O><<<lv.nbt, STHREADS, sm_rc, s>>>(lv.bt, lv.slots, rf, fper, rph, prot, V, dr, lv.S,
-                                                             lv.p_in, lv.p_out);
+            k_stg_back<R, O><<<dim3(lv.nbt, nr), STHREADS, sm_rc, s>>>(lv.bt, lv.slots, rf, fper, rph, prot, V, dr,
+                                                                       lv.S, lv.p_in, lv.p_out, q.rstride, q.ustride);
             fb_count_launch();
         }
     }
@@ -847,11 +866,12 @@ static fb_status stg_level(const StgLevel& lv, int pass_mask, const R* rf, int64
 template <class R>
 static fb_status stg_run(void* plan, const R* rf, int64_t fper, const cx<R>* rph, int prot, const cx<R>* coax,
                          const cx<R>* src, cx<R>* dst, cx<R>* U, cx<R>* V, cudaStream_t s, int nrhs, int64_t rstride,
-                         const StcTabs* tc, const DfTabs* dft, int only_level, int pass_mask) {
+                         const StcTabs* tc, const DfTabs* dft, int only_level, int pass_mask, int nb, int64_t ustride) {
     StgPlanImpl* P = (StgPlanImpl*)plan;
     if (!P) return FB_OK;
     if (!U || !V || !rf) return fb_fail(FB_ERR_STATE, "staged RCR: staging buffers or tables missing");
-    for (int r = 0; r < nrhs; ++r) {
+    for (int r = 0; r < nrhs; r += nb) {
+        const StgRhs q{std::min(nb, nrhs - r), rstride, ustride};
         const cx<R>* sr = src + r * rstride;
         cx<R>* dr = dst + r * rstride;
         for (int li = 0; li < (int)P->levels.size(); ++li) {
@@ -863,11 +883,11 @@ static fb_status stg_run(void* plan, const R* rf, int64_t fper, const cx<R>* rph
                         return fb_fail(FB_ERR_STATE, "staged RCR: double-FP32 tables missing");
                     // the staging buffers hold complex double-FP32 values (16 bytes, as FP64)
                     FB_CHECK((stg_level<df, double>(lv, pass_mask, dft->rf, fper, rph, prot, dft->coax, sr, dr,
-                                                    (cx<df>*)U, (cx<df>*)V, s, nullptr)));
+                                                    (cx<df>*)U, (cx<df>*)V, s, nullptr, q)));
                     continue;
                 }
             }
-            FB_CHECK((stg_level<R, R>(lv, pass_mask, rf, fper, rph, prot, coax, sr, dr, U, V, s, tc)));
+            FB_CHECK((stg_level<R, R>(lv, pass_mask, rf, fper, rph, prot, coax, sr, dr, U, V, s, tc, q)));
         }
     }
     return FB_OK;
@@ -875,15 +895,15 @@ static fb_status stg_run(void* plan, const R* rf, int64_t fper, const cx<R>* rph
 
 fb_status fb_stg_run_f(void* plan, const float* rf, int64_t fper, const cf* rph, int prot, const cf* coax,
                        const cf* src, cf* dst, cf* U, cf* V, cudaStream_t s, int nrhs, int64_t rstride,
-                       const StcTabs& tc, int only_level, int pass_mask) {
+                       const StcTabs& tc, int nb, int64_t ustride, int only_level, int pass_mask) {
     return stg_run<float>(plan, rf, fper, rph, prot, coax, src, dst, U, V, s, nrhs, rstride, &tc, nullptr,
-                          only_level, pass_mask);
+                          only_level, pass_mask, nb, ustride);
 }
 fb_status fb_stg_run_d(void* plan, const double* rf, int64_t fper, const cd* rph, int prot, const cd* coax,
                        const cd* src, cd* dst, cd* U, cd* V, cudaStream_t s, int nrhs, int64_t rstride,
-                       const DfTabs& dft, int only_level, int pass_mask) {
+                       const DfTabs& dft, int nb, int64_t ustride, int only_level, int pass_mask) {
     return stg_run<double>(plan, rf, fper, rph, prot, coax, src, dst, U, V, s, nrhs, rstride, nullptr, &dft,
-                           only_level, pass_mask);
+                           only_level, pass_mask, nb, ustride);
 }
 
 int fb_stg_level_count(const void* plan) {

@@ -42,7 +42,8 @@ struct StcItem {
     int32_t n, part;
     int32_t N, K;     // real columns and summed length
     int32_t g;
-    int32_t uni;      // (set on the device)
+    int32_t uni;      // set on the device: groups of slots with one direction,
+    int64_t rhs, uoff;   // right-hand side and the offset of its u and v
 };
 
 // columns of the folded degree-n block (rows of the table), padded to 16
@@ -77,9 +78,10 @@ fb_status fb_stc_coax_tables(const StcCBlock* blocks, int nblocks, const cd* coa
 
 // Launches the items of a pass: rotation 0 (expansions -> u), back-rotation 1
 // (v -> expansions), coaxial 2 (u -> v); ncol_max bounds their columns; ns is
-// the level's number of slots, u and v are [coefficient][slot].
+// the level's number of slots, u and v are [coefficient][slot].  For nrhs
+// right-hand sides, their expansions rstride and their u and v ustride apart.
 fb_status fb_stc_run(int pass, const StcItem* items, int nitems, int ncol_max, const float* tab, int64_t tper,
                      const StgSlot* slots, const int32_t* cidx, const cf* X, cf* out, int64_t ns, const cf* rph,
-                     int prot, int* err, cudaStream_t s);
+                     int prot, int* err, cudaStream_t s, int nrhs, int64_t rstride, int64_t ustride);
 
 }  // namespace stg

@@ -112,7 +112,8 @@ __host__ __device__ __forceinline__ void stc_dims(int pass, int n, int part, int
 
 struct StcArgs {
     const StcItem* items;
-    int nitems;
+    int nitems, nrhs;         // items per right-hand side
+    int64_t rstride, ustride;   // expansions, u and v of the next right-hand side
     const float* tab;      // R, B: group g's R table at g * 2 tper, B table at g * 2 tper + tper; C: the coaxial blocks
     int64_t tper;
     const StgSlot* slots;
@@ -265,7 +266,7 @@ struct Producer<ST_B> {
                                          int lane, int c) {
         const int j = min(32 * sub + lane, it.ns - 1), left = it.K - c * KC, n = it.n;
         const int64_t es = 8 * a.ns;
-        const char* v = (const char*)(a.X + it.s0 + j) + (n * n + (it.part ? n : 0) + it.part + c * KC) * es;
+        const char* v = (const char*)(a.X + it.uoff + it.s0 + j) + (n * n + (it.part ? n : 0) + it.part + c * KC) * es;
         if (left >= KC) {
 #pragma unroll
             for (int k = 0; k < KC; ++k) nxt[k] = ldg2(v + k * es);
@@ -309,7 +310,7 @@ __device__ __forceinline__ void stc_epilogue(const StcArgs& a, const StcItem& it
         if (PASS == ST_R) {
             tcx::tmem_ld16(acc + (uint32_t)c0, v);
             const int j = 16 * quad + 8 * (lane >> 4) + (lane & 7);
-            char* u = (char*)(a.out + it.s0 + j) + 4 * (lane >> 3 & 1) + (n * n + (part ? n : 0) + part + c0) * es;
+            char* u = (char*)(a.out + it.uoff + it.s0 + j) + 4 * (lane >> 3 & 1) + (n * n + (part ? n : 0) + part + c0) * es;
             const int left = j < ns ? N - c0 : 0;
             if (left >= 16) {
 #pragma unroll
@@ -422,7 +423,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t tmem = tmem_holder;
     // this CTA's items: blockIdx.x, + gridDim.x, ...; the it-th is in ring entry it % STC_RING
-    const int nmine = (a.nitems - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
+    const int nmine = (a.nitems * a.nrhs - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
     auto item_wait = [&](int it) {
         return mbar_wait(smem_u32(&idx_full[it % STC_RING]), (it / STC_RING) & 1, a.wait_limit);
     };
@@ -649,9 +650,9 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                 const int j = tl.s0 + min(q * 32 + lane, tl.ns - 1);
                 d[q] = 0;
                 if (PASS == ST_C) {
-                    o[q] = __ldg(a.cidx + j);
+                    o[q] = __ldg(a.cidx + j) + tl.uoff;
                 } else {
-                    o[q] = PASS == ST_R ? __ldg(&a.slots[j].src_off) : __ldg(&a.slots[j].dst_off);
+                    o[q] = (PASS == ST_R ? __ldg(&a.slots[j].src_off) : __ldg(&a.slots[j].dst_off)) + tl.rhs * a.rstride;
                     d[q] = __ldg(&a.slots[j].dir);
                 }
             }
@@ -661,7 +662,12 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
         const int rot = (int)((int64_t)blockIdx.x * nmine / gridDim.x);
         auto item_of = [&](int it) {
             it += rot;
-            return a.items[blockIdx.x + (int64_t)(it < nmine ? it : it - nmine) * gridDim.x];
+            const int i = (int)blockIdx.x + (it < nmine ? it : it - nmine) * (int)gridDim.x;
+            // the right-hand sides of an item one after the other: they share T
+            StcItem tl = a.items[i / a.nrhs];
+            tl.rhs = i % a.nrhs;
+            tl.uoff = tl.rhs * a.ustride;
+            return tl;
         };
         StcItem cur, nxt;
         int64_t o[2], on[2];
@@ -802,7 +808,7 @@ void fb_stc_group_items(int g, int g0, int g1, int nmax, int pass, int p_in, std
                 int N, K;
                 stc_dims(pass, n, part, p_in, N, K);
                 if (N > 0 && K > 0)
-                    out.push_back(StcItem{toff[2 * n + part], s0, std::min(STC_SLOTS, g1 - s0), n, part, N, K, g, 0});
+                    out.push_back(StcItem{toff[2 * n + part], s0, std::min(STC_SLOTS, g1 - s0), n, part, N, K, g, 0, 0, 0});
             }
 }
 
@@ -816,7 +822,7 @@ void fb_stc_coax_set(int c0, int ns, int64_t cs_off, int pc, int p_in, int p_out
             blocks.push_back(StcCBlock{cs_off, *tfloats, pc, am, r0, nr, K, 0});
             for (int s0 = 0; s0 < ns; s0 += STC_SLOTS)
                 items.push_back(
-                    StcItem{*tfloats, c0 + s0, std::min(STC_SLOTS, ns - s0), am, r0, 2 * nr, 2 * K, 0, 0});
+                    StcItem{*tfloats, c0 + s0, std::min(STC_SLOTS, ns - s0), am, r0, 2 * nr, 2 * K, 0, 0, 0, 0});
             *tfloats += (int64_t)2 * np * kp;
         }
     }
@@ -840,13 +846,17 @@ fb_status fb_stc_coax_tables(const StcCBlock* blocks, int nblocks, const cd* coa
 
 fb_status fb_stc_run(int pass, const StcItem* items, int nitems, int ncol_max, const float* tab, int64_t tper,
                      const StgSlot* slots, const int32_t* cidx, const cf* X, cf* out, int64_t ns, const cf* rph,
-                     int prot, int* err, cudaStream_t s) {
+                     int prot, int* err, cudaStream_t s, int nrhs, int64_t rstride, int64_t ustride) {
     if (nitems == 0) return FB_OK;
     const int npmax = stc_pad16(ncol_max);
+    if ((int64_t)nitems * nrhs > INT32_MAX / 2) return fb_fail(FB_ERR_ARG, "tensor-core staged RCR: too many items");
     if (npmax > STC_COLS) return fb_fail(FB_ERR_ARG, "tensor-core staged RCR: order above 256");
     StcArgs a;
     a.items = items;
     a.nitems = nitems;
+    a.nrhs = nrhs;
+    a.rstride = rstride;
+    a.ustride = ustride;
     a.tab = tab;
     a.tper = tper;
     a.slots = slots;
@@ -881,7 +891,7 @@ fb_status fb_stc_run(int pass, const StcItem* items, int nitems, int ncol_max, c
     int dev = 0, sms = 0;
     FB_CUDA(cudaGetDevice(&dev));
     FB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    const unsigned grid = (unsigned)std::min(sms, nitems);
+    const unsigned grid = (unsigned)std::min<int64_t>(sms, (int64_t)nitems * nrhs);
     if (pass == ST_R)
         k_stg_tc<ST_R><<<grid, STC_THREADS, smem, s>>>(a);
     else if (pass == ST_B)
