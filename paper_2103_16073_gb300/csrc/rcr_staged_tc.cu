@@ -60,6 +60,7 @@ namespace {
 using tcx::canon;
 using tcx::DRAIN_LIMIT;
 using tcx::KC;
+using tcx::mbar_arrive;
 using tcx::mbar_init;
 using tcx::mbar_test;
 using tcx::mbar_wait;
@@ -130,10 +131,6 @@ struct StcArgs {
     int acc_cols, nacc;    // tensor memory columns of an accumulator, accumulators
     int inject_stall;
 };
-
-__device__ __forceinline__ void arrive(uint64_t* bar) {
-    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
-}
 
 // stores a row's 4 K values as TF32 hi and remainder
 __device__ __forceinline__ void split_store(float* st, int plane, const float4& x) {
@@ -395,9 +392,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int nst = a.nst;
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(a.nacc * a.acc_cols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        tcx::tmem_alloc(&tmem_holder, a.nacc * a.acc_cols);
     }
     if (tid == 0) {
         s_fail = 0;
@@ -416,11 +411,11 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
         }
         mbar_init(&done_bar, 1);
         mbar_init(&never_bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tcx::fence_mbar_init();
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    tcx::fence_before_sync();
     __syncthreads();
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    tcx::fence_after_sync();
     const uint32_t tmem = tmem_holder;
     // this CTA's items: blockIdx.x, + gridDim.x, ...; the it-th is in ring entry it % STC_RING
     const int nmine = (a.nitems * a.nrhs - (int)blockIdx.x + (int)gridDim.x - 1) / (int)gridDim.x;
@@ -438,7 +433,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
         auto seek = [&]() -> bool {
             while (c >= nkc) {
                 __syncwarp();
-                if (it >= 0 && lane == 0) arrive(&idx_empty[it % STC_RING]);   // the item is no longer needed
+                if (it >= 0 && lane == 0) mbar_arrive(&idx_empty[it % STC_RING]);   // the item is no longer needed
                 c -= nkc;
                 nkc = 0;
                 if (++it >= nmine) return false;
@@ -477,9 +472,9 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
             }
             p.store(stage0 + (size_t)s * a.stage_floats, sub, lane);
             // generic-proxy stores become visible to the tensor core's reads
-            asm volatile("fence.proxy.async.shared::cta;");
+            tcx::fence_proxy_async();
             __syncwarp();
-            if (lane == 0) arrive(&full_bar[s]);
+            if (lane == 0) mbar_arrive(&full_bar[s]);
             if (next) p.take();
             more = next;
             next = after;
@@ -497,7 +492,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                     break;
                 }
                 const StcItem tl = s_item[r];
-                arrive(&idx_empty[r]);
+                mbar_arrive(&idx_empty[r]);
                 const int blk = 2 * stc_pad16(tl.N) * KC, nkc = (tl.K + KC - 1) / KC;
                 const uint32_t bytes = (uint32_t)(blk * sizeof(float));
                 const float* g = a.tab + tl.tab + (PASS == ST_C ? 0 : ((int64_t)2 * tl.g + (PASS == ST_B)) * a.tper);
@@ -509,11 +504,8 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                     }
                     const uint32_t bb = smem_u32(&b_bar[s]);
                     const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * L::PLANE);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb), "r"(bytes));
-                    asm volatile(
-                        "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                            dB),
-                        "l"(g), "r"(bytes), "r"(bb));
+                    tcx::mbar_expect(bb, bytes);
+                    tcx::bulk_copy(dB, g, bytes, bb);
                     if (++s == nst) {
                         s = 0;
                         ph ^= 1;
@@ -562,7 +554,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                     nK = s_item[r].K;
                 }
                 const int np = stc_pad16(nN), nkc = (nK + KC - 1) / KC;
-                arrive(&idx_empty[r]);
+                mbar_arrive(&idx_empty[r]);
                 iready = false;
                 const int b1 = b + 1 == a.nacc ? 0 : b + 1;
                 const uint32_t ap1 = b1 == 0 ? aph ^ 1 : aph;
@@ -574,7 +566,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                     atomicExch(&s_fail, 1);
                     break;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;");
+                tcx::fence_after_sync();
                 const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols);
                 const uint32_t idesc = tcx::idesc_tf32(STC_M, np);
                 const uint32_t blo = (uint32_t)(np * KC * 4) >> 4;   // from T's hi block to its lo block
@@ -588,7 +580,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                     const int s1 = s + 1 == nst ? 0 : s + 1;
                     const uint32_t p1 = s1 == 0 ? ph ^ 1 : ph;
                     ready = peek_stage(s1, p1);
-                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    tcx::fence_after_sync();
 #pragma unroll
                     for (int ks = 0; ks < KC / 8; ++ks) {
                         const uint32_t aH = a0 + dof + ((ks * 2 * L::LBO) >> 4), bH = b0 + dof + ((ks * 2 * tcx::LBO) >> 4);
@@ -627,15 +619,15 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
                 atomicExch(&s_fail, 1);
                 break;
             }
-            asm volatile("tcgen05.fence::after_thread_sync;");
+            tcx::fence_after_sync();
             stc_epilogue<PASS>(a, s_item[r], s_pos[r], s_dir[r], tmem + (uint32_t)(b * a.acc_cols), quad,
                                (ew / 4 + it) % L::SHARES, lane, sg);
             // this warp's share of the accumulator is read
-            asm volatile("tcgen05.fence::before_thread_sync;");
+            tcx::fence_before_sync();
             __syncwarp();
             if (lane == 0) {
-                arrive(&acc_empty[b]);
-                arrive(&idx_empty[r]);
+                mbar_arrive(&acc_empty[b]);
+                mbar_arrive(&idx_empty[r]);
             }
             if (++b == a.nacc) {
                 b = 0;
@@ -700,7 +692,7 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
             }
             if (lane == 0) s_item[r] = cur;
             __syncwarp();
-            if (lane == 0) arrive(&idx_full[r]);
+            if (lane == 0) mbar_arrive(&idx_full[r]);
             cur = nxt;
             if (it + 2 * STC_IDXW < nmine) nxt = item_of(it + 2 * STC_IDXW);
         }
@@ -709,9 +701,9 @@ __device__ __forceinline__ void stc_body(const StcArgs& a) {
     const bool done = mbar_wait(smem_u32(&done_bar), 0, DRAIN_LIMIT);
     __syncthreads();
     if ((!done || s_fail) && tid == 0) atomicExch(a.err, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    tcx::fence_after_sync();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.nacc * a.acc_cols));
+        tcx::tmem_dealloc(tmem, a.nacc * a.acc_cols);
 }
 
 // rotation (0) and back-rotation (1); coaxial pass

@@ -106,15 +106,16 @@ __device__ __forceinline__ uint32_t cluster_rank() {
     return r;
 }
 __device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;");
-    asm volatile("barrier.cluster.wait.acquire.aligned;");
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 // arrives on `bar` in every CTA of the mask once the MMAs issued so far are complete
 __device__ __forceinline__ void mma_commit_to(uint64_t* bar, uint16_t mask) {
     asm volatile(
         "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
             smem_u32(bar)),
-        "h"(mask));
+        "h"(mask)
+        : "memory");
 }
 
 }  // namespace
@@ -193,19 +194,6 @@ struct TcArgs {
     int nacc, tmem_cols;   // accumulators; columns to allocate
 };
 
-// 32 consecutive accumulator columns of this thread's lane
-__device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&v)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
-        "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];"
-        : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]), "=r"(v[4]), "=r"(v[5]), "=r"(v[6]), "=r"(v[7]),
-          "=r"(v[8]), "=r"(v[9]), "=r"(v[10]), "=r"(v[11]), "=r"(v[12]), "=r"(v[13]), "=r"(v[14]), "=r"(v[15]),
-          "=r"(v[16]), "=r"(v[17]), "=r"(v[18]), "=r"(v[19]), "=r"(v[20]), "=r"(v[21]), "=r"(v[22]), "=r"(v[23]),
-          "=r"(v[24]), "=r"(v[25]), "=r"(v[26]), "=r"(v[27]), "=r"(v[28]), "=r"(v[29]), "=r"(v[30]), "=r"(v[31])
-        : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;");
-}
-
 template <int NB>
 __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     constexpr int PER = tc_period(NB), NP = 2 * PER;   // a producer warp's chunks; its pieces of each per lane
@@ -230,9 +218,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     const int ct0 = blockIdx.x / TC_CLUSTER, ncl = gridDim.x / TC_CLUSTER;
     const TcTile* tiles = a.tiles + rank;   // this CTA's tile of cluster tile ct: tiles[ct * TC_CLUSTER]
     if (warp == 0) {
-        asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_holder)),
-                     "r"(a.tmem_cols));
-        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
+        tcx::tmem_alloc(&tmem_holder, a.tmem_cols);
     }
     if (tid == 0) {
         s_fail = 0;
@@ -251,11 +237,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         }
         mbar_init(&done_bar, 1);
         mbar_init(&never_bar, 1);
-        asm volatile("fence.mbarrier_init.release.cluster;");
+        tcx::fence_mbar_init();
     }
-    asm volatile("tcgen05.fence::before_thread_sync;");
+    tcx::fence_before_sync();
     cluster_sync();   // every CTA's barriers are there before a peer signals them
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    tcx::fence_after_sync();
     const uint32_t tmem = tmem_holder;
 
     if (warp < PROD_WARPS) {
@@ -273,7 +259,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         auto seek = [&]() -> bool {
             while (c >= nkc) {
                 if (it >= 0 && lane == 0)   // the tile's offsets are no longer needed
-                    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_empty[it % TC_RING])) : "memory");
+                    tcx::mbar_arrive(&idx_empty[it % TC_RING]);
                 c -= nkc;
                 nkc = 0;
                 ++it;
@@ -347,10 +333,10 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 cur[i] = nxt[i];
             }
             // generic-proxy stores become visible to the tensor core's reads
-            asm volatile("fence.proxy.async.shared::cta;");
+            tcx::fence_proxy_async();
             __syncwarp();
             if (lane == 0)
-                asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&full_bar[s])) : "memory");
+                tcx::mbar_arrive(&full_bar[s]);
             more = next;
         }
     } else if (warp == 8) {
@@ -376,22 +362,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     }
                     const uint32_t bb = smem_u32(&b_bar[s]);
                     const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_BLOCK + off);
-                    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bb),
-                                 "r"((uint32_t)(NB * blk * sizeof(float))));
+                    tcx::mbar_expect(bb, (uint32_t)(NB * blk * sizeof(float)));
 #pragma unroll
                     for (int h = 0; h < NB; ++h) {
                         const float* gh = g + h * tl.t_blk;
                         const uint32_t dh = dB + (uint32_t)(h * blk * sizeof(float));
                         if (tl.scount == 1)
-                            asm volatile(
-                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-                                    dh),
-                                "l"(gh), "r"((uint32_t)(blk * sizeof(float))), "r"(bb));
+                            tcx::bulk_copy(dh, gh, (uint32_t)(blk * sizeof(float)), bb);
                         else
                             asm volatile(
                                 "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
                                 "[%1], %2, [%3], %4;" ::"r"(dh),
-                                "l"(gh), "r"((uint32_t)(part * sizeof(float))), "r"(bb), "h"(smask));
+                                "l"(gh), "r"((uint32_t)(part * sizeof(float))), "r"(bb), "h"(smask)
+                                : "memory");
                     }
                     if (++s == nst) {
                         s = 0;
@@ -463,7 +446,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     const int s1 = s + 1 == nst ? 0 : s + 1;
                     const uint32_t p1 = s1 == 0 ? ph ^ 1 : ph;
                     ready = mbar_test(smem_u32(&full_bar[s1]), p1) & mbar_test(smem_u32(&b_bar[s1]), p1);
-                    asm volatile("tcgen05.fence::after_thread_sync;");
+                    tcx::fence_after_sync();
 #pragma unroll
                     for (int h = 0; h < NB; ++h)
 #pragma unroll
@@ -519,7 +502,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 s_len[r] = 2 * tl.p_in2;
             }
             __syncwarp();
-            if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&idx_full[r])) : "memory");
+            if (lane == 0) tcx::mbar_arrive(&idx_full[r]);
         }
     } else {
         // ---------------- epilogue: accumulator lanes 32 quad .. 32 quad + 31,
@@ -550,7 +533,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     fail = true;
                     break;
                 }
-                asm volatile("tcgen05.fence::after_thread_sync;");
+                tcx::fence_after_sync();
                 const int npair = min(32, tl.ncol - quad * 32), rows = min(tl.nrow, 2 * tl.p_out2 - tl.row0 - h * tl.nrow);
                 const uint32_t acc = tmem + (uint32_t)(b * a.acc_cols) + ((uint32_t)(quad * 32) << 16);
                 // 16-byte adds where every target of the warp is aligned to them
@@ -558,7 +541,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 int c0 = half * TC_CS;
                 for (; c0 < tl.nrow; c0 += 2 * TC_CS) {
                     uint32_t v[32];   // (columns past the block lie within the accumulator's)
-                    tmem_ld32(acc + (uint32_t)c0, v);
+                    tcx::tmem_ld32(acc + (uint32_t)c0, v);
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
                         *reinterpret_cast<uint4*>(row + 4 * q) = make_uint4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
@@ -588,9 +571,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                     __syncwarp();
                 }
                 // this warp's share of the accumulator is read
-                asm volatile("tcgen05.fence::before_thread_sync;");
+                tcx::fence_before_sync();
                 __syncwarp();
-                if (lane == 0) asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(&acc_empty[b])) : "memory");
+                if (lane == 0) tcx::mbar_arrive(&acc_empty[b]);
                 if (++b == a.nacc) {
                     b = 0;
                     aph ^= 1;
@@ -602,9 +585,9 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     const bool done = mbar_wait(smem_u32(&done_bar), 0, DRAIN_LIMIT);
     __syncthreads();
     if ((!done || s_fail) && tid == 0) atomicExch(a.err, 1);
-    asm volatile("tcgen05.fence::after_thread_sync;");
+    tcx::fence_after_sync();
     if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(a.tmem_cols));
+        tcx::tmem_dealloc(tmem, a.tmem_cols);
     cluster_sync();   // no CTA leaves while a peer may still write its shared memory or signal its barriers
 }
 
