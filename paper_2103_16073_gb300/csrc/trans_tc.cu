@@ -21,13 +21,11 @@
 // Operands:  A = gathered X rows, read as FP32 and split by the producer
 // warps on the way into the canonical layout.  B = T, pre-split and stored in
 // global memory already in the canonical no-swizzle K-major layout, one block
-// (hi then lo) per (row tile, K chunk of 16).  Streaming T for every 128
-// pairs is what bounds a dense level (order 12: 663 KB per 128 pairs, at 6.6
-// TB/s out of L2 0.74 ms of level 7 below), so the tiles of one matrix run in
-// clusters of four that load a share each and multicast it to the others'
-// stages.
+// (hi then lo) per (row tile, K chunk of 16); every CTA copies the blocks of
+// its tile into its own shared memory (tiles of one matrix run side by side,
+// so that all but the first read come out of L2).
 //
-// Persistent: every cluster walks over its share of the tiles with each role
+// Persistent: every CTA walks over its share of the tiles with each role
 // running ahead of the next (a tile's setup, a chain of dependent loads, and
 // its scatter cost as much as its MMAs at order 12):
 //   warps 0-7    A producers: warp w takes every fourth chunk (w % 4) of 64
@@ -36,21 +34,21 @@
 //                the loads of its next chunk in flight (two blocks: every
 //                second chunk of 32 pairs, as only three stages fit);
 //   warp 8       lane 0: bulk copies of T (transaction count);
-//   warp 9       lane 0: MMA issuer (6 MMAs per chunk, commits to the stage's
-//                "empty" barrier in every CTA of the cluster, which keeps the
-//                four in step);
+//   warp 9       lane 0: MMA issuer (6 MMAs per chunk and block, commits to the
+//                stage's "empty" barrier);
 //   warps 10-17  epilogue: accumulator rows (lane = pair) through shared
 //                memory, so that the atomic adds into the targets are
 //                coalesced runs of one pair's coefficients;
 //   warp 18      source offsets of the next tiles into a ring in shared
 //                memory, ahead of the producers.
-// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 0.85 ms (the
+// L-room at 2 kHz, M2L of level 7 (order 12, 952,630 pairs): 0.78 ms (the
 // MMAs alone 0.68 ms); 1.87 ms with pairs as N, one tile per CTA and hi/lo
-// planes of X split in a pass of its own.  The three tensor levels together
-// 1.83 ms against 3.54 ms; of the shoebox at 1 kHz 0.20 against 0.36 ms.
-// What is left is shared-memory bandwidth: the MMAs read 130 bytes per cycle
-// of it at their peak rate, the copies of T, the split X and the epilogue
-// share the rest.
+// planes of X split in a pass of its own, 0.85 ms in clusters of four that
+// shared the loads of T and so kept step with their slowest CTA.  The three
+// tensor levels together 1.66 ms against 3.54 ms (1.83 in clusters); of the
+// shoebox at 1 kHz 0.18 against 0.36 ms.  What is left is shared-memory
+// bandwidth: the MMAs read 130 bytes per cycle of it at their peak rate, the
+// copies of T, the split X and the epilogue share the rest.
 // Every mbarrier wait is bounded; on timeout the kernel records an error
 // flag, drains its own copies and MMAs (bounded) and releases tensor memory.
 #include <algorithm>
@@ -81,12 +79,8 @@ constexpr int TC_THREADS = 32 * (IDX_WARP + 1);
 constexpr int TC_RING = 4;        // tiles of source offsets in shared memory
 constexpr int TC_CS = 32;         // accumulator columns staged per epilogue pass
 constexpr int TC_STAGING = EPI_WARPS * 32 * (TC_CS + 4);   // floats
-constexpr int TC_CLUSTER = 4;     // CTAs per cluster
 // a producer warp takes every fourth chunk, with two blocks every second one
 __host__ __device__ constexpr int tc_period(int nblk) { return nblk == 2 ? 2 : 4; }
-// drain bound of the shared copies: they land within microseconds, but after
-// a peer's timeout a stage may never get that peer's share
-constexpr long long SHARE_DRAIN = 1LL << 20;
 using tcx::canon;
 using tcx::DRAIN_LIMIT;
 using tcx::LBO;
@@ -100,24 +94,6 @@ using tcx::tf32_hi;
 using tcx::umma_desc;
 static_assert(TC_KC == tcx::KC, "one canonical block width");
 
-__device__ __forceinline__ uint32_t cluster_rank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
-__device__ __forceinline__ void cluster_sync() {
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-// arrives on `bar` in every CTA of the mask once the MMAs issued so far are complete
-__device__ __forceinline__ void mma_commit_to(uint64_t* bar, uint16_t mask) {
-    asm volatile(
-        "tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(
-            smem_u32(bar)),
-        "h"(mask)
-        : "memory");
-}
-
 }  // namespace
 
 struct TcTask {
@@ -128,14 +104,12 @@ struct TcTask {
     int32_t p_in2;                      // complex columns P_in
     int64_t src_base, dst_base;         // complex offsets of the source and target levels
 };
-// Columns [col0, col0 + ncol) of a task (ncol = 0 fills a cluster), NB blocks of
-// nrow real rows from row0 on (their chunks of T lie t_blk floats apart).  Its T is shared by the scount (1, 2 or 4) CTAs of the cluster
-// from rank sbase on.  The four tiles of a cluster have the same nkc and nrow.
+// Columns [col0, col0 + ncol) of a task, NB blocks of nrow real rows from row0
+// on (their chunks of T lie t_blk floats apart).
 struct alignas(16) TcTile {
     int64_t t_off, pair_off, src_base, dst_base;
     int32_t p_in2, p_out2, nkc, nrow;
-    int32_t row0, col0;
-    int16_t ncol, sbase, scount, pad;
+    int32_t row0, col0, ncol, pad;
     int64_t t_blk;
 };
 
@@ -177,7 +151,7 @@ __global__ void k_tc_pack(const TcPack* __restrict__ packs, const cd* __restrict
 
 struct TcArgs {
     const TcTile* tiles;
-    int nct;           // clusters of tiles
+    int ntiles;
     const float* T;
     const int32_t* src_idx;
     const int32_t* dst_idx;
@@ -200,7 +174,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     extern __shared__ unsigned char smem_raw[];
     __shared__ __align__(8) uint64_t full_bar[TC_STAGES];    // A producers' stores
     __shared__ __align__(8) uint64_t b_bar[TC_STAGES];       // the bulk copies of T
-    __shared__ __align__(8) uint64_t empty_bar[TC_STAGES];   // the MMAs of every CTA of the cluster
+    __shared__ __align__(8) uint64_t empty_bar[TC_STAGES];   // the MMAs of the stage
     __shared__ __align__(8) uint64_t acc_full[TC_ACC], acc_empty[TC_ACC];
     __shared__ __align__(8) uint64_t done_bar;
     __shared__ __align__(8) uint64_t never_bar;              // test hook: nothing arrives on it
@@ -214,9 +188,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     float* stage0 = (float*)(smem_raw + pad);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int nst = a.nst, rank = (int)cluster_rank();
-    const int ct0 = blockIdx.x / TC_CLUSTER, ncl = gridDim.x / TC_CLUSTER;
-    const TcTile* tiles = a.tiles + rank;   // this CTA's tile of cluster tile ct: tiles[ct * TC_CLUSTER]
+    const int nst = a.nst;
+    const int ct0 = blockIdx.x, ncta = gridDim.x;   // this CTA's tiles: ct0, ct0 + ncta, ...
     if (warp == 0) {
         tcx::tmem_alloc(&tmem_holder, a.tmem_cols);
     }
@@ -225,7 +198,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         for (int s = 0; s < TC_STAGES; ++s) {
             mbar_init(&full_bar[s], PROD_WARPS / PER);   // the warps of a chunk
             mbar_init(&b_bar[s], 1);
-            mbar_init(&empty_bar[s], TC_CLUSTER);
+            mbar_init(&empty_bar[s], 1);
         }
         for (int b = 0; b < TC_ACC; ++b) {
             mbar_init(&acc_full[b], 1);
@@ -240,7 +213,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         tcx::fence_mbar_init();
     }
     tcx::fence_before_sync();
-    cluster_sync();   // every CTA's barriers are there before a peer signals them
+    __syncthreads();
     tcx::fence_after_sync();
     const uint32_t tmem = tmem_holder;
 
@@ -253,7 +226,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         int len = 0;             // floats of a source expansion from the lane's quarter on
         uint32_t has = 0;        // pieces with a pair
         bool al = true;          // every piece 16-byte aligned
-        int c = warp % PER, nkc = 0, it = -1, ct = ct0 - ncl;   // load cursor: chunk of tile it
+        int c = warp % PER, nkc = 0, it = -1, ct = ct0 - ncta;   // load cursor: chunk of tile it
         bool fail = false;
         // moves the cursor to this warp's next chunk; false at the end
         auto seek = [&]() -> bool {
@@ -263,8 +236,8 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 c -= nkc;
                 nkc = 0;
                 ++it;
-                ct += ncl;
-                if (ct >= a.nct) return false;
+                ct += ncta;
+                if (ct >= a.ntiles) return false;
                 const int r = it % TC_RING;
                 const bool ok = mbar_wait(smem_u32(&idx_full[r]), (it / TC_RING) & 1, a.wait_limit);
                 if (!__all_sync(0xffffffffu, ok)) {
@@ -340,20 +313,20 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             more = next;
         }
     } else if (warp == 8) {
-        // ---------------- T: this CTA's share of every stage, to all sharers --
+        // ---------------- chunks of T: one bulk copy per block and stage ------
         if (lane == 0) {
             int64_t cc = 0;
             int s = 0;
             uint32_t ph = 1;
             bool fail = false;
             TcTile tn;
-            if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
-            for (int ct = ct0; ct < a.nct && !fail; ct += ncl) {
+            if (ct0 < a.ntiles) tn = a.tiles[ct0];
+            for (int ct = ct0; ct < a.ntiles && !fail; ct += ncta) {
                 const TcTile tl = tn;
-                if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
-                const int blk = 2 * tl.nrow * TC_KC, part = blk / tl.scount, off = (rank - tl.sbase) * part;
-                const uint16_t smask = (uint16_t)(((1 << tl.scount) - 1) << tl.sbase);
-                const float* g = a.T + tl.t_off + off;
+                if (ct + ncta < a.ntiles) tn = a.tiles[ct + ncta];
+                const int blk = 2 * tl.nrow * TC_KC;
+                const uint32_t bytes = (uint32_t)(blk * sizeof(float));
+                const float* g = a.T + tl.t_off;
                 for (int c = 0; c < tl.nkc; ++c, ++cc, g += blk) {
                     if (cc >= nst && !mbar_wait(smem_u32(&empty_bar[s]), ph, a.wait_limit)) {
                         atomicExch(&s_fail, 1);
@@ -361,31 +334,19 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                         break;
                     }
                     const uint32_t bb = smem_u32(&b_bar[s]);
-                    const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_BLOCK + off);
-                    tcx::mbar_expect(bb, (uint32_t)(NB * blk * sizeof(float)));
+                    const uint32_t dB = smem_u32(stage0 + (size_t)s * a.stage_floats + 2 * A_BLOCK);
+                    tcx::mbar_expect(bb, NB * bytes);
 #pragma unroll
-                    for (int h = 0; h < NB; ++h) {
-                        const float* gh = g + h * tl.t_blk;
-                        const uint32_t dh = dB + (uint32_t)(h * blk * sizeof(float));
-                        if (tl.scount == 1)
-                            tcx::bulk_copy(dh, gh, (uint32_t)(blk * sizeof(float)), bb);
-                        else
-                            asm volatile(
-                                "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.multicast::cluster [%0], "
-                                "[%1], %2, [%3], %4;" ::"r"(dh),
-                                "l"(gh), "r"((uint32_t)(part * sizeof(float))), "r"(bb), "h"(smask)
-                                : "memory");
-                    }
+                    for (int h = 0; h < NB; ++h) tcx::bulk_copy(dB + h * bytes, g + h * tl.t_blk, bytes, bb);
                     if (++s == nst) {
                         s = 0;
                         ph ^= 1;
                     }
                 }
             }
-            // every copy into this CTA lands before it may exit (on success the
-            // MMA issuer has already waited for each of them)
+            // every bulk copy this CTA issued lands before it may exit
             for (int64_t k = cc > nst ? cc - nst : 0; k < cc; ++k)
-                mbar_wait(smem_u32(&b_bar[k % nst]), (uint32_t)(k / nst) & 1, SHARE_DRAIN);
+                mbar_wait(smem_u32(&b_bar[k % nst]), (uint32_t)(k / nst) & 1, DRAIN_LIMIT);
         }
         __syncwarp();
     } else if (warp == 9) {
@@ -408,15 +369,15 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
             // one before is issued.
             bool ready = false;
             int nkc_n = 0, nrow_n = 0;
-            if (ct0 < a.nct) {
-                nkc_n = tiles[(int64_t)ct0 * TC_CLUSTER].nkc;
-                nrow_n = tiles[(int64_t)ct0 * TC_CLUSTER].nrow;
+            if (ct0 < a.ntiles) {
+                nkc_n = a.tiles[ct0].nkc;
+                nrow_n = a.tiles[ct0].nrow;
             }
-            for (int ct = ct0; ct < a.nct && !fail; ct += ncl) {
+            for (int ct = ct0; ct < a.ntiles && !fail; ct += ncta) {
                 const int nkc = nkc_n, nrow = nrow_n;
-                if (ct + ncl < a.nct) {
-                    nkc_n = tiles[(int64_t)(ct + ncl) * TC_CLUSTER].nkc;
-                    nrow_n = tiles[(int64_t)(ct + ncl) * TC_CLUSTER].nrow;
+                if (ct + ncta < a.ntiles) {
+                    nkc_n = a.tiles[ct + ncta].nkc;
+                    nrow_n = a.tiles[ct + ncta].nrow;
                 }
                 uint32_t acc[NB];
                 uint64_t* fullb[NB];
@@ -457,7 +418,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                             mma_tf32(acc[h], desc(aH + ((A_BLOCK * 4) >> 4)), desc(bH), idesc, 1u);
                             mma_tf32(acc[h], desc(aH), desc(bH + blo), idesc, 1u);
                         }
-                    mma_commit_to(&empty_bar[s], (uint16_t)((1 << TC_CLUSTER) - 1));
+                    mma_commit(&empty_bar[s]);
                     dof = s1 == 0 ? dlo : dof + dstep;
                     s = s1;
                     ph = p1;
@@ -473,11 +434,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     } else if (warp == IDX_WARP) {
         // ---------------- source offsets, up to TC_RING tiles ahead -----------
         TcTile tn;
-        if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
+        if (ct0 < a.ntiles) tn = a.tiles[ct0];
         int it = 0;
-        for (int ct = ct0; ct < a.nct; ct += ncl, ++it) {
+        for (int ct = ct0; ct < a.ntiles; ct += ncta, ++it) {
             const TcTile tl = tn;
-            if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
+            if (ct + ncta < a.ntiles) tn = a.tiles[ct + ncta];
             int64_t o[TC_PAIRS / 32];
 #pragma unroll
             for (int q = 0; q < TC_PAIRS / 32; ++q) {
@@ -511,11 +472,11 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
         float* sg = stage0 + (size_t)nst * a.stage_floats + ew * 32 * (TC_CS + 4);
         float* row = sg + lane * (TC_CS + 4);
         TcTile tn;
-        if (ct0 < a.nct) tn = tiles[(int64_t)ct0 * TC_CLUSTER];
+        if (ct0 < a.ntiles) tn = a.tiles[ct0];
         int b = 0;
         uint32_t aph = 0;
         bool fail = false;
-        for (int ct = ct0; ct < a.nct && !fail; ct += ncl) {
+        for (int ct = ct0; ct < a.ntiles && !fail; ct += ncta) {
             const TcTile tl = tn;
             const int j = quad * 32 + lane;   // this lane's pair
             int64_t dst = 0;                  // its target expansion (floats)
@@ -524,7 +485,7 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
                 dst = 2 * ((int64_t)(col - pr * a.nrhs) * a.rstride + tl.dst_base +
                            (int64_t)a.dst_idx[tl.pair_off + pr] * tl.p_out2) + tl.row0;
             }
-            if (ct + ncl < a.nct) tn = tiles[(int64_t)(ct + ncl) * TC_CLUSTER];
+            if (ct + ncta < a.ntiles) tn = a.tiles[ct + ncta];
 #pragma unroll 1
             for (int h = 0; h < NB; ++h, dst += tl.nrow) {
                 const bool full = mbar_wait(smem_u32(&acc_full[b]), aph, a.wait_limit);
@@ -588,7 +549,6 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
     tcx::fence_after_sync();
     if (warp == 0)
         tcx::tmem_dealloc(tmem, a.tmem_cols);
-    cluster_sync();   // no CTA leaves while a peer may still write its shared memory or signal its barriers
 }
 
 // ------------------------------------------------------------- host side ----
@@ -596,12 +556,12 @@ __global__ void __launch_bounds__(TC_THREADS, 1) k_trans_tc(const TcArgs a) {
 struct TcLaunch {
     int rows_max = 0, acc_cols = 0, nblk = 1, nacc = 2, tmem_cols = 0;
     std::vector<int> tasks;
-    int nst = 0, resident = 1;   // pipeline stages, clusters resident at once
+    int nst = 0;   // pipeline stages
     size_t smem = 0;
 };
 struct TcTiles {
     TcTile* d = nullptr;
-    std::vector<int> count;   // clusters of tiles per launch, consecutive in d
+    std::vector<int> count;   // tiles per launch, consecutive in d
 };
 struct TcPlanImpl {
     std::vector<TcTask> h_tasks;
@@ -617,20 +577,6 @@ struct TcPlanImpl {
 static size_t tc_stage_bytes(int rows) { return (size_t)(2 * A_BLOCK + 2 * rows * TC_KC) * sizeof(float); }
 static const void* tc_kernel(int nblk) { return nblk == 2 ? (const void*)k_trans_tc<2> : (const void*)k_trans_tc<1>; }
 
-static void tc_launch_config(const TcLaunch& ln, int clusters, cudaStream_t s, cudaLaunchConfig_t* cfg,
-                             cudaLaunchAttribute* at) {
-    *cfg = {};
-    cfg->gridDim = dim3((unsigned)(TC_CLUSTER * clusters));
-    cfg->blockDim = dim3(TC_THREADS);
-    cfg->dynamicSmemBytes = ln.smem;
-    cfg->stream = s;
-    at->id = cudaLaunchAttributeClusterDimension;
-    at->val.clusterDim.x = TC_CLUSTER;
-    at->val.clusterDim.y = 1;
-    at->val.clusterDim.z = 1;
-    cfg->attrs = at;
-    cfg->numAttrs = 1;
-}
 // Stages and shared memory of a launch (one CTA per SM: at least a share
 // such that no second CTA's allocation waits for tensor memory).  At least as
 // many stages as a producer warp's period of chunks: when it waits for a
@@ -643,31 +589,25 @@ static fb_status tc_configure(TcLaunch& ln) {
     if (ln.nst < tc_period(ln.nblk)) return fb_fail(FB_ERR_STATE, "tensor-core translation: too few pipeline stages");
     ln.smem = std::max(ln.nst * stage + fixed, (size_t)116 * 1024);
     FB_CHECK(fb_smem_cap(tc_kernel(ln.nblk), ln.smem));
-    cudaLaunchConfig_t cfg;
-    cudaLaunchAttribute at;
-    tc_launch_config(ln, 1, nullptr, &cfg, &at);
-    FB_CUDA(cudaOccupancyMaxActiveClusters(&ln.resident, tc_kernel(ln.nblk), &cfg));
-    ln.resident = std::max(1, ln.resident);
     return FB_OK;
 }
 
-// Tiles of the plan for nrhs right-hand sides, in clusters of TC_CLUSTER:
-// per (chunks, rows) whole clusters of one matrix first, then the remaining
-// pairs and single tiles packed together.
+// Tiles of the plan for nrhs right-hand sides: per launch the ones of most
+// work first, those of one matrix side by side.
 static void tc_make_tiles(const TcPlanImpl* pl, int nrhs, std::vector<TcTile>& out, std::vector<int>& count) {
     for (const TcLaunch& ln : pl->launches) {
-        std::map<std::pair<int, int>, std::vector<int>, std::greater<std::pair<int, int>>> by;   // most work first
+        std::map<std::pair<int, int>, std::vector<int>, std::greater<std::pair<int, int>>> by;
         for (int ti : ln.tasks) by[{pl->h_tasks[ti].nkc, pl->h_tasks[ti].rt_rows}].push_back(ti);
         const size_t first = out.size();
-        for (const auto& kv : by) {
-            std::vector<TcTile> two, one;
+        for (const auto& kv : by)
             for (int ti : kv.second) {
                 const TcTask& tk = pl->h_tasks[ti];
-                const int ncol = tk.npairs * nrhs, nc = div_up(ncol, TC_PAIRS);
-                for (int rt = 0; rt < tk.nrt; rt += ln.nblk) {
-                    auto tile = [&](int c, int scount) {
-                        TcTile t;
-                        t.t_off = tk.a_off + (int64_t)rt * tk.nkc * 2 * tk.rt_rows * TC_KC;
+                const int ncol = tk.npairs * nrhs;
+                for (int rt = 0; rt < tk.nrt; rt += ln.nblk)
+                    for (int c0 = 0; c0 < ncol; c0 += TC_PAIRS) {
+                        TcTile t = {};
+                        t.t_blk = (int64_t)tk.nkc * 2 * tk.rt_rows * TC_KC;
+                        t.t_off = tk.a_off + rt * t.t_blk;
                         t.pair_off = tk.pair_off;
                         t.src_base = tk.src_base;
                         t.dst_base = tk.dst_base;
@@ -676,38 +616,12 @@ static void tc_make_tiles(const TcPlanImpl* pl, int nrhs, std::vector<TcTile>& o
                         t.nkc = tk.nkc;
                         t.nrow = tk.rt_rows;
                         t.row0 = rt * tk.rt_rows;
-                        t.col0 = c * TC_PAIRS;
-                        t.ncol = (int16_t)std::min(TC_PAIRS, ncol - c * TC_PAIRS);
-                        t.sbase = 0;
-                        t.scount = (int16_t)scount;
-                        t.pad = 0;
-                        t.t_blk = (int64_t)tk.nkc * 2 * tk.rt_rows * TC_KC;
-                        return t;
-                    };
-                    int c = 0;
-                    for (; c + TC_CLUSTER <= nc; c += TC_CLUSTER)
-                        for (int i = 0; i < TC_CLUSTER; ++i) out.push_back(tile(c + i, TC_CLUSTER));
-                    if (TC_CLUSTER > 2 && c + 2 <= nc) {
-                        two.push_back(tile(c, 2));
-                        two.push_back(tile(c + 1, 2));
-                        c += 2;
+                        t.col0 = c0;
+                        t.ncol = std::min(TC_PAIRS, ncol - c0);
+                        out.push_back(t);
                     }
-                    if (c < nc) one.push_back(tile(c, 1));
-                }
             }
-            out.insert(out.end(), two.begin(), two.end());
-            out.insert(out.end(), one.begin(), one.end());
-            while ((out.size() - first) % TC_CLUSTER) {   // a tile without columns
-                TcTile t = out.back();
-                t.ncol = 0;
-                t.scount = 1;
-                out.push_back(t);
-            }
-        }
-        // rank of the first sharer: groups of 4, 2 and 1 lie aligned to their size
-        for (size_t i = first; i < out.size(); ++i)
-            out[i].sbase = (int16_t)((int)((i - first) % TC_CLUSTER) / out[i].scount * out[i].scount);
-        count.push_back((int)((out.size() - first) / TC_CLUSTER));
+        count.push_back((int)(out.size() - first));
     }
 }
 
@@ -752,7 +666,7 @@ fb_status fb_tc_build_groups(fb_op* op, const std::vector<TcGroup>& groups, cons
         tk.npairs = g.npairs;
         // Two blocks of rows in one tile where that is all rows (orders 11 and
         // 12): X is gathered and split once instead of twice, order 12 0.85
-        // against 1.16 ms (level 7 above).  With more tiles the three stages it
+        // against 1.16 ms (level 7 above, both in clusters).  With more tiles the three stages it
         // leaves cost more than the gathers saved: order 20 in 3 x 2 blocks of
         // 144 0.59 ms, in 4 of 208 0.56 ms.
         tk.nrt = div_up(2 * Pout, TC_RMAX);
@@ -844,22 +758,24 @@ fb_status fb_tc_run(fb_op* op, void* plan, const cf* src, cf* dst, cudaStream_t 
     a.rstride = rstride;
     a.wait_limit = g_wait_limit.load();
     a.inject_stall = g_inject_stall.load();
-    for (size_t i = 0; i < pl->launches.size(); a.tiles += (size_t)tiles->count[i] * TC_CLUSTER, ++i) {
+    int dev = 0, sms = 0;
+    FB_CUDA(cudaGetDevice(&dev));
+    FB_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    for (size_t i = 0; i < pl->launches.size(); a.tiles += tiles->count[i], ++i) {
         const TcLaunch& ln = pl->launches[i];
-        a.nct = tiles->count[i];
+        a.ntiles = tiles->count[i];
         a.acc_cols = ln.acc_cols;
         a.nst = ln.nst;
         a.nacc = ln.nacc;
         a.tmem_cols = ln.tmem_cols;
         a.stage_floats = (int)(tc_stage_bytes(ln.nblk * ln.rows_max) / sizeof(float));
         FB_CHECK(fb_smem_cap(tc_kernel(ln.nblk), ln.smem));
-        cudaLaunchAttribute at;
-        cudaLaunchConfig_t cfg;
-        tc_launch_config(ln, std::min(ln.resident, a.nct), s, &cfg, &at);
+        const unsigned grid = (unsigned)std::min(sms, a.ntiles);
         if (ln.nblk == 2)
-            FB_CUDA(cudaLaunchKernelEx(&cfg, k_trans_tc<2>, a));
+            k_trans_tc<2><<<grid, TC_THREADS, ln.smem, s>>>(a);
         else
-            FB_CUDA(cudaLaunchKernelEx(&cfg, k_trans_tc<1>, a));
+            k_trans_tc<1><<<grid, TC_THREADS, ln.smem, s>>>(a);
+        FB_LAUNCH_CHECK();
         fb_count_launch();
     }
     return FB_OK;

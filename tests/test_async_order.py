@@ -50,3 +50,11 @@ def test_asynchronous_statements_order_memory(path):
             assert '"memory"' in s and "volatile" in s, s
         if "tcgen05.ld" in s:
             assert "tcgen05.wait::ld" in s, s
+
+
+def test_no_load_is_multicast():
+    """The kernels also run with one rank per GPU, where loads stay within a
+    CTA: none names the multicast form."""
+    for p in FILES:
+        for s in statements(open(p).read()):
+            assert "multicast" not in s, (p, s)
