@@ -515,9 +515,11 @@ fb_status upload(T** d, const std::vector<T>& h) {
 
 bool fb_stg_staged(const RcrTask& tk) { return (tk.staged >= 1 && tk.staged <= 3) || tk.staged == 5; }
 
+// A tile works in place on max(p_in, p_out)^2 coefficients per column and needs
+// room for one column and its padding (rcr_tiles.cu).
 bool fb_rcr_tile_fits(int p_in, int p_out, size_t csize) {
-    const size_t per = (size_t)((int64_t)p_in * p_in + std::max<int64_t>((int64_t)p_in * p_in, (int64_t)p_out * p_out));
-    return per * csize <= 200 * 1024;
+    const size_t p = (size_t)std::max(p_in, p_out);
+    return 2 * p * p * csize <= 200 * 1024;
 }
 int fb_rcr_default_staged(int p_in, int p_out, size_t csize) {
     return !fb_rcr_tile_fits(p_in, p_out, csize) || std::max(p_in, p_out) >= FB_STG_PMIN;
