@@ -89,6 +89,7 @@ fb_status time_rcr(fb_op* op, const RcrPlan& base, Pick pick, int staged, void* 
     if (pl.h_tasks.empty()) return FB_OK;
     const size_t csz = op->prec == FB_PREC_MIXED_FMM ? sizeof(cf) : sizeof(cd);
     fb_status st = fb_rcr_upload(op, pl, base.src_idx, base.dst_idx, csz);
+    if (st == FB_OK && pl.stg) fb_stg_reserve(op, nrhs, s);   // as the product does
     if (st == FB_OK) st = time_ms([&]() { return fb_rcr_run_op(op, pl, src, dst, s, nrhs, cnt); }, s, reps, ms);
     cudaStreamSynchronize(s);
     free_rcr(pl);

@@ -429,12 +429,12 @@ struct fb_op {
     // level l; M2M and L2L between levels l-1 and l)
     int stg_m2l[FB_MAXLEV + 1] = {0};
     int stg_pair[FB_MAXLEV + 1] = {0};
-    // staging buffers of the large-order RCR passes (U, V: stg_elems
-    // complex values each, in the operator's precision)
+    // staging buffers of the large-order RCR passes (U, V: stg_elems complex
+    // each), shared by every plan; stg_need: the largest plan's need for one
+    // right-hand side, stg_refused: a size that could not be allocated
     void* stg_u = nullptr;
     void* stg_v = nullptr;
-    int64_t stg_elems = 0;
-    int stg_nrhs = 1;   // right-hand sides they hold
+    int64_t stg_elems = 0, stg_need = 0, stg_refused = 0;
     RcrPlan m2l_rcr, m2m_rcr[FB_MAXLEV + 1], l2l_rcr[FB_MAXLEV + 1];
     // tensor-core (3xTF32) stacked M2L: dense levels (auto) / every level
     void* tc_plan = nullptr;
@@ -516,6 +516,7 @@ fb_status fb_rcr_tiles_run_f(const fb_op* op, RcrPlan& pl, const cf* src, cf* ds
 fb_status fb_rcr_tiles_run_d(const fb_op* op, RcrPlan& pl, const cd* src, cd* dst, cudaStream_t s, int nrhs,
                              int64_t rstride);
 void fb_rcr_tiles_free(RcrTileSet& t);
+void fb_stg_reserve(fb_op* op, int nrhs, cudaStream_t s);
 fb_status fb_rcr_upload(fb_op* op, RcrPlan& pl, const int32_t* src, const int32_t* dst, size_t csize);
 fb_status fb_tree_rotations(fb_tree* t, int P, const std::vector<double>& dirs, cudaStream_t s,
                             const fb_tree::RotSet** out);

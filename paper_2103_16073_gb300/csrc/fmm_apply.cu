@@ -363,8 +363,6 @@ struct RotArgs {
     int64_t fper;
     StcTabs tc;       // tables of the tensor-core staged passes (single precision)
     DfTabs dft;       // tables of the double-FP32 staged passes (FP64 operators)
-    int nb;           // right-hand sides the staging buffers hold, and their stride
-    int64_t ustride;
 };
 template <class R>
 static RotArgs<R> rot_args(const fb_op* op) {
@@ -377,19 +375,17 @@ static RotArgs<R> rot_args(const fb_op* op) {
     a.fper = op->rotf_per;
     a.tc = StcTabs{op->stc_tab, op->stc_per, op->stc_err};
     a.dft = DfTabs{op->rotf_df, op->coax_df};
-    a.nb = op->stg_nrhs;
-    a.ustride = op->stg_elems;
     return a;
 }
 static fb_status stg_run(void* plan, const RotArgs<float>& r, const cf* coax, const cf* src, cf* dst,
-                         cudaStream_t s, int nrhs, int64_t rstride) {
+                         cudaStream_t s, int nrhs, int64_t rstride, int nb, int64_t ustride) {
     return fb_stg_run_f(plan, (const float*)r.rf, r.fper, r.ph, r.prot, coax, src, dst, r.U, r.V, s, nrhs, rstride,
-                        r.tc, r.nb, r.ustride);
+                        r.tc, nb, ustride);
 }
 static fb_status stg_run(void* plan, const RotArgs<double>& r, const cd* coax, const cd* src, cd* dst,
-                         cudaStream_t s, int nrhs, int64_t rstride) {
+                         cudaStream_t s, int nrhs, int64_t rstride, int nb, int64_t ustride) {
     return fb_stg_run_d(plan, (const double*)r.rf, r.fper, r.ph, r.prot, coax, src, dst, r.U, r.V, s, nrhs, rstride,
-                        r.dft, r.nb, r.ustride);
+                        r.dft, nb, ustride);
 }
 
 // Device time (ms, median of 3 after one untimed run, one right-hand side)
@@ -463,8 +459,39 @@ template <class R>
 static fb_status run_rcr(const fb_op* op, RcrPlan& pl, const RotArgs<R>& rot, const cx<R>* coax, const cx<R>* src,
                          cx<R>* dst, cudaStream_t s, int nrhs = 1, int64_t rstride = 0) {
     FB_CHECK(rcr_tiles_run(op, pl, src, dst, s, nrhs, rstride));
-    if (pl.stg) FB_CHECK(stg_run(pl.stg, rot, coax, src, dst, s, nrhs, rstride));
+    if (pl.stg) {   // as many right-hand sides at a time as the staging buffers hold of this plan
+        const int nb = (int)std::min<int64_t>(nrhs, op->stg_elems / std::max<int64_t>(1, pl.stg_elems));
+        FB_CHECK(stg_run(pl.stg, rot, coax, src, dst, s, nrhs, rstride, std::max(1, nb), pl.stg_elems));
+    }
     return FB_OK;
+}
+
+// Grows the staging buffers to nrhs right-hand sides of the largest plan, up
+// to 256 MB a buffer (a level beyond that fills the chip alone): a level too
+// small for a launch of its own per right-hand side takes them all in one,
+// eight sources at 600 Hz 2.59 -> 2.11 ms.  Without room for it (a size that
+// was refused is not asked for again) or in a capture the buffers stay, and
+// the right-hand sides go in smaller batches.
+void fb_stg_reserve(fb_op* op, int nrhs, cudaStream_t s) {
+    const int64_t csize = op->prec == FB_PREC_MIXED_FMM ? sizeof(cf) : sizeof(cd);
+    const int64_t cap0 = (int64_t)(256 << 20) / csize, want = std::min(nrhs * op->stg_need, std::max(op->stg_need, cap0));
+    if (want <= op->stg_elems || (op->stg_refused && want >= op->stg_refused)) return;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) return;
+    void *u = nullptr, *v = nullptr;
+    if (cudaMalloc(&u, (size_t)(want * csize)) != cudaSuccess || cudaMalloc(&v, (size_t)(want * csize)) != cudaSuccess) {
+        cudaGetLastError();
+        cudaFree(u);
+        op->stg_refused = want;
+        return;
+    }
+    cudaStreamSynchronize(s);
+    dfree(op->stg_u);
+    dfree(op->stg_v);
+    op->stg_u = u;
+    op->stg_v = v;
+    op->stg_elems = want;
+    op->buf_gen++;   // captured graphs refer to the old buffers
 }
 
 // Uploads an RCR plan: per-pair tiles for the tasks of moderate order and the
@@ -491,6 +518,7 @@ fb_status fb_rcr_upload(fb_op* op, RcrPlan& pl, const int32_t* src, const int32_
     FB_CHECK(fb_stg_build(pl, op->theta_slot, op->per_dir, op->coax64, &pl.stg, &pl.stg_elems));
     if (fb_stg_uses_tc(pl.stg)) FB_CHECK(fb_stc_tables(op, cudaStreamLegacy));
     if (fb_stg_uses_df(pl.stg)) FB_CHECK(fb_stg_df_tables(op, cudaStreamLegacy));
+    op->stg_need = std::max(op->stg_need, pl.stg_elems);
     if (pl.stg_elems > op->stg_elems) {
         FB_CUDA(cudaDeviceSynchronize());
         dfree(op->stg_u);
@@ -499,7 +527,6 @@ fb_status fb_rcr_upload(fb_op* op, RcrPlan& pl, const int32_t* src, const int32_
         FB_CHECK(dalloc((unsigned char**)&op->stg_u, (size_t)pl.stg_elems * csize));
         FB_CHECK(dalloc((unsigned char**)&op->stg_v, (size_t)pl.stg_elems * csize));
         op->stg_elems = pl.stg_elems;
-        op->stg_nrhs = 1;
         op->buf_gen++;   // captured graphs refer to the old buffers
     }
     return FB_OK;
@@ -547,31 +574,7 @@ static fb_status fmm_apply_t(fb_op* op, const cd* x, cd* y, cudaStream_t s, cons
         op->exp_nrhs = nrhs;
         op->buf_gen++;   // captured graphs of this operator refer to the old buffers
     }
-    // Staging buffers for several right-hand sides at once, where a level is
-    // too small for a launch of its own per right-hand side (up to 256 MB a
-    // buffer; a level beyond that fills the chip alone): eight sources at
-    // 600 Hz 2.59 -> 2.11 ms.  Without room for them, or in a capture, they
-    // go one after the other.
-    if (!scratch && op->stg_elems > 0) {
-        const int nb = (int)std::min<int64_t>(nrhs, std::max<int64_t>(1, (256LL << 20) / (op->stg_elems * (int64_t)sizeof(cx<R>))));
-        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-        if (nb > op->stg_nrhs && cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusNone) {
-            unsigned char *u = nullptr, *v = nullptr;
-            const size_t bytes = (size_t)nb * op->stg_elems * sizeof(cx<R>);
-            if (dalloc(&u, bytes) == FB_OK && dalloc(&v, bytes) == FB_OK) {
-                cudaStreamSynchronize(s);
-                dfree(op->stg_u);
-                dfree(op->stg_v);
-                op->stg_u = u;
-                op->stg_v = v;
-                op->stg_nrhs = nb;
-                op->buf_gen++;
-            } else {
-                dfree(u);
-                cudaGetLastError();
-            }
-        }
-    }
+    if (!scratch) fb_stg_reserve(op, nrhs, s);
     cx<R>* mp = scratch ? (cx<R>*)scratch : (cx<R>*)op->mp;
     cx<R>* loc = scratch ? (cx<R>*)scratch + cnt * nrhs : (cx<R>*)op->loc;
     mark(0);
@@ -736,6 +739,7 @@ fb_status fb_rcr_restage(fb_op* op, const int* m2l, const int* pair) {
         }
     }
     FB_CUDA(cudaDeviceSynchronize());
+    op->stg_refused = 0;   // other plans, another need
     op->buf_gen++;   // captured graphs refer to the plans rebuilt here
     auto redo = [&](RcrPlan& pl) -> fb_status {
         if (pl.h_tasks.empty()) return FB_OK;
@@ -827,7 +831,6 @@ void fb_fmm_destroy(fb_op* op) {
     dfree(op->stg_u);
     dfree(op->stg_v);
     op->stg_elems = 0;
-    op->stg_nrhs = 1;
     if (op->rotf) cudaFree(op->rotf);
     op->rotf = nullptr;
     dfree(op->stc_tab);
