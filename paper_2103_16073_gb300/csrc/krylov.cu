@@ -528,9 +528,10 @@ fb_status fb_self_blocks(const fb_op* op, const int64_t* d_off, cd* out, cudaStr
 
 // In-place Gauss-Jordan inverse with partial pivoting of the block of leaf t
 // (order `scale` x its element count; scale 2 for the indirect system).
-// The block stays in shared memory where it fits (room for `cap` rows), the
-// pivot is found by one warp and a warp updates a row at a time: 1,838 leaves
-// of 29 rows 2.95 ms in global memory with the pivot searched by one thread.
+// The pivot is found by one warp and a warp updates a row at a time (with the
+// pivot searched by one thread 1,838 leaves of up to 77 rows took 2.95 ms of
+// kernel, their preconditioner takes 2.3 ms in all now).  The blocks are in shared
+// memory where every one of the launch fits (`cap` rows; bj_cap).
 __global__ void k_bj_invert(const int32_t* leaf_start, const int64_t* blk_off, cd* blocks, int* piv_scr,
                             int* singular, int scale, int cap) {
     int t = blockIdx.x;
@@ -605,8 +606,13 @@ __global__ void k_bj_invert(const int32_t* leaf_start, const int64_t* blk_off, c
         for (int e = threadIdx.x; e < n * n; e += blockDim.x) ga[e] = a[e];
 }
 
-// Rows a block in shared memory may have and the bytes to launch with, for
-// blocks of up to maxn rows (three CTAs per SM).
+// Rows of the blocks in shared memory (0: all in global memory) and the bytes
+// to launch with, for blocks of up to maxn rows.  All or none: up to 67 rows
+// every block is in shared memory (three CTAs per SM; preconditioner of 96
+// leaves of up to 58 rows 0.72 against 0.75 ms, 3,904 of up to 20 0.48 against
+// 0.49); with larger ones among them the shared memory of the small ones costs
+// the large ones their L1 (56 leaves of up to 68 rows 1.26 ms mixed, 1.06 all
+// in global memory; 7,826 of up to 74 4.27 against 3.9).
 static int bj_cap(int maxn, size_t* smem) {
     const int cap = (size_t)maxn * (maxn + 1) * sizeof(cd) <= 72 * 1024 ? maxn : 0;
     *smem = sizeof(cd) * (size_t)std::max(maxn, 1) * (cap + 1);
