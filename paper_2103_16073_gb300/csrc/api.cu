@@ -60,6 +60,9 @@ void fb_set_error(fb_status code, const std::string& msg) {
     snprintf(g_last_msg, sizeof(g_last_msg), "%s", msg.c_str());
 }
 fb_status fb_fail(fb_status code, const std::string& msg) {
+    // the runtime keeps the error of a refused call until it is read, and the
+    // next launch check would report it for a call that did nothing wrong
+    if (code == FB_ERR_CUDA || code == FB_ERR_OOM) cudaGetLastError();
     fb_set_error(code, msg);
     return code;
 }
