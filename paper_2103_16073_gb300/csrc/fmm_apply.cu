@@ -173,7 +173,7 @@ __device__ __forceinline__ cf nf_entry(uint32_t a) {
 //
 // Bound by reading A and V (one warp per row).  A leaf of some 18 rows is
 // mostly latency: the columns are gathered by all warps at once (offsets of
-// the U-list leaves from one warp scan), the warp's first row of A is on its
+// the U-list leaves from a warp scan), the warp's first row of A is on its
 // way before that, and every batch of LU loads of a row (A, then V, then the
 // next row's A) goes out before the one ahead of it is used.  blockIdx.z
 // splits the rows of a leaf where there are too few leaves.  FP32 with 16-bit
@@ -227,11 +227,11 @@ __global__ void __launch_bounds__(NEAR_THREADS, NEAR_CTAS<R, NB>) k_near_l2p(int
     const int t = blockIdx.x;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int nu = ucnt[t], K = nf_ncol[t];
-    // start and column offset of every U-list leaf (FB_ULIST < 32)
-    __shared__ int s_start[32], s_col[32];
+    // this lane's U-list leaf (FB_ULIST < 32): start and size (in registers of
+    // every warp: the dynamic shared memory of the largest leaves leaves no room)
     const int sl = lane < FB_ULIST ? ulist[(int64_t)t * FB_ULIST + lane] : 0;
     int a0 = 0, len = 0;
-    if (warp == 0 && lane < nu) {
+    if (lane < nu) {
         a0 = leaf_start[sl];
         len = leaf_start[sl + 1] - a0;
     }
@@ -258,31 +258,32 @@ __global__ void __launch_bounds__(NEAR_THREADS, NEAR_CTAS<R, NB>) k_near_l2p(int
         }
     };
     if (r < nrow) load_a(r, 0);
-    if (warp == 0) {
-        int c = len;
+    int col = len;   // its first column (K past the list)
 #pragma unroll
-        for (int o = 1; o < 32; o *= 2) {
-            const int v = __shfl_up_sync(0xffffffffu, c, o);
-            if (lane >= o) c += v;
-        }
-        s_start[lane] = a0;
-        s_col[lane] = lane < nu ? c - len : K;
+    for (int o = 1; o < 32; o *= 2) {
+        const int v = __shfl_up_sync(0xffffffffu, col, o);
+        if (lane >= o) col += v;
     }
+    col = lane < nu ? col - len : K;
+    a0 -= col;
     const int ldx = K + P;              // xs: [nr][K columns, P local coefficients]
     if (loc)
         for (int j = 0; j < nr; ++j)
             for (int q = threadIdx.x; q < P; q += NEAR_THREADS)
                 xs[j * ldx + K + q] = loc[(r0 + j) * lstride + (int64_t)t * P + q];
-    __syncthreads();
     // gather the x values of the U-list leaves in column order
 #pragma unroll 2
-    for (int q = threadIdx.x; q < K; q += NEAR_THREADS) {
+    for (int q0 = 32 * warp; q0 < K; q0 += NEAR_THREADS) {
+        const int q = q0 + lane;
         int i = 0;   // the last leaf that starts at or before column q
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1)
-            if (s_col[i + o] <= q) i += o;
-        const int e = perm[s_start[i] + q - s_col[i]];
-        for (int j = 0; j < nr; ++j) xs[j * ldx + q] = from_d<R>(x[(r0 + j) * xstride + e]);
+            if (__shfl_sync(0xffffffffu, col, i + o) <= q) i += o;
+        const int pos = __shfl_sync(0xffffffffu, a0, i) + q;
+        if (q < K) {
+            const int e = perm[pos];
+            for (int j = 0; j < nr; ++j) xs[j * ldx + q] = from_d<R>(x[(r0 + j) * xstride + e]);
+        }
     }
     __syncthreads();
     constexpr int M = 2 * NR * NB;
