@@ -109,8 +109,9 @@ __device__ __forceinline__ df df_add(df a, df b) {
 }
 // FP64 -> double-FP32 by integer steps (conversion instructions run at the
 // FP64 pipe's rate, a 64th of the integer pipe's): hi is the rounded upper
-// part, lo the 29 remaining bits as a signed count of 2^(E - 52).  Below
-// FP32's normal range the value is flushed to zero, above it is infinite.
+// part, lo the 29 remaining bits as a signed count of 2^(E - 52).  What lies
+// outside [2^-126, 2^127) and is not zero (rare) takes the instructions, which
+// keep subnormals.
 __device__ __forceinline__ df df_from_fast(double v) {
     const uint32_t h = (uint32_t)__double2hiint(v), l = (uint32_t)__double2loint(v);
     const uint32_t e = (h >> 20) & 0x7ff;
@@ -119,13 +120,15 @@ __device__ __forceinline__ df df_from_fast(double v) {
     const int r = (int)low - (int)(up << 29);
     float lo = (__int2float_rn(r) * 2.220446049250313e-16f) * __uint_as_float((e - 896) << 23);
     if (e - 897 >= 253u) {
-        mag = e < 897 ? 0u : (e == 0x7ff ? 0x7fffffffu : 0x7f800000u);
+        if ((h & 0x7fffffffu) | l) return df_from(v);
+        mag = 0;
         lo = 0.f;
     }
     return df(__uint_as_float(mag | sign), __uint_as_float(__float_as_uint(lo) ^ sign));
 }
 // double-FP32 -> FP64 the same way: the normalised low part is a signed
-// count of ulps added to the significand of the high part.
+// count of ulps added to the significand of the high part (subnormal, infinite
+// and NaN: the instructions).
 __device__ __forceinline__ double df_to_fast(df a) {
     const float s = __fadd_rn(a.hi, a.lo);
     const float bb = __fsub_rn(s, a.hi);
@@ -138,8 +141,10 @@ __device__ __forceinline__ double df_to_fast(df a) {
     if (b >> 31) q = -q;
     if ((mag & 0x7fffffu) == 0 && q < 0) q *= 2;   // below a power of two the ulps are half as large
     uint32_t hi = (mag >> 3) + (896u << 20), lo = mag << 29;
-    if (e == 0) hi = lo = 0, q = 0;                                    // zero (FP32 denormals are flushed)
-    if (e == 255) hi = 0x7ff00000u | ((mag & 0x7fffffu) >> 3), lo = mag << 29, q = 0;   // infinity, NaN
+    if (e - 1 >= 254u) {
+        if (mag) return df_to(a);
+        hi = lo = 0, q = 0;   // zero
+    }
     const uint64_t w = (((uint64_t)hi << 32) | lo) + (uint64_t)(int64_t)q;
     return __longlong_as_double((long long)(w | ((uint64_t)(b & 0x80000000u) << 32)));
 }
