@@ -40,6 +40,10 @@
 // 19.7 -> 8.1-8.6 ms (its multiply-adds alone 5.3 ms, 62 % of the FP32 pipe;
 // loads 1.0 ms, the 274 M FP64 atomics 1.7 ms), FP64 44.5 -> 21.1 ms, FP32
 // 3.68 -> 1.78 ms (multiply-adds 1.05 ms).
+//
+// Double-FP32: the load and store steps (phases, x_m +- x_-m, y_+-m') run in
+// FP64 and round once, as in the staged passes; in 48 bits they added 11 % to
+// the error against FP64 for 1 % of a product (L-room 29.4 against 29.8 ms).
 #include <algorithm>
 #include <cstdlib>
 #include <map>
@@ -95,18 +99,6 @@ __host__ __device__ __forceinline__ int rt_rot_off(int n, int part) {
 }
 
 // ------------------------------------------------------ double-FP32 steps ----
-__device__ __forceinline__ df df_mul(df a, df b) {
-    const float p = __fmul_rn(a.hi, b.hi);
-    float e = __fmaf_rn(a.hi, b.hi, -p);
-    e = __fmaf_rn(a.hi, b.lo, e);
-    return df(p, __fmaf_rn(a.lo, b.hi, e));
-}
-__device__ __forceinline__ df df_add(df a, df b) {
-    const float s = __fadd_rn(a.hi, b.hi);
-    const float bb = __fsub_rn(s, a.hi);
-    const float err = __fadd_rn(__fsub_rn(a.hi, __fsub_rn(s, bb)), __fsub_rn(b.hi, bb));
-    return df(s, __fadd_rn(__fadd_rn(a.lo, b.lo), err));
-}
 // FP64 -> double-FP32 by integer steps (conversion instructions run at the
 // FP64 pipe's rate, a 64th of the integer pipe's): hi is the rounded upper
 // part, lo the 29 remaining bits as a signed count of 2^(E - 52).  What lies
@@ -149,7 +141,8 @@ __device__ __forceinline__ double df_to_fast(df a) {
     return __longlong_as_double((long long)(w | ((uint64_t)(b & 0x80000000u) << 32)));
 }
 
-// conversions and arithmetic of the load and store steps in the type R
+// conversions between the expansions' type O and the arithmetic type R: the
+// load and store steps (phases, sums and differences) run in O
 template <class R, class O>
 __device__ __forceinline__ cx<R> rt_in(const cx<O>& a) { return a; }
 template <>
@@ -159,20 +152,6 @@ __device__ __forceinline__ cx<O> rt_out(const cx<R>& a) { return a; }
 template <>
 __device__ __forceinline__ cd rt_out<double, df>(const cx<df>& a) { return mk(df_to_fast(a.re), df_to_fast(a.im)); }
 
-template <class R>
-__device__ __forceinline__ cx<R> rt_mul(const cx<R>& a, const cx<R>& b) { return a * b; }
-template <>
-__device__ __forceinline__ cx<df> rt_mul(const cx<df>& a, const cx<df>& b) {
-    return mk(fma(-a.im, b.im, df_mul(a.re, b.re)), fma(a.im, b.re, df_mul(a.re, b.im)));
-}
-template <class R>
-__device__ __forceinline__ cx<R> rt_add(const cx<R>& a, const cx<R>& b) { return a + b; }
-template <>
-__device__ __forceinline__ cx<df> rt_add(const cx<df>& a, const cx<df>& b) {
-    return mk(df_add(a.re, b.re), df_add(a.im, b.im));
-}
-template <class R>
-__device__ __forceinline__ cx<R> rt_neg(const cx<R>& a) { return mk(-a.re, -a.im); }
 template <class R>
 __device__ __forceinline__ cx<R> rt_conj(const cx<R>& a) { return mk(a.re, -a.im); }
 __device__ __forceinline__ float rt_half(float a) { return 0.5f * a; }
@@ -337,15 +316,14 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rcr(const RtArgs<R, O> a) {
         for (int b = warp; b < tl.ncol; b += nw) {
             const cx<O>* x = s_src[b] + c0;
             cx<R>* o = B + (n * n + m) * cwp + b;
-            const cx<R> xp = rt_in<R, O>(x[m]);
+            const cx<O> xp = x[m];
             if (m == 0) {
-                o[0] = xp;
+                o[0] = rt_in<R, O>(xp);
             } else {
-                const cx<R> xm = rt_in<R, O>(x[-m]);
-                const cx<R> ph = rt_in<R, O>(s_ph[b][m]);
-                const cx<R> u = rt_mul(xp, ph), v = rt_mul(xm, rt_conj(ph));
-                o[0] = rt_add(u, v);
-                o[n * cwp] = rt_add(u, rt_neg(v));
+                const cx<O> xm = x[-m], ph = s_ph[b][m];
+                const cx<O> u = xp * ph, v = xm * rt_conj(ph);
+                o[0] = rt_in<R, O>(u + v);
+                o[n * cwp] = rt_in<R, O>(u - v);
             }
         }
     }
@@ -400,9 +378,9 @@ __global__ void __launch_bounds__(RT_THREADS, 1) k_rcr(const RtArgs<R, O> a) {
             } else {
                 cx<R> ym = o[n * cwp];
                 ym = mk(rt_half(ym.re), rt_half(ym.im));
-                const cx<R> ph = rt_in<R, O>(s_ph[b][m]);
-                rt_atomic(d + m, rt_out<O, R>(rt_mul(rt_add(yp, ym), rt_conj(ph))));
-                rt_atomic(d - m, rt_out<O, R>(rt_mul(rt_add(yp, rt_neg(ym)), ph)));
+                const cx<O> ph = s_ph[b][m], a1 = rt_out<O, R>(yp), a2 = rt_out<O, R>(ym);
+                rt_atomic(d + m, (a1 + a2) * rt_conj(ph));
+                rt_atomic(d - m, (a1 - a2) * ph);
             }
         }
     }
