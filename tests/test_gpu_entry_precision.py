@@ -9,7 +9,7 @@ torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 import paper_2103_16073_gb300 as fb
-from _cases import oracle_mesh, workload
+from _cases import oracle_mesh, seeded_vector, workload
 
 LD = np.longdouble
 PI = LD("3.14159265358979323846264338327950288")
@@ -92,3 +92,45 @@ def test_closed_form_entries():
     x, n, v, area = xc[I], xn[J], v[J].astype(float), area[J].astype(float)
     plain = (int_inv_r(x, v, n) + smooth(k, x, v, area)) / (4 * np.pi)
     assert rms((got - exact) / exact) < 1.05 * rms((plain - exact) / exact)
+
+
+def gauss(v):
+    T = v.dtype.type
+    b = [[T(2) / 3 if i == q else T(1) / 6 for i in range(3)] for q in range(3)]
+    return np.stack([sum(w * v[:, i] for i, w in enumerate(r)) for r in b], 1)
+
+
+def field(k, x, y, c, n, area, beta, psi, gam, rc):
+    """L q - M psi at the points x by the three-point rule, elements within r_c left out."""
+    out = []
+    for r in x:
+        d = y - r
+        R = np.sqrt(dot(d, d))
+        e = np.cos(k * R) + 1j * np.sin(k * R)
+        w = (area / 3)[:, None] / (4 * np.pi if R.dtype == float else 4 * PI)
+        L = (w * e / R).sum(1)
+        M = (w * dot(n[:, None, :], d) / R ** 3 * (e * (-1 + 1j * k * R))).sum(1)
+        z = L * (gam + 1j * k * beta * psi) - M * psi
+        out.append(z[dot(c - r, c - r) >= rc * rc].sum())
+    return np.array(out)
+
+
+def test_receivers_at_a_low_wavenumber():
+    """Receivers farther than r_c from every wall, where k R stays small and its rounding does not dominate."""
+    wl, v, c, n, area = geometry("sub")
+    k, rc = 2.0, oracle_mesh("sub").rc
+    rng = np.random.default_rng(5)
+    x = rc + (np.array(wl.room) - 2 * rc) * rng.uniform(0.0, 1.0, size=(400, 3))
+    psi, gam = seeded_vector(wl.n, 1), seeded_vector(wl.n, 2)
+    mesh = fb.fb_mesh_create(wl.verts, wl.tris)
+    fb.fb_mesh_set_admittance(mesh, wl.beta)
+    try:
+        xc, xn = fb.fb_mesh_geometry(mesh)
+        out = torch.empty(400, dtype=torch.complex128, device="cuda")
+        got = fb.fb_eval_field(mesh, k, *(torch.tensor(a, device="cuda") for a in (psi, gam, x)), out).cpu().numpy()
+    finally:
+        fb.fb_mesh_destroy(mesh)
+    rest = (wl.beta, psi, gam, rc)
+    exact = field(LD(k), x.astype(LD), gauss(v), c, n, area, *rest)
+    plain = field(k, x, gauss(v.astype(float)), xc, xn, area.astype(float), *rest)
+    assert rms(got - exact) < 1.05 * rms(plain - exact)
