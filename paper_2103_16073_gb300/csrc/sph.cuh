@@ -54,11 +54,14 @@ __device__ inline void sph_bessel_j(int nmax, double x, double* j) {
         return;
     }
     int start = nmax + 24 + (int)x;
-    const double ix = 1.0 / x;
+    // (2n + 1) / x as a multiple of 1/x in two parts: one part alone is the
+    // functions at a rounded argument, 4 to 8 times the error for n, x of 20 to 160
+    const double ix = 1.0 / x, ir = fma(-x, ix, 1.0) * ix;
     double fp = 0.0, f = 1e-280;
     for (int n = 0; n <= nmax; ++n) j[n] = 0.0;
     for (int n = start; n >= 1; --n) {
-        double fm = (2.0 * n + 1.0) * ix * f - fp;
+        const double c = 2.0 * n + 1.0;
+        double fm = fma(c, ix, c * ir) * f - fp;
         fp = f;
         f = fm;             // f = f_{n-1}, fp = f_n
         if (n - 1 <= nmax) j[n - 1] = f;
