@@ -588,13 +588,9 @@ fb_status fb_operator_export(const fb_op* op, int which, int level, int64_t inde
         if (out) {
             const int64_t off = (int64_t)op->dir_of_code[index] * op->per_dir + (int64_t)n * (2 * n - 1) * (2 * n + 1) / 3;
             std::vector<double> h((size_t)w * w);
-            if (op->prec == FB_PREC_MIXED_FMM) {
-                std::vector<float> f((size_t)w * w);
-                FB_CUDA(cudaMemcpy(f.data(), op->rotd32 + off, sizeof(float) * f.size(), cudaMemcpyDeviceToHost));
-                for (size_t i = 0; i < f.size(); ++i) h[i] = f[i];
-            } else {
-                FB_CUDA(cudaMemcpy(h.data(), op->rotd64 + off, sizeof(double) * h.size(), cudaMemcpyDeviceToHost));
-            }
+            FB_CUDA(cudaMemcpy(h.data(), op->rotd64 + off, sizeof(double) * h.size(), cudaMemcpyDeviceToHost));
+            if (op->prec == FB_PREC_MIXED_FMM)   // as the FP32 passes round them
+                for (double& v : h) v = (float)v;
             for (size_t i = 0; i < h.size(); ++i) {
                 out[2 * i] = h[i];
                 out[2 * i + 1] = 0.0;

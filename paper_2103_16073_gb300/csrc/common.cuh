@@ -199,7 +199,6 @@ struct fb_tree {
     struct RotSet {
         cd* r64 = nullptr;          // complex blocks, degrees < Pc (composed matrices)
         double* d64 = nullptr;      // real factors, degrees < P
-        float* d32 = nullptr;
         cd* ph64 = nullptr;         // phase tables e^{i m phi}
         cf* ph32 = nullptr;
         int P = 0, Pc = 0, ndir = 0;
@@ -400,7 +399,7 @@ struct fb_op {
     int Prot = 0;
     int64_t per_dir = 0;
     cd* rot64 = nullptr;                     // complex rotation blocks, degrees < FB_COMPOSE_PMAX
-    double* rotd64 = nullptr; float* rotd32 = nullptr;   // real parts d (owned by the tree)
+    double* rotd64 = nullptr;                // real parts d (owned by the tree)
     cd* rph64 = nullptr; cf* rph32 = nullptr;            // phase tables (owned by the tree)
     cd* coax64 = nullptr; cf* coax32 = nullptr;
     int64_t coax_count = 0, rot_count = 0;
@@ -411,9 +410,7 @@ struct fb_op {
     void* rotf = nullptr;                    // folded rotation tables (staged RCR), per group
     int64_t rotf_per = 0;                    // values per group and table
     float* stc_tab = nullptr;                // pre-split canonical tables of the tensor-core staged passes
-    int64_t* stc_off = nullptr;              // their block offsets per (degree, part)
     int64_t stc_per = 0;                     // floats per group and table
-    int stc_P = 0;
     int* stc_err = nullptr;                  // error flag of the tensor-core staged passes
     const fb_op* near_donor = nullptr;       // during creation: an FP64 FMM operator of the same
                                              // mesh, tree, k and kind whose near-field entries are copied

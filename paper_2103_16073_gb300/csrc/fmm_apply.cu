@@ -824,7 +824,6 @@ void fb_fmm_destroy(fb_op* op) {
     }
     op->rot64 = nullptr;   // owned by the tree
     op->rotd64 = nullptr;
-    op->rotd32 = nullptr;
     op->rph64 = nullptr;
     op->rph32 = nullptr;
     dfree(op->coax64);
@@ -835,7 +834,6 @@ void fb_fmm_destroy(fb_op* op) {
     if (op->rotf) cudaFree(op->rotf);
     op->rotf = nullptr;
     dfree(op->stc_tab);
-    dfree(op->stc_off);
     dfree(op->stc_err);
     dfree(op->rotf_df);
     dfree(op->coax_df);

@@ -638,7 +638,7 @@ __global__ void k_box_centers(const uint32_t* keys, int n, int level, double ox,
 // 1e-12 up to degree 318).  Also writes the phase tables ph[m + P - 1] = e^{i m phi}
 // and, for degrees n < Pc, the complex blocks D = d e^{i m phi} the
 // composed matrices use.  grid: (entry chunk, n, dir)
-__global__ void k_rot_delta(const cd* delta, const double* dirs, int ndir, int P, int Pc, double* d64, float* d32,
+__global__ void k_rot_delta(const cd* delta, const double* dirs, int ndir, int P, int Pc, double* d64,
                             cd* ph64, cf* ph32, cd* r64) {
     __shared__ double cs[FB_ROT_PMAX], sn[FB_ROT_PMAX];
     int n = blockIdx.y, dd = blockIdx.z;
@@ -673,7 +673,6 @@ __global__ void k_rot_delta(const cd* delta, const double* dirs, int ndir, int P
     int64_t per_dir = (int64_t)P * (2 * P - 1) * (2 * P + 1) / 3;
     int64_t o = (int64_t)dd * per_dir + off + e;
     d64[o] = acc;
-    d32[o] = (float)acc;
     if (n < Pc) {
         double sp, cp;
         sincos((double)m * phi, &sp, &cp);
@@ -731,9 +730,9 @@ fb_status fb_tree_rotations(fb_tree* t, int P, const std::vector<double>& dirs, 
     rs.per_dir = per_dir;
     rs.per_dir_c = per_c;
     rs.ndir = ndir;
-    auto free_rs = [&]() { dfree(rs.r64); dfree(rs.d64); dfree(rs.d32); dfree(rs.ph64); dfree(rs.ph32); };
+    auto free_rs = [&]() { dfree(rs.r64); dfree(rs.d64); dfree(rs.ph64); dfree(rs.ph32); };
     if ((st = dalloc(&rs.r64, (size_t)ndir * per_c)) || (st = dalloc(&rs.d64, (size_t)ndir * per_dir)) ||
-        (st = dalloc(&rs.d32, (size_t)ndir * per_dir)) || (st = dalloc(&rs.ph64, (size_t)ndir * (2 * Prot - 1))) ||
+        (st = dalloc(&rs.ph64, (size_t)ndir * (2 * Prot - 1))) ||
         (st = dalloc(&rs.ph32, (size_t)ndir * (2 * Prot - 1)))) {
         free_tmp();
         free_rs();
@@ -741,7 +740,7 @@ fb_status fb_tree_rotations(fb_tree* t, int P, const std::vector<double>& dirs, 
     }
     {
         dim3 grid(div_up((2 * Prot - 1) * (2 * Prot - 1), 128), Prot, ndir);
-        k_rot_delta<<<grid, 128, 0, s>>>(delta, ddirs, ndir, Prot, Pc, rs.d64, rs.d32, rs.ph64, rs.ph32, rs.r64);
+        k_rot_delta<<<grid, 128, 0, s>>>(delta, ddirs, ndir, Prot, Pc, rs.d64, rs.ph64, rs.ph32, rs.r64);
     }
     FB_LAUNCH_CHECK();
     cudaError_t e = cudaStreamSynchronize(s);
@@ -1065,7 +1064,6 @@ fb_status fb_fmm_create(fb_op* op, double d0, int pmin, cudaStream_t s) {
     coax = nullptr;
     op->rot64 = rot;
     op->rotd64 = rset->d64;
-    op->rotd32 = rset->d32;
     op->rph64 = rset->ph64;
     op->rph32 = rset->ph32;
     op->rot_count = (int64_t)ndir * per_dir;

@@ -908,22 +908,27 @@ fb_status fb_stc_tables(fb_op* op, cudaStream_t s) {
     if (ng == 0 || P < 1) return fb_fail(FB_ERR_STATE, "tensor-core staged RCR: no rotation groups");
     std::vector<int64_t> toff;
     const int64_t tper = stg::fb_stc_layout(P, toff);
-    int* d_dirs = nullptr;
-    FB_CHECK(dalloc(&d_dirs, (size_t)ng));
-    FB_CHECK(dalloc(&op->stc_off, toff.size()));
-    FB_CHECK(dalloc(&op->stc_tab, (size_t)ng * 2 * tper));
     if (!op->stc_err) {
         FB_CHECK(dalloc(&op->stc_err, 1));
         FB_CUDA(cudaMemsetAsync(op->stc_err, 0, sizeof(int), s));
     }
+    int* d_dirs = nullptr;
+    int64_t* d_off = nullptr;
+    fb_status st;
+    if ((st = dalloc(&d_dirs, (size_t)ng)) || (st = dalloc(&d_off, toff.size())) ||
+        (st = dalloc(&op->stc_tab, (size_t)ng * 2 * tper))) {
+        dfree(d_dirs);
+        dfree(d_off);
+        return st;
+    }
     FB_CUDA(cudaMemcpyAsync(d_dirs, op->theta_dirs.data(), sizeof(int) * ng, cudaMemcpyHostToDevice, s));
-    FB_CUDA(cudaMemcpyAsync(op->stc_off, toff.data(), sizeof(int64_t) * toff.size(), cudaMemcpyHostToDevice, s));
-    k_stc_tables<<<dim3(P, ng), 256, 0, s>>>(op->rotd64, op->per_dir, d_dirs, op->stc_off, tper, op->stc_tab);
+    FB_CUDA(cudaMemcpyAsync(d_off, toff.data(), sizeof(int64_t) * toff.size(), cudaMemcpyHostToDevice, s));
+    k_stc_tables<<<dim3(P, ng), 256, 0, s>>>(op->rotd64, op->per_dir, d_dirs, d_off, tper, op->stc_tab);
     cudaError_t e = cudaStreamSynchronize(s);
     dfree(d_dirs);
+    dfree(d_off);
     if (e != cudaSuccess) return fb_fail(FB_ERR_CUDA, std::string("tensor-core rotation tables: ") + cudaGetErrorString(e));
     op->stc_per = tper;
-    op->stc_P = P;
     fb_count_launch();
     return FB_OK;
 }

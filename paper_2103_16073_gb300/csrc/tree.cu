@@ -427,7 +427,6 @@ void fb_tree_free(fb_tree* t) {
     for (auto& rs : t->rot_sets) {
         dfree(rs.r64);
         dfree(rs.d64);
-        dfree(rs.d32);
         dfree(rs.ph64);
         dfree(rs.ph32);
     }
