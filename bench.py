@@ -304,6 +304,15 @@ def fp64_only_forms(tune):
     return out
 
 
+def tune_summary(tune):
+    """Per operator and level the autotuner's choice bits and the times (ms)
+    of the candidates it ran."""
+    return {op: levels if isinstance(levels, str) else   # forms given on the command line
+            {l: {**{k: round(v, 3) for k, v in t.items() if isinstance(v, float)}, "choice": t["choice"]}
+             for l, t in (levels or {}).items()}
+            for op, levels in tune.items()}
+
+
 def m2l_levels(tune, p, pairs):
     """Per level of an autotuned operator whose M2L is not staged: (form,
     device ms of its M2L pass, algorithmic flops) from the autotuner's
@@ -665,7 +674,7 @@ def run_ours(args):
         "solution_rel_diff_mixed_vs_plain": sol_diff,
         "learned": "side study, not in the timed step (the trained network did not reduce the outer "
                    "iterations of the inner-outer solve)",
-        "autotune": P["tune"],
+        "autotune": tune_summary(P["tune"]),
         "graphs": True,
         "measured_alu_peaks_tflops": {"fp32": round(fp32_peak, 2), "fp64": round(fp64_peak, 3)},
         "e2e": {"value": round(1.0 / e2e_s, 5), "unit": "solves/s", "h2d_bytes_per_step": 16 * n,
