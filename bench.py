@@ -243,10 +243,9 @@ def level_counts(fb, op, tree):
 
 
 def rot_flops(p_out, p_in):
-    """Algorithmic flops of the two rotations of one RCR translation: sum
-    (2n+1)^2 over n < p_in (rotate) and n < p_out (rotate back), complex-by-
-    real MACs counted as complex MACs x 8 (the unfolded count; the folded
-    kernels execute about half)."""
+    """Flops of the two rotations of one RCR translation as the method states
+    them (Sec. 3.3): sum (2n+1)^2 over n < p_in (rotate) and n < p_out (rotate
+    back) complex MACs of 8.  The rooflines count folded_rot_flops."""
     return 8.0 * (sum((2 * n + 1) ** 2 for n in range(p_in)) + sum((2 * n + 1) ** 2 for n in range(p_out)))
 
 
@@ -260,6 +259,18 @@ def rcr_flops(p_out, p_in):
     """Algorithmic flops of one RCR translation (rotations + coaxial step),
     about (10/3) p^3 x 8 for p_out = p_in."""
     return rot_flops(p_out, p_in) + coax_flops(p_out, p_in)
+
+
+def folded_rot_flops(p_out, p_in):
+    """Flops of the two rotations after folding the orders +-m (rcr_tiles.cu):
+    (n+1)^2 + n^2 real-by-complex MACs of 4 per degree.  Every kernel form
+    runs the folded rotations (the composed one a single dense product)."""
+    return 4.0 * (sum((n + 1) ** 2 + n ** 2 for n in range(p_in)) + sum((n + 1) ** 2 + n ** 2 for n in range(p_out)))
+
+
+def folded_rcr_flops(p_out, p_in):
+    """Flops of one RCR translation with folded rotations."""
+    return folded_rot_flops(p_out, p_in) + coax_flops(p_out, p_in)
 
 
 # double-FP32 multiply-accumulate: 12 FP32-pipe operations (df.cuh)
@@ -331,7 +342,7 @@ def m2l_levels(tune, p, pairs):
             form, ms = "tiles", t["m2l_rcr"]
         if ms is None:
             continue
-        out[l] = (form, ms, float(pairs[l]) * rcr_flops(int(p[l]), int(p[l])))
+        out[l] = (form, ms, float(pairs[l]) * folded_rcr_flops(int(p[l]), int(p[l])))
     return out
 
 
@@ -374,7 +385,7 @@ def roofline(fb, P, iters, true_mv, pk, fp32_peak, fp64_peak):
         p = fb.fb_operator_info(P[op])[2]
         for l, d in fb.fb_operator_staged_pass_times(P[op]).items():
             pl, npair = int(p[l]), float(pairs[l])
-            rot, cox = npair * rot_flops(pl, pl), npair * coax_flops(pl, pl)
+            rot, cox = npair * folded_rot_flops(pl, pl), npair * coax_flops(pl, pl)
             cw = 16 if prec == "f32" else 32   # bytes per complex coefficient read + written
             if d["form"] == "df":
                 add("k_stg<df>", "df", key, l, count, d["rot"] + d["coax"] + d["back"], rot + cox)
@@ -411,11 +422,12 @@ def roofline(fb, P, iters, true_mv, pk, fp32_peak, fp64_peak):
     if d["unit"] == "TB/s":
         work = "algorithmic bytes per box pair: 16 B per complex coefficient read and written (32 B in FP64)"
     elif dom in ("k_stg_tc", "k_stg_rot+back<float>"):
-        work = "algorithmic flops per box pair: rotations 8 x 2 sum_{n<p}(2n+1)^2 (unfolded count)"
+        work = "algorithmic flops per box pair: folded rotations 4 x 2 sum_{n<p}((n+1)^2 + n^2)"
     elif dom in ("k_stc_coax", "k_stg_coax<float>"):
         work = "algorithmic flops per box pair: coaxial step 8 x sum_m (p-|m|)^2"
     else:
-        work = "algorithmic flops per box pair: rotations 8 x 2 sum_{n<p}(2n+1)^2 + coaxial 8 x sum_m (p-|m|)^2"
+        work = ("algorithmic flops per box pair: folded rotations 4 x 2 sum_{n<p}((n+1)^2 + n^2) "
+                "+ coaxial 8 x sum_m (p-|m|)^2")
     rf = {"kernel": dom, "bound": d["bound"], "achieved": d["achieved"], "peak": d["peak"], "unit": d["unit"],
           "frac": d["frac"], "traffic": traffic_for(dom), "peak_kind": d["peak_kind"], "what": d["what"],
           "est_ms_per_step": d["est_ms_per_step"],

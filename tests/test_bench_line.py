@@ -29,3 +29,17 @@ def test_tuning_summary_is_small_and_complete():
             assert {k: v for k, v in s[op][l].items() if k != "choice"} == {
                 k: round(v, 3) for k, v in t.items() if k in TIMES and v is not None}
     assert len(json.dumps(s)) < 5000 < len(json.dumps(tune))
+
+
+def test_folded_rotation_counts():
+    """(n+1)^2 + n^2 = ((2n+1)^2 + 1) / 2: p (2p-1)(2p+1)/6 + p/2 over the degrees below p, 4 flops each."""
+    for p in (1, 2, 12, 89, 159):
+        assert bench.folded_rot_flops(p, p) == 4.0 * (p * (2 * p - 1) * (2 * p + 1) / 3 + p)
+        assert bench.folded_rcr_flops(p, p) == bench.folded_rot_flops(p, p) + bench.coax_flops(p, p)
+    assert bench.folded_rot_flops(5, 3) == 4.0 * ((1 + 5 + 13) + (1 + 5 + 13 + 25 + 41))
+
+
+def test_rooflines_count_what_the_kernels_execute():
+    tune = {6: {"choice": 256, "m2l_tiles_df": 2.0, "m2l_rcr": 3.0, "m2l_tensor": None}}
+    form, ms, flops = bench.m2l_levels(tune, [0] * 6 + [12], [0] * 6 + [1000])[6]
+    assert (form, ms, flops) == ("tiles_df", 2.0, 1000.0 * bench.folded_rcr_flops(12, 12))
