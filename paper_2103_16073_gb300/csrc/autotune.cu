@@ -10,7 +10,7 @@
 //     arithmetic (as are the FP64 per-pair tiles),
 //   * mixed precision only: the stacked tensor-core GEMM of composed
 //     matrices (3xTF32),
-// for M2L and for the M2M / L2L passes into that level.  The tensor-core
+// for M2L and for the M2M / L2L passes into that level.  The composed
 // candidate of an M2L level is skipped when its order exceeds 20, when it
 // has fewer than 16 box pairs per translation vector on average, or when
 // its composed matrices would exceed a memory cap.  The result replaces the
@@ -56,17 +56,37 @@ fb_status time_ms(F&& f, cudaStream_t s, int reps, double* out) {
 
 void free_rcr(RcrPlan& p) { fb_rcr_free(p); }
 
-// Candidates worth timing (measured crossovers on GB300: per-pair tiles lose
-// to the staged passes from order ~40 on and by ~5x at 89; the staged passes
-// lose below order ~30, where a level's coefficient blocks are small).  A
-// level always keeps at least one candidate.
+// Candidates worth timing.  M2L in ms of a level of 8,928 box pairs (composed
+// matrices also of 113,472), the level above it included and the same for all
+// forms of a line:
+//   FP32  order   tiles  staged  rot. tc  rot.+coax. tc  composed | tiles  composed
+//          8      0.056   0.154    0.121     0.098         0.060  | 0.396    0.331
+//         16      0.113   0.283    0.201     0.146         0.184  | 1.024    0.907
+//         20      0.160   0.408    0.275     0.195         0.330  | 1.448    1.442
+//         24      0.295   0.582    0.397     0.289         0.641  | 3.288    3.690
+//         32      0.428   0.801    0.512     0.346         1.686  |
+//         48      1.18    1.46     0.84      0.53                 |
+//         56      2.00    1.99     1.17      0.76                 |
+//         80      6.56    4.11     2.22      1.19                 |
+//   FP64  order   tiles  staged  df tiles  df staged
+//         16       1.96    5.71     1.73      3.04
+//         32      11.0    20.0      8.84     12.0
+//         48      20.3    34.0     13.4      18.1
+//         64      50.2    61.5     33.2      35.4
+//         72      77.5    83.3     54.8      44.7
+//         80     105     111       71.8      59.3
+// So tiles lead up to order 24 in FP32 (then the tensor-core passes; the
+// CUDA-core ones cross tiles at 56), as long as they fit in FP64 and up to 64
+// in double-FP32; composed matrices from some 100,000 pairs a level to order
+// 20.  The lines below leave the losers of both sides out with room to spare,
+// but for FP64 tiles of orders 60 to 80, which lead by a few percent.  A level
+// always keeps at least one candidate.
 bool rcr_tile_candidate(int p, size_t csz) { return fb_rcr_tile_fits(p, p, csz) && p < 60; }
 bool rcr_staged_candidate(int p, size_t csz) { return p >= 24 || !rcr_tile_candidate(p, csz); }
-// double-FP32 passes: their arithmetic runs several times faster than FP64,
-// which moves the crossover with the FP64 tiles to lower orders
+// double-FP32 passes: ahead of the FP64 passes at every order
 bool rcr_df_candidate(int p) { return p >= 16; }
-// staged passes with tensor-core rotations: their degree blocks pack into
-// one tile up to 256 columns, so low orders stay worth timing
+// staged passes with tensor-core rotations: behind the tiles below order 24,
+// ahead of composed matrices on levels of few pairs
 bool rcr_stc_candidate(int p) { return p >= 12; }
 
 }  // namespace

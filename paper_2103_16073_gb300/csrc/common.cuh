@@ -284,9 +284,12 @@ struct RcrTables {
 // Large orders run as staged batched GEMM passes (rcr_staged.cu) instead of
 // per-pair tiles: a pair's rotation and coaxial blocks must then be shared
 // by many pairs to be read at a useful rate.  By default a level is staged
-// from order FB_STG_PMIN on, and always when a pair's working set
-// (p_in^2 + max(p_in, p_out)^2 coefficients) exceeds what one CTA's shared
-// memory holds; the autotuner and fb_operator_set_forms choose per level.
+// from order FB_STG_PMIN on, and always when a tile of one column does not
+// fit one CTA's shared memory (fb_rcr_tile_fits); the autotuner and
+// fb_operator_set_forms choose per level.  The line was set with an earlier
+// tile kernel: the present one is ahead of the CUDA-core passes up to order 56
+// in FP32 (0.72 against 1.11 ms at 40) and as long as it fits in FP64 (table
+// in autotune.cu), so programs that neither tune nor restore forms lose there.
 constexpr int FB_STG_PMIN = 40;
 bool fb_rcr_tile_fits(int p_in, int p_out, size_t csize);
 int fb_rcr_default_staged(int p_in, int p_out, size_t csize);
