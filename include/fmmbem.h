@@ -381,9 +381,9 @@ FB_API fb_status fb_precond_use_graphs(fb_precond* pc, int enable);
  *     arithmetic,
  *   - mixed precision only: the stacked tensor-core GEMM of composed
  *     matrices (3xTF32).
- * Tiles are timed below order 60, the staged passes from order 24 on, with tensor-core rotations from order
- * 12 on, in double-FP32 from order 16 on; a level keeps at least one
- * candidate.
+ * Tiles are timed below order 60, the staged passes from order 24 on, with
+ * tensor-core rotations from order 12 on, in double-FP32 from order 16 on; a
+ * level keeps at least one candidate.
  * times: FB_TUNE_TIMES*13 doubles or NULL, times[FB_TUNE_TIMES l + 0..13] =
  * M2L RCR tiles, M2L tensor, M2M+L2L RCR tiles, M2M+L2L tensor, M2L RCR
  * staged, M2M+L2L RCR staged, M2L RCR staged with tensor-core rotations,

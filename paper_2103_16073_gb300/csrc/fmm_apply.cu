@@ -3,10 +3,13 @@
 // for the plain FP64 path, float for the mixed path); input and output
 // vectors are complex128 in the caller's element order.
 //
-// Translations use the stacked form: all box pairs of one level that share a
-// translation vector share one p^2 x p^2 matrix, so each (level, offset)
-// group is one complex GEMM  Y = T X  with X gathered from the source boxes
-// and Y scatter-added into the target boxes.
+// Translations run per level in the form chosen for it: per-pair tiles
+// (rcr_tiles.cu), staged passes (rcr_staged.cu, rcr_staged_tc.cu) or composed
+// matrices on the tensor cores (trans_tc.cu).  k_trans below is the composed
+// form on CUDA cores (FB_TRANS_COMPOSED): all box pairs of one level that share
+// a translation vector share one p^2 x p^2 matrix, so each (level, offset)
+// group is one complex GEMM  Y = T X  with X gathered from the source boxes and
+// Y scatter-added into the target boxes.
 #include <algorithm>
 #include <mutex>
 #include <string>

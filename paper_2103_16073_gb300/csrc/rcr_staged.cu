@@ -779,11 +779,7 @@ fb_status fb_stg_df_tables(fb_op* op, cudaStream_t s) {
     return FB_OK;
 }
 
-// Runs the staged passes of a plan for nrhs right-hand sides (set r of the
-// expansions at src / dst + r * rstride), one level and as many right-hand
-// sides at a time as the staging buffers hold (nb, ustride apart): pre-pass (src -> V), rotation (V -> U), coaxial (U -> V),
-// back-rotation (V -> dst).
-// right-hand sides of one launch
+// right-hand sides of one launch, their expansions and staging buffers apart
 struct StgRhs {
     int n;
     int64_t rstride, ustride;
@@ -866,6 +862,10 @@ static fb_status stg_level(const StgLevel& lv, int pass_mask, const R* rf, int64
     return FB_OK;
 }
 
+// Runs the staged passes of a plan for nrhs right-hand sides (set r of the
+// expansions at src / dst + r * rstride), one level and nb right-hand sides at
+// a time (their staging buffers ustride apart): pre-pass (src -> V), rotation
+// (V -> U), coaxial (U -> V), back-rotation (V -> dst).
 template <class R>
 static fb_status stg_run(void* plan, const R* rf, int64_t fper, const cx<R>* rph, int prot, const cx<R>* coax,
                          const cx<R>* src, cx<R>* dst, cx<R>* U, cx<R>* V, cudaStream_t s, int nrhs, int64_t rstride,
