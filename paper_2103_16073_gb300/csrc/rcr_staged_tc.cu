@@ -38,8 +38,8 @@
 //                added (atomics) in runs of one target's coefficients;
 //   warps 18-19  items and their slots into a ring in shared memory, ahead of
 //                the others.
-// Room of 240 leaf boxes at 7.5 kHz (orders 116 and 66, M2L): R 0.44 ms, C
-// 0.34 ms, B 0.46 ms over both levels; together 3.34 ms with one tile per
+// Room of 240 leaf boxes at 7.5 kHz (orders 116 and 66, M2L): R 0.45 ms, C
+// 0.34 ms, B 0.47 ms over both levels; together 3.34 ms with one tile per
 // CTA, degree-major u and v, and lanes along a row's K values.  C moves 1 GB
 // per pass out of L2 at 6 TB/s; R and B are bound by their warps' issue rate
 // around the waits of a chunk.
