@@ -52,9 +52,9 @@ def test_asynchronous_statements_order_memory(path):
             assert "tcgen05.wait::ld" in s, s
 
 
-def test_no_load_is_multicast():
-    """The kernels also run with one rank per GPU, where loads stay within a
-    CTA: none names the multicast form."""
-    for p in FILES:
-        for s in statements(open(p).read()):
-            assert "multicast" not in s, (p, s)
+def test_bulk_copies_stay_within_a_cta():
+    """The kernels also run with one rank per GPU, where a copy goes to the
+    CTA that issues it: the plain form, without a mask of further CTAs."""
+    plain = re.compile(r"cp\.async\.bulk\.shared::cluster\.global\.mbarrier::complete_tx::bytes \[%0\], \[%1\], %2, \[%3\];")
+    copies = [s for p in FILES for s in statements(open(p).read()) if "cp.async.bulk" in s]
+    assert copies and all(plain.search(s) for s in copies)
